@@ -392,7 +392,7 @@ im_status im_graph_create(const int64_t *in_off, const int32_t *in_src, const ui
 im_status im_graph_destroy(im_graph *g) {
     if (!g) return IM_ERR_INVALID_ARG;
     DeviceGuard dg(g->device);
-    for (void *b : {(void *)g->in_off, (void *)g->in_src, (void *)g->w, (void *)g->lt_vrec,
+    for (void *b : {(void *)g->in_off, (void *)g->in_src, (void *)g->w, (void *)g->ic_rec, (void *)g->lt_vrec,
                     (void *)g->lt_leaf, (void *)g->lt_tree, (void *)g->lt_guide,
                     (void *)g->out_off, (void *)g->out_rec})
         cudaFree(b);

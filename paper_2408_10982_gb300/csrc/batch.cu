@@ -344,6 +344,8 @@ im_status im_solve_batch(im_batch *b, const im_query *qs, int32_t nq, int32_t km
                 set_error("im_solve_batch: LT query on a graph whose in-weights exceed 1");
                 return IM_ERR_INVALID_ARG;
             }
+        } else {
+            IM_TRY(build_ic_index(const_cast<im_graph *>(Q.graph), st));
         }
         n_total += Q.graph->n;
         sets_total += Q.theta;

@@ -193,6 +193,7 @@ struct QueryView {
     const int64_t *in_off;
     const int32_t *in_src;
     const uint32_t *w;
+    const uint4 *ic_rec;
     const uint4 *lt_vrec;
     const unsigned long long *lt_leaf;
     const unsigned long long *lt_tree;
@@ -211,6 +212,8 @@ struct im_graph {
     int64_t *in_off;     // [n+1]
     int32_t *in_src;     // [m]
     uint32_t *w;         // [m], 16-byte aligned
+    uint4 *ic_rec;       // [n] {first in-edge, in-degree, common weight, 1 if all in-edges have it};
+                         // built on first IC use
     // LT search index, built on first LT use: per-vertex records, per-edge
     // leaves (running weight sum << 31 | source) and upper tree levels
     uint4 *lt_vrec;                  // [n] {edge offset, in-degree, tree offset | levels << 28, equal in-weight or 0}
@@ -397,6 +400,7 @@ QueryView query_view(const im_graph *g, uint64_t seed, uint64_t first);
 im_status sample_append(const im_graph *g, im_model model, uint64_t seed, uint64_t first,
                         uint64_t count, im_pool *pool, cudaStream_t st);
 im_status build_lt_index(im_graph *g, cudaStream_t st);
+im_status build_ic_index(im_graph *g, cudaStream_t st);
 
 // index.cu
 im_status build_index(im_pool *p, cudaStream_t st);

@@ -4,10 +4,9 @@
 // Every sampler is a persistent kernel that takes the next sample id from a
 // global counter (dynamic balancing: set sizes are heavy tailed on R-MAT).
 // IC (Def. 3 under the IC live-edge world): one warp per sample expands up to
-// 32 queued vertices at once; their in-edge ranges are split into aligned
-// groups of four edges, so each lane makes one Philox call (four coins) and
-// one 16-byte load of weights and one of sources per group.  Sets longer than
-// the warp's queue are re-run by k_sample_ic_big, one block per sample.  LT:
+// 32 queued vertices at once, four coins to a Philox call; live edges are
+// listed and followed 32 at a time.  Sets that percolate, or outgrow the warp's
+// queue, are finished by k_sample_ic_big, one block per sample.  LT:
 // k_sample_lt1 (default) runs one walk per thread; the picked in-edge (first
 // edge whose running weight sum exceeds the draw) comes from one division when
 // the vertex's in-edges weigh the same, else from a cut-point table in O(1)
@@ -31,14 +30,22 @@ namespace {
 
 constexpr int kSampleThreads = 256;          // 8 warps per block
 constexpr int kWarps = kSampleThreads / 32;
-constexpr int64_t kSmemVisBits = 1 << 16;    // visited bitmap in smem when n <= this
+constexpr int64_t kSmemVisBits = 1 << 15;    // IC visited bitmap in shared memory when n <= this
 constexpr int kPathSmem = 256;               // LT path entries mirrored in smem (warp walks)
 constexpr int kPathSmemGroup = 64;           // ... per walk when a warp runs several walks
 constexpr int64_t kQueueCapIC = 1 << 14;     // per-warp queue entries (first pass)
 constexpr int64_t kQueueCapLT = 1 << 11;
-constexpr int kICU = 2;                      // IC edge groups per lane in flight
 constexpr int kWarpSortBytes = 4096;         // per-warp smem sort buffer
 constexpr int kBlockSortCap = 16384;         // ... by one block in shared memory (int32)
+
+// An IC sample that a warp gave up: its members so far are hand[off .. off +
+// tail), of which the first `head` are expanded (examined in-edges so far);
+// off < 0: start again from the root.
+struct Handed {
+    int64_t off;
+    unsigned long long examined;
+    int32_t head, tail;
+};
 
 struct SampleArgs {
     const QueryView *qv;      // [nq] graphs and streams of the queries of this launch
@@ -61,6 +68,11 @@ struct SampleArgs {
     int64_t *ovf_list;
     unsigned long long *ovf_count;
     int *status;
+    struct Handed *handed;    // [count] state of the samples in ovf_list (IC)
+    int32_t *hand;            // their members
+    int64_t hand_cap;
+    unsigned long long *hand_cursor;
+    uint32_t rk[20];          // Philox round keys of the launch's query, when it has only one
 };
 
 // The query that flattened sample index j belongs to (largest q, qstart[q] <= j).
@@ -74,187 +86,432 @@ __device__ __forceinline__ int find_query(const SampleArgs &a, int64_t j) {
     return lo;
 }
 
-__device__ __forceinline__ int64_t next_item(const SampleArgs &a, int lane) {
-    unsigned long long j = 0;
-    if (lane == 0) j = atomicAdd(a.work, 1ull);
-    j = __shfl_sync(kFull, j, 0);
-    if (j >= (unsigned long long)a.count) return -1;
-    return a.list ? a.list[j] : (int64_t)j;
-}
-
-// Move the finished set q[0..len) to the stage and record where it went.
-__device__ __forceinline__ void emit_set(const SampleArgs &a, int64_t j, const int32_t *q,
-                                         int64_t len, int lane) {
-    unsigned long long pos = 0;
-    if (lane == 0) pos = atomicAdd(a.stage_cursor, (unsigned long long)len);
-    pos = __shfl_sync(kFull, pos, 0);
-    if ((int64_t)pos + len > a.stage_cap) {
-        if (lane == 0) {
-            raise_status(a.status, kDevStageOverflow);
-            a.sizes[j] = 0;
-            a.stage_off[j] = 0;
-        }
-        return;
-    }
-    for (int64_t i = lane; i < len; i += 32) a.stage[pos + i] = q[i];
-    if (lane == 0) {
-        a.stage_off[j] = (int64_t)pos;
-        a.sizes[j] = (int32_t)len;
-    }
-}
-
-__device__ __forceinline__ void mark_overflow(const SampleArgs &a, int64_t j, int lane) {
-    if (lane == 0) {
-        a.sizes[j] = -1;
-        a.stage_off[j] = 0;
-        unsigned long long at = atomicAdd(a.ovf_count, 1ull);
-        a.ovf_list[at] = j;
-    }
-}
 
 // ---------------------------------------------------------------------------
 // IC: stochastic reverse BFS.  Edge e of sample s is live iff lane (e & 3) of
 // Philox(s, e >> 2 (low word), e >> 34, coin tag) is below w[e].
+//
+// The bound is the coins: every in-edge of every member takes one, four to a
+// Philox call, so the kernels are built around an inner loop that is little
+// more than the ten rounds.  Three things keep it that small.
+//   - m < 2^31, so the counter's third word is 0 and the first word is the
+//     sample id: of the first three rounds only two products depend on the
+//     edge (CoinStream), the rest is computed once a sample.
+//   - A vertex whose in-edges all weigh the same (weighted cascade, uniform p)
+//     takes its threshold from its record (im_graph.ic_rec): no weights are
+//     read at all.  Sources are read only for live edges.
+//   - Live edges are rare (a few per hundred, or per ten thousand under
+//     weighted cascade).  The loop only lists them, in shared memory; when a
+//     warp has 32, its lanes take one each: source, visited test, append.
+//     So the long-latency part (source load, bitmap atomic) runs with 32
+//     lanes busy and once per 32 live edges, not inside the coin loop.
+// A warp expands up to 32 queued vertices together: those with at least
+// kICWide edge groups one after another on all lanes (no search for an edge's
+// owner), the short lists packed.
+// Measured against one lane loop that loaded weights and sources with every
+// group and claimed live sources where it found them: weighted cascade on the
+// LiveJournal shape (IMM, 1.6 x 10^11 coins) 597 -> 139 ms, U[0, 0.1] at scale
+// 20 (9.8 x 10^9 coins) 55 -> 24.5 ms, trivalency on the LiveJournal shape
+// (6.3 x 10^9) 45 -> 20.7 ms.  ncu, weighted cascade at scale 15: 141
+// instructions per 128 coins, issue 71 % and ALU and FMA-heavy pipes 62 % busy
+// while DRAM is idle, so what is left is the instructions of the coins.  Tried
+// and not kept: one call site for all kinds of lists (a state machine; fewer
+// instruction-fetch stalls, more instructions: 31.5 against 23.5 ms at scale
+// 20); lists from 12 groups on for the whole warp (26.1 against 23.5 ms).
 // ---------------------------------------------------------------------------
-template <bool kSmemVis>
-__global__ void __launch_bounds__(kSampleThreads, 4) k_sample_ic(SampleArgs a) {
-    extern __shared__ uint32_t smem_vis[];
+constexpr int kICWide = 24;                  // edge groups from which a vertex gets the whole warp
+constexpr int kCandCap = 32 + 128;           // listed live edges of a warp: < 32 left over + 128 new
+constexpr int kICQueueSmem = 384;            // queue entries of a warp in shared memory
+constexpr int kICHash = 1024;                // visited-set slots of a warp (n > kSmemVisBits)
+constexpr int kICHashMax = kICQueueSmem;              // members from which the visited set spills to a bitmap
+// A warp leaves a sample to the second pass when it has expanded this many
+// in-edges and this many members wait to be expanded.
+constexpr uint32_t kICWideEdges = 1u << 16;
+constexpr int32_t kICWarpFront = 1024;
+constexpr int64_t kICHandCap = 1 << 23;      // members handed over to the second pass (32 MB)
+
+// The coins of one sample: Philox4x32-10 of counter (s, g, 0, coin tag), with
+// what does not depend on g computed by begin().  KEYS: the round keys come
+// from rk (kernel parameters, so constant-bank operands); else they are
+// derived from k0, k1 as the rounds go.
+template <bool KEYS>
+struct CoinStream {
+    uint32_t k0, k1;
+    uint32_t gx, c1, ca, cb, cc;
+    __device__ __forceinline__ uint32_t K0(const uint32_t *rk, int r) const {
+        return KEYS ? rk[2 * r] : k0 + (uint32_t)r * 0x9E3779B9u;
+    }
+    __device__ __forceinline__ uint32_t K1(const uint32_t *rk, int r) const {
+        return KEYS ? rk[2 * r + 1] : k1 + (uint32_t)r * 0xBB67AE85u;
+    }
+    __device__ __forceinline__ void begin(const uint32_t *rk, uint32_t s, uint32_t key0,
+                                          uint32_t key1) {
+        k0 = key0;
+        k1 = key1;
+        gx = K0(rk, 0);                                           // round 0: x = g ^ gx
+        const uint32_t z1 = __umulhi(0xD2511F53u, s) ^ kStreamCoin ^ K1(rk, 0);
+        c1 = (0xD2511F53u * s) ^ K1(rk, 1);                       // round 1: z = hi(a) ^ c1
+        const uint32_t x2 = __umulhi(0xCD9E8D57u, z1) ^ K0(rk, 1);
+        ca = (0xCD9E8D57u * z1) ^ K0(rk, 2);                      // round 2: x = hi(b) ^ ca
+        cb = __umulhi(0xD2511F53u, x2) ^ K1(rk, 2);               //          z = lo(a) ^ cb
+        cc = (0xD2511F53u * x2) ^ K1(rk, 3);                      // round 3: z = hi(a) ^ cc
+    }
+    __device__ __forceinline__ uint4 operator()(const uint32_t *rk, uint32_t g) const {
+        auto wide = [](uint32_t m, uint32_t x, uint32_t &lo, uint32_t &hi) {
+            const unsigned long long p = (unsigned long long)m * x;
+            lo = (uint32_t)p;
+            hi = (uint32_t)(p >> 32);
+        };
+        uint32_t al, ah, bl, bh, dl, dh, el, eh;
+        wide(0xD2511F53u, g ^ gx, al, ah);
+        wide(0xCD9E8D57u, ah ^ c1, bl, bh);
+        wide(0xD2511F53u, bh ^ ca, dl, dh);
+        wide(0xCD9E8D57u, al ^ cb, el, eh);
+        uint4 x = make_uint4(eh ^ bl ^ K0(rk, 3), el, dh ^ cc, dl);
+#pragma unroll
+        for (int r = 4; r < 10; ++r) {
+            wide(0xD2511F53u, x.x, al, ah);
+            wide(0xCD9E8D57u, x.z, bl, bh);
+            x = make_uint4(bh ^ x.y ^ K0(rk, r), bl, ah ^ x.w ^ K1(rk, r), al);
+        }
+        return x;
+    }
+};
+
+// What a warp expands: the in-edge lists of up to 32 vertices, one per lane.
+struct ICItem {
+    uint32_t eb, ee;     // in-edges [eb, ee)
+    uint32_t w;          // their common threshold, when equal
+    uint32_t equal;      // 1: all in-edges weigh w
+};
+
+__device__ __forceinline__ ICItem ic_item(const uint4 *rec, uint32_t v) {
+    const uint4 r = __ldg(rec + v);
+    return ICItem{r.x, r.x + r.y, r.z, r.w};
+}
+
+// Edge groups (of four, aligned) of an item; 0 when no in-edge can be live.
+__device__ __forceinline__ uint32_t ic_groups(const ICItem &it) {
+    if (it.ee == it.eb || (it.equal && it.w == 0u)) return 0u;
+    return ((it.ee - 1u) >> 2) - (it.eb >> 2) + 1u;
+}
+
+// Live edges of group g within [eb, ee), as four bits, from its coins c and
+// thresholds wv.
+__device__ __forceinline__ uint32_t ic_live(const uint4 c, const uint4 wv, uint32_t g, uint32_t eb,
+                                            uint32_t ee) {
+    uint32_t m = (c.x < wv.x ? 1u : 0u) | (c.y < wv.y ? 2u : 0u) | (c.z < wv.z ? 4u : 0u) |
+                 (c.w < wv.w ? 8u : 0u);
+    const uint32_t e0 = g << 2;
+    if (e0 < eb) m &= 15u << (eb - e0);                // first group
+    if (e0 + 4u > ee) m &= 15u >> (e0 + 4u - ee);      // last group
+    return m;
+}
+
+// Lists the live edges of the warp's groups (bits m of the group starting at
+// edge e0) after the ncand listed before.
+__device__ __forceinline__ void ic_list(uint32_t m, uint32_t e0, uint32_t *cand, int &ncand,
+                                        int lane) {
+    const unsigned lt = (1u << lane) - 1u;
+#pragma unroll
+    for (int c = 0; c < 4; ++c) {
+        const unsigned b = __ballot_sync(kFull, m >> c & 1u);
+        if (m >> c & 1u) cand[ncand + __popc(b & lt)] = e0 + c;
+        ncand += __popc(b);
+    }
+}
+
+// Calls visit(m, e0) for the groups with a live edge among groups [t0, n) of
+// one in-list.  Equal weights: pairs of groups per lane, and the smallest coin
+// of the warp's 64 groups decides whether any edge is live; the bits, and what
+// lies outside the list in its first and last group, are looked at only then.
+// Unequal weights: the next groups' are loaded while these are tested.
+template <bool KEYS, typename F>
+__device__ __forceinline__ void ic_expand_wide(const CoinStream<KEYS> &cs, const uint32_t *rk,
+                                               const uint32_t *wgt, const ICItem &o, uint32_t t0,
+                                               uint32_t n, int lane, F &&visit) {
+    const uint32_t g0 = o.eb >> 2;
+    if (o.equal) {
+        while (n - t0 >= 64u) {
+            const uint32_t g = g0 + t0 + lane;
+            const uint4 c0 = cs(rk, g), c1 = cs(rk, g + 32u);
+            t0 += 64u;
+            const uint32_t least = min(min(min(c0.x, c0.y), min(c0.z, c0.w)),
+                                       min(min(c1.x, c1.y), min(c1.z, c1.w)));
+            if (__any_sync(kFull, least < o.w)) {
+                const uint4 wv = make_uint4(o.w, o.w, o.w, o.w);
+                uint32_t m = ic_live(c0, wv, g, o.eb, o.ee), e0 = g << 2;
+                uint32_t m1 = ic_live(c1, wv, g + 32u, o.eb, o.ee);
+#pragma unroll 1
+                for (int u = 0; u < 2; ++u) {
+                    if (__any_sync(kFull, m)) visit(m, e0);
+                    m = m1;
+                    e0 += 128u;
+                }
+            }
+        }
+    }
+    if (t0 >= n) return;
+    uint4 wv = make_uint4(o.w, o.w, o.w, o.w);
+    const uint4 *wp = reinterpret_cast<const uint4 *>(wgt) + g0 + lane;
+    if (!o.equal && t0 + lane < n) wv = __ldg(wp + t0);
+#pragma unroll 1
+    for (; t0 < n; t0 += 32u) {
+        const uint32_t g = g0 + t0 + lane;
+        uint4 wn = wv;
+        if (!o.equal && t0 + 32u + lane < n) wn = __ldg(wp + t0 + 32u);
+        const uint4 c = cs(rk, g);
+        uint32_t m = 0;
+        if (t0 + lane < n) m = ic_live(c, wv, g, o.eb, o.ee);
+        if (__any_sync(kFull, m)) visit(m, g << 2);
+        wv = wn;
+    }
+}
+
+// The same for the lists of a warp's lanes (ng groups in this lane's): those of
+// at least kICWide groups one after another on all lanes, the others packed.
+template <bool KEYS, typename F>
+__device__ __forceinline__ void ic_expand(const CoinStream<KEYS> &cs, const uint32_t *rk,
+                                          const uint32_t *wgt, const ICItem &it, uint32_t ng,
+                                          int lane, F &&visit) {
+    unsigned wide = __ballot_sync(kFull, ng >= (uint32_t)kICWide);
+    while (wide) {
+        const int l = __ffs(wide) - 1;
+        wide &= wide - 1u;
+        const ICItem o{__shfl_sync(kFull, it.eb, l), __shfl_sync(kFull, it.ee, l),
+                       __shfl_sync(kFull, it.w, l), __shfl_sync(kFull, it.equal, l)};
+        ic_expand_wide<KEYS>(cs, rk, wgt, o, 0u, __shfl_sync(kFull, ng, l), lane, visit);
+    }
+    const uint32_t ns = ng >= (uint32_t)kICWide ? 0u : ng;
+    const uint32_t incl = warp_incl_scan<uint32_t>(ns, lane);
+    const uint32_t total = __shfl_sync(kFull, incl, 31);
+#pragma unroll 1
+    for (uint32_t t0 = 0; t0 < total; t0 += 32) {
+        const uint32_t t = t0 + lane;
+        int owner = 0;                       // first lane whose inclusive count exceeds t
+#pragma unroll
+        for (int step = 16; step > 0; step >>= 1)
+            if (__shfl_sync(kFull, incl, owner + step - 1) <= t) owner += step;
+        const uint32_t before = __shfl_sync(kFull, incl - ns, owner);
+        const uint32_t eb = __shfl_sync(kFull, it.eb, owner);
+        const uint32_t ee = __shfl_sync(kFull, it.ee, owner);
+        const uint32_t w = __shfl_sync(kFull, it.w, owner);
+        const bool equal = __shfl_sync(kFull, it.equal, owner) != 0u;
+        const uint32_t g = (eb >> 2) + (t - before);
+        uint4 wv = make_uint4(w, w, w, w);
+        if (!equal && t < total) wv = __ldg(reinterpret_cast<const uint4 *>(wgt) + g);
+        const uint4 c = cs(rk, g);
+        uint32_t m = 0;
+        if (t < total) m = ic_live(c, wv, g, eb, ee);
+        if (__any_sync(kFull, m)) visit(m, g << 2);
+    }
+}
+
+__device__ __forceinline__ uint32_t ic_hash(uint32_t u) {
+    return (u * 0x9E3779B1u) >> (32 - 10);
+}
+static_assert(kICHash == 1 << 10, "ic_hash gives a slot of kICHash");
+
+// One warp per sample.  BITS: the visited set is an n-bit bitmap in shared
+// memory (n <= kSmemVisBits).  Otherwise it is a hash set of kICHash slots in
+// shared memory -- an RRR set of a large graph is mostly a few dozen members,
+// and a bitmap of its own in global memory would cost a DRAM access per probe
+// -- which moves to the warp's bitmap in global memory (cleared by the warp on
+// its first use, and kept clear) when the set passes kICHashMax members.
+// Shared memory of a warp: visited words, kICQueueSmem queue entries (later
+// entries in global memory), kCandCap listed edges.  Three blocks an SM with
+// the round keys in the arguments (80 registers; four blocks at 64 measured 4 %
+// slower), four without (three: 3 % slower on the batched mix).
+template <bool BITS, bool KEYS>
+__global__ void __launch_bounds__(kSampleThreads, KEYS ? 3 : 4) k_sample_ic(const __grid_constant__ SampleArgs a) {
+    extern __shared__ uint32_t ic_smem[];
     const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
+    const unsigned lt = (1u << lane) - 1u;
     const int64_t gw = (int64_t)blockIdx.x * kWarps + wib;
-    uint32_t *vis = kSmemVis ? smem_vis + (size_t)wib * a.vis_words
-                             : a.gvis + (size_t)gw * (size_t)a.vis_words;
+    const int svis = BITS ? (int)((a.vis_words + 3) & ~(int64_t)3) : kICHash;
+    uint32_t *vis = ic_smem + (size_t)wib * (svis + kICQueueSmem + kCandCap);
+    int32_t *sq = reinterpret_cast<int32_t *>(vis + svis);
+    uint32_t *cand = reinterpret_cast<uint32_t *>(sq + kICQueueSmem);
+    uint32_t *gvis = BITS ? nullptr : a.gvis + (size_t)gw * (size_t)a.vis_words;
     int32_t *q = a.queues + (size_t)gw * (size_t)a.qcap;
-    if (kSmemVis)
-        for (int64_t i = lane; i < a.vis_words; i += 32) vis[i] = 0;
+    constexpr uint32_t kClear = BITS ? 0u : 0xffffffffu;
+    for (int i = lane; i < svis; i += 32) vis[i] = kClear;
     __syncwarp();
+    bool gclear = false;                     // the global bitmap has been cleared
     unsigned long long exam = 0, abytes = 0;
+    // the next sample index is taken while this one's set is built
+    unsigned long long jn = 0;
+    if (lane == 0) jn = atomicAdd(a.work, 1ull);
     for (;;) {
-        const int64_t j = next_item(a, lane);
-        if (j < 0) break;
-        const int qi = find_query(a, j);
+        const unsigned long long jw = __shfl_sync(kFull, jn, 0);
+        if (jw >= (unsigned long long)a.count) break;
+        if (lane == 0) jn = atomicAdd(a.work, 1ull);
+        const int64_t j = a.list ? a.list[jw] : (int64_t)jw;
+        const int qi = a.nq == 1 ? 0 : find_query(a, j);
         const QueryView &V = a.qv[qi];
-        const int64_t *in_off = V.in_off;
+        const uint4 *rec = V.ic_rec;
         const int32_t *in_src = V.in_src;
         const uint32_t *wgt = V.w;
         const uint64_t seed = V.seed;
-        const uint32_t k0 = seed_lo(seed), k1 = seed_hi(seed);
         const uint32_t s = V.first + (uint32_t)(j - __ldg(a.qstart + qi));
         const uint32_t root = rrr_root(seed, s, V.n);
+        CoinStream<KEYS> cs;
+        cs.begin(a.rk, s, seed_lo(seed), seed_hi(seed));
+        int32_t head = 0, tail = 1;
+        int ncand = 0;
+        bool spilled = false, lost = false;
+        uint32_t work = 0;                   // in-edges of the expanded members (saturating)
+        unsigned long long sexam = 0;
         if (lane == 0) {
-            atomicOr(&vis[root >> 5], 1u << (root & 31));
-            q[0] = (int32_t)root;
+            if (BITS) vis[root >> 5] |= 1u << (root & 31);
+            else vis[ic_hash(root)] = root;
+            sq[0] = (int32_t)root;
         }
         __syncwarp();
-        int64_t head = 0, tail = 1;
-        bool overflow = false;
-        unsigned long long sexam = 0;
-        while (head < tail && !overflow) {
-            const int nb = (int)(tail - head < 32 ? tail - head : 32);
-            int64_t eb = 0, ee = 0;
-            if (lane < nb) {
-                const int32_t v = q[head + lane];
-                eb = __ldg(in_off + v);
-                ee = __ldg(in_off + v + 1);
-                sexam += (unsigned long long)(ee - eb);
-            }
-            head += nb;
-            const int64_t g0 = eb >> 2;
-            const int64_t ng = ee > eb ? ((ee - 1) >> 2) - g0 + 1 : 0;
-            const int64_t incl = warp_incl_scan<int64_t>(ng, lane);
-            const int64_t total = __shfl_sync(kFull, incl, 31);
-            // kICU edge groups per lane per iteration: their loads and coin
-            // draws are independent, so they overlap
-            for (int64_t base = 0; base < total; base += 32 * kICU) {
-                uint4 wv[kICU];
-                int4 sv[kICU];
-                int64_t gg[kICU], lo[kICU], hi[kICU];
-#pragma unroll
-                for (int uu = 0; uu < kICU; ++uu) {
-                    const int64_t t = base + uu * 32 + lane;
-                    int owner = 0;   // first lane whose inclusive group count exceeds t
-#pragma unroll
-                    for (int step = 16; step > 0; step >>= 1) {
-                        const int64_t c = __shfl_sync(kFull, incl, owner + step - 1);
-                        if (c <= t) owner += step;
-                    }
-                    const int64_t o_incl = __shfl_sync(kFull, incl, owner);
-                    const int64_t o_ng = __shfl_sync(kFull, ng, owner);
-                    const int64_t o_g0 = __shfl_sync(kFull, g0, owner);
-                    lo[uu] = __shfl_sync(kFull, eb, owner);
-                    hi[uu] = __shfl_sync(kFull, ee, owner);
-                    gg[uu] = -1;
-                    if (t < total) {
-                        gg[uu] = o_g0 + (t - (o_incl - o_ng));
-                        wv[uu] = __ldg(reinterpret_cast<const uint4 *>(wgt) + gg[uu]);
-                        sv[uu] = __ldg(reinterpret_cast<const int4 *>(in_src) + gg[uu]);
-                    }
+        // the last min(32, ncand) listed edges: source, visited test, append
+        auto flush = [&]() {
+            const int take = ncand < 32 ? ncand : 32;
+            ncand -= take;
+            __syncwarp();
+            uint32_t u = 0;
+            bool fresh = false;
+            if (lane < take) u = (uint32_t)__ldg(in_src + cand[ncand + lane]);
+            if (!BITS && !spilled && tail + 32 > kICHashMax) {
+                // the hash set moves to the warp's bitmap in global memory
+                if (!gclear) {
+                    for (int64_t i = lane; i < a.vis_words; i += 32) gvis[i] = 0u;
+                    gclear = true;
+                    __syncwarp();
                 }
-                unsigned fresh = 0;
-                int32_t src[4 * kICU];
-#pragma unroll
-                for (int uu = 0; uu < kICU; ++uu) {
-                    src[4 * uu + 0] = src[4 * uu + 1] = src[4 * uu + 2] = src[4 * uu + 3] = 0;
-                    if (gg[uu] < 0) continue;
-                    const int64_t g = gg[uu];
-                    const uint4 coin = philox4x32_10(
-                        make_uint4(s, (uint32_t)g, (uint32_t)((uint64_t)g >> 32), kStreamCoin), k0,
-                        k1);
-                    const uint32_t cv[4] = {coin.x, coin.y, coin.z, coin.w};
-                    const uint32_t wq[4] = {wv[uu].x, wv[uu].y, wv[uu].z, wv[uu].w};
-                    src[4 * uu + 0] = sv[uu].x;
-                    src[4 * uu + 1] = sv[uu].y;
-                    src[4 * uu + 2] = sv[uu].z;
-                    src[4 * uu + 3] = sv[uu].w;
-                    const int64_t e0 = g << 2;
-#pragma unroll
-                    for (int c = 0; c < 4; ++c) {
-                        const int64_t e = e0 + c;
-                        if (e >= lo[uu] && e < hi[uu] && cv[c] < wq[c]) {
-                            const uint32_t u = (uint32_t)src[4 * uu + c];
-                            const uint32_t bit = 1u << (u & 31);
-                            if (!(atomicOr(&vis[u >> 5], bit) & bit)) fresh |= 1u << (4 * uu + c);
-                        }
-                    }
+                for (int32_t i = lane; i < tail; i += 32) {
+                    const uint32_t x = (uint32_t)sq[i];
+                    atomicOr(&gvis[x >> 5], 1u << (x & 31));
                 }
-                const int nf = __popc(fresh);
-                const int inclf = warp_incl_scan<int>(nf, lane);
-                const int totf = __shfl_sync(kFull, inclf, 31);
-                if (totf == 0) continue;
-                if (tail + totf > a.qcap) {
-                    // drop this sample; un-mark what was just marked
-#pragma unroll
-                    for (int c = 0; c < 4 * kICU; ++c)
-                        if (fresh >> c & 1) {
-                            const uint32_t u = (uint32_t)src[c];
-                            atomicAnd(&vis[u >> 5], ~(1u << (u & 31)));
-                        }
-                    overflow = true;
-                    break;
-                }
-                int64_t pos = tail + inclf - nf;
-#pragma unroll
-                for (int c = 0; c < 4 * kICU; ++c)
-                    if (fresh >> c & 1) q[pos++] = src[c];
-                tail += totf;
+                spilled = true;
                 __syncwarp();
             }
+            if (lane < take) {
+                const uint32_t bit = 1u << (u & 31);
+                if (BITS) {
+                    fresh = !(atomicOr(&vis[u >> 5], bit) & bit);
+                } else if (spilled) {
+                    fresh = !(atomicOr(&gvis[u >> 5], bit) & bit);
+                } else {
+                    uint32_t h = ic_hash(u);
+                    for (;;) {           // at most kICHashMax of kICHash slots are taken
+                        const uint32_t old = atomicCAS(&vis[h], 0xffffffffu, u);
+                        if (old == 0xffffffffu) fresh = true;
+                        if (old == 0xffffffffu || old == u) break;
+                        h = (h + 1) & (kICHash - 1);
+                    }
+                }
+            }
+            const unsigned fm = __ballot_sync(kFull, fresh);
+            const int nf = __popc(fm);
+            if ((int64_t)tail + nf > a.qcap) {
+                // a queue overflow: the sample starts again in the second pass;
+                // un-mark what was just marked (bitmaps only: the hash set
+                // holds at most kICHashMax <= qcap)
+                if (fresh) atomicAnd(BITS ? &vis[u >> 5] : &gvis[u >> 5], ~(1u << (u & 31)));
+                lost = true;
+                ncand = 0;
+                __syncwarp();
+                return;
+            }
+            if (fresh) {
+                const int32_t at = tail + __popc(fm & lt);
+                if (at < kICQueueSmem) sq[at] = (int32_t)u;
+                else q[at] = (int32_t)u;
+            }
+            tail += nf;
+            __syncwarp();
+        };
+        bool leave = false;
+        while (!lost) {
+            if (head == tail || leave) {
+                if (ncand == 0) break;
+                flush();
+                continue;
+            }
+            // a set that percolates: its frontier feeds a whole block.  (A long
+            // set with a narrow frontier -- weighted cascade grows them thin and
+            // deep -- stays: the block's levels would leave most warps idle, 152
+            // against 139 ms of IMM on the LiveJournal shape.)
+            leave = work >= kICWideEdges && tail - head >= kICWarpFront;
+            if (leave) continue;
+            const int nb = tail - head < 32 ? tail - head : 32;
+            ICItem it{0u, 0u, 0u, 1u};
+            if (lane < nb) {
+                const int32_t x = head + lane;
+                it = ic_item(rec, (uint32_t)(x < kICQueueSmem ? sq[x] : q[x]));
+            }
+            const uint32_t deg = it.ee - it.eb;
+            work = min(work + __reduce_add_sync(kFull, deg < (1u << 25) ? deg : 1u << 25),
+                       kICWideEdges);
+            sexam += (unsigned long long)deg;
+            head += nb;
+            ic_expand<KEYS>(cs, a.rk, wgt, it, ic_groups(it), lane, [&](uint32_t m, uint32_t e0) {
+                if (lost) return;
+                ic_list(m, e0, cand, ncand, lane);
+                while (ncand >= 32) flush();
+            });
         }
+        const bool overflow = lost || head < tail;
         __syncwarp();
         if (overflow) {
-            mark_overflow(a, j, lane);
+            // second pass: the state goes along if there is room for it
+            const unsigned long long ex = warp_sum<unsigned long long>(sexam);
+            unsigned long long off = ~0ull;
+            if (lane == 0 && !lost) {
+                off = atomicAdd(a.hand_cursor, (unsigned long long)tail);
+                if ((int64_t)off + tail > a.hand_cap) off = ~0ull;
+            }
+            off = __shfl_sync(kFull, off, 0);
+            if (off != ~0ull)
+                for (int32_t i = lane; i < tail; i += 32)
+                    a.hand[off + i] = i < kICQueueSmem ? sq[i] : q[i];
+            if (lane == 0) {
+                a.sizes[j] = -1;
+                a.stage_off[j] = 0;
+                const unsigned long long at = atomicAdd(a.ovf_count, 1ull);
+                a.ovf_list[at] = j;
+                a.handed[at] = Handed{(int64_t)off, ex, head, tail};
+            }
         } else {
-            emit_set(a, j, q, tail, lane);
+            unsigned long long pos = 0;
+            if (lane == 0) pos = atomicAdd(a.stage_cursor, (unsigned long long)tail);
+            pos = __shfl_sync(kFull, pos, 0);
+            if ((int64_t)pos + tail > a.stage_cap) {
+                if (lane == 0) {
+                    raise_status(a.status, kDevStageOverflow);
+                    a.sizes[j] = 0;
+                    a.stage_off[j] = 0;
+                }
+            } else {
+                for (int32_t i = lane; i < tail; i += 32)
+                    a.stage[pos + i] = i < kICQueueSmem ? sq[i] : q[i];
+                if (lane == 0) {
+                    a.stage_off[j] = (int64_t)pos;
+                    a.sizes[j] = tail;
+                }
+            }
             exam += sexam;
-            // 16 B offsets + 4 B write per member, 8 B per examined edge, 8 B per set
+            // 16 B record + 4 B write per member, 8 B per examined edge, 8 B per set
             abytes += 8ull * sexam + (lane == 0 ? 20ull * (unsigned long long)tail + 8ull : 0ull);
         }
-        // reset the visited bits of this sample
-        if (tail > a.vis_words) {
-            for (int64_t i = lane; i < a.vis_words; i += 32) vis[i] = 0;
+        // reset the visited set
+        if (BITS && tail <= svis) {
+            for (int32_t i = lane; i < tail; i += 32)
+                vis[(uint32_t)(i < kICQueueSmem ? sq[i] : q[i]) >> 5] = 0u;
         } else {
-            for (int64_t i = lane; i < tail; i += 32) {
-                const uint32_t u = (uint32_t)q[i];
-                vis[u >> 5] = 0;
+            for (int i = lane; i < svis; i += 32) vis[i] = kClear;
+        }
+        if (spilled) {
+            if (tail > a.vis_words) {
+                for (int64_t i = lane; i < a.vis_words; i += 32) gvis[i] = 0u;
+            } else {
+                for (int32_t i = lane; i < tail; i += 32)
+                    gvis[(uint32_t)(i < kICQueueSmem ? sq[i] : q[i]) >> 5] = 0u;
             }
         }
         __syncwarp();
@@ -268,71 +525,34 @@ __global__ void __launch_bounds__(kSampleThreads, 4) k_sample_ic(SampleArgs a) {
 // IC, one block per sample: the second pass for the sets longer than a warp's
 // queue.  The giant sets of hub-heavy graphs (hundreds of thousands of
 // members, tens of millions of examined in-edges) are a level-synchronous
-// BFS whose 32 warps take 32 queued vertices of the current level at a time
-// and expand their in-edges four per lane (one Philox call per group of four,
-// as in k_sample_ic), appending what they reach with one block-level atomic
-// per warp and step.  The queue and visited bitmap (n entries / n bits per
-// block) live in global memory.  The set is copied to the stage by the block.
+// BFS: the 32 warps take 32 queued vertices of the level at a time and expand
+// them as k_sample_ic does; in-lists of at least kICHubGroups groups are put
+// aside and shared out over the whole block at the end of the level, so that
+// no warp is left alone with a hub.  The queue and visited bitmap (n entries /
+// n bits per block) live in global memory; a warp appends what 32 listed live
+// edges reach with one block-level atomic.  The set is copied to the stage by
+// the block.
 constexpr int kICBigThreads = 1024;
-constexpr int kICBigU = 2;          // edge groups per lane in flight (k_sample_ic_big)
+constexpr uint32_t kICHubGroups = 512;       // edge groups from which a list is shared by the block
+constexpr int kICHubCap = 256;               // shared lists a level holds (others stay with their warp)
 
-// One group of four in-edges of sample s: coins of edge group g (edges
-// 4g .. 4g+3 inside [eb, ee)) against its loaded weights wv, with sources sv;
-// marks the live edges' fresh sources visited and returns their bits (the
-// sources in src[]).
-__device__ __forceinline__ unsigned ic_group_loaded(const uint4 wv, const int4 sv, int64_t g,
-                                                    int64_t eb, int64_t ee, uint32_t s,
-                                                    uint32_t k0, uint32_t k1, uint32_t *vis,
-                                                    int32_t (&src)[4]) {
-    const uint4 coin = philox4x32_10(
-        make_uint4(s, (uint32_t)g, (uint32_t)((uint64_t)g >> 32), kStreamCoin), k0, k1);
-    const uint32_t cv[4] = {coin.x, coin.y, coin.z, coin.w};
-    const uint32_t wq[4] = {wv.x, wv.y, wv.z, wv.w};
-    src[0] = sv.x;
-    src[1] = sv.y;
-    src[2] = sv.z;
-    src[3] = sv.w;
-    unsigned fresh = 0;
-    const int64_t e0 = g << 2;
-#pragma unroll
-    for (int c = 0; c < 4; ++c) {
-        const int64_t e = e0 + c;
-        if (e >= eb && e < ee && cv[c] < wq[c]) {
-            const uint32_t u = (uint32_t)src[c];
-            const uint32_t bit = 1u << (u & 31);
-            if (!(atomicOr(&vis[u >> 5], bit) & bit)) fresh |= 1u << c;
-        }
-    }
-    return fresh;
-}
-
-// Appends each lane's fresh sources to the block queue (one atomic per warp).
-__device__ __forceinline__ void ic_append(unsigned fresh, const int32_t (&src)[4], int lane,
-                                          unsigned long long *tail, int32_t *q) {
-    const int nf = __popc(fresh);
-    const int inclf = warp_incl_scan<int>(nf, lane);
-    const int totf = __shfl_sync(kFull, inclf, 31);
-    if (totf == 0) return;
-    long long at = 0;
-    if (lane == 31) at = (long long)atomicAdd(tail, (unsigned long long)totf);
-    at = __shfl_sync(kFull, at, 31);
-    int64_t pos = at + inclf - nf;
-#pragma unroll
-    for (int c = 0; c < 4; ++c)
-        if (fresh >> c & 1) q[pos++] = src[c];
-}
-
-__global__ void __launch_bounds__(kICBigThreads) k_sample_ic_big(SampleArgs a) {
-    __shared__ unsigned long long s_item, s_tail, s_cursor, s_pos;
-    __shared__ unsigned long long s_red[2][kICBigThreads / 32];
+template <bool KEYS>
+__global__ void __launch_bounds__(kICBigThreads) k_sample_ic_big(const __grid_constant__ SampleArgs a) {
+    __shared__ unsigned long long s_item, s_pos;
+    __shared__ unsigned int s_tail, s_cursor, s_nhub;
+    __shared__ ICItem s_hub[kICHubCap];
+    __shared__ uint32_t s_cand[kICBigThreads / 32][kCandCap];
+    __shared__ unsigned long long s_red[kICBigThreads / 32];
 
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const unsigned lt = (1u << lane) - 1u;
     int32_t *q = a.queues + (size_t)blockIdx.x * (size_t)a.qcap;
     uint32_t *vis = a.gvis + (size_t)blockIdx.x * (size_t)a.vis_words;
+    uint32_t *cand = s_cand[warp];
     for (;;) {
         if (threadIdx.x == 0) {
             s_item = atomicAdd(a.work, 1ull);
-            s_tail = 0;
+            s_nhub = 0;
         }
         __syncthreads();
         const unsigned long long jw = s_item;
@@ -340,90 +560,113 @@ __global__ void __launch_bounds__(kICBigThreads) k_sample_ic_big(SampleArgs a) {
         const int64_t j = a.list ? a.list[jw] : (int64_t)jw;
         const int qi = find_query(a, j);
         const QueryView &V = a.qv[qi];
-        const int64_t *in_off = V.in_off;
+        const uint4 *rec = V.ic_rec;
         const int32_t *in_src = V.in_src;
         const uint32_t *wgt = V.w;
-        const uint32_t k0 = seed_lo(V.seed), k1 = seed_hi(V.seed);
         const uint32_t s = V.first + (uint32_t)(j - __ldg(a.qstart + qi));
-        if (threadIdx.x == 0) {
+        CoinStream<KEYS> cs;
+        cs.begin(a.rk, s, seed_lo(V.seed), seed_hi(V.seed));
+        unsigned long long sexam = 0;
+        unsigned int head = 0;
+        const Handed hd = a.handed[jw];
+        if (hd.off >= 0) {                   // go on where the warp stopped
+            for (int32_t x = threadIdx.x; x < hd.tail; x += kICBigThreads) {
+                const int32_t u = a.hand[hd.off + x];
+                q[x] = u;
+                atomicOr(&vis[u >> 5], 1u << (u & 31));
+            }
+            head = (unsigned)hd.head;
+            if (threadIdx.x == 0) {
+                s_tail = (unsigned)hd.tail;
+                sexam = hd.examined;
+            }
+        } else if (threadIdx.x == 0) {
             const uint32_t root = rrr_root(V.seed, s, V.n);
             atomicOr(&vis[root >> 5], 1u << (root & 31));
             q[0] = (int32_t)root;
             s_tail = 1;
         }
         __syncthreads();
-        unsigned long long sexam = 0;
-        long long head = 0;
+        int ncand = 0;
+        // the last min(32, ncand) listed edges: source, visited test, append
+        // (the queue holds n entries, so it cannot overflow)
+        auto flush = [&]() {
+            const int take = ncand < 32 ? ncand : 32;
+            ncand -= take;
+            __syncwarp();
+            uint32_t u = 0;
+            bool fresh = false;
+            if (lane < take) {
+                u = (uint32_t)__ldg(in_src + cand[ncand + lane]);
+                const uint32_t bit = 1u << (u & 31);
+                // most live edges of a giant set reach a member: a load answers
+                // those, an atomic the rest
+                if (!(__ldcg(vis + (u >> 5)) & bit))
+                    fresh = !(atomicOr(&vis[u >> 5], bit) & bit);
+            }
+            const unsigned fm = __ballot_sync(kFull, fresh);
+            if (fm) {
+                unsigned int at = 0;
+                if (lane == 0) at = atomicAdd(&s_tail, (unsigned int)__popc(fm));
+                at = __shfl_sync(kFull, at, 0);
+                if (fresh) q[at + __popc(fm & lt)] = (int32_t)u;
+            }
+            __syncwarp();
+        };
+        auto visit = [&](uint32_t m, uint32_t e0) {
+            ic_list(m, e0, cand, ncand, lane);
+            while (ncand >= 32) flush();
+        };
         for (;;) {
-            const long long lvl_end = (long long)s_tail;
+            const unsigned int lvl_end = s_tail;
             if (head >= lvl_end) break;
-            if (threadIdx.x == 0) s_cursor = (unsigned long long)head;
+            __syncthreads();                 // everyone has read s_tail
+            if (threadIdx.x == 0) s_cursor = head;
             __syncthreads();
             for (;;) {
-                long long base = 0;
-                if (lane == 0) base = (long long)atomicAdd(&s_cursor, 32ull);
+                unsigned int base = 0;
+                if (lane == 0) base = atomicAdd(&s_cursor, 32u);
                 base = __shfl_sync(kFull, base, 0);
                 if (base >= lvl_end) break;
-                const int nb = (int)(lvl_end - base < 32 ? lvl_end - base : 32);
-                int64_t eb = 0, ee = 0;
-                if (lane < nb) {
-                    const int32_t v = q[base + lane];
-                    eb = __ldg(in_off + v);
-                    ee = __ldg(in_off + v + 1);
-                    sexam += (unsigned long long)(ee - eb);
+                ICItem it{0u, 0u, 0u, 1u};
+                if (base + lane < lvl_end) {
+                    it = ic_item(rec, (uint32_t)q[base + lane]);
+                    sexam += (unsigned long long)(it.ee - it.eb);
                 }
-                const int64_t g0 = eb >> 2;
-                const int64_t ng = ee > eb ? ((ee - 1) >> 2) - g0 + 1 : 0;
-                const int64_t incl = warp_incl_scan<int64_t>(ng, lane);
-                const int64_t total = __shfl_sync(kFull, incl, 31);
-                // kICBigU edge groups per lane in flight: their loads are issued
-                // together before any coin is drawn
-                for (int64_t gb = 0; gb < total; gb += 32 * kICBigU) {
-                    int64_t grp[kICBigU], geb[kICBigU], gee[kICBigU];
-                    uint4 wv[kICBigU];
-                    int4 sv[kICBigU];
-#pragma unroll
-                    for (int u = 0; u < kICBigU; ++u) {
-                        const int64_t t = gb + u * 32 + lane;
-                        int owner = 0;   // first lane whose inclusive group count exceeds t
-#pragma unroll
-                        for (int step = 16; step > 0; step >>= 1) {
-                            const int64_t c = __shfl_sync(kFull, incl, owner + step - 1);
-                            if (c <= t) owner += step;
-                        }
-                        const int64_t o_incl = __shfl_sync(kFull, incl, owner);
-                        const int64_t o_ng = __shfl_sync(kFull, ng, owner);
-                        const int64_t o_g0 = __shfl_sync(kFull, g0, owner);
-                        geb[u] = __shfl_sync(kFull, eb, owner);
-                        gee[u] = __shfl_sync(kFull, ee, owner);
-                        grp[u] = t < total ? o_g0 + (t - (o_incl - o_ng)) : -1;
-                        if (grp[u] >= 0) {
-                            wv[u] = __ldg(reinterpret_cast<const uint4 *>(wgt) + grp[u]);
-                            sv[u] = __ldg(reinterpret_cast<const int4 *>(in_src) + grp[u]);
-                        }
-                    }
-#pragma unroll
-                    for (int u = 0; u < kICBigU; ++u) {
-                        unsigned fresh = 0;
-                        int32_t src[4] = {0, 0, 0, 0};
-                        if (grp[u] >= 0)
-                            fresh = ic_group_loaded(wv[u], sv[u], grp[u], geb[u], gee[u], s, k0, k1,
-                                                    vis, src);
-                        ic_append(fresh, src, lane, &s_tail, q);
+                uint32_t ng = ic_groups(it);
+                if (ng >= kICHubGroups) {    // shared by the block below
+                    const unsigned int h = atomicAdd(&s_nhub, 1u);
+                    if (h < (unsigned)kICHubCap) {
+                        s_hub[h] = it;
+                        ng = 0;
                     }
                 }
+                __syncwarp();
+                ic_expand<KEYS>(cs, a.rk, wgt, it, ng, lane, visit);
             }
             __syncthreads();
+            const int nhub = (int)(s_nhub < (unsigned)kICHubCap ? s_nhub : (unsigned)kICHubCap);
+            for (int h = 0; h < nhub; ++h) {  // this warp's slice of every shared list
+                const ICItem it = s_hub[h];
+                const uint32_t n = ic_groups(it);
+                const uint32_t per =
+                    ((n + kICBigThreads / 32 - 1) / (kICBigThreads / 32) + 31u) & ~31u;
+                const uint32_t t = min(n, warp * per);
+                ic_expand_wide<KEYS>(cs, a.rk, wgt, it, t, min(n, t + per), lane, visit);
+            }
+            while (ncand > 0) flush();
+            __syncthreads();
+            if (threadIdx.x == 0) s_nhub = 0;
             head = lvl_end;
         }
         // emit: reserve the stage range, copy the queue, record size and offset
         const long long len = (long long)s_tail;
-        unsigned long long ex = warp_sum<unsigned long long>(sexam);
-        if (lane == 0) s_red[0][warp] = ex;
+        const unsigned long long ex = warp_sum<unsigned long long>(sexam);
+        if (lane == 0) s_red[warp] = ex;
         __syncthreads();
         if (threadIdx.x == 0) {
             unsigned long long tot = 0;
-            for (int w2 = 0; w2 < kICBigThreads / 32; ++w2) tot += s_red[0][w2];
+            for (int w2 = 0; w2 < kICBigThreads / 32; ++w2) tot += s_red[w2];
             s_pos = atomicAdd(a.stage_cursor, (unsigned long long)len);
             if ((long long)s_pos + len > a.stage_cap) {
                 raise_status(a.status, kDevStageOverflow);
@@ -434,7 +677,7 @@ __global__ void __launch_bounds__(kICBigThreads) k_sample_ic_big(SampleArgs a) {
                 a.stage_off[j] = (int64_t)s_pos;
                 a.sizes[j] = (int32_t)len;
                 atomicAdd(a.examined, tot);
-                // 16 B offsets + 4 B write per member, 8 B per examined edge, 8 B per set
+                // 16 B record + 4 B write per member, 8 B per examined edge, 8 B per set
                 atomicAdd(a.alg_bytes, 8ull * tot + 20ull * (unsigned long long)len + 8ull);
             }
         }
@@ -448,6 +691,53 @@ __global__ void __launch_bounds__(kICBigThreads) k_sample_ic_big(SampleArgs a) {
             for (long long x = threadIdx.x; x < len; x += blockDim.x) vis[q[x] >> 5] = 0u;
         }
         __syncthreads();
+    }
+}
+
+// In-edge records of the IC kernels: {first in-edge, in-degree, common weight,
+// 1 if all in-edges have it}.  A lane looks at up to kICRecLane in-edges of
+// its own vertex -- with unequal weights that settles nearly every list -- and
+// the warp scans the rest of the undecided lists together, until the first
+// difference.
+constexpr int kICRecLane = 4;
+
+__global__ void __launch_bounds__(256) k_ic_records(const int64_t *in_off, const uint32_t *w,
+                                                    int64_t n, uint4 *rec) {
+    const int lane = threadIdx.x & 31;
+    const int64_t warps = (int64_t)gridDim.x * (blockDim.x >> 5);
+    for (int64_t v0 = ((int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5)) * 32; v0 < n;
+         v0 += warps * 32) {
+        const int64_t v = v0 + lane;
+        int64_t b = 0, e = 0;
+        if (v < n) {
+            b = in_off[v];
+            e = in_off[v + 1];
+        }
+        const uint32_t w0 = e > b ? __ldg(w + b) : 0u;
+        bool same = true;
+#pragma unroll
+        for (int i = 1; i < kICRecLane; ++i)
+            if (b + i < e) same &= __ldg(w + b + i) == w0;
+        unsigned open = __ballot_sync(kFull, same && e - b > kICRecLane);
+        while (open) {
+            const int l = __ffs(open) - 1;
+            open &= open - 1u;
+            const int64_t lb = __shfl_sync(kFull, b, l), le = __shfl_sync(kFull, e, l);
+            const uint32_t lw = __shfl_sync(kFull, w0, l);
+            bool ok = true;
+            for (int64_t i0 = lb + kICRecLane; i0 < le && ok; i0 += 256) {
+                bool mine = true;
+#pragma unroll
+                for (int u = 0; u < 8; ++u) {
+                    const int64_t i = i0 + u * 32 + lane;
+                    if (i < le) mine &= __ldg(w + i) == lw;
+                }
+                ok = __all_sync(kFull, mine);
+            }
+            if (lane == l) same = ok;
+        }
+        if (v < n)
+            rec[v] = make_uint4((uint32_t)b, (uint32_t)(e - b), w0, same ? 1u : 0u);
     }
 }
 
@@ -1584,7 +1874,7 @@ im_status segmented_sort_impl(Key *keys, const int64_t *seg_off, int64_t nseg, c
     return IM_OK;
 }
 
-static std::mutex g_lt_index_mu;   // graphs are shared by serving workers
+static std::mutex g_lt_index_mu;   // graphs are shared by serving workers (LT and IC records)
 
 im_status build_lt_index(im_graph *g, cudaStream_t st) {
     std::lock_guard<std::mutex> lk(g_lt_index_mu);
@@ -1682,11 +1972,32 @@ im_status build_lt_index(im_graph *g, cudaStream_t st) {
     return IM_OK;
 }
 
+// In-edge records of the IC samplers (k_ic_records), built on the first IC use
+// of a graph and kept with it.
+im_status build_ic_index(im_graph *g, cudaStream_t st) {
+    std::lock_guard<std::mutex> lk(g_lt_index_mu);
+    if (g->ic_rec) return IM_OK;   // set only once the records are complete
+    uint4 *rec = nullptr;
+    IM_CUDA(cudaMalloc((void **)&rec, (size_t)g->n * sizeof(uint4)));
+    cudaError_t e;
+    {
+        KernelTimer kt(st, "ic_index");
+        k_ic_records<<<num_sms() * 8, 256, 0, st>>>(g->in_off, g->w, g->n, rec);
+    }
+    if ((e = cudaGetLastError()) != cudaSuccess || (e = cudaStreamSynchronize(st)) != cudaSuccess) {
+        cudaFree(rec);
+        return cuda_fail(e, "IC index");
+    }
+    g->ic_rec = rec;
+    return IM_OK;
+}
+
 QueryView query_view(const im_graph *g, uint64_t seed, uint64_t first) {
     QueryView v;
     v.in_off = g->in_off;
     v.in_src = g->in_src;
     v.w = g->w;
+    v.ic_rec = g->ic_rec;
     v.lt_vrec = g->lt_vrec;
     v.lt_leaf = g->lt_leaf;
     v.lt_tree = g->lt_tree;
@@ -1709,6 +2020,7 @@ im_status run_sampling(const SamplingJob &job, const std::function<im_status(siz
     const int64_t cnt = qstart[nq];
     const int64_t n = job.n_max;
     const bool smem_vis = model == IM_IC && n <= kSmemVisBits;
+    const bool one_key = nq == 1;                    // the round keys go in the launch's arguments
     const int64_t vis_words = (n + 31) / 32;
 
     // launch shape: persistent, occupancy-sized
@@ -1723,19 +2035,23 @@ im_status run_sampling(const SamplingJob &job, const std::function<im_status(siz
                               : G == 8  ? (const void *)k_sample_lt<8>
                               : G == 16 ? (const void *)k_sample_lt<16>
                                         : (const void *)k_sample_lt<32>)
-                       : smem_vis ? (const void *)k_sample_ic<true>
-                                  : (const void *)k_sample_ic<false>;
+                       : smem_vis ? (one_key ? (const void *)k_sample_ic<true, true>
+                                             : (const void *)k_sample_ic<true, false>)
+                                  : (one_key ? (const void *)k_sample_ic<false, true>
+                                             : (const void *)k_sample_ic<false, false>);
     const int threads = lt1 ? kLT1Threads : kSampleThreads;
-    const size_t dyn_smem = smem_vis ? (size_t)kWarps * vis_words * 4
-                            : lt1    ? (size_t)kBloomWords * kLT1Threads * 4
-                                     : 0;
+    const size_t ic_words = (smem_vis ? (vis_words + 3) & ~(int64_t)3 : kICHash) + kICQueueSmem +
+                            kCandCap;                // a warp's shared memory
+    const size_t dyn_smem = model == IM_IC ? (size_t)kWarps * ic_words * 4
+                            : lt1          ? (size_t)kBloomWords * kLT1Threads * 4
+                                           : 0;
     if (dyn_smem > 48 * 1024)
         IM_TRY(raise_dyn_smem(kern, dyn_smem));
     int blocks = blocks_for(kern, threads, dyn_smem);
-    // global visited bitmaps are n bits per warp: keep them within ~2 GB
+    // global visited bitmaps are n bits per warp: keep them within ~4 GB
     if (model == IM_IC && !smem_vis) {
         int64_t cap_blocks = std::max<int64_t>(
-            num_sms(), (int64_t)(2ll << 30) / ((int64_t)kWarps * vis_words * 4));
+            num_sms(), (int64_t)(4ll << 30) / ((int64_t)kWarps * vis_words * 4));
         blocks = (int)std::min<int64_t>(blocks, cap_blocks);
     }
     const int64_t warps = (int64_t)blocks * (threads / 32);
@@ -1758,6 +2074,9 @@ im_status run_sampling(const SamplingJob &job, const std::function<im_status(siz
     const size_t o_ovf = take((size_t)cnt * 8);
     const size_t o_scan = take(scan_tmp_bytes(cnt));
     const size_t o_sort = take((size_t)(2 + 2 * cnt) * 8);
+    const size_t o_handed = take(model == IM_IC ? (size_t)cnt * sizeof(Handed) : 0);
+    const int64_t hand_cap = model == IM_IC ? std::min<int64_t>(kICHandCap, cnt * qcap) : 0;
+    const size_t o_hand = take((size_t)hand_cap * 4);
     const size_t o_q = take((size_t)slots * qcap * 4);
     const size_t o_vis = take(model == IM_IC && !smem_vis ? (size_t)warps * vis_words * 4 : 0);
     void *base = nullptr;
@@ -1766,14 +2085,12 @@ im_status run_sampling(const SamplingJob &job, const std::function<im_status(siz
     char *B = (char *)base;
     unsigned long long *ctr = (unsigned long long *)(B + o_ctr);
     // ctr: 0 work, 1 stage cursor, 2 examined, 3 overflow count, 4 status (int),
-    //      5 algorithmic bytes
+    //      5 algorithmic bytes, 6 handed-over members
     IM_CUDA(cudaMemsetAsync(ctr, 0, 8 * sizeof(unsigned long long), st));
     IM_CUDA(cudaMemcpyAsync(B + o_views, job.views.data(), (size_t)nq * sizeof(QueryView),
                             cudaMemcpyHostToDevice, st));
     IM_CUDA(cudaMemcpyAsync(B + o_qstart, qstart.data(), (size_t)(nq + 1) * 8,
                             cudaMemcpyHostToDevice, st));
-    if (o_vis && model == IM_IC && !smem_vis)
-        IM_CUDA(cudaMemsetAsync(B + o_vis, 0, (size_t)warps * vis_words * 4, st));
 
     SampleArgs a;
     a.qv = (const QueryView *)(B + o_views);
@@ -1796,6 +2113,15 @@ im_status run_sampling(const SamplingJob &job, const std::function<im_status(siz
     a.ovf_list = (int64_t *)(B + o_ovf);
     a.ovf_count = ctr + 3;
     a.status = (int *)(ctr + 4);
+    a.handed = (Handed *)(B + o_handed);
+    a.hand = (int32_t *)(B + o_hand);
+    a.hand_cap = hand_cap;
+    a.hand_cursor = ctr + 6;
+    for (int r = 0; r < 10; ++r) {
+        a.rk[2 * r] = one_key ? (uint32_t)job.views[0].seed + (uint32_t)r * 0x9E3779B9u : 0u;
+        a.rk[2 * r + 1] =
+            one_key ? (uint32_t)(job.views[0].seed >> 32) + (uint32_t)r * 0xBB67AE85u : 0u;
+    }
 
     auto launch = [&](int nblocks, int group) {
         KernelTimer kt(st, model == IM_LT ? "sample_lt" : "sample_ic");
@@ -1809,9 +2135,11 @@ im_status run_sampling(const SamplingJob &job, const std::function<im_status(siz
             else if (group == 16) k_sample_lt<16><<<nblocks, kSampleThreads, 0, st>>>(a);
             else k_sample_lt<32><<<nblocks, kSampleThreads, 0, st>>>(a);
         } else if (smem_vis) {
-            k_sample_ic<true><<<nblocks, kSampleThreads, dyn_smem, st>>>(a);
+            if (one_key) k_sample_ic<true, true><<<nblocks, kSampleThreads, dyn_smem, st>>>(a);
+            else k_sample_ic<true, false><<<nblocks, kSampleThreads, dyn_smem, st>>>(a);
         } else {
-            k_sample_ic<false><<<nblocks, kSampleThreads, 0, st>>>(a);
+            if (one_key) k_sample_ic<false, true><<<nblocks, kSampleThreads, dyn_smem, st>>>(a);
+            else k_sample_ic<false, false><<<nblocks, kSampleThreads, dyn_smem, st>>>(a);
         }
     };
     launch(blocks, G);
@@ -1821,20 +2149,25 @@ im_status run_sampling(const SamplingJob &job, const std::function<im_status(siz
     IM_CUDA(cudaMemcpyAsync(hc, ctr, sizeof(hc), cudaMemcpyDeviceToHost, st));
     IM_CUDA(cudaStreamSynchronize(st));
     int dev_status = (int)(hc[4] & 0xffffffffu);
-    if (dev_status == kDevOk && hc[3] > 0 && qcap < n) {
-        // second pass for sets longer than the per-walk queue: a few warps
-        // with queues of n entries re-run exactly those samples
+    if (dev_status == kDevOk && hc[3] > 0) {
+        // second pass for the sets the first gave up (LT: longer than the
+        // per-walk queue; IC: longer than that, or of too many in-edges for one
+        // warp), with queues of n entries
         const int64_t novf = (int64_t)hc[3];
         const bool ic_big = model == IM_IC;
         // IC: one block per sample; LT: one walk per warp
         const int64_t per_unit = (int64_t)n * 4 + (ic_big ? vis_words * 4 : 0);
         int64_t units = ic_big ? std::min<int64_t>(novf, (int64_t)num_sms())
                                : std::min<int64_t>((novf + kWarps - 1) / kWarps, num_sms()) * kWarps;
-        if (ic_big) units = std::max<int64_t>(1, std::min<int64_t>(units, (2ll << 30) / per_unit));
+        if (ic_big) units = std::max<int64_t>(1, std::min<int64_t>(units, (4ll << 30) / per_unit));
         const int nb2 = (int)(ic_big ? units : std::max<int64_t>(1, units / kWarps));
         const size_t need2 = (size_t)units * (size_t)per_unit;
+        // the first pass's queues and bitmaps are free by now, and mostly enough
+        // (mapping fresh memory took 2 to 5 ms a call)
         int32_t *q2 = nullptr;
-        IM_CUDA(cudaMallocAsync((void **)&q2, need2, st));
+        const bool own = need2 > off - o_q;
+        if (own) IM_CUDA(cudaMallocAsync((void **)&q2, need2, st));
+        else q2 = (int32_t *)(B + o_q);
         uint32_t *vis2 = (uint32_t *)((char *)q2 + (size_t)units * (size_t)n * 4);
         if (ic_big) IM_CUDA(cudaMemsetAsync(vis2, 0, (size_t)units * vis_words * 4, st));
         IM_CUDA(cudaMemsetAsync(ctr, 0, sizeof(unsigned long long), st));
@@ -1849,12 +2182,13 @@ im_status run_sampling(const SamplingJob &job, const std::function<im_status(siz
         a = a2;
         if (ic_big) {
             KernelTimer kt(st, "sample_ic_big");
-            k_sample_ic_big<<<nb2, kICBigThreads, 0, st>>>(a);
+            if (one_key) k_sample_ic_big<true><<<nb2, kICBigThreads, 0, st>>>(a);
+            else k_sample_ic_big<false><<<nb2, kICBigThreads, 0, st>>>(a);
         } else {
             launch(nb2, 32);   // one walk per warp: queues of n entries for the longest walks
         }
         IM_CUDA(cudaGetLastError());
-        IM_CUDA(cudaFreeAsync(q2, st));
+        if (own) IM_CUDA(cudaFreeAsync(q2, st));
         IM_CUDA(cudaMemcpyAsync(hc, ctr, sizeof(hc), cudaMemcpyDeviceToHost, st));
         IM_CUDA(cudaStreamSynchronize(st));
         dev_status = (int)(hc[4] & 0xffffffffu);
@@ -1917,6 +2251,8 @@ im_status sample_append(const im_graph *gc, im_model model, uint64_t seed, uint6
             set_error("LT sampling needs every vertex's in-weights to sum to at most 2^32");
             return IM_ERR_INVALID_ARG;
         }
+    } else {
+        IM_TRY(build_ic_index(g, st));
     }
     if (count == 0) return IM_OK;
     if (pool->theta + (int64_t)count > pool->max_sets) {
