@@ -447,7 +447,7 @@ im_status greedy_select(im_pool *p, int32_t k, bool lazy, int32_t *d_seeds, int6
 // SelectSeeds (index build + the cover opts asks for) with its coverage
 // read back to the host.
 im_status sample_growing(const im_graph *g, im_model model, uint64_t seed, uint64_t first,
-                         uint64_t count, im_pool *p, cudaStream_t st);
+                         uint64_t count, im_pool *p, cudaStream_t st, bool sized = false);
 im_status select_seeds(im_pool *p, int32_t k, const im_cover_opts *o, int32_t *d_seeds,
                        int64_t *d_gains, int32_t *d_ns, int64_t *d_cov, int *d_status,
                        int64_t *coverage, cudaStream_t st);
