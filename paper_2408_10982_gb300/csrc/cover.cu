@@ -1151,35 +1151,205 @@ __global__ void __launch_bounds__(kRGThreads) k_rg_stream_masks(RGArgs a) {
     }
 }
 
+// Streaming buckets, one block each, over a bitmap in shared memory (Alg. 5, run
+// after the local greedy has finished; theta <= kSmallBits).  For short
+// streams and many buckets: the stage is then a chain of decisions, not a
+// scan, and the chain of one bucket lives within one SM -- block barriers where
+// k_rg_stream_masks has grid barriers, and no bucket waits for another's cut.
+//
+// The block takes kSmallThreads stream slots at a time, keeps those whose
+// subset reaches the bucket's threshold at all, and counts the gains of 32 of
+// them against the bucket as it stands, in pieces of kSmallPiece entries over
+// all warps.  The first that reaches the threshold is accepted (the slots
+// before it saw the same bucket); the slots behind it that fell short still
+// do, since gains only shrink, so only those that passed are counted again.
+// Hence a group costs one count and one short recount per accepted seed.
+// Bound by that chain (a few hundred cycles a link), not by memory.  OPIM at
+// k = 1,000 (94 buckets, 37,000 slots, 10,780 sets): 36.6 -> 2.07 ms against a
+// cluster per bucket counting one candidate at a time.
+// The line to the masks: with B <= 64 the masks read every subset once for all
+// buckets, a block here reads it for its own.  At 2.7 x 10^6 members the masks
+// take 0.56 ms, the blocks 0.69; over the 24 RandGreedi queries of the batched
+// mix 12.5 ms with the line at 2^20 members, 13.4 without the blocks, 40.4 with
+// it at 2^24.  With B > 64 the other choice is the cluster kernel, which reads
+// as much and one candidate at a time.
+constexpr int kSmallThreads = 512;
+constexpr int kSmallPiece = 256;             // entries of a subset a warp counts at once
+constexpr int64_t kSmallBits = 1600 * 1024;  // sets whose bitmap fits (200 KB)
+constexpr int64_t kSmallTotal = 1 << 20;     // pool members from which a stream counts as long
+
+// The stream's slots as {element or -1, |S(x)|} and the subset's first entry.
+__global__ void k_rg_slots(RGArgs a) {
+    const int64_t nslots = (int64_t)a.trunc * a.P;
+    for (int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; t < nslots;
+         t += (int64_t)gridDim.x * blockDim.x) {
+        const int32_t x = a.flags[t] == 1u ? a.elems[t] : -1;
+        const int64_t b = x >= 0 ? a.vtx_off[x] : 0;
+        a.slot_x[t] = x;
+        a.slot_beg[t] = b;
+        a.slot_len[t] = x >= 0 ? a.vtx_off[x + 1] - b : 0;
+    }
+}
+
+__global__ void __launch_bounds__(kSmallThreads) k_rg_stream_small(RGArgs a) {
+    extern __shared__ uint32_t bits[];       // [ceil(theta / 32)]
+    constexpr int kWarpsS = kSmallThreads / 32;
+    __shared__ int32_t s_x[kSmallThreads], s_len[kSmallThreads];
+    __shared__ int64_t s_beg[kSmallThreads];
+    __shared__ int32_t s_gain[32], s_off[33];
+    __shared__ int32_t s_wcnt[kWarpsS];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const unsigned lt = (1u << lane) - 1u;
+    const int64_t nslots = (int64_t)a.trunc * a.P;
+    for (int b = blockIdx.x; b < a.B; b += gridDim.x) {
+        for (int64_t x = threadIdx.x; x < a.words; x += blockDim.x) bits[x] = 0u;
+        const int64_t T = a.thr[b];
+        const uint64_t t_begin = global_ns();
+        long long n_eval = 0, scanned = 0;
+        int32_t bn = 0;
+        int64_t bcov = 0;
+        for (int64_t base = 0; base < nslots && bn < a.k; base += kSmallThreads) {
+            // ---- the window's slots that can pass, in stream order
+            __syncthreads();                 // the last group has been read; bits are cleared
+            const int64_t t = base + threadIdx.x;
+            const int32_t x = t < nslots ? __ldg(a.slot_x + t) : -1;
+            const int64_t len = t < nslots ? __ldg(a.slot_len + t) : 0;
+            const bool keep = x >= 0 && len >= T;
+            const unsigned km = __ballot_sync(kFull, keep);
+            if (lane == 0) s_wcnt[warp] = __popc(km);
+            __syncthreads();
+            int before = 0, nc = 0;
+            for (int w = 0; w < kWarpsS; ++w) {
+                if (w < warp) before += s_wcnt[w];
+                nc += s_wcnt[w];
+            }
+            if (keep) {
+                const int at = before + __popc(km & lt);
+                s_x[at] = x;
+                s_len[at] = (int32_t)len;    // |S(x)| <= theta <= kSmallBits
+                s_beg[at] = __ldg(a.slot_beg + t);
+            }
+            __syncthreads();
+            for (int c0 = 0; c0 < nc && bn < a.k; c0 += 32) {
+                // lane u of every warp stands for slot c0 + u
+                const int32_t my_len = c0 + lane < nc ? s_len[c0 + lane] : 0;
+                unsigned todo = nc - c0 < 32 ? (1u << (nc - c0)) - 1u : kFull;
+                n_eval += __popc(todo);
+                for (;;) {
+                    if (warp == 0) {
+                        const int32_t pieces = todo >> lane & 1u ? (my_len + kSmallPiece - 1) / kSmallPiece : 0;
+                        const int32_t incl = warp_incl_scan<int32_t>(pieces, lane);
+                        s_off[lane] = incl - pieces;
+                        if (lane == 31) s_off[32] = incl;
+                        s_gain[lane] = 0;
+                    }
+                    __syncthreads();         // also: the accepted subset is in the bitmap
+                    const int32_t my_off = s_off[lane], total = s_off[32];
+                    for (int32_t c = warp; c < total; c += kWarpsS) {
+                        // the last slot of todo that starts at or before piece c
+                        const unsigned at = __ballot_sync(kFull, (todo >> lane & 1u) && my_off <= c);
+                        const int u = 31 - __clz(at);
+                        const int32_t e0 = (c - __shfl_sync(kFull, my_off, u)) * kSmallPiece;
+                        const int32_t n = s_len[c0 + u];
+                        const int32_t *ids = a.set_ids + s_beg[c0 + u];
+                        int32_t id[kSmallPiece / 32];
+#pragma unroll
+                        for (int q = 0; q < kSmallPiece / 32; ++q) {
+                            const int32_t i = e0 + q * 32 + lane;
+                            id[q] = i < n ? __ldg(ids + i) : -1;
+                        }
+                        int miss = 0;
+#pragma unroll
+                        for (int q = 0; q < kSmallPiece / 32; ++q)
+                            if (id[q] >= 0) miss += !((bits[id[q] >> 5] >> (id[q] & 31)) & 1u);
+                        miss = __reduce_add_sync(kFull, miss);
+                        if (lane == 0 && miss) atomicAdd(&s_gain[u], miss);
+                    }
+                    __syncthreads();
+                    const int32_t g = s_gain[lane];
+                    const unsigned pass = __ballot_sync(kFull, (todo >> lane & 1u) && (int64_t)g >= T);
+                    scanned += (long long)__reduce_add_sync(kFull, todo >> lane & 1u ? my_len : 0);
+                    if (!pass) break;
+                    const int u = __ffs(pass) - 1;
+                    const int32_t gain = __shfl_sync(kFull, g, u);
+                    if (threadIdx.x == 0) {
+                        a.bucket_seeds[(int64_t)b * a.k + bn] = s_x[c0 + u];
+                        a.bucket_gains[(int64_t)b * a.k + bn] = gain;
+                    }
+                    ++bn;
+                    bcov += gain;
+                    if (bn == a.k) break;
+                    const int32_t n = s_len[c0 + u];
+                    const int32_t *ids = a.set_ids + s_beg[c0 + u];
+                    for (int32_t i = threadIdx.x; i < n; i += kSmallThreads) {
+                        const int32_t id = __ldg(ids + i);
+                        atomicOr(&bits[id >> 5], 1u << (id & 31));
+                    }
+                    todo = pass & ~((2u << u) - 1u);
+                    if (!todo) break;
+                    __syncthreads();         // s_gain and s_off have been read by every warp
+                }
+                __syncthreads();             // likewise, and the bitmap is complete
+            }
+        }
+        if (threadIdx.x == 0) {
+            a.bucket_n[b] = bn;
+            a.bucket_cov[b] = bcov;
+            if (a.stats) {
+                long long *st = a.stats + 6 * ((int64_t)a.P + b);
+                st[0] = (long long)t_begin;
+                st[1] = (long long)global_ns();
+                st[2] = n_eval;
+                st[3] = bn;
+                st[4] = scanned;
+                st[5] = 0;
+            }
+        }
+        __syncthreads();
+    }
+}
+
 // Alg. 4's final compare: best bucket (ties: smallest b) against the best
-// local solution (ties: smallest p); the bucket wins ties.
-__global__ void k_rg_final(RGArgs a, int32_t *seeds, int64_t *gains, int32_t *nseeds,
-                           int64_t *coverage, int32_t *chosen) {
-    if (threadIdx.x != 0 || blockIdx.x != 0) return;
-    int bstar = 0;
-    for (int b = 1; b < a.B; ++b)
-        if (a.bucket_cov[b] > a.bucket_cov[bstar]) bstar = b;
-    int pbest = 0;
-    for (int p = 1; p < a.P; ++p)
-        if (a.local_cov[p] > a.local_cov[pbest]) pbest = p;
-    if (a.bucket_cov[bstar] >= a.local_cov[pbest]) {
-        *chosen = -1;
-        const int32_t m = a.bucket_n[bstar];
-        for (int32_t j = 0; j < m; ++j) {
-            seeds[j] = a.bucket_seeds[(int64_t)bstar * a.k + j];
-            gains[j] = a.bucket_gains[(int64_t)bstar * a.k + j];
-        }
+// local solution (ties: smallest p); the bucket wins ties.  One block: maxima by
+// block reductions, the winner's seeds copied by all threads (one thread
+// walking both lists took 85 us at P = 148, k = 1,000).
+constexpr int kFinalThreads = 256;
+
+// The largest of cov[0 .. n) and its smallest index, by the whole block.
+__device__ __forceinline__ int64_t best_coverage(const int64_t *cov, int n, int *at,
+                                                 unsigned long long *shm) {
+    unsigned long long m = 0;                // coverage + 1
+    for (int i = threadIdx.x; i < n; i += blockDim.x) {
+        const unsigned long long c = (unsigned long long)cov[i] + 1ull;
+        m = c > m ? c : m;
+    }
+    m = block_max_u64(m, shm);
+    unsigned long long k = 0;                // 2^32 - index
+    for (int i = threadIdx.x; i < n; i += blockDim.x)
+        if ((unsigned long long)cov[i] + 1ull == m && (1ull << 32) - i > k) k = (1ull << 32) - i;
+    *at = (int)((1ull << 32) - block_max_u64(k, shm));
+    return (int64_t)m - 1;
+}
+
+__global__ void __launch_bounds__(kFinalThreads) k_rg_final(RGArgs a, int32_t *seeds, int64_t *gains,
+                                                            int32_t *nseeds, int64_t *coverage,
+                                                            int32_t *chosen) {
+    __shared__ unsigned long long shm[33];
+    int b, p;
+    const int64_t bcov = best_coverage(a.bucket_cov, a.B, &b, shm);
+    const int64_t pcov = best_coverage(a.local_cov, a.P, &p, shm);
+    const bool bucket = bcov >= pcov;
+    const int32_t m = bucket ? a.bucket_n[b] : a.local_n[p];
+    const int32_t *s = bucket ? a.bucket_seeds + (int64_t)b * a.k : a.local_seeds + (int64_t)p * a.k;
+    const int64_t *g = bucket ? a.bucket_gains + (int64_t)b * a.k : a.local_gains + (int64_t)p * a.k;
+    for (int32_t j = threadIdx.x; j < m; j += kFinalThreads) {
+        seeds[j] = s[j];
+        gains[j] = g[j];
+    }
+    if (threadIdx.x == 0) {
+        *chosen = bucket ? -1 : p;
         *nseeds = m;
-        *coverage = a.bucket_cov[bstar];
-    } else {
-        *chosen = pbest;
-        const int32_t m = a.local_n[pbest];
-        for (int32_t j = 0; j < m; ++j) {
-            seeds[j] = a.local_seeds[(int64_t)pbest * a.k + j];
-            gains[j] = a.local_gains[(int64_t)pbest * a.k + j];
-        }
-        *nseeds = m;
-        *coverage = a.local_cov[pbest];
+        *coverage = bucket ? bcov : pcov;
     }
 }
 
@@ -1388,18 +1558,23 @@ im_status randgreedi(im_pool *p, int32_t k, const im_cover_opts *o, int32_t *d_s
         return at;
     };
     const size_t o_cov = take((size_t)P * words * 4);
-    const size_t o_bcov = take((size_t)B * words * 4);
     const size_t o_flags = take((size_t)trunc * P * 4);
     const size_t o_elems = take((size_t)trunc * P * 4);
     const size_t o_l = take(64);
-    // bucket-mask stage (two-launch mode, automatic layout, B <= 64)
-    const bool use_masks = !naive && o->fused == 0 && tune_value(IM_TUNE_RG_CLUSTER) == 0 && B <= 64;
+    // two-launch mode, automatic layout: a block per bucket where the bitmaps fit
+    // and the stream is short (kSmallTotal) or has more buckets than a mask has
+    // bits; else the bucket-mask stage (B <= 64)
+    const bool automatic = !naive && o->fused == 0 && tune_value(IM_TUNE_RG_CLUSTER) == 0;
+    const bool use_small = automatic && theta <= kSmallBits && (p->total <= kSmallTotal || B > 64);
+    const bool use_masks = automatic && !use_small && B <= 64;
     const size_t o_mask = use_masks ? take((size_t)std::max<int64_t>(theta, 1) * 8) : 0;
     const size_t o_gbuf = use_masks ? take((size_t)2 * kMaskG * 64 * 4) : 0;
     const size_t o_bar = use_masks ? take(sizeof(GridBarrier)) : 0;
-    const size_t o_sx = use_masks ? take((size_t)trunc * P * 4) : 0;
-    const size_t o_sb = use_masks ? take((size_t)trunc * P * 8) : 0;
-    const size_t o_sl = use_masks ? take((size_t)trunc * P * 8) : 0;
+    const size_t o_bcov = take(use_masks || use_small || naive ? 0 : (size_t)B * words * 4);
+    const bool slots = use_masks || use_small;
+    const size_t o_sx = slots ? take((size_t)trunc * P * 4) : 0;
+    const size_t o_sb = slots ? take((size_t)trunc * P * 8) : 0;
+    const size_t o_sl = slots ? take((size_t)trunc * P * 8) : 0;
     const size_t o_lazy = naive ? take(lazy_greedy_scratch(n, theta)) : 0;
     void *base = nullptr;
     s = pool_scratch(p, off, &base);
@@ -1456,9 +1631,9 @@ im_status randgreedi(im_pool *p, int32_t k, const im_cover_opts *o, int32_t *d_s
     a.mask = use_masks ? (unsigned long long *)(Bs + o_mask) : nullptr;
     a.gbuf = use_masks ? (uint32_t *)(Bs + o_gbuf) : nullptr;
     a.bar = use_masks ? (GridBarrier *)(Bs + o_bar) : nullptr;
-    a.slot_x = use_masks ? (int32_t *)(Bs + o_sx) : nullptr;
-    a.slot_beg = use_masks ? (int64_t *)(Bs + o_sb) : nullptr;
-    a.slot_len = use_masks ? (int64_t *)(Bs + o_sl) : nullptr;
+    a.slot_x = slots ? (int32_t *)(Bs + o_sx) : nullptr;
+    a.slot_beg = slots ? (int64_t *)(Bs + o_sb) : nullptr;
+    a.slot_len = slots ? (int64_t *)(Bs + o_sl) : nullptr;
     if (use_masks) IM_CUDA(cudaMemsetAsync(Bs + o_bar, 0, sizeof(GridBarrier), st));
 
     IM_TRY(raise_dyn_smem((const void *)k_randgreedi, prod_smem));
@@ -1505,6 +1680,13 @@ im_status randgreedi(im_pool *p, int32_t k, const im_cover_opts *o, int32_t *d_s
                                    p->rg_bucket_cov, p->lz_stats, d_status, st,
                                    p->rg_local_seeds, p->rg_local_n, P, trunc, k);
             if (s != IM_OK) return s;
+        } else if (use_small) {
+            const size_t smem = (size_t)words * 4;
+            IM_TRY(raise_dyn_smem((const void *)k_rg_stream_small, smem));
+            KernelTimer kt(st, "randgreedi_stream");
+            k_rg_slots<<<num_sms(), 256, 0, st>>>(a);
+            k_rg_stream_small<<<B, kSmallThreads, smem, st>>>(a);
+            IM_CUDA(cudaGetLastError());
         } else if (use_masks) {
             // buckets: one pass over each streamed subset serves all buckets
             int per = 0;
@@ -1527,7 +1709,7 @@ im_status randgreedi(im_pool *p, int32_t k, const im_cover_opts *o, int32_t *d_s
             if (csmem <= kClusterSmemCap) break;
         }
         if (want < 0) CS = 16;   // global-memory bitmaps requested
-        if (naive || use_masks) {
+        if (naive || use_masks || use_small) {
             // done above
         } else if (CS <= 8) {
             unsigned *counter = (unsigned *)(Bs + o_l) + 2;
@@ -1561,7 +1743,7 @@ im_status randgreedi(im_pool *p, int32_t k, const im_cover_opts *o, int32_t *d_s
     int32_t *d_chosen = (int32_t *)(Bs + o_l);   // l is no longer needed
     {
         KernelTimer kt(st, "randgreedi_final");
-        k_rg_final<<<1, 32, 0, st>>>(a, d_seeds, d_gains, d_nseeds, d_cov, d_chosen);
+        k_rg_final<<<1, kFinalThreads, 0, st>>>(a, d_seeds, d_gains, d_nseeds, d_cov, d_chosen);
     }
     IM_CUDA(cudaGetLastError());
     int32_t chosen = 0;
