@@ -419,6 +419,7 @@ im_status im_solve_batch(im_batch *b, const im_query *qs, int32_t nq, int32_t km
         // 1. sampling: one launch per model
         int64_t added = 0, examined = 0;
         bool capacity = false;
+        unsigned long long long_sets = 0;
         int64_t done_sets = 0;
         for (int mi = 0; mi < 2 && !capacity; ++mi) {
             const im_model model = mi == 0 ? IM_IC : IM_LT;
@@ -469,6 +470,7 @@ im_status im_solve_batch(im_batch *b, const im_query *qs, int32_t nq, int32_t km
             }
             done_sets += nsets;
             added += r.added;
+            long_sets += r.long_sets;
             examined += r.examined;
         }
         if (capacity) {
@@ -491,7 +493,8 @@ im_status im_solve_batch(im_batch *b, const im_query *qs, int32_t nq, int32_t km
                                       scan_tmp_bytes(sets_total), st);
         if (s != IM_OK) return s;
         int32_t *members = (int32_t *)(A + o_mem);
-        s = segmented_sort_sets(members, set_off, sets_total, stage, stage_off, tmp, n_max, st);
+        s = segmented_sort_sets(members, set_off, sets_total, stage, stage_off, tmp, n_max,
+                                long_sets, st);
         if (s != IM_OK) return s;
         // 3. one vertex space, one index
         IM_CUDA(cudaMemcpyAsync(A + o_bq, bq.data(), (size_t)nq * sizeof(BatchQuery),

@@ -391,11 +391,14 @@ struct SamplingResult {
     int64_t added;           // members written to the stage
     int64_t examined;
     int64_t alg_bytes;
+    unsigned long long long_sets;   // sets that a warp does not sort, plus 2^32 for every one
+                                    // that a block does not either (for segmented_sort_sets)
 };
 im_status run_sampling(const SamplingJob &job, const std::function<im_status(size_t, void **)> &alloc,
                        cudaStream_t st, SamplingResult *res);
 im_status segmented_sort_sets(int32_t *dst, const int64_t *seg_off, int64_t nseg, const int32_t *stage,
-                              const int64_t *stage_off, void *tmp, int64_t n_max, cudaStream_t st);
+                              const int64_t *stage_off, void *tmp, int64_t n_max,
+                              unsigned long long long_sets, cudaStream_t st);
 QueryView query_view(const im_graph *g, uint64_t seed, uint64_t first);
 im_status sample_append(const im_graph *g, im_model model, uint64_t seed, uint64_t first,
                         uint64_t count, im_pool *pool, cudaStream_t st);

@@ -35,7 +35,9 @@ constexpr int kPathSmem = 256;               // LT path entries mirrored in smem
 constexpr int kPathSmemGroup = 64;           // ... per walk when a warp runs several walks
 constexpr int64_t kQueueCapIC = 1 << 14;     // per-warp queue entries (first pass)
 constexpr int64_t kQueueCapLT = 1 << 11;
-constexpr int kWarpSortBytes = 4096;         // per-warp smem sort buffer
+constexpr int kWarpSortKeys = 1024;          // sets up to this length are sorted by one warp
+// set in stage_off of a set that lies in the stage in ascending order already
+constexpr int64_t kStageAscending = (int64_t)1 << 62;
 constexpr int kBlockSortCap = 16384;         // ... by one block in shared memory (int32)
 
 // An IC sample that a warp gave up: its members so far are hand[off .. off +
@@ -72,6 +74,8 @@ struct SampleArgs {
     int32_t *hand;            // their members
     int64_t hand_cap;
     unsigned long long *hand_cursor;
+    unsigned long long *nlong;    // sets longer than kWarpSortKeys, plus 2^32 for every
+                                  // unsorted one longer than kBlockSortCap
     uint32_t rk[20];          // Philox round keys of the launch's query, when it has only one
 };
 
@@ -493,6 +497,7 @@ __global__ void __launch_bounds__(kSampleThreads, KEYS ? 3 : 4) k_sample_ic(cons
                 if (lane == 0) {
                     a.stage_off[j] = (int64_t)pos;
                     a.sizes[j] = tail;
+                    if (tail > kWarpSortKeys) atomicAdd(a.nlong, 1ull);
                 }
             }
             exam += sexam;
@@ -659,8 +664,13 @@ __global__ void __launch_bounds__(kICBigThreads) k_sample_ic_big(const __grid_co
             if (threadIdx.x == 0) s_nhub = 0;
             head = lvl_end;
         }
-        // emit: reserve the stage range, copy the queue, record size and offset
+        // emit: reserve the stage range, write the set, record size and offset.
+        // A long set is read off its bitmap, in ascending order (so that it
+        // needs no sorting: 0.9 ms a set when the sort marked and read a bitmap
+        // of its own), which also clears it; a short one is copied from the
+        // queue.
         const long long len = (long long)s_tail;
+        const bool ascending = len > kBlockSortCap || (len > kWarpSortKeys && a.vis_words <= 64 * len);
         const unsigned long long ex = warp_sum<unsigned long long>(sexam);
         if (lane == 0) s_red[warp] = ex;
         __syncthreads();
@@ -674,21 +684,52 @@ __global__ void __launch_bounds__(kICBigThreads) k_sample_ic_big(const __grid_co
                 a.stage_off[j] = 0;
                 s_pos = ~0ull;
             } else {
-                a.stage_off[j] = (int64_t)s_pos;
+                a.stage_off[j] = (int64_t)s_pos | (ascending ? kStageAscending : 0);
                 a.sizes[j] = (int32_t)len;
+                if (len > kWarpSortKeys) atomicAdd(a.nlong, 1ull);
                 atomicAdd(a.examined, tot);
                 // 16 B record + 4 B write per member, 8 B per examined edge, 8 B per set
                 atomicAdd(a.alg_bytes, 8ull * tot + 20ull * (unsigned long long)len + 8ull);
             }
         }
         __syncthreads();
-        if (s_pos != ~0ull)
-            for (long long x = threadIdx.x; x < len; x += blockDim.x) a.stage[s_pos + x] = q[x];
-        // clear this sample's visited bits
-        if (len > a.vis_words) {
-            for (int64_t x = threadIdx.x; x < a.vis_words; x += blockDim.x) vis[x] = 0u;
+        if (ascending && s_pos != ~0ull) {
+            // each warp a run of words: the members before it, then its own
+            const int64_t run = ((a.vis_words + kICBigThreads - 1) / kICBigThreads) * 32;
+            const int64_t w0 = min(a.vis_words, warp * run), w1 = min(a.vis_words, w0 + run);
+            int cnt = 0;
+#pragma unroll 4
+            for (int64_t x = w0 + lane; x < w1; x += 32) cnt += __popc(__ldcg(vis + x));
+            cnt = __reduce_add_sync(kFull, cnt);
+            if (lane == 0) s_red[warp] = (unsigned long long)cnt;
+            __syncthreads();
+            const int incl = warp_incl_scan<int>((int)s_red[lane], lane);
+            int64_t at = (int64_t)s_pos + (warp ? __shfl_sync(kFull, incl, warp - 1) : 0);
+            uint32_t next = w0 + lane < w1 ? __ldcg(vis + w0 + lane) : 0u;
+            for (int64_t x0 = w0; x0 < w1; x0 += 32) {
+                const int64_t x = x0 + lane;
+                uint32_t bitset = next;
+                next = x + 32 < w1 ? __ldcg(vis + x + 32) : 0u;
+                if (bitset) vis[x] = 0u;
+                const int mine = __popc(bitset);
+                const int upto = warp_incl_scan<int>(mine, lane);
+                int64_t p = at + upto - mine;
+                while (bitset) {
+                    const int c = __ffs(bitset) - 1;
+                    bitset &= bitset - 1u;
+                    a.stage[p++] = (int32_t)(x * 32 + c);
+                }
+                at += __shfl_sync(kFull, upto, 31);
+            }
         } else {
-            for (long long x = threadIdx.x; x < len; x += blockDim.x) vis[q[x] >> 5] = 0u;
+            if (s_pos != ~0ull)
+                for (long long x = threadIdx.x; x < len; x += blockDim.x) a.stage[s_pos + x] = q[x];
+            // clear this sample's visited bits
+            if (len > a.vis_words) {
+                for (int64_t x = threadIdx.x; x < a.vis_words; x += blockDim.x) vis[x] = 0u;
+            } else {
+                for (long long x = threadIdx.x; x < len; x += blockDim.x) vis[q[x] >> 5] = 0u;
+            }
         }
         __syncthreads();
     }
@@ -938,6 +979,8 @@ __global__ void __launch_bounds__(kSampleThreads, G == 32 ? 8 : 5) k_sample_lt(S
                     if (gl == 0) {
                         a.stage_off[j] = (int64_t)pos;
                         a.sizes[j] = len;
+                        if (len > kWarpSortKeys)
+                            atomicAdd(a.nlong, 1ull + (len > kBlockSortCap ? 1ull << 32 : 0ull));
                     }
                 }
                 exam += sexam;
@@ -1623,13 +1666,11 @@ __device__ __forceinline__ void thread_bitonic(Key (&v)[N]) {
 
 // One segment sorted by the whole warp (len > kLaneSort): copied from the
 // stage and sorted in registers, or in the warp's shared buffer, or listed in
-// `big` for k_sort_block / k_sort_giant.
+// `big` for k_sort_block.
 template <typename Key>
-__device__ __forceinline__ void warp_sort_segment(Key *out, const Key *src, int64_t len,
-                                                  bool from_stage, int64_t i, Key *buf,
-                                                  int64_t *big, unsigned long long *nbig,
+__device__ __forceinline__ void warp_sort_segment(Key *out, const Key *src, int64_t len, int64_t i,
+                                                  Key *buf, int64_t *big, unsigned long long *nbig,
                                                   int lane) {
-    constexpr int kCapW = kWarpSortBytes / (int)sizeof(Key);
     if (len <= 32) {
         Key v = lane < len ? src[lane] : key_max<Key>();
         v = warp_bitonic32<Key>(v, lane);
@@ -1642,23 +1683,20 @@ __device__ __forceinline__ void warp_sort_segment(Key *out, const Key *src, int6
         warp_sort_copy<Key, 8>(out, src, len, lane);
     } else if (len <= 512 && sizeof(Key) == 4) {
         warp_sort_copy<Key, 16>(out, src, len, lane);
-    } else if (len <= kCapW) {
+    } else if (len <= kWarpSortKeys) {
         int P = 64;
         while (P < len) P <<= 1;
         for (int t = lane; t < P; t += 32) buf[t] = t < len ? src[t] : key_max<Key>();
         __syncwarp();
         bitonic_smem<Key>(buf, P, lane, 32, false);
         for (int t = lane; t < len; t += 32) out[t] = buf[t];
-    } else {
-        if (from_stage)
-            for (int64_t t = lane; t < len; t += 32) out[t] = src[t];
-        if (lane == 0) big[atomicAdd(nbig, 1ull)] = i;
+    } else if (lane == 0) {
+        big[atomicAdd(nbig, 1ull)] = i;
     }
     __syncwarp();
 }
 
-// Copies stage segments into place (when `stage` is non-null) and sorts the
-// short ones.  A warp takes 32 consecutive segments at once (their offsets in
+// Copies stage segments into place and sorts the short ones.  A warp takes 32 consecutive segments at once (their offsets in
 // one coalesced load each): segments of at most kLaneSort keys -- most RRR
 // sets -- are sorted by their own lane in registers; the longer ones are
 // listed in `mid` for k_sort_mid, one warp each.
@@ -1670,8 +1708,7 @@ __global__ void __launch_bounds__(256) k_sort_small(Key *dst, const int64_t *seg
                                                     int64_t *mid, unsigned long long *nmid,
                                                     bool inline_long, int64_t *big,
                                                     unsigned long long *nbig) {
-    constexpr int kCapW = kWarpSortBytes / (int)sizeof(Key);
-    __shared__ Key sbuf[8][kCapW];
+    __shared__ Key sbuf[8][kWarpSortKeys];
     const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
     const int64_t nw = (int64_t)gridDim.x * 8;
     for (int64_t i0 = ((int64_t)blockIdx.x * 8 + wib) * 32; i0 < nseg; i0 += nw * 32) {
@@ -1681,11 +1718,11 @@ __global__ void __launch_bounds__(256) k_sort_small(Key *dst, const int64_t *seg
         if (i < nseg) {
             o = seg_off[i];
             len = seg_off[i + 1] - o;
-            src = stage ? stage + stage_off[i] : dst + o;
+            src = stage + (stage_off[i] & ~kStageAscending);
         }
         Key *out = dst + o;
         if (len == 1) {
-            if (stage) out[0] = src[0];
+            out[0] = src[0];
         } else if (len > 1 && len <= kLaneSort) {
             Key v[kLaneSort];
 #pragma unroll
@@ -1703,8 +1740,7 @@ __global__ void __launch_bounds__(256) k_sort_small(Key *dst, const int64_t *seg
                 const int64_t ol = __shfl_sync(kFull, o, l);
                 const int64_t ll = __shfl_sync(kFull, len, l);
                 const Key *sl = (const Key *)__shfl_sync(kFull, (unsigned long long)src, l);
-                warp_sort_segment<Key>(dst + ol, sl, ll, stage != nullptr, i0 + l, sbuf[wib], big,
-                                       nbig, lane);
+                warp_sort_segment<Key>(dst + ol, sl, ll, i0 + l, sbuf[wib], big, nbig, lane);
             }
         } else if (longer) {
             unsigned long long base = 0;
@@ -1724,8 +1760,7 @@ __global__ void __launch_bounds__(256) k_sort_mid(Key *dst, const int64_t *seg_o
                                                   const int64_t *mid,
                                                   const unsigned long long *nmid, int64_t *big,
                                                   unsigned long long *nbig) {
-    constexpr int kCapW = kWarpSortBytes / (int)sizeof(Key);
-    __shared__ Key sbuf[8][kCapW];
+    __shared__ Key sbuf[8][kWarpSortKeys];
     const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
     const int64_t nw = (int64_t)gridDim.x * 8;
     const int64_t cnt = (int64_t)*nmid;
@@ -1733,19 +1768,20 @@ __global__ void __launch_bounds__(256) k_sort_mid(Key *dst, const int64_t *seg_o
         const int64_t i = mid[x];
         const int64_t o = seg_off[i];
         const int64_t len = seg_off[i + 1] - o;
-        warp_sort_segment<Key>(dst + o, stage ? stage + stage_off[i] : dst + o, len,
-                               stage != nullptr, i, sbuf[wib], big, nbig, lane);
+        warp_sort_segment<Key>(dst + o, stage + (stage_off[i] & ~kStageAscending), len, i,
+                               sbuf[wib], big, nbig, lane);
     }
 }
 
-// One block per listed segment longer than a warp's buffer and at most kCap
-// keys: bitonic sort in shared memory.
-template <typename Key, int kCap>
+// One block per listed segment longer than a warp's buffer: copied from the
+// stage when it is ascending there, else sorted in shared memory, or listed in
+// `giant` for k_sort_giant when it has more than kBlockSortCap keys.
+template <typename Key>
 __global__ void __launch_bounds__(1024) k_sort_block(Key *dst, const int64_t *seg_off,
+                                                     const Key *stage, const int64_t *stage_off,
                                                      const int64_t *big,
                                                      const unsigned long long *nbig,
-                                                     int64_t *giant,
-                                                     unsigned long long *ngiant) {
+                                                     int64_t *giant, unsigned long long *ngiant) {
     extern __shared__ unsigned char sraw[];
     Key *buf = reinterpret_cast<Key *>(sraw);
     const int64_t nb = (int64_t)*nbig;
@@ -1753,14 +1789,32 @@ __global__ void __launch_bounds__(1024) k_sort_block(Key *dst, const int64_t *se
         const int64_t i = big[b];
         const int64_t o = seg_off[i];
         const int64_t len = seg_off[i + 1] - o;
-        if (len > kCap) {
-            if (threadIdx.x == 0 && giant) giant[atomicAdd(ngiant, 1ull)] = i;
+        const int64_t so = stage_off[i];
+        const Key *src = stage + (so & ~kStageAscending);
+        if (so & kStageAscending) {
+            constexpr int U = 8;
+            for (int64_t t0 = threadIdx.x; t0 < len; t0 += (int64_t)U * blockDim.x) {
+                Key v[U];
+#pragma unroll
+                for (int u = 0; u < U; ++u) {
+                    const int64_t t = t0 + (int64_t)u * blockDim.x;
+                    if (t < len) v[u] = src[t];
+                }
+#pragma unroll
+                for (int u = 0; u < U; ++u) {
+                    const int64_t t = t0 + (int64_t)u * blockDim.x;
+                    if (t < len) dst[o + t] = v[u];
+                }
+            }
+            continue;
+        }
+        if (len > kBlockSortCap) {
+            if (threadIdx.x == 0) giant[atomicAdd(ngiant, 1ull)] = i;
             continue;
         }
         int P = 64;
         while (P < len) P <<= 1;
-        for (int t = threadIdx.x; t < P; t += blockDim.x)
-            buf[t] = t < len ? dst[o + t] : key_max<Key>();
+        for (int t = threadIdx.x; t < P; t += blockDim.x) buf[t] = t < len ? src[t] : key_max<Key>();
         __syncthreads();
         bitonic_smem<Key>(buf, P, threadIdx.x, blockDim.x, true);
         for (int t = threadIdx.x; t < len; t += blockDim.x) dst[o + t] = buf[t];
@@ -1768,9 +1822,12 @@ __global__ void __launch_bounds__(1024) k_sort_block(Key *dst, const int64_t *se
     }
 }
 
-// Segments longer than kBlockSortCap of distinct vertex ids: mark them in an
-// n-bit bitmap (one per block) and read the bitmap back in order.
+// Unsorted segments longer than kBlockSortCap (LT walks) of distinct vertex
+// ids: mark them in an n-bit bitmap (one per block) and read the bitmap back in
+// order.
 __global__ void __launch_bounds__(1024) k_sort_giant(int32_t *dst, const int64_t *seg_off,
+                                                     const int32_t *stage,
+                                                     const int64_t *stage_off,
                                                      const int64_t *giant,
                                                      const unsigned long long *ngiant,
                                                      uint32_t *bitmaps, int64_t words) {
@@ -1782,8 +1839,9 @@ __global__ void __launch_bounds__(1024) k_sort_giant(int32_t *dst, const int64_t
         const int64_t i = giant[b];
         const int64_t o = seg_off[i];
         const int64_t len = seg_off[i + 1] - o;
+        const int64_t so = stage_off[i];
         for (int64_t t = threadIdx.x; t < len; t += blockDim.x) {
-            const uint32_t u = (uint32_t)dst[o + t];
+            const uint32_t u = (uint32_t)stage[so + t];
             atomicOr(&bm[u >> 5], 1u << (u & 31));
         }
         __syncthreads();
@@ -1826,53 +1884,6 @@ int blocks_for(const void *kernel, int threads, size_t smem) {
 }
 
 }  // namespace
-
-template <typename Key>
-im_status segmented_sort_impl(Key *keys, const int64_t *seg_off, int64_t nseg, const Key *stage,
-                              const int64_t *stage_off, void *tmp, size_t tmp_bytes,
-                              int64_t *ngiant_host, cudaStream_t st, const char *warp_name,
-                              const char *block_name) {
-    // tmp layout: [2 counters][big list nseg][giant list nseg]; the giant
-    // list's space and second counter first hold the list for k_sort_mid
-    if (tmp_bytes < (size_t)(2 + 2 * nseg) * 8) return IM_ERR_INVALID_ARG;
-    unsigned long long *ctr = (unsigned long long *)tmp;
-    int64_t *big = (int64_t *)tmp + 2;
-    int64_t *giant = big + nseg;
-    IM_CUDA(cudaMemsetAsync(ctr, 0, 2 * sizeof(unsigned long long), st));
-    if (nseg == 0) return IM_OK;
-    const int gs = blocks_for((const void *)k_sort_small<Key>, 256, 0);
-    const int gm = blocks_for((const void *)k_sort_mid<Key>, 256, 0);
-    // with at least four groups of 32 segments per warp the longer segments
-    // spread over the warps anyway: each warp sorts its own; with fewer, they
-    // are listed and k_sort_mid gives each its own warp
-    const bool inline_long = nseg >= (int64_t)gs * 8 * 32 * 4;
-    {
-        KernelTimer kt(st, warp_name);
-        k_sort_small<Key><<<gs, 256, 0, st>>>(keys, seg_off, nseg, stage, stage_off, giant,
-                                               ctr + 1, inline_long, big, ctr);
-        if (!inline_long)
-            k_sort_mid<Key><<<gm, 256, 0, st>>>(keys, seg_off, stage, stage_off, giant, ctr + 1,
-                                                 big, ctr);
-    }
-    IM_CUDA(cudaGetLastError());
-    IM_CUDA(cudaMemsetAsync(ctr + 1, 0, sizeof(unsigned long long), st));
-    constexpr int kCap = kBlockSortCap * 4 / (int)sizeof(Key);
-    const size_t smem = (size_t)kCap * sizeof(Key);
-    IM_TRY(raise_dyn_smem((const void *)k_sort_block<Key, kCap>, smem));
-    {
-        KernelTimer kt(st, block_name);
-        k_sort_block<Key, kCap><<<num_sms(), 1024, smem, st>>>(keys, seg_off, big, ctr,
-                                                              giant, ctr + 1);
-    }
-    IM_CUDA(cudaGetLastError());
-    if (ngiant_host) {
-        unsigned long long ng = 0;
-        IM_CUDA(cudaMemcpyAsync(&ng, ctr + 1, sizeof(ng), cudaMemcpyDeviceToHost, st));
-        IM_CUDA(cudaStreamSynchronize(st));
-        *ngiant_host = (int64_t)ng;
-    }
-    return IM_OK;
-}
 
 static std::mutex g_lt_index_mu;   // graphs are shared by serving workers (LT and IC records)
 
@@ -2085,7 +2096,7 @@ im_status run_sampling(const SamplingJob &job, const std::function<im_status(siz
     char *B = (char *)base;
     unsigned long long *ctr = (unsigned long long *)(B + o_ctr);
     // ctr: 0 work, 1 stage cursor, 2 examined, 3 overflow count, 4 status (int),
-    //      5 algorithmic bytes, 6 handed-over members
+    //      5 algorithmic bytes, 6 handed-over members, 7 long sets (SampleArgs::nlong)
     IM_CUDA(cudaMemsetAsync(ctr, 0, 8 * sizeof(unsigned long long), st));
     IM_CUDA(cudaMemcpyAsync(B + o_views, job.views.data(), (size_t)nq * sizeof(QueryView),
                             cudaMemcpyHostToDevice, st));
@@ -2117,6 +2128,7 @@ im_status run_sampling(const SamplingJob &job, const std::function<im_status(siz
     a.hand = (int32_t *)(B + o_hand);
     a.hand_cap = hand_cap;
     a.hand_cursor = ctr + 6;
+    a.nlong = ctr + 7;
     for (int r = 0; r < 10; ++r) {
         a.rk[2 * r] = one_key ? (uint32_t)job.views[0].seed + (uint32_t)r * 0x9E3779B9u : 0u;
         a.rk[2 * r + 1] =
@@ -2145,7 +2157,7 @@ im_status run_sampling(const SamplingJob &job, const std::function<im_status(siz
     launch(blocks, G);
     IM_CUDA(cudaGetLastError());
 
-    unsigned long long hc[6];
+    unsigned long long hc[8];
     IM_CUDA(cudaMemcpyAsync(hc, ctr, sizeof(hc), cudaMemcpyDeviceToHost, st));
     IM_CUDA(cudaStreamSynchronize(st));
     int dev_status = (int)(hc[4] & 0xffffffffu);
@@ -2208,29 +2220,61 @@ im_status run_sampling(const SamplingJob &job, const std::function<im_status(siz
     res->added = (int64_t)hc[1];
     res->examined = (int64_t)hc[2];
     res->alg_bytes = (int64_t)hc[5];
+    res->long_sets = hc[7];
     return IM_OK;
 }
 
 // Copies every set from the stage into dst at seg_off and sorts it ascending.
+// long_sets: what the sampling counted (SamplingResult::long_sets), so that the
+// passes for long sets are launched only when there are any.  tmp: (2 + 2 nseg)
+// * 8 bytes.
 im_status segmented_sort_sets(int32_t *dst, const int64_t *seg_off, int64_t nseg, const int32_t *stage,
-                              const int64_t *stage_off, void *tmp, int64_t n_max, cudaStream_t st) {
-    int64_t ngiant = 0;
-    im_status rs = segmented_sort_impl<int32_t>(dst, seg_off, nseg, stage, stage_off, tmp,
-                                                (size_t)(2 + 2 * nseg) * 8, &ngiant, st,
-                                                "sort_sets_warp", "sort_sets_block");
-    if (rs != IM_OK) return rs;
+                              const int64_t *stage_off, void *tmp, int64_t n_max,
+                              unsigned long long long_sets, cudaStream_t st) {
+    // tmp layout: [2 counters][list for k_sort_block, nseg][list for k_sort_mid, nseg]
+    unsigned long long *ctr = (unsigned long long *)tmp;
+    int64_t *big = (int64_t *)tmp + 2;
+    int64_t *mid = big + nseg;
+    if (nseg == 0) return IM_OK;
+    IM_CUDA(cudaMemsetAsync(ctr, 0, 2 * sizeof(unsigned long long), st));
+    const int gs = blocks_for((const void *)k_sort_small<int32_t>, 256, 0);
+    // with at least four groups of 32 segments per warp the longer segments
+    // spread over the warps anyway: each warp sorts its own; with fewer, they
+    // are listed and k_sort_mid gives each its own warp
+    const bool inline_long = nseg >= (int64_t)gs * 8 * 32 * 4;
+    {
+        KernelTimer kt(st, "sort_sets_warp");
+        k_sort_small<int32_t><<<gs, 256, 0, st>>>(dst, seg_off, nseg, stage, stage_off, mid,
+                                                   ctr + 1, inline_long, big, ctr);
+        if (!inline_long) {
+            const int gm = blocks_for((const void *)k_sort_mid<int32_t>, 256, 0);
+            k_sort_mid<int32_t><<<gm, 256, 0, st>>>(dst, seg_off, stage, stage_off, mid, ctr + 1,
+                                                     big, ctr);
+        }
+    }
+    IM_CUDA(cudaGetLastError());
+    if (long_sets == 0) return IM_OK;
+    const size_t smem = (size_t)kBlockSortCap * 4;
+    IM_TRY(raise_dyn_smem((const void *)k_sort_block<int32_t>, smem));
+    IM_CUDA(cudaMemsetAsync(ctr + 1, 0, sizeof(unsigned long long), st));
+    {
+        KernelTimer kt(st, "sort_sets_block");
+        k_sort_block<int32_t><<<num_sms(), 1024, smem, st>>>(dst, seg_off, stage, stage_off, big,
+                                                             ctr, mid, ctr + 1);
+    }
+    IM_CUDA(cudaGetLastError());
+    const int64_t ngiant = (int64_t)(long_sets >> 32);
     if (ngiant > 0) {
-        // giant sets (> block sort cap) need an n-bit bitmap per block
+        // an n-bit bitmap per block
         const int64_t gwords = (n_max + 31) / 32;
         const int blocks3 = (int)std::min<int64_t>(ngiant, num_sms());
         uint32_t *gbm = nullptr;
         IM_CUDA(cudaMallocAsync((void **)&gbm, (size_t)blocks3 * gwords * 4, st));
         IM_CUDA(cudaMemsetAsync(gbm, 0, (size_t)blocks3 * gwords * 4, st));
-        unsigned long long *sctr = (unsigned long long *)tmp;
-        int64_t *giant = (int64_t *)tmp + 2 + nseg;
         {
             KernelTimer kt(st, "sort_sets_bitmap");
-            k_sort_giant<<<blocks3, 1024, 0, st>>>(dst, seg_off, giant, sctr + 1, gbm, gwords);
+            k_sort_giant<<<blocks3, 1024, 0, st>>>(dst, seg_off, stage, stage_off, mid, ctr + 1,
+                                                   gbm, gwords);
         }
         IM_CUDA(cudaGetLastError());
         IM_CUDA(cudaFreeAsync(gbm, st));
@@ -2280,7 +2324,8 @@ im_status sample_append(const im_graph *gc, im_model model, uint64_t seed, uint6
     rs = exclusive_scan_i32_to_i64(r.sizes, so, cnt, so, r.scan_tmp, scan_tmp_bytes(cnt), st);
     if (rs != IM_OK) return rs;
     // copy stage -> members and sort each set ascending
-    rs = segmented_sort_sets(pool->members, so, cnt, job.stage, r.stage_off, r.sort_tmp, g->n, st);
+    rs = segmented_sort_sets(pool->members, so, cnt, job.stage, r.stage_off, r.sort_tmp, g->n,
+                             r.long_sets, st);
     if (rs != IM_OK) return rs;
     pool->theta += cnt;
     pool->total += r.added;

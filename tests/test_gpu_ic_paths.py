@@ -78,3 +78,23 @@ def test_ic_hash_set_spills(im, weights):
                                          (50_021, 900_001, "trivalency"), (33_000, 300_000, "ic0.9999")])
 def test_ic_handed_over(im, n, m, weights):
     check(im, inputs.rmat_graph(n, m, 9, weights), 21, 96)
+
+
+# chains: sets of every length up to n = 20,011, one member a level -- past a
+# warp's sort (1,024), its queue (16,384) and a block's sort (16,384)
+@pytest.mark.parametrize("model", [0, 1])
+def test_long_chains(im, model):
+    n = 20_011
+    src = np.arange(n - 1, dtype=np.int64)
+    in_off, in_src = inputs.in_csr(n, src, src + 1)
+    g = inputs.Graph(n, in_off, in_src, np.full(n - 1, 2**32 - 1, np.uint32))
+    G = im.Graph(g)
+    P = im.Pool(G, 40, 40 * n)
+    P.sample(model, 17, 0, 40)
+    set_off, members = P.export()
+    ref = oracle.sample(oracle.LT if model else oracle.IC, g, 17, 0, 40)
+    assert np.array_equal(set_off, ref.set_off)
+    assert np.array_equal(members, ref.members)
+    assert np.diff(ref.set_off).max() > 16384
+    P.close()
+    G.close()
