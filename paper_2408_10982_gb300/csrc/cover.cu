@@ -147,6 +147,10 @@ struct GreedyArgs {
     int32_t *ctl;                       // [4] hub rows, candidates, max |S(v)|, 0
     int32_t hub_cap, hub_shift, cand_shift;
     unsigned long long *work;           // [2] per-step chunk counters
+    // pieces of long newly covered sets: first member << 16 | members << 5 | set
+    // id mod 32, and how many this step has
+    unsigned long long *piece;          // [2 T / kGreedyPiece + 1]
+    unsigned long long *npiece;         // [1]
 };
 
 constexpr int kHubRep = 32;             // partial counts of a hub (one per set id mod 32)
@@ -154,6 +158,13 @@ constexpr int kHubRep = 32;             // partial counts of a hub (one per set 
 // hold hundreds of members each, so small chunks spread the decrements over
 // more warps (the step waits for the slowest one).
 constexpr int kGreedyChunk = 16;
+// A newly covered set longer than this is put aside in pieces of this many
+// members, which the whole grid shares after the claims of the step: the
+// percolating sets of equal-probability IC hold 10^4 to 10^6 members each, and
+// the ~100 warps that claim S(v*) would walk them alone (4,096 sets of U[0, 0.1]
+// at scale 20, 1.1 x 10^8 members: 42.1 -> 1.9 ms; no change where sets are
+// short).
+constexpr int kGreedyPiece = 1024;
 constexpr int kHubCap = 4096;           // hub rows at most
 constexpr int kHubShift = 6;            // hubs: |S(v)| >= max |S(v)| / 64
 
@@ -230,6 +241,13 @@ __global__ void __launch_bounds__(kGreedyThreads, 2) k_greedy(GreedyArgs a) {
         nhub = min(__ldcg(a.ctl + 0), a.hub_cap);
         ncand = __ldcg(a.ctl + 1);
     }
+    // a newly covered set of id = rep (mod 32) holds batch vertex mv
+    auto decrement = [&](int32_t mv, int rep) {
+        const int64_t u = mv - a.vshift;
+        const int32_t hr = a.hub_rank ? __ldcg(a.hub_rank + u) : -1;
+        if (hr >= 0) red_add_s32(a.hub_cnt + (int64_t)hr * kHubRep + rep, -1);
+        else if (hr == -1) red_add_s32(a.counts + slot(u), -1);   // -2: frozen
+    };
     int64_t cov = 0;
     int32_t j = 0;
     while (j < a.k) {
@@ -320,6 +338,17 @@ __global__ void __launch_bounds__(kGreedyThreads, 2) k_greedy(GreedyArgs a) {
                     mo = a.set_off[i];
                     ml = a.set_off[i + 1] - mo;
                 }
+                if (a.piece && ml > kGreedyPiece) {
+                    const int64_t np = (ml + kGreedyPiece - 1) / kGreedyPiece;
+                    unsigned long long *to = a.piece + atomicAdd(a.npiece, (unsigned long long)np);
+                    for (int64_t q = 0; q < np; ++q) {
+                        const int64_t left = ml - q * kGreedyPiece;
+                        to[q] = (unsigned long long)(mo + q * kGreedyPiece) << 16 |
+                                (unsigned long long)(left < kGreedyPiece ? left : kGreedyPiece) << 5 |
+                                (unsigned long long)(i & (kHubRep - 1));
+                    }
+                    ml = 0;
+                }
                 const int64_t incl = warp_incl_scan<int64_t>(ml, lane);
                 const int64_t tot = __shfl_sync(kFull, incl, 31);
                 constexpr int U = 4;
@@ -341,21 +370,34 @@ __global__ void __launch_bounds__(kGreedyThreads, 2) k_greedy(GreedyArgs a) {
                         mv[uu] = q < tot ? __ldg(a.members + o_mo + (q - (o_incl - o_ml))) : -1;
                     }
 #pragma unroll
-                    for (int uu = 0; uu < U; ++uu) {
-                        if (mv[uu] < 0) continue;
-                        const int64_t u = mv[uu] - a.vshift;
-                        const int32_t hr = a.hub_rank ? __ldcg(a.hub_rank + u) : -1;
-                        if (hr >= 0)
-                            red_add_s32(a.hub_cnt + (int64_t)hr * kHubRep + (ms[uu] & (kHubRep - 1)),
-                                        -1);
-                        else if (hr == -1)
-                            red_add_s32(a.counts + slot(u), -1);   // -2: frozen
-                    }
+                    for (int uu = 0; uu < U; ++uu)
+                        if (mv[uu] >= 0) decrement(mv[uu], ms[uu] & (kHubRep - 1));
                 }
             }
             if (!work) base += nwarps * kGreedyChunk;
         }
         if (!grid_sync(a.bar, nb, a.status)) return;
+        const int64_t np = a.piece ? (int64_t)__ldcg(a.npiece) : 0;
+        if (np > 0) {                                // (grid-uniform)
+            for (int64_t p = gwarp; p < np; p += nwarps) {
+                const unsigned long long pc = __ldcg(a.piece + p);
+                const int32_t *mem = a.members + (pc >> 16);
+                const int len = (int)(pc >> 5 & 2047), rep = (int)(pc & (kHubRep - 1));
+                constexpr int U = 8;
+                for (int x0 = lane; x0 < len; x0 += 32 * U) {
+                    int32_t mv[U];
+#pragma unroll
+                    for (int uu = 0; uu < U; ++uu)
+                        mv[uu] = x0 + uu * 32 < len ? __ldg(mem + x0 + uu * 32) : -1;
+#pragma unroll
+                    for (int uu = 0; uu < U; ++uu)
+                        if (mv[uu] >= 0) decrement(mv[uu], rep);
+                }
+            }
+            if (!grid_sync(a.bar, nb, a.status)) return;
+            // (the next pieces are put aside after the next barrier)
+            if (blockIdx.x == 0 && threadIdx.x == 0) *a.npiece = 0ull;
+        }
         ++j;
     }
     if (blockIdx.x == 0 && threadIdx.x == 0) {
@@ -1386,14 +1428,15 @@ im_status greedy_plain(im_pool *p, int32_t k, int32_t *d_seeds, int64_t *d_gains
                  o_best = take((size_t)grid * 8), o_bar = take(sizeof(GridBarrier)),
                  o_work = take(16), o_hrank = take((size_t)n * 4),
                  o_hcnt = take((size_t)kHubCap * kHubRep * 4), o_hlist = take((size_t)kHubCap * 4),
-                 o_cand = take((size_t)n * 4), o_ctl = take(16);
+                 o_cand = take((size_t)n * 4), o_ctl = take(32),
+                 o_piece = take((size_t)(2 * p->total / kGreedyPiece + 1) * 8);
     void *base = nullptr;
     im_status s = pool_scratch(p, off, &base);
     if (s != IM_OK) return s;
     char *B = (char *)base;
     IM_CUDA(cudaMemsetAsync(B + o_bar, 0, sizeof(GridBarrier), st));
     IM_CUDA(cudaMemsetAsync(B + o_work, 0, 16, st));
-    IM_CUDA(cudaMemsetAsync(B + o_ctl, 0, 16, st));
+    IM_CUDA(cudaMemsetAsync(B + o_ctl, 0, 32, st));
     IM_CUDA(cudaMemsetAsync(d_nseeds, 0, sizeof(int32_t), st));
     IM_CUDA(cudaMemsetAsync(d_cov, 0, sizeof(int64_t), st));
     GreedyArgs a;
@@ -1424,6 +1467,8 @@ im_status greedy_plain(im_pool *p, int32_t k, int32_t *d_seeds, int64_t *d_gains
     a.hub_shift = kHubShift;
     a.cand_shift = cand_shift;
     a.work = (unsigned long long *)(B + o_work);
+    a.piece = (unsigned long long *)(B + o_piece);
+    a.npiece = (unsigned long long *)(B + o_ctl + 16);
     void *args[] = {&a};
     KernelTimer kt(st, "greedy");
     IM_CUDA(cudaLaunchCooperativeKernel((const void *)k_greedy, dim3(grid), dim3(kGreedyThreads),
