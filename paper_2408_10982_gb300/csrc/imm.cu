@@ -187,7 +187,7 @@ im_status im_solve(const im_graph *g, im_model model, int32_t k, double eps, dou
     }
     int32_t *d_seeds = (int32_t *)res;
     int64_t *d_gains = (int64_t *)((char *)res + (((size_t)k * 4 + 15) & ~(size_t)15));
-    int64_t *d_cov = (int64_t *)((char *)res + (size_t)k * 12 + 128);
+    int64_t *d_cov = (int64_t *)((char *)res + (((size_t)k * 12 + 128 + 15) & ~(size_t)15));
     int32_t *d_ns = (int32_t *)((char *)d_cov + 8);
     int *d_status = (int *)((char *)d_cov + 16);
 
