@@ -74,6 +74,7 @@ struct SampleArgs {
     int32_t *hand;            // their members
     int64_t hand_cap;
     unsigned long long *hand_cursor;
+    uint2 *recs;              // LT walks: {sample, first entry} of finished walks, [warp][k][lane]
     unsigned long long *nlong;    // sets longer than kWarpSortKeys, plus 2^32 for every
                                   // unsorted one longer than kBlockSortCap
     uint32_t rk[20];          // Philox round keys of the launch's query, when it has only one
@@ -134,12 +135,13 @@ constexpr uint32_t kICWideEdges = 1u << 16;
 constexpr int32_t kICWarpFront = 1024;
 constexpr int64_t kICHandCap = 1 << 23;      // members handed over to the second pass (32 MB)
 
-// The coins of one sample: Philox4x32-10 of counter (s, g, 0, coin tag), with
-// what does not depend on g computed by begin().  KEYS: the round keys come
-// from rk (kernel parameters, so constant-bank operands); else they are
-// derived from k0, k1 as the rounds go.
-template <bool KEYS>
-struct CoinStream {
+// One sample's draws of one kind (TAG: coins of edge group g, or the LT pick of
+// vertex g): Philox4x32-10 of counter (s, g, 0, TAG), with what does not depend
+// on g computed by begin().  KEYS: the round keys come from rk (kernel
+// parameters, so constant-bank operands); else they are derived from k0, k1 as
+// the rounds go.
+template <uint32_t TAG, bool KEYS>
+struct DrawStream {
     uint32_t k0, k1;
     uint32_t gx, c1, ca, cb, cc;
     __device__ __forceinline__ uint32_t K0(const uint32_t *rk, int r) const {
@@ -153,7 +155,7 @@ struct CoinStream {
         k0 = key0;
         k1 = key1;
         gx = K0(rk, 0);                                           // round 0: x = g ^ gx
-        const uint32_t z1 = __umulhi(0xD2511F53u, s) ^ kStreamCoin ^ K1(rk, 0);
+        const uint32_t z1 = __umulhi(0xD2511F53u, s) ^ TAG ^ K1(rk, 0);
         c1 = (0xD2511F53u * s) ^ K1(rk, 1);                       // round 1: z = hi(a) ^ c1
         const uint32_t x2 = __umulhi(0xCD9E8D57u, z1) ^ K0(rk, 1);
         ca = (0xCD9E8D57u * z1) ^ K0(rk, 2);                      // round 2: x = hi(b) ^ ca
@@ -181,6 +183,11 @@ struct CoinStream {
         return x;
     }
 };
+
+template <bool KEYS>
+using CoinStream = DrawStream<kStreamCoin, KEYS>;
+template <bool KEYS>
+using PickStream = DrawStream<kStreamPick, KEYS>;
 
 // What a warp expands: the in-edge lists of up to 32 vertices, one per lane.
 struct ICItem {
@@ -1009,24 +1016,50 @@ __global__ void __launch_bounds__(kSampleThreads, G == 32 ? 8 : 5) k_sample_lt(S
 // one dependent load: the source of in-edge floor(x / u) when all in-edges of
 // the vertex weigh u (1/in-degree weights, for one), else one guide entry (see
 // k_lt_guide), with a binary search over the running sums only when the draw
-// lies past the guide's edge.  The revisit test goes through a 1024-bit Bloom filter of
-// the walk in shared memory (two hashes); a walk whose pick hits the filter
-// waits (takes no step) until kLT1Flush walks of its warp wait, or every active
-// one does, and the whole warp then checks them exactly, scanning kLT1Group of
-// their paths together so that those loads are in flight at once.  Finished
-// walks are copied to the stage by the whole warp as well, kLT1Group paths at
-// a time, after one warp-wide reservation.
-// A warp takes sample indices kLT1Chunk at a time, and all its lanes then draw
-// the roots of that chunk together (one Philox call each) into a per-warp ring
-// in shared memory, from which a lane starting a walk reads its root.
+// lies past the guide's edge.
+//
+// The two dependent loads are what a step cannot do without; a warp hides them
+// behind the other 31 of its SM.  Everything else a walk needs -- its start, the
+// check for a revisit, its way to the stage -- happens once in tens of steps of
+// a lane, but with 32 lanes nearly every iteration has some lane at one of them,
+// and each costs a warp a round trip to L2.  So each is put off until it serves
+// many lanes or many walks:
+//   - A warp takes sample indices kLT1Chunk at a time; its lanes draw the roots
+//     and look at their records together, write the sets of roots without
+//     in-edges (half of an R-MAT graph) at once, and keep the others in a ring in
+//     shared memory.  Lanes without a walk wait until kLT1Refill of them do.
+//   - A revisit is noticed by a 1024-bit Bloom filter of the walk in shared
+//     memory (two hashes).  The walk goes on: after a true revisit it repeats
+//     its cycle (a vertex's pick is the same in the whole sample), so the next
+//     source is in the filter too, and a source that is not proves the hit before
+//     it false.  Only after two hits in a row is the first one checked, exactly,
+//     by the whole warp over the walk's path, two walks at a time.
+//   - Finished walks stay in the lane's buffer, one behind the other, and are
+//     moved to the stage when some lane has kLT1Flush members of them: one
+//     reservation and one coalesced copy of all the lanes' finished walks.
 // Waiting changes no draw: a walk's steps are the same whenever they run.
+//
+// Measured at 4,194,304 sets on R-MAT scale 20 with 1/in-degree weights (1.7 x
+// 10^8 steps): 4.14 + 0.98 -> 3.7 ms, the 0.98 a second pass for walks longer
+// than the 512 entries a lane had; U[0, 0.1] weights (1.6 x 10^7 members) 1.51 ->
+// 0.80 ms.  What is left is the two random reads: ncu shows 12.8 instructions a
+// step (19.2), issue 41 % busy, half of the reads missing L2, and 24 warps an SM
+// only 4 % slower than 32.  Not kept: 16-byte in-edge records (source and its
+// vertex record) for one read a step: 4.76 ms, every one of them from DRAM (268
+// MB against 84 MB of records and sources); five blocks an SM (spills) 5.4 ms;
+// streaming stores to the stage, kLT1Flush 64 to 384, kLT1Refill 2 to 5,
+// kLT1Check 1 to 3: within 2 %.
 constexpr int kLT1Threads = 256;
 constexpr int kLT1Warps = kLT1Threads / 32;
 constexpr int kBloomWords = 32;              // 1024 bits per walk
-constexpr int64_t kQueueCapLT1 = 512;
+constexpr int64_t kQueueCapLT1 = 1024;       // entries of a lane's buffer at most
 constexpr unsigned kLT1Chunk = 32;           // sample indices a warp takes at once (one per lane)
-constexpr int kLT1Flush = 2;                 // flagged walks that trigger the exact checks
-constexpr int kLT1Group = 2;                 // paths scanned or copied together
+constexpr int kLT1Refill = 3;                // lanes without a walk that start new ones
+constexpr int kLT1Check = 2;                 // walks waiting for an exact check that start it
+constexpr int kLT1Group = 2;                 // paths scanned together
+constexpr int kLT1Flush = 192;               // finished members of a lane that start a flush
+constexpr int kLT1Recs = 32;                 // finished walks a lane keeps at most
+constexpr int kLT1Blocks = 4;                // blocks an SM
 // The work items of one launch stay below this count, so that the warp's chunk
 // bounds fit 32 bits (a larger job takes the grouped kernel).
 constexpr int64_t kLT1MaxCount = (1ll << 32) - (1ll << 28);
@@ -1072,160 +1105,214 @@ __device__ __forceinline__ uint64_t l2_policy_evict_first() {
 // CP (IM_TUNE_LT_CACHE): 0 plain loads; 1 the vertex records (n x 16 B, read
 // at every step) are kept in L2 ahead of other lines (evict_last); 2 as 1, and
 // the cut points (m x 16 B, mostly single-use) leave L2 first (evict_first).
-// Launched with a.count <= kLT1MaxCount.  Four blocks per SM: the 63 registers
-// the grouped scans want, with no spills (five blocks at 48 registers measured
-// slower).
-template <int CP>
-__global__ void __launch_bounds__(kLT1Threads, 4) k_sample_lt1(SampleArgs a) {
+// KEYS: the launch has one query, whose round keys are in the arguments.
+// Launched with a.count <= kLT1MaxCount.
+// A lane's buffer (a.qcap entries): finished walks in [fb, wb), the current one
+// in [wb, wb + len); its finished walks' {sample, first entry} in a.recs.
+template <int CP, bool KEYS>
+__global__ void __launch_bounds__(kLT1Threads, kLT1Blocks) k_sample_lt1(const __grid_constant__ SampleArgs a) {
     extern __shared__ uint32_t bloom[];          // [kBloomWords][kLT1Threads]
-    // roots, sample ids and query indices of the warp's last two chunks
-    __shared__ uint32_t ring_root[kLT1Warps][2 * kLT1Chunk];
-    __shared__ uint32_t ring_s[kLT1Warps][2 * kLT1Chunk];
-    __shared__ int32_t ring_q[kLT1Warps][2 * kLT1Chunk];
-    // per warp: examined edges and algorithmic bytes of its finished walks
-    __shared__ unsigned long long wsum[kLT1Warps][2];
+    // drawn roots with in-edges, their sample ids, indices and queries
+    constexpr uint32_t kRing = 2 * kLT1Chunk;
+    __shared__ uint32_t ring_root[kLT1Warps][kRing], ring_s[kLT1Warps][kRing], ring_j[kLT1Warps][kRing];
+    __shared__ int32_t ring_q[kLT1Warps][kRing];
     const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
+    const unsigned lt = (1u << lane) - 1u;
     uint32_t *bl = bloom + threadIdx.x;
-    int32_t *q = a.queues + ((int64_t)blockIdx.x * kLT1Threads + threadIdx.x) * a.qcap;
-    if (lane == 0) {
-        wsum[wib][0] = 0ull;
-        wsum[wib][1] = 0ull;
-    }
-    // with one query in the launch, every walk has the same graph and key
-    const bool one_query = a.nq == 1;
-    const uint4 *vrec = one_query ? a.qv[0].lt_vrec : nullptr;
-    const int32_t *srcs = one_query ? a.qv[0].in_src : nullptr;
-    uint32_t k0 = one_query ? seed_lo(a.qv[0].seed) : 0u;
-    uint32_t k1 = one_query ? seed_hi(a.qv[0].seed) : 0u;
-    bool active = false, exhausted = false;
-    bool pend = false;                           // waiting for an exact revisit check of u
-    uint32_t j = 0, s = 0, cur = 0, u = 0;
-    int32_t qi = 0, len = 0;
-    unsigned long long sexam = 0;
-    uint32_t sbytes = 0;
-    // the warp's current chunk is [wend - kLT1Chunk, wend); [wnext, wend) is not
-    // taken yet; the chunk's roots are in half `half` of the ring (warp-uniform)
-    uint32_t wnext = 0, wend = 0;
-    int half = 1;
-    __syncwarp();
+    const int32_t cap = (int32_t)a.qcap;
+    const int64_t warp_id = (int64_t)blockIdx.x * kLT1Warps + wib;
+    int32_t *q = a.queues + (warp_id * 32 + lane) * a.qcap;
+    uint2 *recs = a.recs + warp_id * 32 * kLT1Recs + lane;
+    const uint4 *vrec = a.qv[0].lt_vrec;
+    const int32_t *srcs = a.qv[0].in_src;
+    PickStream<KEYS> ps;
+    bool active = false, pend = false, exhausted = false;
+    uint32_t j = 0, cur = 0;
+    int32_t qi = 0, len = 0, fb = 0, wb = 0, nrec = 0;
+    // hits: filter hits in a row at the end of the path (0 to 2); the first of
+    // them is path entry `hit`.  What the steps from there on examined and moved
+    // counts only once the hit is known to be false (pexam, pbytes).
+    int32_t hits = 0, hit = 0;
+    unsigned long long sexam = 0, pexam = 0, tot_exam = 0, tot_bytes = 0;
+    uint32_t sbytes = 0, pbytes = 0;
+    uint32_t rhead = 0, rcnt = 0;                // the ring (warp-uniform)
     for (;;) {
-        // ---- lanes without a walk take the next samples of the warp's chunk
-        const bool want = !active && !exhausted;
-        const unsigned need = __ballot_sync(kFull, want);
-        if (need) {
-            const uint32_t nneed = (uint32_t)__popc(need);
-            const uint32_t rank = (uint32_t)__popc(need & ((1u << lane) - 1u));
-            const uint32_t avail = wend - wnext;
-            uint32_t jw = wnext + rank;
-            uint32_t cb = wend - kLT1Chunk;          // first index of jw's chunk
-            int hw = half;                           // and the ring half holding it
-            if (avail < nneed) {                     // the rest of this chunk, then a new one
-                unsigned long long nb64 = 0;
-                if (lane == 0) nb64 = atomicAdd(a.work, (unsigned long long)kLT1Chunk);
-                const uint32_t nb = (uint32_t)__shfl_sync(kFull, nb64, 0);
-                half ^= 1;
-                const uint32_t jc = nb + (uint32_t)lane;
-                if ((int64_t)jc < a.count) {         // lane draws the root of sample nb + lane
-                    const int64_t jj = a.list ? a.list[jc] : (int64_t)jc;
-                    const int qc = one_query ? 0 : find_query(a, jj);
-                    const QueryView &V = a.qv[qc];
-                    const uint32_t sc = V.first + (uint32_t)(jj - __ldg(a.qstart + qc));
-                    ring_root[wib][half * kLT1Chunk + lane] = rrr_root(V.seed, sc, V.n);
-                    ring_s[wib][half * kLT1Chunk + lane] = sc;
-                    ring_q[wib][half * kLT1Chunk + lane] = qc;
-                }
-                __syncwarp();
-                if (rank >= avail) {
-                    jw = nb + (rank - avail);
-                    cb = nb;
-                    hw = half;
-                }
-                wnext = nb + (nneed - avail);
-                wend = nb + kLT1Chunk;
-            } else {
-                wnext += nneed;
-            }
-            if (want) {
-                if ((int64_t)jw < a.count) {
-                    const int e = hw * (int)kLT1Chunk + (int)(jw - cb);
-                    j = a.list ? (uint32_t)a.list[jw] : jw;
-                    cur = ring_root[wib][e];
-                    s = ring_s[wib][e];
-                    qi = ring_q[wib][e];
-                    if (!one_query) {
-                        const QueryView &V = a.qv[qi];
-                        vrec = V.lt_vrec;
-                        srcs = V.in_src;
-                        k0 = seed_lo(V.seed);
-                        k1 = seed_hi(V.seed);
-                    }
-                    q[0] = (int32_t)cur;
-#pragma unroll
-                    for (int w = 0; w < kBloomWords; ++w) bl[w * kLT1Threads] = 0u;
-                    bloom_add(bl, cur);
-                    len = 1;
-                    sexam = 0;
-                    sbytes = 8u + 4u;                // set offset, root write
-                    active = true;
-                } else {
+        // ---- lanes without a walk take the next drawn roots
+        const unsigned idle = __ballot_sync(kFull, !active);
+        if (idle == kFull && exhausted && rcnt == 0) break;
+        if ((__popc(idle) >= kLT1Refill || idle == kFull) && (rcnt > 0 || !exhausted)) {
+            if (rcnt < (uint32_t)__popc(idle) && !exhausted) {
+                unsigned long long nb = 0;
+                if (lane == 0) nb = atomicAdd(a.work, (unsigned long long)kLT1Chunk);
+                nb = __shfl_sync(kFull, nb, 0);
+                if (nb >= (unsigned long long)a.count) {
                     exhausted = true;
+                } else {
+                    const int64_t jc = (int64_t)nb + lane;
+                    const bool have = jc < a.count;
+                    uint32_t root = 0, sc = 0, d = 0;
+                    int qc = 0;
+                    if (have) {
+                        qc = KEYS ? 0 : find_query(a, jc);
+                        const QueryView &V = a.qv[qc];
+                        sc = V.first + (uint32_t)(jc - __ldg(a.qstart + qc));
+                        root = rrr_root(V.seed, sc, V.n);
+                        d = __ldg(reinterpret_cast<const uint32_t *>(V.lt_vrec + root) + 1);
+                    }
+                    // roots without in-edges are sets of their own
+                    const unsigned sm = __ballot_sync(kFull, have && d == 0u);
+                    if (sm) {
+                        unsigned long long pos = 0;
+                        if (lane == 0) pos = atomicAdd(a.stage_cursor, (unsigned long long)__popc(sm));
+                        pos = __shfl_sync(kFull, pos, 0);
+                        if (have && d == 0u) {
+                            const int64_t at = (int64_t)pos + __popc(sm & lt);
+                            if (at < a.stage_cap) {
+                                a.stage[at] = (int32_t)root;
+                                a.stage_off[jc] = at;
+                                a.sizes[jc] = 1;
+                                tot_bytes += 8u + 4u + 16u;   // set offset, root write, record
+                            } else {
+                                raise_status(a.status, kDevStageOverflow);
+                            }
+                        }
+                    }
+                    const unsigned wm = __ballot_sync(kFull, have && d != 0u);
+                    if (have && d != 0u) {
+                        const uint32_t e = (rhead + rcnt + (uint32_t)__popc(wm & lt)) & (kRing - 1);
+                        ring_root[wib][e] = root;
+                        ring_s[wib][e] = sc;
+                        ring_j[wib][e] = (uint32_t)jc;
+                        if (!KEYS) ring_q[wib][e] = qc;
+                    }
+                    rcnt += (uint32_t)__popc(wm);
+                    __syncwarp();
                 }
             }
+            const uint32_t rank = (uint32_t)__popc(idle & lt);
+            if (!active && rank < rcnt) {
+                const uint32_t e = (rhead + rank) & (kRing - 1);
+                cur = ring_root[wib][e];
+                j = ring_j[wib][e];
+                if (KEYS) {
+                    ps.begin(a.rk, ring_s[wib][e], 0u, 0u);
+                } else {
+                    qi = ring_q[wib][e];
+                    const QueryView &V = a.qv[qi];
+                    vrec = V.lt_vrec;
+                    srcs = V.in_src;
+                    ps.begin(a.rk, ring_s[wib][e], seed_lo(V.seed), seed_hi(V.seed));
+                }
+                if (fb == wb) fb = wb = 0;           // nothing finished is left in the buffer
+                q[wb] = (int32_t)cur;
+#pragma unroll
+                for (int w = 0; w < kBloomWords; ++w) bl[w * kLT1Threads] = 0u;
+                bloom_add(bl, cur);
+                len = 1;
+                hits = 0;
+                sexam = pexam = 0;
+                pbytes = 0;
+                sbytes = 8u + 4u;                    // set offset, root write
+                active = true;
+            }
+            const uint32_t took = min(rcnt, (uint32_t)__popc(idle));
+            rhead += took;
+            rcnt -= took;
+            __syncwarp();
         }
-        if (!__any_sync(kFull, active)) break;
 
-        // ---- one step of every active walk that is not waiting for its revisit check
-        bool ending = false, accept = false;
+        // ---- one step of every walk that is not waiting for its exact check
+        bool ending = false;
         if (active && !pend) {
-            const uint32_t x = philox4x32_10(make_uint4(s, cur, 0u, kStreamPick), k0, k1).x;
+            const uint32_t x = ps(a.rk, cur).x;
+            uint32_t u = 0, e = 0xffffffffu;         // the pick: source and index
+            uint32_t stepb = 16u;                    // vertex record
             // (the L2 policies are made where they are used: one instruction,
             // and no registers held across the loop)
             const uint4 vr =
                 CP >= 1 ? ldg_policy(vrec + cur, l2_policy_evict_last()) : __ldg(vrec + cur);
             const uint32_t d = vr.y;
-            int64_t e = -1;
-            sbytes += 16u;                           // vertex record
-            if (vr.w != 0u) {                        // equal in-weights: edge floor(x / weight)
-                const uint32_t ei = x / vr.w;
+            if (vr.w != 0u) {
+                // equal in-weights: edge floor(x / weight), from the reciprocal in
+                // the record, at most 2 too small
+                uint32_t ei = __umulhi(x, vr.z), rem = x - ei * vr.w;
+                if (rem >= vr.w) { ++ei; rem -= vr.w; }
+                if (rem >= vr.w) ++ei;
                 if (ei < d) {
                     e = ei;
                     u = (uint32_t)__ldg(srcs + vr.x + ei);
-                    sbytes += 4u;                    // source of the pick
+                    stepb += 4u;                     // source of the pick
                 }
             } else if (d > 0) {
                 const QueryView &V = a.qv[qi];
                 const uint4 *gp = V.lt_guide + vr.x + __umulhi(x, d);
                 const uint4 gv = CP >= 2 ? ldg_policy(gp, l2_policy_evict_first()) : __ldg(gp);
                 const unsigned long long cum = ((unsigned long long)gv.y << 32) | gv.x;
-                sbytes += 16u;                       // cut point
+                stepb += 16u;                        // cut point
                 if ((unsigned long long)x < cum) {
                     e = gv.w;
                     u = gv.z;
                 } else {
-                    const unsigned long long *leaf = V.lt_leaf;
-                    uint32_t lo = gv.w + 1, hi = d;  // first edge past the guide's with x < sum
+                    // the first edge past the guide's with x < sum: with unequal
+                    // weights that is about every second draw, and mostly the next
+                    // edge, so the search doubles its stride from there (halving
+                    // all that is left of the list read log2 d scattered sums)
+                    const unsigned long long *leaf = V.lt_leaf + vr.x;
+                    uint32_t lo = gv.w + 1, hi = d, stride = 1;
+                    unsigned long long at = 0;       // the sum and source of edge hi < d
                     while (lo < hi) {
-                        const uint32_t mid = (lo + hi) >> 1;
-                        if ((unsigned long long)x < (__ldg(leaf + vr.x + mid) >> 31)) hi = mid;
-                        else lo = mid + 1;
-                        sbytes += 8u;                // search probe
+                        const uint32_t p = hi < d ? (lo + hi) >> 1 : min(lo + stride - 1u, d - 1u);
+                        const unsigned long long r = __ldg(leaf + p);
+                        stepb += 8u;                 // search probe
+                        if ((unsigned long long)x < (r >> 31)) {
+                            hi = p;
+                            at = r;
+                        } else {
+                            lo = p + 1;
+                        }
+                        stride <<= 1;
                     }
-                    if (lo < d) {
-                        e = lo;
-                        u = (uint32_t)(__ldg(leaf + vr.x + lo) & 0x7fffffffull);
-                        sbytes += 8u;                // picked leaf
+                    if (hi < d) {
+                        e = hi;
+                        u = (uint32_t)(at & 0x7fffffffull);
+                        stepb += 8u;                 // picked leaf
                     }
                 }
             }
-            sexam += e >= 0 ? (unsigned long long)(e + 1) : (unsigned long long)d;
-            if (e < 0) ending = true;                // no in-edge picked: the walk stops
-            else if (bloom_has(bl, u)) pend = true;  // maybe a revisit: check exactly
-            else accept = true;
+            if (e == 0xffffffffu) {                  // no in-edge picked: the walk stops, and
+                sexam += pexam + d;                  // hits before this were false
+                sbytes += pbytes + stepb;
+                ending = true;
+            } else {
+                const unsigned long long stepx = (unsigned long long)e + 1ull;
+                if (!bloom_has(bl, u)) {             // a new vertex, so earlier hits were false
+                    sexam += pexam + stepx;
+                    sbytes += pbytes + stepb + 4u;   // ... and a member write
+                    pexam = 0;
+                    pbytes = 0;
+                    hits = 0;
+                    bloom_add(bl, u);
+                } else if (hits == 0) {              // maybe a revisit, which this step found
+                    sexam += stepx;
+                    sbytes += stepb;
+                    pbytes = 4u;
+                    hits = 1;
+                    hit = len;
+                } else {                             // again: check the first
+                    pexam = stepx;
+                    pbytes += stepb + 4u;
+                    pend = true;
+                }
+                q[wb + len] = (int32_t)u;            // (room: see the end of the loop)
+                ++len;
+                cur = u;
+            }
         }
-        // ---- exact revisit checks of the flagged walks, once kLT1Flush of them wait
-        // (or every active walk does); kLT1Group paths are scanned together
+        // ---- exact checks of the walks that wait for one, once kLT1Check do (or
+        // every active walk does): is path entry `hit` among those before it?
         const unsigned pm = __ballot_sync(kFull, pend);
-        if (pm && (__popc(pm) >= kLT1Flush || pm == __ballot_sync(kFull, active))) {
+        if (pm && (__popc(pm) >= kLT1Check || pm == __ballot_sync(kFull, active && !ending))) {
+            __syncwarp();                            // the paths are read across lanes
             bool seen = false;
             unsigned rest = pm;
             do {
@@ -1235,12 +1322,13 @@ __global__ void __launch_bounds__(kLT1Threads, 4) k_sample_lt1(SampleArgs a) {
                     l[g] = rest ? __ffs(rest) - 1 : l[0];
                     rest &= rest - 1u;
                 }
-                int32_t ug[kLT1Group], lg[kLT1Group];
+                int32_t lg[kLT1Group], at[kLT1Group], ug[kLT1Group];
                 int32_t lmax = 0;
 #pragma unroll
                 for (int g = 0; g < kLT1Group; ++g) {
-                    ug[g] = __shfl_sync(kFull, (int32_t)u, l[g]);
-                    lg[g] = __shfl_sync(kFull, len, l[g]);
+                    lg[g] = __shfl_sync(kFull, hit, l[g]);
+                    at[g] = __shfl_sync(kFull, wb, l[g]);
+                    ug[g] = __ldcg(q + (int64_t)(l[g] - lane) * a.qcap + at[g] + lg[g]);
                     lmax = max(lmax, lg[g]);
                 }
                 bool f[kLT1Group];
@@ -1250,7 +1338,7 @@ __global__ void __launch_bounds__(kLT1Threads, 4) k_sample_lt1(SampleArgs a) {
                     int32_t v[kLT1Group];
 #pragma unroll
                     for (int g = 0; g < kLT1Group; ++g)      // lane l[g]'s path entry i
-                        v[g] = i < lg[g] ? __ldcg(q + (int64_t)(l[g] - lane) * a.qcap + i) : -1;
+                        v[g] = i < lg[g] ? __ldcg(q + (int64_t)(l[g] - lane) * a.qcap + at[g] + i) : -1;
 #pragma unroll
                     for (int g = 0; g < kLT1Group; ++g) f[g] |= v[g] == ug[g];
                 }
@@ -1261,94 +1349,142 @@ __global__ void __launch_bounds__(kLT1Threads, 4) k_sample_lt1(SampleArgs a) {
                 }
             } while (rest);
             if (pend) {
-                if (seen) ending = true;             // a revisit: the walk stops
-                else accept = true;
                 pend = false;
+                if (seen) {                          // a revisit: the walk stopped before it
+                    len = hit;
+                    ending = true;
+                } else {                             // a new vertex; the hit after it is now the first
+                    sexam += pexam;
+                    sbytes += pbytes - 4u;
+                    pexam = 0;
+                    pbytes = 4u;
+                    ++hit;
+                }
             }
         }
-        bool ovf = false;
-        if (accept) {
-            if (len < a.qcap) {
-                q[len] = (int32_t)u;
-                bloom_add(bl, u);
-                ++len;
-                sbytes += 4u;                        // member write
-                cur = u;
-            } else {
-                ovf = true;                          // longer than the queue: second pass
-                ending = true;
-                a.sizes[j] = -1;
-                a.stage_off[j] = 0;
-                a.ovf_list[atomicAdd(a.ovf_count, 1ull)] = (int64_t)j;
-            }
+        if (ending) {                                // stays in the buffer
+            a.sizes[j] = len;
+            recs[nrec * 32] = make_uint2(j, (uint32_t)wb);
+            ++nrec;
+            wb += len;
+            tot_exam += sexam;
+            tot_bytes += sbytes;
+            active = false;
+            len = 0;
         }
-        // ---- finished walks go to the stage, kLT1Group paths copied together
-        const bool emit = ending && !ovf;
-        unsigned em = __ballot_sync(kFull, emit);
-        if (em) {
-            const int32_t my = emit ? len : 0;
-            const int32_t incl = warp_incl_scan<int32_t>(my, lane);
-            const int32_t tot = __shfl_sync(kFull, incl, 31);
+        // ---- the finished walks of all lanes go to the stage when one lane has many
+        // of them, or has no room for its next member (without a walk: for a root
+        // and the member after it)
+        const bool tight = wb + len + (active ? 0 : 1) >= cap;
+        if (__any_sync(kFull, wb - fb >= kLT1Flush || nrec == kLT1Recs || tight)) {
+            __syncwarp();                            // the buffers are read across lanes
+            const int32_t mine = wb - fb;
+            const int32_t upto = warp_incl_scan<int32_t>(mine, lane), excl = upto - mine;
+            const int32_t tot = __shfl_sync(kFull, upto, 31);
             unsigned long long base = 0;
             if (lane == 0) base = atomicAdd(a.stage_cursor, (unsigned long long)tot);
             base = __shfl_sync(kFull, base, 0);
-            const bool fits = (int64_t)base + tot <= a.stage_cap;
-            if (emit) {
-                if (fits) {
-                    a.stage_off[j] = (int64_t)base + incl - my;
-                    a.sizes[j] = len;
-                    atomicAdd(&wsum[wib][0], sexam);
-                    atomicAdd(&wsum[wib][1], (unsigned long long)sbytes);
-                } else {
-                    raise_status(a.status, kDevStageOverflow);
-                    a.sizes[j] = 0;
-                    a.stage_off[j] = 0;
+            if ((int64_t)base + tot <= a.stage_cap) {
+                const int32_t most = __reduce_max_sync(kFull, nrec);
+#pragma unroll 4
+                for (int32_t k = 0; k < most; ++k)
+                    if (k < nrec) {
+                        const uint2 r = __ldcg(recs + k * 32);
+                        a.stage_off[r.x] = (int64_t)base + excl + ((int32_t)r.y - fb);
+                    }
+                const int64_t from = fb - excl;      // the lane's entry for position 0
+                constexpr int U = 4;
+                for (int32_t t0 = 0; t0 < tot; t0 += 32 * U) {
+                    int32_t v[U];
+#pragma unroll
+                    for (int uu = 0; uu < U; ++uu) {
+                        const int32_t t = t0 + uu * 32 + lane;
+                        int owner = 0;               // first lane whose inclusive count exceeds t
+#pragma unroll
+                        for (int step = 16; step > 0; step >>= 1)
+                            if (__shfl_sync(kFull, upto, owner + step - 1) <= t) owner += step;
+                        const int64_t o_from = __shfl_sync(kFull, from, owner);
+                        v[uu] = t < tot ? __ldcg(q + (int64_t)(owner - lane) * a.qcap + o_from + t) : 0;
+                    }
+#pragma unroll
+                    for (int uu = 0; uu < U; ++uu) {
+                        const int32_t t = t0 + uu * 32 + lane;
+                        if (t < tot) a.stage[(int64_t)base + t] = v[uu];
+                    }
                 }
+            } else if (lane == 0) {
+                raise_status(a.status, kDevStageOverflow);
             }
-            if (fits) {
-                __syncwarp();
-                do {
-                    int l[kLT1Group];
-#pragma unroll
-                    for (int g = 0; g < kLT1Group; ++g) {
-                        l[g] = em ? __ffs(em) - 1 : l[0];
-                        em &= em - 1u;
+            fb = wb;
+            nrec = 0;
+            // lanes without room: the current walk moves to the front of the
+            // buffer, or is longer than it (second pass)
+            unsigned full = __ballot_sync(kFull, tight && active);
+            while (full) {
+                const int l = __ffs(full) - 1;
+                full &= full - 1u;
+                const int32_t lw = __shfl_sync(kFull, wb, l), ln = __shfl_sync(kFull, len, l);
+                if (lw == 0) {
+                    if (lane == l) {
+                        a.sizes[j] = -1;
+                        a.stage_off[j] = 0;
+                        a.ovf_list[atomicAdd(a.ovf_count, 1ull)] = (int64_t)j;
+                        active = pend = false;
+                        len = 0;
                     }
-                    int32_t lg[kLT1Group], og[kLT1Group];
-                    int32_t lmax = 0;
-#pragma unroll
-                    for (int g = 0; g < kLT1Group; ++g) {
-                        lg[g] = __shfl_sync(kFull, len, l[g]);
-                        og[g] = __shfl_sync(kFull, incl - my, l[g]);   // offset from base
-                        lmax = max(lmax, lg[g]);
-                    }
-                    for (int32_t i = lane; i < lmax; i += 32) {
-                        int32_t v[kLT1Group];
-#pragma unroll
-                        for (int g = 0; g < kLT1Group; ++g)
-                            v[g] = i < lg[g] ? __ldcg(q + (int64_t)(l[g] - lane) * a.qcap + i) : 0;
-#pragma unroll
-                        for (int g = 0; g < kLT1Group; ++g)
-                            if (i < lg[g]) a.stage[(int64_t)base + og[g] + i] = v[g];
-                    }
-                } while (em);
+                    continue;
+                }
+                int32_t *b = q + (int64_t)(l - lane) * a.qcap;
+                for (int32_t i0 = 0; i0 < ln; i0 += 32) {   // (read before it is overwritten)
+                    const int32_t i = i0 + lane;
+                    const int32_t v = i < ln ? __ldcg(b + lw + i) : 0;
+                    __syncwarp();
+                    if (i < ln) b[i] = v;
+                    __syncwarp();
+                }
+                if (lane == l) fb = wb = 0;
             }
+            if (!active) fb = wb = 0;                // nothing is left in the buffer
         }
-        if (ending) active = false;
         __syncwarp();
     }
-    if (lane == 0) {
-        if (wsum[wib][0]) atomicAdd(a.examined, wsum[wib][0]);
-        if (wsum[wib][1]) atomicAdd(a.alg_bytes, wsum[wib][1]);
+    // what the lanes still hold
+    {
+        const int32_t mine = wb - fb;
+        const int32_t upto = warp_incl_scan<int32_t>(mine, lane), excl = upto - mine;
+        const int32_t tot = __shfl_sync(kFull, upto, 31);
+        unsigned long long base = 0;
+        if (lane == 0 && tot) base = atomicAdd(a.stage_cursor, (unsigned long long)tot);
+        base = __shfl_sync(kFull, base, 0);
+        if ((int64_t)base + tot <= a.stage_cap) {
+            for (int32_t k = 0; k < nrec; ++k) {
+                const uint2 r = __ldcg(recs + k * 32);
+                a.stage_off[r.x] = (int64_t)base + excl + ((int32_t)r.y - fb);
+            }
+            for (int l = 0; l < 32; ++l) {
+                const int32_t n = __shfl_sync(kFull, mine, l), o = __shfl_sync(kFull, excl, l);
+                const int32_t f = __shfl_sync(kFull, fb, l);
+                for (int32_t i = lane; i < n; i += 32)
+                    a.stage[(int64_t)base + o + i] = __ldcg(q + (int64_t)(l - lane) * a.qcap + f + i);
+            }
+        } else if (lane == 0) {
+            raise_status(a.status, kDevStageOverflow);
+        }
     }
+    tot_exam = warp_sum<unsigned long long>(tot_exam);
+    tot_bytes = warp_sum<unsigned long long>(tot_bytes);
+    if (lane == 0 && tot_exam) atomicAdd(a.examined, tot_exam);
+    if (lane == 0 && tot_bytes) atomicAdd(a.alg_bytes, tot_bytes);
 }
 
-// LT search index.  vrec[v] = {eb, d, tree offset | L << 28, u} with L the
-// number of upper tree levels (tree offsets stay below 2^28 since m < 2^31) and
-// u the common weight of v's in-edges when they all carry the same nonzero
-// weight (0 otherwise).  For such a vertex the pick needs no table: the running
-// sum of edge i is (i + 1) u, so a draw x picks edge floor(x / u) when that is
-// below d and nothing otherwise.
+// LT search index.  vrec[v] = {eb, d, z, u} with u the common weight of v's
+// in-edges when they all carry the same nonzero weight (0 otherwise).  For such
+// a vertex the pick needs no table: the running sum of edge i is (i + 1) u, so a
+// draw x picks edge floor(x / u) when that is below d and nothing otherwise; z is
+// then floor((2^32 - 1) / u), which gives the quotient as the high word of x z,
+// at most 2 too small (x / u - x z / 2^32 < 1 + x / 2^32).  Otherwise z is the
+// tree offset | L << 28 with L the number of upper tree levels (tree offsets stay
+// below 2^28 since m < 2^31).
 // For vertex v with in-edges [eb, eb + d):
 //   leaf[e] = (sum of w over v's in-edges up to and including e) << 31 | src(e)
 // (the running sum is at most 2^32 for valid LT weights -- 33 bits -- and
@@ -1363,6 +1499,10 @@ __device__ __forceinline__ int64_t lt_tree_size(int64_t d) {
         total += d;
     }
     return total;
+}
+
+__device__ __forceinline__ uint4 lt_record(int64_t b, int64_t d, uint32_t tree, uint32_t w) {
+    return make_uint4((uint32_t)b, (uint32_t)d, w ? 0xffffffffu / w : tree, w);
 }
 
 // In-degree above which one block, not one warp, builds a vertex's running
@@ -1403,7 +1543,7 @@ __global__ void k_lt_index_small(const int64_t *in_off, const int32_t *in_src, c
         }
         if (c > (1ull << 32)) atomicExch(invalid, 1);
         if (d > 0 && !(same && w0 != 0u)) invalid[2] = 1;   // the cut points are needed
-        vrec[v] = make_uint4((uint32_t)b, (uint32_t)d, (uint32_t)tree_off[v], same ? w0 : 0u);
+        vrec[v] = lt_record(b, d, (uint32_t)tree_off[v], same ? w0 : 0u);
     }
 }
 
@@ -1437,8 +1577,7 @@ __global__ void k_lt_index(const int64_t *in_off, const int32_t *in_src, const u
         int L = 0;
         for (int64_t t = d; t > 32; t = (t + 31) >> 5) ++L;
         if (lane == 0)
-            vrec[v] = make_uint4((uint32_t)b, (uint32_t)d,
-                                 (uint32_t)tree_off[v] | ((uint32_t)L << 28), same ? w0 : 0u);
+            vrec[v] = lt_record(b, d, (uint32_t)tree_off[v] | ((uint32_t)L << 28), same ? w0 : 0u);
         __syncwarp();
         if (!leaf) continue;
         // upper levels, top-down
@@ -1503,8 +1642,7 @@ __global__ void __launch_bounds__(256) k_lt_index_block(
         int L = 0;
         for (int64_t t = d; t > 32; t = (t + 31) >> 5) ++L;
         if (tid == 0)
-            vrec[v] = make_uint4((uint32_t)b, (uint32_t)d,
-                                 (uint32_t)tree_off[v] | ((uint32_t)L << 28), same ? w0 : 0u);
+            vrec[v] = lt_record(b, d, (uint32_t)tree_off[v] | ((uint32_t)L << 28), same ? w0 : 0u);
         __syncthreads();   // every leaf of v written by the block is visible to it
         if (!leaf) continue;   // (block-uniform)
         unsigned long long *lvl = tree + tree_off[v];
@@ -2028,6 +2166,12 @@ QueryView query_view(const im_graph *g, uint64_t seed, uint64_t first) {
     return v;
 }
 
+static void (*lt1_kernel(int cache, bool one_key))(const SampleArgs) {
+    if (cache == 0) return one_key ? k_sample_lt1<0, true> : k_sample_lt1<0, false>;
+    if (cache == 1) return one_key ? k_sample_lt1<1, true> : k_sample_lt1<1, false>;
+    return one_key ? k_sample_lt1<2, true> : k_sample_lt1<2, false>;
+}
+
 // ---------------------------------------------------------------------------
 // One sampling launch over a table of queries (see SamplingJob).
 // ---------------------------------------------------------------------------
@@ -2049,9 +2193,7 @@ im_status run_sampling(const SamplingJob &job, const std::function<im_status(siz
     const int lt_cache = (int)tune_value(IM_TUNE_LT_CACHE);
     const bool lt1 = model == IM_LT && G == 1;      // one walk per thread
     const void *kern = model == IM_LT
-                           ? (G == 1    ? (lt_cache == 0   ? (const void *)k_sample_lt1<0>
-                                            : lt_cache == 1 ? (const void *)k_sample_lt1<1>
-                                                            : (const void *)k_sample_lt1<2>)
+                           ? (G == 1    ? (const void *)lt1_kernel(lt_cache, one_key)
                               : G == 8  ? (const void *)k_sample_lt<8>
                               : G == 16 ? (const void *)k_sample_lt<16>
                                         : (const void *)k_sample_lt<32>)
@@ -2076,8 +2218,10 @@ im_status run_sampling(const SamplingJob &job, const std::function<im_status(siz
     }
     const int64_t warps = (int64_t)blocks * (threads / 32);
     const int64_t slots = warps * (32 / G);           // one queue per walk in flight
-    const int64_t qcap = std::min<int64_t>(
-        n, lt1 ? kQueueCapLT1 : model == IM_LT ? kQueueCapLT : kQueueCapIC);
+    // (a walk of one thread goes up to two entries past its end)
+    const int64_t qcap =
+        lt1 ? std::min<int64_t>((n + 3 + 3) & ~(int64_t)3, kQueueCapLT1)
+            : std::min<int64_t>(n, model == IM_LT ? kQueueCapLT : kQueueCapIC);
 
     // scratch layout
     size_t off = 0;
@@ -2097,6 +2241,7 @@ im_status run_sampling(const SamplingJob &job, const std::function<im_status(siz
     const size_t o_handed = take(model == IM_IC ? (size_t)cnt * sizeof(Handed) : 0);
     const int64_t hand_cap = model == IM_IC ? std::min<int64_t>(kICHandCap, cnt * qcap) : 0;
     const size_t o_hand = take((size_t)hand_cap * 4);
+    const size_t o_recs = take(lt1 ? (size_t)slots * kLT1Recs * sizeof(uint2) : 0);
     const size_t o_q = take((size_t)slots * qcap * 4);
     const size_t o_vis = take(model == IM_IC && !smem_vis ? (size_t)warps * vis_words * 4 : 0);
     void *base = nullptr;
@@ -2137,6 +2282,7 @@ im_status run_sampling(const SamplingJob &job, const std::function<im_status(siz
     a.hand = (int32_t *)(B + o_hand);
     a.hand_cap = hand_cap;
     a.hand_cursor = ctr + 6;
+    a.recs = (uint2 *)(B + o_recs);
     a.nlong = ctr + 7;
     for (int r = 0; r < 10; ++r) {
         a.rk[2 * r] = one_key ? (uint32_t)job.views[0].seed + (uint32_t)r * 0x9E3779B9u : 0u;
@@ -2147,11 +2293,7 @@ im_status run_sampling(const SamplingJob &job, const std::function<im_status(siz
     auto launch = [&](int nblocks, int group) {
         KernelTimer kt(st, model == IM_LT ? "sample_lt" : "sample_ic");
         if (model == IM_LT) {
-            if (group == 1) {
-                if (lt_cache == 0) k_sample_lt1<0><<<nblocks, kLT1Threads, dyn_smem, st>>>(a);
-                else if (lt_cache == 1) k_sample_lt1<1><<<nblocks, kLT1Threads, dyn_smem, st>>>(a);
-                else k_sample_lt1<2><<<nblocks, kLT1Threads, dyn_smem, st>>>(a);
-            }
+            if (group == 1) lt1_kernel(lt_cache, one_key)<<<nblocks, kLT1Threads, dyn_smem, st>>>(a);
             else if (group == 8) k_sample_lt<8><<<nblocks, kSampleThreads, 0, st>>>(a);
             else if (group == 16) k_sample_lt<16><<<nblocks, kSampleThreads, 0, st>>>(a);
             else k_sample_lt<32><<<nblocks, kSampleThreads, 0, st>>>(a);
