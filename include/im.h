@@ -235,9 +235,9 @@ im_status im_pool_sample_bytes(const im_pool *p, int64_t *bytes);
  *                       it); -1 keeps the bitmaps in global memory (one block
  *                       per bucket).
  *   IM_TUNE_INDEX_REPLICAS  covering-subset build: 0 (default) a stable radix
- *                       sort of the (vertex, set id) pairs by vertex, 8 bits a
- *                       pass, with 12 bytes of pool scratch per member (set ids
- *                       come out ascending inside every S(v); without the
+ *                       sort of the (vertex, set id) pairs by vertex, up to 10
+ *                       bits a pass, with 0, 8 or 12 bytes of pool scratch per
+ *                       member (1, 2 or 3 passes; set ids come out ascending inside every S(v); without the
  *                       memory, the counting build with 4 replicas runs
  *                       instead); 1, 2, 4 or 8: a counting build, histogram
  *                       and scatter through per-vertex counters and cursors

@@ -1,11 +1,12 @@
 // index.cu -- covering subsets S(v) (Sec. 3.2) and the RandGreedi partition
 // structures (Alg. 3).
 //
-// S(v) is the transpose of the RRR CSR: a histogram of member ids, an
-// exclusive scan into vtx_off, and a scatter of set ids.  On one GPU this is
-// the paper's all-to-all shuffle of covering subsets (Alg. 3), done in place.
-// Set ids inside one S(v) land in atomic order; nothing downstream depends on
-// that order.
+// S(v) is the transpose of the RRR CSR.  On one GPU this is the paper's all-to-all
+// shuffle of covering subsets (Alg. 3), done in place: by a stable radix sort of
+// the (vertex, set id) pairs, or, as a tuning-knob alternative and without the
+// memory for it, by a histogram of member ids, an exclusive scan into vtx_off
+// and a scatter of set ids, which then land in atomic order inside one S(v)
+// (nothing downstream depends on that order).
 //
 // For RandGreedi every vertex gets a Philox label part(v) in [0, P); the
 // vertices of each part are listed in ascending id (part_off / part_vtx), and
@@ -105,16 +106,30 @@ __global__ void k_scatter(const int64_t *set_off, const int32_t *members, int64_
 //                 warp by warp, item by item, lanes in order), places them in
 //                 digit order there, and writes each digit's run to its offset
 //                 (consecutive threads write consecutive positions).
-// The first pass reads the members and derives each pair's set id from
-// set_off; the last writes the set ids to S(v) and the keys to a buffer from
-// which k_rx_bounds counts |S(v)| (start and end of every run of equal keys).
+// The first pass reads the members; a pair's set id is the number of set starts
+// up to its position, from a bitmap of the tile's set starts.  The last pass
+// writes the set ids to S(v) only, and adds |S(v)| up from the runs of equal keys
+// in its tiles.
+//
+// What bounds a pass is the ranking in shared memory (its 16 bytes a pair would
+// take 0.4 of its 1.4 ms at 1.7 x 10^8 pairs): instructions, bank conflicts and
+// the chain from item to item.  Hence digits of 10 bits: 2^20 vertices take two
+// passes, 2^10 one.  The peers of an item's digit come from ballots of its bits
+// or from __match_any_sync, which runs on a pipe of its own (75 % busy when it
+// found them all): every third item's by match is the best mix.
+// 1.7 x 10^8 pairs, 2^20 vertices, scans apart: 5.44 + 0.32 ms (|S(v)| in a pass
+// of its own) with 7-bit digits in three passes, all by match; now 3.4 ms (all by
+// match 4.0, all by ballots 3.6, every second item by match 3.35, but 10 % more
+// with few bits).  The count of a pass, 0.62 -> 0.23 ms, was atomics of a warp on
+// the same counters.
 // ---------------------------------------------------------------------------
 constexpr int kRxThreads = 512;
 constexpr int kRxWarps = kRxThreads / 32;
 constexpr int kRxItems = 16;
 constexpr int kRxTile = kRxThreads * kRxItems;   // pairs per tile
-constexpr int kRxMaxBits = 8;
+constexpr int kRxMaxBits = 10;
 constexpr int kRxMaxBins = 1 << kRxMaxBits;
+constexpr int kRxCopies = 4;                     // of every counter of k_rx_count
 
 // Position of item j of lane `lane` of warp w in tile `tile`: warp w holds the
 // tile's w-th run of 32 kRxItems positions, item j its j-th run of 32.
@@ -122,148 +137,195 @@ __device__ __forceinline__ int64_t rx_pos(int64_t tile, int w, int j, int lane) 
     return tile * kRxTile + (int64_t)w * (32 * kRxItems) + j * 32 + lane;
 }
 
+// The set that holds the first pair of every tile (sets are not empty).
+__global__ void k_rx_tile_sets(const int64_t *set_off, int64_t theta, int32_t *tile_set) {
+    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < theta;
+         i += (int64_t)gridDim.x * blockDim.x) {
+        const int64_t b = set_off[i], e = set_off[i + 1];
+        for (int64_t t = (b + kRxTile - 1) / kRxTile; t * kRxTile < e; ++t) tile_set[t] = (int32_t)i;
+    }
+}
+
+// Every counter has kRxCopies copies side by side, taken by lane: hub vertices
+// give many lanes the same digit, and atomics of a warp on one address run one
+// after the other.
 __global__ void __launch_bounds__(kRxThreads) k_rx_count(const int32_t *keys, int64_t T, int shift,
                                                          int bits, int64_t ntiles, int32_t *table) {
-    __shared__ int32_t h[kRxWarps][kRxMaxBins];
+    __shared__ int4 h[kRxMaxBins];               // [digit][kRxCopies]
+    static_assert(kRxCopies == 4, "the copies of a counter are an int4");
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     const uint32_t mask = (1u << bits) - 1u;
     const int bins = 1 << bits;
+    int32_t *mine = reinterpret_cast<int32_t *>(h) + (lane & (kRxCopies - 1));
     for (int64_t tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
-        for (int i = threadIdx.x; i < kRxWarps * kRxMaxBins; i += kRxThreads) (&h[0][0])[i] = 0;
-        __syncthreads();
-#pragma unroll 4
+        for (int d = threadIdx.x; d < bins; d += kRxThreads) h[d] = make_int4(0, 0, 0, 0);
+        uint32_t key[kRxItems];
+#pragma unroll
         for (int j = 0; j < kRxItems; ++j) {
             const int64_t t = rx_pos(tile, w, j, lane);
-            if (t < T) atomicAdd(&h[w][((uint32_t)__ldg(keys + t) >> shift) & mask], 1);
+            key[j] = t < T ? (uint32_t)__ldg(keys + t) : 0u;
         }
         __syncthreads();
+#pragma unroll
+        for (int j = 0; j < kRxItems; ++j)
+            if (rx_pos(tile, w, j, lane) < T)
+                atomicAdd(mine + ((key[j] >> shift) & mask) * kRxCopies, 1);
+        __syncthreads();
         for (int d = threadIdx.x; d < bins; d += kRxThreads) {
-            int32_t c = 0;
-            for (int q = 0; q < kRxWarps; ++q) c += h[q][d];
-            table[(int64_t)d * ntiles + tile] = c;
+            const int4 c = h[d];
+            table[(int64_t)d * ntiles + tile] = c.x + c.y + c.z + c.w;
         }
         __syncthreads();
     }
 }
 
-// kFirst: the keys are the members and the values the set ids, found from
-// set_off (lane 0 of a warp searches the set of the warp's first position, then
-// every lane advances through set_off as its positions grow).
-template <bool kFirst>
+// Shared memory of k_rx_scatter (dynamic).
+struct RxSmem {
+    int32_t key[kRxTile], val[kRxTile];
+    uint16_t wc[kRxWarps][kRxMaxBins];           // per warp and digit: count, then start
+    int64_t go[kRxMaxBins];                      // output offset of every digit, less its start here
+    uint32_t starts[kRxTile / 32];               // FIRST: bitmap of the tile's set starts
+    int32_t before[kRxTile / 32];                // ... and how many before each word
+    int32_t wsum[kRxWarps];
+};
+
+// RB: ballots that find the peers of a digit (bits <= RB; the bits above are 0).
+template <int RB, bool FIRST, bool LAST>
 __global__ void __launch_bounds__(kRxThreads, 2) k_rx_scatter(
-    const int32_t *kin, const int32_t *vin, const int64_t *set_off, int64_t theta, int64_t T,
-    int shift, int bits, int64_t ntiles, const int64_t *goff, int32_t *kout, int32_t *vout) {
-    extern __shared__ int32_t rx_smem[];          // [kRxTile] keys, then [kRxTile] values
-    int32_t *skey = rx_smem, *sval = rx_smem + kRxTile;
-    __shared__ int32_t wc[kRxWarps][kRxMaxBins];  // per warp and digit: count, then start
-    __shared__ int32_t dstart[kRxMaxBins];        // first local index of every digit
-    __shared__ int64_t sgo[kRxMaxBins];           // output offset of every digit's run
-    __shared__ int32_t wsum[kRxMaxBins / 32];
+    const int32_t *kin, const int32_t *vin, const int64_t *set_off, const int32_t *tile_set,
+    int64_t theta, int64_t T, int shift, int bits, int64_t ntiles, const int64_t *goff,
+    int32_t *kout, int32_t *vout, uint32_t *cnt) {
+    extern __shared__ __align__(16) unsigned char rx_raw[];
+    RxSmem &S = *reinterpret_cast<RxSmem *>(rx_raw);
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     const uint32_t mask = (1u << bits) - 1u;
     const int bins = 1 << bits;
     const unsigned lt = (1u << lane) - 1u;
+    // thread i looks after digits 2 i and 2 i + 1, as two 16-bit halves
+    uint32_t *wc2 = reinterpret_cast<uint32_t *>(&S.wc[0][0]) + threadIdx.x;
+    const bool owns = 2 * (int)threadIdx.x < bins;
     for (int64_t tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
-        for (int i = threadIdx.x; i < kRxWarps * kRxMaxBins; i += kRxThreads) (&wc[0][0])[i] = 0;
-        for (int d = threadIdx.x; d < bins; d += kRxThreads)
-            sgo[d] = goff[(int64_t)d * ntiles + tile];
-        __syncthreads();
+#pragma unroll
+        for (int q = 0; q < kRxWarps; ++q) wc2[q * (kRxMaxBins / 2)] = 0u;
+        int64_t go0 = 0, go1 = 0;
+        if (owns) {
+            go0 = __ldg(goff + (int64_t)(2 * threadIdx.x) * ntiles + tile);
+            if (bins > 1) go1 = __ldg(goff + (int64_t)(2 * threadIdx.x + 1) * ntiles + tile);
+        }
+        const int64_t t0 = tile * kRxTile;
+        const bool full = t0 + kRxTile <= T;
+        const int32_t *kp = kin + t0 + w * (32 * kRxItems) + lane;
+        const int32_t *vp = vin + t0 + w * (32 * kRxItems) + lane;
+        const int32_t tn = full ? kRxTile : (int32_t)(T - t0);
+        const int32_t p0 = w * (32 * kRxItems) + lane;
         uint32_t key[kRxItems];
+#pragma unroll
+        for (int j = 0; j < kRxItems; ++j)
+            // past the end: the largest digit, so that they rank behind every pair
+            key[j] = full || p0 + j * 32 < tn ? (uint32_t)__ldg(kp + j * 32) : mask << shift;
+        int32_t s0 = 0;
+        if (FIRST) {
+            s0 = __ldg(tile_set + tile);
+            if (threadIdx.x < kRxTile / 32) S.starts[threadIdx.x] = 0u;
+            __syncthreads();
+            for (int64_t s = s0 + 1 + threadIdx.x; s < theta; s += kRxThreads) {
+                const int64_t p = __ldg(set_off + s) - t0;
+                if (p >= kRxTile) break;
+                atomicOr(&S.starts[p >> 5], 1u << (p & 31));
+            }
+        }
+        __syncthreads();
+        if (FIRST && w == 0) {
+            int32_t c[kRxTile / 1024], sum = 0;  // eight words a lane
+#pragma unroll
+            for (int q = 0; q < kRxTile / 1024; ++q) {
+                c[q] = sum;
+                sum += __popc(S.starts[lane * (kRxTile / 1024) + q]);
+            }
+            const int32_t excl = warp_incl_scan<int32_t>(sum, lane) - sum;
+#pragma unroll
+            for (int q = 0; q < kRxTile / 1024; ++q)
+                S.before[lane * (kRxTile / 1024) + q] = excl + c[q];
+        }
+        // rank of every pair among the warp's earlier pairs of its digit
         uint32_t rk[kRxItems / 2];                 // two 16-bit ranks per register
 #pragma unroll
         for (int j = 0; j < kRxItems; ++j) {
-            const int64_t t = rx_pos(tile, w, j, lane);
-            key[j] = t < T ? (uint32_t)__ldg(kin + t) : 0u;
-        }
-        // rank of every pair among the warp's earlier pairs of its digit
+            const uint32_t d = (key[j] >> shift) & mask;
+            unsigned peers = kFull;
+            if (j % 3 == 2) {                    // (see above)
+                peers = __match_any_sync(kFull, d);
+            } else {
 #pragma unroll
-        for (int j = 0; j < kRxItems; ++j) {
-            const bool ok = rx_pos(tile, w, j, lane) < T;
-            const uint32_t d = ok ? (key[j] >> shift) & mask : (uint32_t)(kRxMaxBins + lane);
-            const unsigned peers = __match_any_sync(kFull, d);
-            int32_t base = 0;
-            if (ok) base = wc[w][d];
+                for (int q = 0; q < RB; ++q) {
+                    const unsigned v = __ballot_sync(kFull, d & (1u << q));
+                    peers &= v ^ ((d >> q & 1u) - 1u);
+                }
+            }
+            const uint32_t base = S.wc[w][d], mine = (uint32_t)__popc(peers & lt);
             __syncwarp();
-            if (ok && lane == __ffs(peers) - 1) wc[w][d] = base + __popc(peers);
+            if (lane == 31 - __clz((int)peers)) S.wc[w][d] = (uint16_t)(base + mine + 1u);
             __syncwarp();
-            const uint32_t r = (uint32_t)(base + __popc(peers & lt));
+            const uint32_t r = base + mine;
             rk[j >> 1] = (j & 1) ? (rk[j >> 1] | (r << 16)) : r;
         }
         __syncthreads();
-        // digit-major starts: digit d's run of warp q begins after every
-        // smaller digit and after digit d's pairs of warps < q
-        int32_t tot = 0;
-        if (threadIdx.x < bins) {
-            for (int q = 0; q < kRxWarps; ++q) {
-                const int32_t c = wc[q][threadIdx.x];
-                wc[q][threadIdx.x] = tot;
-                tot += c;
-            }
-        }
-        const int32_t incl = warp_incl_scan<int32_t>(tot, lane);
-        if (lane == 31 && w < kRxMaxBins / 32) wsum[w] = incl;
+        // digit-major starts: digit d's run of warp q begins after every smaller
+        // digit and after digit d's pairs of the warps before q
+        uint32_t tot = 0;
+        if (owns)
+#pragma unroll
+            for (int q = 0; q < kRxWarps; ++q) tot += wc2[q * (kRxMaxBins / 2)];
+        const int32_t both = (int32_t)((tot & 0xffffu) + (tot >> 16));
+        const int32_t incl = warp_incl_scan<int32_t>(both, lane);
+        if (lane == 31) S.wsum[w] = incl;
         __syncthreads();
-        if (threadIdx.x < bins) {
-            int32_t before = 0;
-            for (int q = 0; q < w; ++q) before += wsum[q];
-            const int32_t ds = before + incl - tot;
-            dstart[threadIdx.x] = ds;
-            for (int q = 0; q < kRxWarps; ++q) wc[q][threadIdx.x] += ds;
+        int32_t ds = incl - both;
+        for (int q = 0; q < w; ++q) ds += S.wsum[q];
+        if (owns) {
+            const int32_t ds1 = ds + (int32_t)(tot & 0xffffu);
+            S.go[2 * threadIdx.x] = go0 - ds;
+            S.go[2 * threadIdx.x + 1] = go1 - ds1;
+            uint32_t run = (uint32_t)ds | (uint32_t)ds1 << 16;
+#pragma unroll
+            for (int q = 0; q < kRxWarps; ++q) {
+                const uint32_t c = wc2[q * (kRxMaxBins / 2)];
+                wc2[q * (kRxMaxBins / 2)] = run;
+                run += c;
+            }
         }
         __syncthreads();
         // place every pair at its local sorted index
-        int64_t cur = 0;
-        if (kFirst) {
-            const int64_t t0 = rx_pos(tile, w, 0, 0);
-            if (lane == 0 && t0 < T) {
-                int64_t lo = 0, hi = theta - 1;       // largest s with set_off[s] <= t0
-                while (lo < hi) {
-                    const int64_t mid = (lo + hi + 1) >> 1;
-                    if (__ldg(set_off + mid) <= t0) lo = mid;
-                    else hi = mid - 1;
-                }
-                cur = lo;
-            }
-            cur = __shfl_sync(kFull, cur, 0);
-        }
 #pragma unroll
         for (int j = 0; j < kRxItems; ++j) {
-            const int64_t t = rx_pos(tile, w, j, lane);
-            if (t < T) {
-                const uint32_t d = (key[j] >> shift) & mask;
-                const int32_t idx = wc[w][d] + (int32_t)((rk[j >> 1] >> (16 * (j & 1))) & 0xffffu);
-                skey[idx] = (int32_t)key[j];
-                if (kFirst) {
-                    while (__ldg(set_off + cur + 1) <= t) ++cur;
-                    sval[idx] = (int32_t)cur;
-                } else {
-                    sval[idx] = __ldg(vin + t);
-                }
+            const uint32_t d = (key[j] >> shift) & mask;
+            const uint32_t idx = S.wc[w][d] + ((rk[j >> 1] >> (16 * (j & 1))) & 0xffffu);
+            S.key[idx] = (int32_t)key[j];
+            if (FIRST) {
+                const int word = w * kRxItems + j;
+                S.val[idx] = s0 + S.before[word] + __popc(S.starts[word] & (lt | 1u << lane));
+            } else if (full || p0 + j * 32 < tn) {
+                S.val[idx] = __ldg(vp + j * 32);
             }
         }
         __syncthreads();
-        const int64_t t0 = tile * kRxTile;
-        const int32_t tn = (int32_t)min((int64_t)kRxTile, T - t0);
+#pragma unroll 4
         for (int32_t i = threadIdx.x; i < tn; i += kRxThreads) {
-            const uint32_t k = (uint32_t)skey[i];
-            const uint32_t d = (k >> shift) & mask;
-            const int64_t pos = sgo[d] + (i - dstart[d]);
-            vout[pos] = sval[i];
-            kout[pos] = (int32_t)k;
+            const uint32_t k = (uint32_t)S.key[i];
+            const int64_t pos = S.go[(k >> shift) & mask] + i;
+            vout[pos] = S.val[i];
+            if (!LAST) {
+                kout[pos] = (int32_t)k;
+            } else {
+                // a run of key k over [b, e) adds e - b to cnt[k]: -b at its first
+                // pair, e at its last (modulo 2^32; the total is below 2^31)
+                const bool first = i == 0 || (uint32_t)S.key[i - 1] != k;
+                const bool last = i == tn - 1 || (uint32_t)S.key[i + 1] != k;
+                if (first || last)
+                    atomicAdd(cnt + k, (last ? (uint32_t)(i + 1) : 0u) - (first ? (uint32_t)i : 0u));
+            }
         }
         __syncthreads();
-    }
-}
-
-// |S(v)| from the sorted keys: a run of key v over positions [b, e) adds
-// e - b to cnt[v] (as -b at its first position and +e at its last, modulo
-// 2^32; the total is below 2^31).
-__global__ void k_rx_bounds(const int32_t *keys, int64_t T, uint32_t *cnt) {
-    for (int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; p < T;
-         p += (int64_t)gridDim.x * blockDim.x) {
-        const int32_t k = keys[p];
-        if (p == 0 || keys[p - 1] != k) atomicAdd(cnt + k, 0u - (uint32_t)p);
-        if (p == T - 1 || keys[p + 1] != k) atomicAdd(cnt + k, (uint32_t)(p + 1));
     }
 }
 
@@ -404,73 +466,90 @@ im_status build_index_raw(const int64_t *set_off, const int32_t *members, int64_
 
 static size_t up256(size_t x) { return (x + 255) & ~(size_t)255; }
 
+namespace {
+
+template <int RB>
+auto rx_scatter(bool first, bool last) {
+    return first ? (last ? k_rx_scatter<RB, true, true> : k_rx_scatter<RB, true, false>)
+                 : (last ? k_rx_scatter<RB, false, true> : k_rx_scatter<RB, false, false>);
+}
+
+// Digits of a build: nbits = bit length of n - 1, split evenly over the passes.
+struct RxPlan {
+    int nbits = 0, passes, width;
+    explicit RxPlan(int64_t n) {
+        while (nbits < 63 && ((int64_t)1 << nbits) < n) ++nbits;
+        passes = std::max(1, (nbits + kRxMaxBits - 1) / kRxMaxBits);
+        width = (nbits + passes - 1) / passes;
+    }
+};
+
+}  // namespace
+
 size_t radix_index_bytes(int64_t T, int64_t n) {
+    const RxPlan plan(n);
     const int64_t ntiles = (T + kRxTile - 1) / kRxTile;
-    const int64_t cells = (int64_t)kRxMaxBins * ntiles;
-    return 3 * up256((size_t)T * 4) + up256((size_t)cells * 4) + up256((size_t)(cells + 1) * 8) +
+    const int64_t cells = ((int64_t)1 << plan.width) * ntiles;
+    // keys of all passes but the last (two buffers in turn), values of the last but one
+    return std::min(plan.passes, 3) * (plan.passes > 1 ? up256((size_t)T * 4) : 0) +
+           up256((size_t)ntiles * 4) + up256((size_t)cells * 4) + up256((size_t)(cells + 1) * 8) +
            std::max(scan_tmp_bytes(cells), scan_tmp_bytes(n)) + 256;
 }
 
 im_status build_index_radix(const int64_t *set_off, const int32_t *members, int64_t theta,
                             int64_t T, int64_t n, int64_t *vtx_off, int32_t *set_ids,
                             int32_t *cnt, void *scratch, cudaStream_t st) {
+    const RxPlan plan(n);
+    const int passes = plan.passes;
     const int64_t ntiles = (T + kRxTile - 1) / kRxTile;
-    const int64_t cells = (int64_t)kRxMaxBins * ntiles;
+    const int64_t cells = ((int64_t)1 << plan.width) * ntiles;
     char *b = (char *)scratch;
     auto take = [&](size_t bytes) {
         char *r = b;
         b += up256(bytes);
         return r;
     };
-    int32_t *kA = (int32_t *)take((size_t)T * 4), *kB = (int32_t *)take((size_t)T * 4),
-            *vB = (int32_t *)take((size_t)T * 4);
+    int32_t *vB = passes > 1 ? (int32_t *)take((size_t)T * 4) : nullptr;
+    int32_t *kA = passes > 1 ? (int32_t *)take((size_t)T * 4) : nullptr;
+    int32_t *kB = passes > 2 ? (int32_t *)take((size_t)T * 4) : nullptr;
+    int32_t *tile_set = (int32_t *)take((size_t)ntiles * 4);
     int32_t *table = (int32_t *)take((size_t)cells * 4);
     int64_t *goff = (int64_t *)take((size_t)(cells + 1) * 8);
     void *stmp = take(0);
     const size_t stmp_bytes = std::max(scan_tmp_bytes(cells), scan_tmp_bytes(n));
-    // digits: nbits = bit length of n - 1, split evenly over ceil(nbits / 8) passes
-    int nbits = 0;
-    while (nbits < 63 && ((int64_t)1 << nbits) < n) ++nbits;
-    const int passes = std::max(1, (nbits + kRxMaxBits - 1) / kRxMaxBits);
-    const int width = (nbits + passes - 1) / passes;
     IM_CUDA(cudaMemsetAsync(cnt, 0, (size_t)n * 4, st));
     if (T > 0) {
         const int grid = (int)std::min<int64_t>(ntiles, (int64_t)num_sms() * 2);
-        const size_t smem = (size_t)2 * kRxTile * 4;
-        // the scatter's 64 KB of dynamic shared memory (a per-device attribute)
-        IM_TRY(raise_dyn_smem((const void *)k_rx_scatter<true>, smem));
-        IM_TRY(raise_dyn_smem((const void *)k_rx_scatter<false>, smem));
+        const size_t smem = sizeof(RxSmem);
         const int32_t *kin = members, *vin = nullptr;
         for (int ps = 0; ps < passes; ++ps) {
-            const int shift = ps * width;
-            const int bits = std::max(0, std::min(width, nbits - shift));
+            const int shift = ps * plan.width;
+            const int bits = std::max(0, std::min(plan.width, plan.nbits - shift));
+            const bool first = ps == 0, last = ps == passes - 1;
             int32_t *kout = (ps & 1) ? kB : kA;
             int32_t *vout = ((passes - 1 - ps) & 1) ? vB : set_ids;
             {
                 KernelTimer kt(st, "index_radix");
-                k_rx_count<<<grid, kRxThreads, 0, st>>>(kin, T, shift, bits, ntiles, table);
+                if (first)
+                    k_rx_tile_sets<<<num_sms() * 4, 256, 0, st>>>(set_off, theta, tile_set);
+                k_rx_count<<<(int)std::min<int64_t>(ntiles, (int64_t)num_sms() * 4), kRxThreads, 0,
+                             st>>>(kin, T, shift, bits, ntiles, table);
             }
             IM_CUDA(cudaGetLastError());
             const int64_t used = ((int64_t)1 << bits) * ntiles;
             IM_TRY(exclusive_scan_i32_to_i64(table, goff, used, nullptr, stmp, stmp_bytes, st));
             {
+                auto kern = bits <= 8 ? rx_scatter<8>(first, last) : rx_scatter<10>(first, last);
+                // 110 KB of dynamic shared memory (a per-device attribute)
+                IM_TRY(raise_dyn_smem((const void *)kern, smem));
                 KernelTimer kt(st, "index_radix");
-                if (ps == 0)
-                    k_rx_scatter<true><<<grid, kRxThreads, smem, st>>>(
-                        kin, vin, set_off, theta, T, shift, bits, ntiles, goff, kout, vout);
-                else
-                    k_rx_scatter<false><<<grid, kRxThreads, smem, st>>>(
-                        kin, vin, set_off, theta, T, shift, bits, ntiles, goff, kout, vout);
+                kern<<<grid, kRxThreads, smem, st>>>(kin, vin, set_off, tile_set, theta, T, shift,
+                                                     bits, ntiles, goff, kout, vout, (uint32_t *)cnt);
             }
             IM_CUDA(cudaGetLastError());
             kin = kout;
             vin = vout;
         }
-        {
-            KernelTimer kt(st, "index_bounds");
-            k_rx_bounds<<<num_sms() * 8, 256, 0, st>>>(kin, T, (uint32_t *)cnt);
-        }
-        IM_CUDA(cudaGetLastError());
     }
     return exclusive_scan_i32_to_i64(cnt, vtx_off, n, nullptr, stmp, stmp_bytes, st);
 }
