@@ -5,7 +5,9 @@
 // Run r simulates the live-edge world of RRR sample r -- the same IC coins
 // and LT picks the sampler uses -- forward from S by a BFS
 // over out-edges (one block per run, level by level, each warp expanding 32
-// queued vertices at a time).
+// queued vertices at a time).  Under LT a run that activates a large part of the
+// graph is finished by k_spread_pull, which draws every vertex's pick once
+// instead of once per in-edge from an activated vertex.
 //   IC: in-edge e is live iff lane (e & 3) of Philox(r, e >> 2, e >> 34, coin
 //       tag) is below w[e];
 //   LT: in-edge e into v is live iff v's pick draw x = Philox(r, v, 0, pick
@@ -71,12 +73,22 @@ struct SpreadArgs {
     const uint4 *out_rec;
     uint32_t *vis;                    // [blocks][words]
     int64_t words;
-    int32_t *queues;                  // [blocks][n]
+    int32_t *queues;                  // [blocks][qcap]
+    int64_t qcap;
     unsigned long long *work;
     unsigned long long *total;
     int64_t *activated;               // [runs] or null
     uint8_t *root_hit;                // [runs] or null
     int *status;
+    // LT: runs that examined more than `budget` out-edges, for k_spread_pull
+    unsigned long long budget;
+    uint32_t *wide;                   // [runs]
+    unsigned long long *nwide;
+    QueryView view;                   // LT: the graph's pick tables
+    int32_t *next;                    // [groups][n] k_spread_pull
+    GridBarrier *bars;                // [groups]
+    unsigned long long *left;         // [groups][4] per-round and result counters
+    int32_t groups;
 };
 
 // One run per block: a level-synchronous BFS whose warps take 32 vertices
@@ -84,16 +96,17 @@ struct SpreadArgs {
 // the block's queue (one atomic per warp and step).
 __global__ void __launch_bounds__(kSpreadThreads) k_spread(SpreadArgs a) {
     __shared__ unsigned long long s_run;
-    __shared__ unsigned long long s_tail, s_cursor;
+    __shared__ unsigned long long s_tail, s_cursor, s_work;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     uint32_t *vis = a.vis + (int64_t)blockIdx.x * a.words;
-    int32_t *q = a.queues + (int64_t)blockIdx.x * a.n;
+    int32_t *q = a.queues + (int64_t)blockIdx.x * a.qcap;
     const uint32_t k0 = seed_lo(a.seed), k1 = seed_hi(a.seed);
     unsigned long long my_total = 0;
     for (;;) {
         if (threadIdx.x == 0) {
             s_run = atomicAdd(a.work, 1ull);
             s_tail = 0;
+            s_work = 0;
         }
         __syncthreads();
         const unsigned long long i = s_run;
@@ -123,14 +136,21 @@ __global__ void __launch_bounds__(kSpreadThreads) k_spread(SpreadArgs a) {
         }
         __syncthreads();
         long long head = 0;
+        bool wide = false;                   // (block-uniform)
         for (;;) {
             const long long lvl_end = (long long)s_tail;
+            if (a.wide && s_work > a.budget) {
+                wide = true;
+                break;
+            }
             if (head >= lvl_end) break;
+            __syncthreads();                 // everyone has read s_tail and s_work
             if (threadIdx.x == 0) s_cursor = (unsigned long long)head;
             __syncthreads();
             for (;;) {
-                long long base = 0;
-                if (lane == 0) base = (long long)atomicAdd(&s_cursor, 32ull);
+                long long base = lvl_end;    // over budget: leave the level
+                if (lane == 0 && !(a.wide && *(volatile unsigned long long *)&s_work > a.budget))
+                    base = (long long)atomicAdd(&s_cursor, 32ull);
                 base = __shfl_sync(kFull, base, 0);
                 if (base >= lvl_end) break;
                 const int nb = (int)(lvl_end - base < 32 ? lvl_end - base : 32);
@@ -143,6 +163,11 @@ __global__ void __launch_bounds__(kSpreadThreads) k_spread(SpreadArgs a) {
                 const int64_t len = oe - ob;
                 const int64_t incl = warp_incl_scan<int64_t>(len, lane);
                 const int64_t total = __shfl_sync(kFull, incl, 31);
+                if (a.wide) {                // over budget: the run is redone by pulling
+                    unsigned long long w = 0;
+                    if (lane == 0) w = atomicAdd(&s_work, (unsigned long long)total) + (unsigned long long)total;
+                    if (__shfl_sync(kFull, w, 0) > a.budget) break;
+                }
                 for (int64_t eb = 0; eb < total; eb += 32) {
                     const int64_t t = eb + lane;
                     int owner = 0;   // first lane whose inclusive count exceeds t
@@ -193,7 +218,9 @@ __global__ void __launch_bounds__(kSpreadThreads) k_spread(SpreadArgs a) {
             head = lvl_end;
         }
         const long long tail = (long long)s_tail;
-        if (threadIdx.x == 0) {
+        if (wide) {
+            if (threadIdx.x == 0) a.wide[atomicAdd(a.nwide, 1ull)] = (uint32_t)i;
+        } else if (threadIdx.x == 0) {
             const uint32_t root = rrr_root(a.seed, s, (uint32_t)a.n);
             const bool hit = (vis[root >> 5] >> (root & 31)) & 1u;
             if (a.activated) a.activated[i] = tail;
@@ -210,6 +237,130 @@ __global__ void __launch_bounds__(kSpreadThreads) k_spread(SpreadArgs a) {
         __syncthreads();
     }
     if (threadIdx.x == 0 && my_total) atomicAdd(a.total, my_total);
+}
+
+// The source that vertex v picks in sample s (draw x), or -1: the rules of the LT
+// sampler over its tables (equal in-weights by the record's reciprocal, else the
+// cut point and, past it, a search of doubling stride in the running sums).
+__device__ __forceinline__ int32_t lt_pick_source(const QueryView &V, uint32_t v, uint32_t x) {
+    const uint4 vr = __ldg(V.lt_vrec + v);
+    const uint32_t d = vr.y;
+    if (vr.w != 0u) {
+        uint32_t e = __umulhi(x, vr.z), rem = x - e * vr.w;
+        if (rem >= vr.w) { ++e; rem -= vr.w; }
+        if (rem >= vr.w) ++e;
+        return e < d ? __ldg(V.in_src + vr.x + e) : -1;
+    }
+    if (d == 0u) return -1;
+    const uint4 gv = __ldg(V.lt_guide + vr.x + __umulhi(x, d));
+    if ((unsigned long long)x < (((unsigned long long)gv.y << 32) | gv.x)) return (int32_t)gv.z;
+    const unsigned long long *leaf = V.lt_leaf + vr.x;
+    uint32_t lo = gv.w + 1, hi = d, stride = 1;
+    unsigned long long at = 0;
+    while (lo < hi) {
+        const uint32_t p = hi < d ? (lo + hi) >> 1 : min(lo + stride - 1u, d - 1u);
+        const unsigned long long r = __ldg(leaf + p);
+        if ((unsigned long long)x < (r >> 31)) {
+            hi = p;
+            at = r;
+        } else {
+            lo = p + 1;
+        }
+        stride <<= 1;
+    }
+    return hi < d ? (int32_t)(at & 0x7fffffffull) : -1;
+}
+
+// LT runs that activate a large part of the graph.  In an LT world every vertex
+// keeps at most one in-edge, so the world is one pointer a vertex, and v is
+// activated iff its chain of pointers reaches a seed.  A group of blocks draws
+// the n pointers of a run (next[v]: the pick; -1: a seed; -2: nothing picked),
+// then lets every pointer jump to where its target points until no more chain
+// ends at a seed or at nothing; what is still unresolved runs into a cycle.  (A
+// round with an unresolved chain that ends always resolves one: the unresolved
+// vertex nearest its end points at a resolved one.)  Concurrent jumps only ever
+// shorten chains, so rounds work in place.
+// n draws and about ten rounds of n gathers in L2 instead of a draw per out-edge
+// of an activated vertex (1.5 x 10^7 of 1.7 x 10^7 at scale 20 from 100 of the
+// largest vertices): 256 runs 79.9 -> 5.3 ms, 0.7 of them the forward pass.  The groups' pointers together stay
+// below kPullBytes, so that the gathers hit L2.
+constexpr int kPullThreads = 1024;
+constexpr int64_t kPullBytes = 64ll << 20;
+constexpr int kPullU = 4;                    // gathers in flight per thread
+
+__global__ void __launch_bounds__(kPullThreads) k_spread_pull(const __grid_constant__ SpreadArgs a) {
+    __shared__ unsigned long long s_cnt[kPullThreads / 32];
+    const int group = blockIdx.x % a.groups;             // blocks of a group on different SMs
+    const uint32_t rank = blockIdx.x / a.groups, nb = (gridDim.x - group + a.groups - 1) / a.groups;
+    int32_t *next = a.next + (int64_t)group * a.n;
+    GridBarrier *bar = a.bars + group;
+    unsigned long long *left = a.left + 4 * group;       // [0], [1] resolved in a round, [2] activated
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int64_t tid = (int64_t)rank * kPullThreads + threadIdx.x, stride = (int64_t)nb * kPullThreads;
+    const uint32_t k0 = seed_lo(a.seed), k1 = seed_hi(a.seed);
+    const int64_t nruns = (int64_t)*a.nwide;
+    // adds the block's counts to *to
+    auto block_add = [&](unsigned int mine, unsigned long long *to) {
+        mine = __reduce_add_sync(kFull, mine);
+        if (lane == 0) s_cnt[warp] = mine;
+        __syncthreads();
+        if (warp == 0) {
+            const unsigned long long t = warp_sum<unsigned long long>(s_cnt[lane]);
+            if (lane == 0 && t) atomicAdd(to, t);
+        }
+        __syncthreads();
+    };
+    for (int64_t i = group; i < nruns; i += a.groups) {
+        const uint32_t run = a.wide[i];
+        const uint32_t s = (uint32_t)(a.first + run);
+        for (int64_t v = tid; v < a.n; v += stride) {
+            const int32_t u = lt_pick_source(
+                a.view, (uint32_t)v, philox4x32_10(make_uint4(s, (uint32_t)v, 0u, kStreamPick), k0, k1).x);
+            next[v] = u >= 0 ? u : -2;
+        }
+        if (tid == 0) left[0] = left[1] = left[2] = 0ull;
+        if (!grid_sync(bar, nb, a.status)) return;
+        for (int64_t b = tid; b < a.k; b += stride) next[a.seeds[b]] = -1;
+        if (!grid_sync(bar, nb, a.status)) return;
+        for (int round = 0;; ++round) {
+            unsigned int resolved = 0;
+            for (int64_t v0 = tid; v0 < a.n; v0 += stride * kPullU) {
+                int32_t p[kPullU], q[kPullU];
+#pragma unroll
+                for (int u = 0; u < kPullU; ++u) {
+                    const int64_t v = v0 + u * stride;
+                    p[u] = v < a.n ? __ldcg(next + v) : -1;
+                }
+#pragma unroll
+                for (int u = 0; u < kPullU; ++u) q[u] = p[u] >= 0 ? __ldcg(next + p[u]) : 0;
+#pragma unroll
+                for (int u = 0; u < kPullU; ++u)
+                    if (p[u] >= 0) {
+                        next[v0 + u * stride] = q[u];
+                        resolved += q[u] < 0;
+                    }
+            }
+            block_add(resolved, left + (round & 1));
+            if (!grid_sync(bar, nb, a.status)) return;
+            const unsigned long long any = *(volatile unsigned long long *)(left + (round & 1));
+            // (the other counter's last readers passed the barrier above)
+            if (tid == 0) left[(round + 1) & 1] = 0ull;
+            if (any == 0ull) break;
+            if (!grid_sync(bar, nb, a.status)) return;
+        }
+        unsigned int act = 0;
+        for (int64_t v = tid; v < a.n; v += stride) act += __ldcg(next + v) == -1;
+        block_add(act, left + 2);
+        if (!grid_sync(bar, nb, a.status)) return;
+        if (tid == 0) {
+            const unsigned long long t = *(volatile unsigned long long *)(left + 2);
+            const uint32_t root = rrr_root(a.seed, s, (uint32_t)a.n);
+            if (a.activated) a.activated[run] = (int64_t)t;
+            if (a.root_hit) a.root_hit[run] = __ldcg(next + root) == -1 ? 1 : 0;
+            atomicAdd(a.total, t);
+        }
+        if (!grid_sync(bar, nb, a.status)) return;       // before next and left are rewritten
+    }
 }
 
 std::mutex g_out_index_mu;   // graphs are shared between threads
@@ -295,7 +446,12 @@ extern "C" im_status im_spread(const im_graph *gc, im_model model, const int32_t
     // queue (n entries) and bitmap within about 2 GB
     int per_sm = 0;
     IM_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_spread, kSpreadThreads, 0));
-    const int64_t per_block = (int64_t)n * 4 + words * 4;
+    const bool pull = model == IM_LT;
+    // LT: out-edges from which drawing all n picks is the cheaper way; a run
+    // examines no more of them here, so its queue holds no more either
+    const int64_t budget = std::max<int64_t>(n / 8, 1 << 16);
+    const int64_t qcap = pull ? std::min<int64_t>(n, budget + k) : n;
+    const int64_t per_block = qcap * 4 + words * 4;
     int64_t blocks = std::max(1, per_sm) * (int64_t)num_sms();
     blocks = std::min<int64_t>(blocks, std::max<int64_t>(1, (2ll << 30) / per_block));
     blocks = std::min<int64_t>(blocks, (int64_t)runs);
@@ -309,8 +465,9 @@ extern "C" im_status im_spread(const im_graph *gc, im_model model, const int32_t
         off += (bytes + 255) & ~(size_t)255;
         return at;
     };
+    const size_t o_wide = take(pull ? (size_t)runs * 4 : 0);
     const size_t o_ctr = take(4 * 8), o_seeds = take((size_t)std::max(k, 1) * 4),
-                 o_vis = take((size_t)warps * words * 4), o_q = take((size_t)warps * n * 4),
+                 o_vis = take((size_t)warps * words * 4), o_q = take((size_t)warps * qcap * 4),
                  o_act = take(host_act ? (size_t)runs * 8 : 0),
                  o_hit = take(host_hit ? (size_t)runs : 0);
     char *B = nullptr;
@@ -335,6 +492,15 @@ extern "C" im_status im_spread(const im_graph *gc, im_model model, const int32_t
     a.work = ctr;
     a.total = ctr + 1;
     a.status = (int *)(ctr + 2);
+    a.nwide = ctr + 3;
+    a.wide = pull ? (uint32_t *)(B + o_wide) : nullptr;
+    a.budget = (unsigned long long)budget;
+    a.qcap = qcap;
+    a.view = query_view(g, seed, first_run);
+    a.next = nullptr;
+    a.bars = nullptr;
+    a.left = nullptr;
+    a.groups = 0;
     a.activated = host_act ? (int64_t *)(B + o_act) : activated;
     a.root_hit = host_hit ? (uint8_t *)(B + o_hit) : root_hit;
     {
@@ -342,10 +508,41 @@ extern "C" im_status im_spread(const im_graph *gc, im_model model, const int32_t
         k_spread<<<(unsigned)blocks, kSpreadThreads, 0, st>>>(a);
     }
     IM_CUDA(cudaGetLastError());
-    unsigned long long hc[3] = {0, 0, 0};
+    unsigned long long hc[4] = {0, 0, 0, 0};
+    int32_t *next = nullptr;
+    if (pull) {
+        IM_CUDA(cudaMemcpyAsync(hc, ctr, sizeof(hc), cudaMemcpyDeviceToHost, st));
+        IM_CUDA(cudaStreamSynchronize(st));
+    }
+    if (hc[3] > 0 && (int)(hc[2] & 0xffffffffu) == kDevOk) {
+        int per = 0;
+        IM_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_spread_pull, kPullThreads, 0));
+        if (per < 1) return IM_ERR_UNSUPPORTED;
+        const int grid = per * num_sms();
+        a.groups = (int32_t)std::max<int64_t>(
+            1, std::min<int64_t>({(int64_t)hc[3], (int64_t)grid / 4, kPullBytes / (n * 4)}));
+        // the forward pass's queues are free by now
+        const size_t o_bars = ((size_t)a.groups * n * 4 + 255) & ~(size_t)255;
+        const size_t o_left = o_bars + (((size_t)a.groups * sizeof(GridBarrier) + 255) & ~(size_t)255);
+        const size_t need = o_left + (size_t)a.groups * 4 * 8;
+        char *N = B + o_q;
+        if (need > (size_t)warps * qcap * 4) {
+            IM_CUDA(cudaMallocAsync((void **)&next, need, st));
+            N = (char *)next;
+        }
+        a.next = (int32_t *)N;
+        a.bars = (GridBarrier *)(N + o_bars);
+        a.left = (unsigned long long *)(N + o_left);
+        IM_CUDA(cudaMemsetAsync(N + o_bars, 0, need - o_bars, st));
+        void *args[] = {&a};
+        KernelTimer kt(st, "spread_pull");
+        IM_CUDA(cudaLaunchCooperativeKernel((const void *)k_spread_pull, dim3(grid),
+                                            dim3(kPullThreads), args, 0, st));
+    }
     IM_CUDA(cudaMemcpyAsync(hc, ctr, sizeof(hc), cudaMemcpyDeviceToHost, st));
     if (host_act) IM_CUDA(cudaMemcpyAsync(activated, B + o_act, (size_t)runs * 8, cudaMemcpyDeviceToHost, st));
     if (host_hit) IM_CUDA(cudaMemcpyAsync(root_hit, B + o_hit, (size_t)runs, cudaMemcpyDeviceToHost, st));
+    if (next) IM_CUDA(cudaFreeAsync(next, st));
     IM_CUDA(cudaFreeAsync(B, st));
     IM_CUDA(cudaStreamSynchronize(st));
     (void)host_seeds;
