@@ -39,7 +39,10 @@ namespace {
 
 constexpr int kGreedyThreads = 512;
 constexpr int kRGThreads = 512;
-constexpr int kProdThreads = 1024;           // producer blocks of the two-launch mode
+constexpr int kProdThreads = 1024;           // producer blocks of the two-launch mode, at most
+constexpr int kProdMinThreads = 512;         // ... and at least (64 a candidate, see scan_ids)
+constexpr size_t kProdSmemCap = 200 * 1024;  // their keys, and what fits beside them
+constexpr size_t kProdInfoCap = 56 * 1024;   // keys and subsets beside a bitmap in global memory
 constexpr int kBatch = 256;                  // stream slots a consumer reads at once
 constexpr int kUnroll = 8;                   // independent loads in flight per lane in scans
 constexpr int kSpec = 32;                    // largest speculative group of stream elements
@@ -61,22 +64,6 @@ __device__ __forceinline__ unsigned long long block_max_u64(unsigned long long v
     }
     __syncthreads();
     const unsigned long long r = sh[32];
-    __syncthreads();
-    return r;
-}
-
-__device__ __forceinline__ long long block_sum_i64(long long v, long long *sh) {
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    v = warp_sum<long long>(v);
-    if (lane == 0) sh[warp] = v;
-    __syncthreads();
-    if (warp == 0) {
-        long long x = lane < (int)(blockDim.x >> 5) ? sh[lane] : 0ll;
-        x = warp_sum<long long>(x);
-        if (lane == 0) sh[32] = x;
-    }
-    __syncthreads();
-    const long long r = sh[32];
     __syncthreads();
     return r;
 }
@@ -416,7 +403,9 @@ struct RGArgs {
     const int32_t *set_ids;
     const int32_t *part_off;
     const int32_t *part_vtx;
-    uint32_t *covered;        // [P][words] producer bitmaps
+    uint4 *cinfo;             // [n] by part position: first entry (64 bits), length and vertex of S(v),
+    int32_t cinfo_smem;       // unless the producers keep it in shared memory
+    uint32_t *covered;        // [P][words] producer bitmaps (unless in shared memory)
     uint32_t *bcovered;       // [B][words] bucket bitmaps
     int32_t *local_seeds;
     int64_t *local_gains;
@@ -450,168 +439,201 @@ struct RGArgs {
 // exact, which picks exactly the standard greedy's sequence.
 //
 // cmax[c] is the largest packed key (gain << 32 | ~l) of the 32 candidates of
-// chunk c.  A round takes the best candidate of each of the kProdW chunks with
-// the largest cmax and re-evaluates the stale ones at once (blockDim / kProdW
-// threads each) against the part's covered bitmap; then, if the overall
-// largest key is exact, it is taken.  Evaluating more candidates than the
-// sequential rule would only replaces upper bounds by exact values, so the
-// sequence of picks is unchanged while a pick takes one or two rounds instead
-// of one round per stale candidate.
+// chunk c.  A round takes the best candidate of each of the W chunks with the
+// largest cmax and re-evaluates the stale ones at once (blockDim / W threads
+// each) against the part's covered bitmap; then, if the overall largest key is
+// exact, it is taken.  Evaluating more candidates than the sequential rule
+// would only replaces upper bounds by exact values, so the sequence of picks is
+// unchanged while a pick takes one or two rounds instead of one round per stale
+// candidate.
+//
+// A round is a chain: select, read the candidates' subsets, probe the bitmap,
+// add up.  Warp 0 does all that is serial (keys, chunk maxima, the selection of
+// the next round, by 32-bit reductions) while the others wait at one barrier or,
+// after a pick, cover its subset meanwhile; a candidate's subset comes in one
+// read.  With few sets the bitmap lies in shared memory (SB), where 32
+// probes take a few cycles; in global memory they take one L1 line each, and at
+// 4 x 10^6 sets that is what bounds the part (2.7 x 10^6 probes and 0.6 x 10^6
+// marks a part, 0.63 of them a cycle).  148 parts of R-MAT scale 20, k = 100, 4.2 x
+// 10^6 LT sets: 3.13 -> 2.82 ms; 512 parts, 2.1 x 10^6 weighted-cascade sets (two
+// blocks an SM): 3.58 -> 1.74 ms; 64 parts, 2 x 10^5 sets: 0.40 -> 0.30 ms.
 constexpr int kProdW = 8;
 
 __device__ __forceinline__ unsigned long long prod_key(int32_t g, int32_t l) {
     return g > 0 ? ((unsigned long long)(uint32_t)g << 32) | (0xffffffffu - (uint32_t)l) : 0ull;
 }
 
+// The largest packed key of a warp's lanes (distinct unless 0).
+__device__ __forceinline__ unsigned long long warp_max_key(unsigned long long v) {
+    const uint32_t hi = __reduce_max_sync(kFull, (uint32_t)(v >> 32));
+    const uint32_t lo = __reduce_max_sync(kFull, (uint32_t)(v >> 32) == hi ? (uint32_t)v : 0u);
+    return (unsigned long long)hi << 32 | lo;
+}
+
 // cmax of chunk c, by one warp
 __device__ __forceinline__ void prod_chunk_max(const int32_t *key, unsigned long long *cmax,
                                                int32_t np, int32_t c, int lane) {
     const int32_t l = c * 32 + lane;
-    const unsigned long long v = warp_max_u64(l < np ? prod_key(key[l], l) : 0ull);
+    const unsigned long long v = warp_max_key(l < np ? prod_key(key[l], l) : 0ull);
     if (lane == 0) cmax[c] = v;
 }
 
-__device__ void produce(const RGArgs &a, int p, int32_t *key, unsigned long long *shm,
-                        long long *shs) {
-    __shared__ int32_t s_cand[kProdW];
-    __shared__ int32_t s_cnt[kProdW];
-    __shared__ unsigned long long s_top;
+template <bool SB>
+__device__ void produce(const RGArgs &a, int p, int32_t *key) {
+    __shared__ int32_t s_cand[kProdW];           // the round's candidates, -1: none
+    __shared__ int32_t s_stale[kProdW];          // ... 1: to be evaluated
+    __shared__ int32_t s_cnt[kProdW];            // ... their gains
+    __shared__ int64_t s_beg[kProdW];            // ... their subsets
+    __shared__ int32_t s_len[kProdW];
+    __shared__ int s_act;                        // 0 done, 1 evaluate, 2 take candidate 0
     const int32_t vb = a.part_off[p], np = a.part_off[p + 1] - vb;
-    const int32_t *vtx = a.part_vtx + vb;
     int32_t *stamp = key + a.max_np;
     unsigned long long *cmax = reinterpret_cast<unsigned long long *>(key + 2 * a.max_np);
     const int32_t nch = (np + 31) / 32;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarp = blockDim.x >> 5;
-    uint32_t *cov = a.covered + (size_t)p * (size_t)a.words;
+    unsigned char *rest = reinterpret_cast<unsigned char *>(cmax + ((a.max_np + 63) / 64) * 2);
+    uint4 *cinfo = a.cinfo_smem ? reinterpret_cast<uint4 *>(rest) : a.cinfo + vb;
+    if (a.cinfo_smem) rest += (size_t)a.max_np * sizeof(uint4);
+    uint32_t *cov = SB ? reinterpret_cast<uint32_t *>(rest) : a.covered + (size_t)p * (size_t)a.words;
     for (int64_t x = threadIdx.x; x < a.words; x += blockDim.x) cov[x] = 0u;
     for (int32_t l = threadIdx.x; l < np; l += blockDim.x) {
-        const int32_t v = vtx[l];
-        key[l] = (int32_t)(a.vtx_off[v + 1] - a.vtx_off[v]);
+        const int32_t v = a.part_vtx[vb + l];
+        const int64_t b = a.vtx_off[v], n = a.vtx_off[v + 1] - b;
+        cinfo[l] = make_uint4((uint32_t)b, (uint32_t)((uint64_t)b >> 32), (uint32_t)n, (uint32_t)v);
+        key[l] = (int32_t)n;
         stamp[l] = 0;                                   // exact: nothing is covered yet
     }
     __syncthreads();
     for (int32_t c = warp; c < nch; c += nwarp) prod_chunk_max(key, cmax, np, c, lane);
     __syncthreads();
     const uint64_t t_begin = global_ns();
-    long long n_rounds = 0, n_evals = 0, eval_entries = 0, cover_entries = 0;
+    long long n_rounds = 0, n_evals = 0, eval_entries = 0, cover_entries = 0;   // (warp 0's)
     int64_t total = 0;
     int32_t j = 0;
     const int W = a.evals;
     const int gsz = blockDim.x / W, grp = threadIdx.x / gsz, gt = threadIdx.x % gsz;
-    while (j < a.k) {
-        ++n_rounds;
-        // ---- the W chunks with the largest maxima (warp 0, by repeated max)
-        if (warp == 0) {
-            unsigned long long taken = 0ull;    // chunks already chosen, as keys
-            for (int w = 0; w < W; ++w) {
-                unsigned long long best = 0ull;
-                for (int32_t c = lane; c < nch; c += 32) {
-                    const unsigned long long v = cmax[c];
-                    // skip chunks chosen earlier this round (their keys are distinct)
-                    if (v > best && (w == 0 || v < taken)) best = v;
-                }
-                const unsigned long long m = warp_max_u64(best);
-                if (lane == 0) {
-                    s_cand[w] = m ? (int32_t)(0xffffffffu - (uint32_t)(m & 0xffffffffu)) : -1;
-                    s_cnt[w] = 0;
-                    if (w == 0) s_top = m;
-                }
-                taken = m;
-                if (!m) {
-                    for (int w2 = w + 1; w2 < W && lane == 0; ++w2) s_cand[w2] = -1;
-                    break;
-                }
+    // warp 0: the candidates of the next round, and what to do with them
+    auto select = [&]() {
+        unsigned long long taken = ~0ull;        // the last one chosen; keys are distinct
+        int32_t mine = -1;                       // candidate of lane w
+        unsigned long long top = 0ull;
+        for (int w = 0; w < W; ++w) {
+            unsigned long long best = 0ull;
+            for (int32_t c = lane; c < nch; c += 32) {
+                const unsigned long long v = cmax[c];
+                if (v > best && v < taken) best = v;
             }
+            const unsigned long long m = warp_max_key(best);
+            if (m == 0ull) break;
+            if (w == 0) top = m;
+            if (lane == w) mine = (int32_t)(0xffffffffu - (uint32_t)m);
+            taken = m;
+            // an exact top is taken: no need of the others
+            if (w == 0 && stamp[0xffffffffu - (uint32_t)m] == j) break;
         }
-        __syncthreads();
-        if (s_top == 0ull) break;                       // every gain is zero
-        {
-            const int32_t l0 = s_cand[0];
-            if (stamp[l0] != j) {
-                // ---- re-evaluate every stale candidate of the round at once
-                const int32_t l = s_cand[grp];
-                const bool mine = l >= 0 && stamp[l] != j;
-                if (mine) {
-                    const int32_t v = vtx[l];
-                    const int64_t sb = a.vtx_off[v], se = a.vtx_off[v + 1];
-                    int miss = 0;
-                    // L1-cached probes: the bitmap is written only by this
-                    // block (atomics, ordered before these loads by the block
-                    // barriers), and S(v) is scanned in ascending set order
-                    // when the index comes from the radix build, so
-                    // neighbouring ids share cached lines
-                    scan_ids<4>(a.set_ids, sb, se - sb, gt, gsz, [&](int32_t i) {
-                        if (i >= 0) miss += !((__ldca(cov + (i >> 5)) >> (i & 31)) & 1u);
-                    });
-                    miss = warp_sum<int>(miss);
-                    if (lane == 0 && miss) atomicAdd(&s_cnt[grp], miss);
-                }
-                __syncthreads();
-                if (mine && gt == 0) {
-                    key[l] = s_cnt[grp];
-                    stamp[l] = j;
-                    const int32_t v = vtx[l];
+        bool stale = false;
+        if (mine >= 0) {
+            stale = stamp[mine] != j;
+            const uint4 ci = cinfo[mine];
+            s_beg[lane] = (int64_t)((uint64_t)ci.y << 32 | ci.x);
+            s_len[lane] = (int32_t)ci.z;
+        }
+        if (lane < W) {
+            s_cand[lane] = mine;
+            s_stale[lane] = stale;
+            s_cnt[lane] = 0;
+        }
+        const bool top_stale = __shfl_sync(kFull, stale, 0);
+        if (lane == 0) s_act = top == 0ull ? 0 : top_stale ? 1 : 2;
+        __syncwarp();
+    };
+    if (warp == 0) select();
+    __syncthreads();
+    while (s_act != 0) {
+        if (s_act == 1) {
+            // ---- re-evaluate every stale candidate of the round at once
+            ++n_rounds;
+            if (s_stale[grp]) {
+                int miss = 0;
+                // global bitmap: L1-cached probes.  It is written only by this block
+                // (atomics, ordered before these loads by the block barriers), and
+                // S(v) is scanned in ascending set order when the index comes from
+                // the radix build, so neighbouring ids share cached lines
+                scan_ids<4>(a.set_ids, s_beg[grp], s_len[grp], gt, gsz, [&](int32_t i) {
+                    if (i >= 0)
+                        miss += !(((SB ? cov[i >> 5] : __ldca(cov + (i >> 5))) >> (i & 31)) & 1u);
+                });
+                miss = __reduce_add_sync(kFull, miss);
+                if (lane == 0 && miss) atomicAdd(&s_cnt[grp], miss);
+            }
+            __syncthreads();
+            if (warp == 0) {
+                for (int w = 0; w < W; ++w) {
+                    if (!s_stale[w]) continue;
+                    const int32_t l = s_cand[w];
+                    if (lane == 0) {
+                        key[l] = s_cnt[w];
+                        stamp[l] = j;
+                    }
                     ++n_evals;
-                    eval_entries += a.vtx_off[v + 1] - a.vtx_off[v];
+                    eval_entries += s_len[w];
+                    __syncwarp();
+                    prod_chunk_max(key, cmax, np, l >> 5, lane);
+                    __syncwarp();
                 }
-                __syncthreads();
-                // refresh the maxima of the chunks that changed, then the top
-                if (warp < W && s_cand[warp] >= 0)
-                    prod_chunk_max(key, cmax, np, s_cand[warp] >> 5, lane);
-                __syncthreads();
-                if (warp == 0) {
-                    unsigned long long best = 0ull;
-                    for (int32_t c = lane; c < nch; c += 32) best = cmax[c] > best ? cmax[c] : best;
-                    best = warp_max_u64(best);
-                    if (lane == 0) s_top = best;
+                select();
+            }
+        } else {
+            // ---- take candidate 0; the next round's are selected meanwhile
+            const int32_t l = s_cand[0];
+            const int64_t sb = s_beg[0];
+            const int32_t n = s_len[0];
+            __syncthreads();                     // everyone has read the candidate
+            if (warp == 0) {
+                const int32_t gain = key[l];
+                __syncwarp();                    // every lane has read it
+                if (lane == 0) {
+                    const int32_t v = (int32_t)cinfo[l].w;
+                    a.local_seeds[(int64_t)p * a.k + j] = v;
+                    a.local_gains[(int64_t)p * a.k + j] = gain;
+                    if (j < a.trunc) {
+                        a.elems[(int64_t)j * a.P + p] = v;
+                        st_release_u32(&a.flags[(int64_t)j * a.P + p], 1u);
+                    }
+                    key[l] = 0;
                 }
-                __syncthreads();
-                if (s_top == 0ull) break;
+                total += gain;
+                cover_entries += n;
+                __syncwarp();
+                prod_chunk_max(key, cmax, np, l >> 5, lane);
+                __syncwarp();
+            }
+            ++j;
+            if (j < a.k) {
+                if (warp == 0) select();
+                else
+                    scan_ids<4>(a.set_ids, sb, n, (int)threadIdx.x - 32, (int)blockDim.x - 32, [&](int32_t i) {
+                        if (i >= 0) atomicOr(&cov[i >> 5], 1u << (i & 31));
+                    });
+            } else if (threadIdx.x == 0) {
+                s_act = 0;
             }
         }
-        const unsigned long long top = s_top;
-        const int32_t l = (int32_t)(0xffffffffu - (uint32_t)(top & 0xffffffffu));
-        if (stamp[l] != j) continue;                    // the top is still an upper bound
-        // ---- take it
-        const int32_t v = vtx[l];
-        const int64_t sb = a.vtx_off[v], se = a.vtx_off[v + 1];
-        const int64_t gain = (int64_t)(top >> 32);
-        if (threadIdx.x == 0) {
-            a.local_seeds[(int64_t)p * a.k + j] = v;
-            a.local_gains[(int64_t)p * a.k + j] = gain;
-            if (j < a.trunc) {
-                a.elems[(int64_t)j * a.P + p] = v;
-                st_release_u32(&a.flags[(int64_t)j * a.P + p], 1u);
-            }
-            key[l] = 0;
-        }
-        total += gain;
-        cover_entries += se - sb;
-        scan_ids<4>(a.set_ids, sb, se - sb, threadIdx.x, blockDim.x, [&](int32_t i) {
-            if (i >= 0) atomicOr(&cov[i >> 5], 1u << (i & 31));
-        });
         __syncthreads();
-        if (warp == 0) prod_chunk_max(key, cmax, np, l >> 5, lane);
-        __syncthreads();
-        ++j;
     }
-    (void)shm;
-    (void)shs;
     if (threadIdx.x == 0) {
         a.local_n[p] = j;
         a.local_cov[p] = total;
         for (int32_t jj = j; jj < a.trunc; ++jj) st_release_u32(&a.flags[(int64_t)jj * a.P + p], 2u);
-    }
-    n_evals = block_sum_i64(n_evals, shs);
-    eval_entries = block_sum_i64(eval_entries, shs);
-    if (threadIdx.x == 0 && a.stats) {
-        long long *st = a.stats + 6 * (int64_t)p;
-        st[0] = (long long)t_begin;
-        st[1] = (long long)global_ns();
-        st[2] = n_rounds;
-        st[3] = n_evals;
-        st[4] = eval_entries;
-        st[5] = cover_entries;
+        if (a.stats) {
+            long long *st = a.stats + 6 * (int64_t)p;
+            st[0] = (long long)t_begin;
+            st[1] = (long long)global_ns();
+            st[2] = n_rounds + j;
+            st[3] = n_evals;
+            st[4] = eval_entries;
+            st[5] = cover_entries;
+        }
     }
     __syncthreads();
 }
@@ -772,21 +794,19 @@ __device__ void consume(const RGArgs &a, int b, long long *shs) {
     __syncthreads();
 }
 
-// The producers alone (two-launch mode): one block of kProdThreads per part.
+// The producers alone (two-launch mode): one block per part.
+template <bool SB>
 __global__ void __launch_bounds__(kProdThreads) k_rg_local(RGArgs a) {
     extern __shared__ int32_t key[];
-    __shared__ unsigned long long shm[33];
-    __shared__ long long shs[33];
-    for (int p = blockIdx.x; p < a.P; p += gridDim.x) produce(a, p, key, shm, shs);
+    for (int p = blockIdx.x; p < a.P; p += gridDim.x) produce<SB>(a, p, key);
 }
 
 __global__ void __launch_bounds__(kRGThreads) k_randgreedi(RGArgs a) {
     extern __shared__ int32_t key[];
-    __shared__ unsigned long long shm[33];
     __shared__ long long shs[33];
     const int r = blockIdx.x;
     if (a.first_role == 0 && r < a.nprod) {
-        for (int p = r; p < a.P; p += a.nprod) produce(a, p, key, shm, shs);
+        for (int p = r; p < a.P; p += a.nprod) produce<false>(a, p, key);
     } else {
         const int c = a.first_role == 0 ? r - a.nprod : r;
         for (int b = c; b < a.B; b += a.ncons) consume(a, b, shs);
@@ -1552,9 +1572,10 @@ im_status randgreedi(im_pool *p, int32_t k, const im_cover_opts *o, int32_t *d_s
     IM_CUDA(cudaStreamSynchronize(st));
     int32_t max_np = 0;
     for (int q = 0; q < P; ++q) max_np = std::max(max_np, hoff[q + 1] - hoff[q]);
+    max_np = std::max((max_np + 1) & ~1, 2);             // (16-byte steps in shared memory)
     // key + stamp (4 bytes each per candidate) + one 8-byte maximum per 32
-    const size_t prod_smem = (size_t)std::max(max_np, 1) * 8 + (size_t)((max_np + 31) / 32) * 8;
-    if (prod_smem > 200 * 1024) {
+    size_t prod_smem = (size_t)max_np * 8 + (size_t)((max_np + 63) / 64) * 16;
+    if (prod_smem > kProdSmemCap) {
         set_error("RandGreedi: a vertex part is too large for shared memory; use more partitions");
         return IM_ERR_UNSUPPORTED;
     }
@@ -1602,7 +1623,21 @@ im_status randgreedi(im_pool *p, int32_t k, const im_cover_opts *o, int32_t *d_s
         off += align256(bytes);
         return at;
     };
-    const size_t o_cov = take((size_t)P * words * 4);
+    // two-launch mode: the candidates' subsets, and the producers' bitmaps, in
+    // shared memory where they fit beside the keys.  A bitmap in global memory
+    // wants the L1 cache, which is what shared memory leaves of an SM's 256 KB:
+    // beside one, the subsets go there only below kProdInfoCap (at 7,100
+    // candidates and 4 x 10^6 sets, 177 KB: 3.49 ms against 2.82; at 2,050 and 2 x
+    // 10^6, 49 KB: 1.74 against 1.94).
+    const bool two = naive || o->fused == 0;
+    const size_t info_bytes = (size_t)max_np * sizeof(uint4), bits_bytes = (size_t)words * 4;
+    const bool smem_info = two && (prod_smem + info_bytes + bits_bytes <= kProdSmemCap ||
+                                   prod_smem + info_bytes <= kProdInfoCap);
+    if (smem_info) prod_smem += info_bytes;
+    const size_t bits_smem = prod_smem + bits_bytes;
+    const bool smem_bits = two && bits_smem <= kProdSmemCap;
+    const size_t o_cov = take(smem_bits ? 0 : (size_t)P * words * 4);
+    const size_t o_cinfo = take(smem_info ? 0 : (size_t)n * sizeof(uint4));
     const size_t o_flags = take((size_t)trunc * P * 4);
     const size_t o_elems = take((size_t)trunc * P * 4);
     const size_t o_l = take(64);
@@ -1657,6 +1692,8 @@ im_status randgreedi(im_pool *p, int32_t k, const im_cover_opts *o, int32_t *d_s
     a.part_off = p->part_off;
     a.part_vtx = p->part_vtx;
     a.covered = (uint32_t *)(Bs + o_cov);
+    a.cinfo = (uint4 *)(Bs + o_cinfo);
+    a.cinfo_smem = smem_info;
     a.bcovered = (uint32_t *)(Bs + o_bcov);
     a.local_seeds = p->rg_local_seeds;
     a.local_gains = p->rg_local_gains;
@@ -1670,7 +1707,7 @@ im_status randgreedi(im_pool *p, int32_t k, const im_cover_opts *o, int32_t *d_s
     a.flags = (uint32_t *)(Bs + o_flags);
     a.elems = (int32_t *)(Bs + o_elems);
     a.status = d_status;
-    a.max_np = std::max(max_np, 1);
+    a.max_np = max_np;
     a.evals = (int32_t)std::min<int64_t>(kProdW, std::max<int64_t>(1, tune_value(IM_TUNE_RG_EVALS)));
     a.stats = p->rg_stats;
     a.mask = use_masks ? (unsigned long long *)(Bs + o_mask) : nullptr;
@@ -1699,17 +1736,24 @@ im_status randgreedi(im_pool *p, int32_t k, const im_cover_opts *o, int32_t *d_s
                                             prod_smem, st));
     } else {
         // producers alone, then consumers alone (the stream is complete by then)
-        IM_TRY(raise_dyn_smem((const void *)k_rg_local, prod_smem));
+        const size_t local_smem = smem_bits ? bits_smem : prod_smem;
+        const void *local = smem_bits ? (const void *)k_rg_local<true> : (const void *)k_rg_local<false>;
+        IM_TRY(raise_dyn_smem(local, local_smem));
+        // more parts than SMs: smaller blocks, so that two parts share one
+        int threads = kProdThreads;
         int per_l = 0;
-        IM_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_l, k_rg_local, kProdThreads,
-                                                              prod_smem));
+        for (;; threads /= 2) {
+            IM_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_l, local, threads, local_smem));
+            if (per_l * num_sms() >= P || threads <= kProdMinThreads) break;
+        }
         if (per_l < 1) return IM_ERR_UNSUPPORTED;
         a.nprod = std::min<int32_t>(P, per_l * num_sms());
         a.ncons = 0;
         a.first_role = 0;
         {
             KernelTimer kt(st, "randgreedi_local");
-            k_rg_local<<<a.nprod, kProdThreads, prod_smem, st>>>(a);
+            if (smem_bits) k_rg_local<true><<<a.nprod, threads, local_smem, st>>>(a);
+            else k_rg_local<false><<<a.nprod, threads, local_smem, st>>>(a);
         }
         IM_CUDA(cudaGetLastError());
         const int64_t want = tune_value(IM_TUNE_RG_CLUSTER);   // 0 auto, -1 off, 1..8
