@@ -191,6 +191,25 @@ im_status dev_alloc(void **p, size_t bytes) {
     return IM_OK;
 }
 
+im_status call_alloc(void **p, size_t bytes, cudaStream_t st) {
+    *p = nullptr;
+    DevHeap *h = nullptr;
+    IM_CUDA(dev_heap(&h));
+    if (bytes == 0) bytes = 16;
+    cudaError_t e = cudaMallocFromPoolAsync(p, bytes, h->pool, st);
+    if (e == cudaErrorMemoryAllocation) {
+        cudaGetLastError();
+        IM_CUDA(cudaDeviceSynchronize());
+        cudaMemPoolTrimTo(h->pool, 0);
+        e = cudaMallocFromPoolAsync(p, bytes, h->pool, st);
+    }
+    if (e != cudaSuccess) {
+        *p = nullptr;
+        return cuda_fail(e, "device allocation");
+    }
+    return IM_OK;
+}
+
 im_status raise_dyn_smem(const void *func, size_t bytes) {
     constexpr size_t kDefault = 48 * 1024;   // the limit without opting in
     if (bytes <= kDefault) return IM_OK;

@@ -356,6 +356,12 @@ inline im_status dev_alloc(T **p, size_t bytes) {
     return dev_alloc(reinterpret_cast<void **>(p), bytes);
 }
 
+// A call's temporary memory, from the same cached memory pool but ordered on the
+// call's stream (free it there with cudaFreeAsync): the default memory pool
+// unmaps what is freed at the next synchronisation, and mapping it again cost
+// im_spread 2.6 ms a call.
+im_status call_alloc(void **p, size_t bytes, cudaStream_t st);
+
 // scratch arena of a pool: returns a pointer to at least `bytes` (256-aligned)
 im_status pool_scratch(im_pool *p, size_t bytes, void **out);
 

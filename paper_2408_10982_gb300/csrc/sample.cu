@@ -2063,10 +2063,10 @@ im_status build_lt_index(im_graph *g, cudaStream_t st) {
         }
     } x;
     const int64_t big_cap = m / (kLtBlockDeg + 1) + 1;
-    IM_CUDA(cudaMallocAsync((void **)&t.sizes, (size_t)n * 4, st));
-    IM_CUDA(cudaMallocAsync((void **)&t.big, (size_t)big_cap * 4, st));
-    IM_CUDA(cudaMallocAsync((void **)&t.toff, (size_t)(n + 1) * 8 + scan_tmp_bytes(n) + 256, st));
-    IM_CUDA(cudaMallocAsync((void **)&t.flags, 3 * sizeof(int), st));
+    IM_TRY(call_alloc((void **)&t.sizes, (size_t)n * 4, st));
+    IM_TRY(call_alloc((void **)&t.big, (size_t)big_cap * 4, st));
+    IM_TRY(call_alloc((void **)&t.toff, (size_t)(n + 1) * 8 + scan_tmp_bytes(n) + 256, st));
+    IM_TRY(call_alloc((void **)&t.flags, 3 * sizeof(int), st));
     IM_CUDA(cudaMemsetAsync(t.flags, 0, 3 * sizeof(int), st));
     {
         KernelTimer kt(st, "lt_index");
@@ -2329,7 +2329,7 @@ im_status run_sampling(const SamplingJob &job, const std::function<im_status(siz
         // (mapping fresh memory took 2 to 5 ms a call)
         int32_t *q2 = nullptr;
         const bool own = need2 > off - o_q;
-        if (own) IM_CUDA(cudaMallocAsync((void **)&q2, need2, st));
+        if (own) IM_TRY(call_alloc((void **)&q2, need2, st));
         else q2 = (int32_t *)(B + o_q);
         uint32_t *vis2 = (uint32_t *)((char *)q2 + (size_t)units * (size_t)n * 4);
         if (ic_big) IM_CUDA(cudaMemsetAsync(vis2, 0, (size_t)units * vis_words * 4, st));
@@ -2420,7 +2420,7 @@ im_status segmented_sort_sets(int32_t *dst, const int64_t *seg_off, int64_t nseg
         const int64_t gwords = (n_max + 31) / 32;
         const int blocks3 = (int)std::min<int64_t>(ngiant, num_sms());
         uint32_t *gbm = nullptr;
-        IM_CUDA(cudaMallocAsync((void **)&gbm, (size_t)blocks3 * gwords * 4, st));
+        IM_TRY(call_alloc((void **)&gbm, (size_t)blocks3 * gwords * 4, st));
         IM_CUDA(cudaMemsetAsync(gbm, 0, (size_t)blocks3 * gwords * 4, st));
         {
             KernelTimer kt(st, "sort_sets_bitmap");

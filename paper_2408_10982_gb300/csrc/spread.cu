@@ -387,8 +387,8 @@ im_status build_out_index(im_graph *g, cudaStream_t st) {
             if (scan_tmp) cudaFreeAsync(scan_tmp, st);
         }
     } t{st};
-    IM_CUDA(cudaMallocAsync((void **)&t.cnt, (size_t)n * 4, st));
-    IM_CUDA(cudaMallocAsync(&t.scan_tmp, scan_tmp_bytes(n), st));
+    IM_TRY(call_alloc((void **)&t.cnt, (size_t)n * 4, st));
+    IM_TRY(call_alloc(&t.scan_tmp, scan_tmp_bytes(n), st));
     IM_CUDA(cudaMalloc(&t.off, (size_t)(n + 1) * 8));
     IM_CUDA(cudaMalloc(&t.rec, (size_t)std::max<int64_t>(m, 1) * sizeof(uint4)));
     IM_CUDA(cudaMemsetAsync(t.cnt, 0, (size_t)n * 4, st));
@@ -471,7 +471,7 @@ extern "C" im_status im_spread(const im_graph *gc, im_model model, const int32_t
                  o_act = take(host_act ? (size_t)runs * 8 : 0),
                  o_hit = take(host_hit ? (size_t)runs : 0);
     char *B = nullptr;
-    IM_CUDA(cudaMallocAsync((void **)&B, off, st));
+    IM_TRY(call_alloc((void **)&B, off, st));
     IM_CUDA(cudaMemsetAsync(B + o_ctr, 0, 4 * 8, st));
     IM_CUDA(cudaMemsetAsync(B + o_vis, 0, (size_t)warps * words * 4, st));
     if (k > 0) IM_CUDA(cudaMemcpyAsync(B + o_seeds, seeds, (size_t)k * 4, cudaMemcpyDefault, st));
@@ -527,7 +527,7 @@ extern "C" im_status im_spread(const im_graph *gc, im_model model, const int32_t
         const size_t need = o_left + (size_t)a.groups * 4 * 8;
         char *N = B + o_q;
         if (need > (size_t)warps * qcap * 4) {
-            IM_CUDA(cudaMallocAsync((void **)&next, need, st));
+            IM_TRY(call_alloc((void **)&next, need, st));
             N = (char *)next;
         }
         a.next = (int32_t *)N;
