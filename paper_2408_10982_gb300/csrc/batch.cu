@@ -7,8 +7,8 @@
 //      run_sampling in sample.cu);
 //   2. one scan and one segmented sort over all sets;
 //   3. members are moved into one vertex space (query q's vertex u becomes
-//      vbase[q] + u) so that one histogram / scan / scatter builds the covering
-//      subsets of every query at once;
+//      vbase[q] + u) so that one radix sort builds the covering subsets of every
+//      query at once;
 //   4. one greedy launch, one block per query, running the lazy greedy of
 //      Alg. 2 with exact tie handling -- the standard greedy's result -- over
 //      a tournament: stale gains of the query's vertices in global memory,
@@ -75,19 +75,45 @@ __global__ void k_localize(int32_t *set_ids, const int64_t *vtx_off, int64_t n, 
         set_ids[t] -= (int32_t)sbase;
 }
 
-__global__ void k_globalize(const int64_t *set_off, int32_t *members, int64_t nsets,
-                            const int64_t *qset, const int64_t *vbase, int32_t nq) {
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < nsets;
-         i += (int64_t)gridDim.x * blockDim.x) {
-        int lo = 0, hi = nq - 1;
+// Moves the members into the batch's vertex space: those of query q, positions
+// [bounds[q], bounds[q + 1]), gain vbase[q].  A warp takes kGlobalRun positions.
+constexpr int kGlobalRun = 1024;
+
+__global__ void __launch_bounds__(256) k_globalize(int32_t *members, int64_t T, const int64_t *bounds,
+                                                   const int64_t *vbase, int32_t nq) {
+    const int lane = threadIdx.x & 31;
+    const int64_t warps = ((int64_t)gridDim.x * blockDim.x) >> 5;
+    for (int64_t t0 = (((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5) * kGlobalRun; t0 < T;
+         t0 += warps * kGlobalRun) {
+        int lo = 0, hi = nq - 1;                 // the query of the run's first position
         while (lo < hi) {
             const int mid = (lo + hi + 1) >> 1;
-            if (qset[mid] <= i) lo = mid;
+            if (__ldg(bounds + mid) <= t0) lo = mid;
             else hi = mid - 1;
         }
-        const int32_t vb = (int32_t)vbase[lo];
-        for (int64_t t = set_off[i]; t < set_off[i + 1]; ++t) members[t] += vb;
+        int64_t end = __ldg(bounds + lo + 1);
+        int32_t vb = (int32_t)__ldg(vbase + lo);
+#pragma unroll 8
+        for (int i = 0; i < kGlobalRun; i += 32) {
+            const int64_t t = t0 + i + lane;
+            if (t >= T) break;
+            while (t >= end) {
+                ++lo;
+                end = __ldg(bounds + lo + 1);
+                vb = (int32_t)__ldg(vbase + lo);
+            }
+            members[t] += vb;
+        }
     }
+}
+
+// Stage offsets of the second sampling launch, relative to its part of the
+// stage, become relative to the stage (kept apart from the flag in their top bits
+// by being far below it).
+__global__ void k_shift(const int64_t *in, int64_t count, int64_t by, int64_t *out) {
+    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < count;
+         i += (int64_t)gridDim.x * blockDim.x)
+        out[i] = in[i] + by;
 }
 
 __device__ __forceinline__ unsigned long long bmax(unsigned long long v, unsigned long long *sh) {
@@ -454,20 +480,11 @@ im_status im_solve_batch(im_batch *b, const im_query *qs, int32_t nq, int32_t km
             // gather sizes and stage offsets (relative to `stage`) in batch order
             IM_CUDA(cudaMemcpyAsync(sizes + done_sets, r.sizes, (size_t)nsets * 4,
                                     cudaMemcpyDeviceToDevice, st));
-            if (added == 0) {
-                IM_CUDA(cudaMemcpyAsync(stage_off + done_sets, r.stage_off, (size_t)nsets * 8,
-                                        cudaMemcpyDeviceToDevice, st));
-            } else {
-                // offsets of the second launch are relative to stage + added: shift them
-                std::vector<int64_t> h(nsets);
-                IM_CUDA(cudaMemcpyAsync(h.data(), r.stage_off, (size_t)nsets * 8,
-                                        cudaMemcpyDeviceToHost, st));
-                IM_CUDA(cudaStreamSynchronize(st));
-                for (auto &x : h) x += added;
-                IM_CUDA(cudaMemcpyAsync(stage_off + done_sets, h.data(), (size_t)nsets * 8,
-                                        cudaMemcpyHostToDevice, st));
-                IM_CUDA(cudaStreamSynchronize(st));
+            {
+                KernelTimer kt(st, "batch_shift");
+                k_shift<<<num_sms() * 4, 256, 0, st>>>(r.stage_off, nsets, added, stage_off + done_sets);
             }
+            IM_CUDA(cudaGetLastError());
             done_sets += nsets;
             added += r.added;
             long_sets += r.long_sets;
@@ -501,17 +518,31 @@ im_status im_solve_batch(im_batch *b, const im_query *qs, int32_t nq, int32_t km
                                 cudaMemcpyHostToDevice, st));
         IM_CUDA(cudaMemcpyAsync(A + o_qset, qset.data(), (size_t)(nq + 1) * 8, cudaMemcpyHostToDevice, st));
         IM_CUDA(cudaMemcpyAsync(A + o_vbase, vbase.data(), (size_t)nq * 8, cudaMemcpyHostToDevice, st));
-        if (sets_total > 0) {
+        int64_t *d_bounds = (int64_t *)(A + o_bounds);
+        {
+            KernelTimer kt(st, "batch_bounds");
+            k_query_bounds<<<std::max(1, std::min(num_sms(), (nq + 256) / 256)), 256, 0, st>>>(
+                set_off, (const int64_t *)(A + o_qset), nq, d_bounds);
+        }
+        if (added > 0) {
             KernelTimer kt(st, "batch_globalize");
-            k_globalize<<<num_sms() * 4, 256, 0, st>>>(set_off, members, sets_total,
-                                                       (const int64_t *)(A + o_qset),
+            k_globalize<<<num_sms() * 8, 256, 0, st>>>(members, added, d_bounds,
                                                        (const int64_t *)(A + o_vbase), nq);
         }
         IM_CUDA(cudaGetLastError());
         int64_t *vtx_off = (int64_t *)(A + o_voff);
         int32_t *set_ids = (int32_t *)(A + o_sids);
-        s = build_index_raw(set_off, members, sets_total, added, n_total, vtx_off, set_ids,
-                            (int32_t *)(A + o_cur), 1, tmp, st);
+        // the radix build where its buffers fit (the sampling scratch is free by
+        // now; 12 bytes a member), else the counting build
+        s = tune_value(IM_TUNE_INDEX_REPLICAS) == 0
+                ? grow(&b->sscratch, &b->sscratch_bytes, radix_index_bytes(added, n_total))
+                : IM_ERR_UNSUPPORTED;
+        if (s == IM_OK)
+            s = build_index_radix(set_off, members, sets_total, added, n_total, vtx_off, set_ids,
+                                  (int32_t *)(A + o_cur), b->sscratch, st);
+        else
+            s = build_index_raw(set_off, members, sets_total, added, n_total, vtx_off, set_ids,
+                                (int32_t *)(A + o_cur), 1, tmp, st);
         if (s != IM_OK) return s;
         // 4. seed selection.  A block-per-query lazy greedy suits many small
         // queries; a query holding a large share of the batch's members would
@@ -525,13 +556,6 @@ im_status im_solve_batch(im_batch *b, const im_query *qs, int32_t nq, int32_t km
         int64_t *d_gains = (int64_t *)(A + o_out + up256((size_t)nq * kmax * 4));
         int32_t *d_ns = (int32_t *)((char *)d_gains + up256((size_t)nq * kmax * 8));
         int64_t *d_cov = (int64_t *)((char *)d_ns + up256((size_t)nq * 4));
-        int64_t *d_bounds = (int64_t *)(A + o_bounds);
-        {
-            KernelTimer kt(st, "batch_bounds");
-            k_query_bounds<<<std::max(1, std::min(num_sms(), (nq + 256) / 256)), 256, 0, st>>>(
-                set_off, (const int64_t *)(A + o_qset), nq, d_bounds);
-        }
-        IM_CUDA(cudaGetLastError());
         std::vector<int64_t> hb(nq + 1);
         IM_CUDA(cudaMemcpyAsync(hb.data(), d_bounds, (size_t)(nq + 1) * 8, cudaMemcpyDeviceToHost, st));
         IM_CUDA(cudaStreamSynchronize(st));

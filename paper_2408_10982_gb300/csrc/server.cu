@@ -67,7 +67,7 @@ struct im_server {
 namespace {
 
 // device bytes a request needs inside a batch: stage + members + covering
-// subsets (12 B per member), set offsets and sizes (20 B per set), the
+// subsets (12 B per member) and the buffers of their sort (12 B), set offsets and sizes (20 B per set), the
 // covered bitmap, and per-vertex greedy state (24 B per vertex)
 int64_t footprint(im_server *s, const im_query &q) {
     auto it = s->per_set.find({q.graph, q.model});
@@ -77,7 +77,7 @@ int64_t footprint(im_server *s, const im_query &q) {
         const int64_t P = q.cover.partitions > 0 ? q.cover.partitions : 148;
         rg = P * ((q.theta + 31) / 32) * 4 + q.theta * 8 + q.graph->n * 16;
     }
-    return (int64_t)((double)q.theta * per * 1.5 * 12.0) + q.theta * 20 + q.theta / 8 +
+    return (int64_t)((double)q.theta * per * 1.5 * 24.0) + q.theta * 20 + q.theta / 8 +
            q.graph->n * 24 + rg + 4096;
 }
 
