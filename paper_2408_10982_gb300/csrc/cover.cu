@@ -48,6 +48,7 @@ constexpr int kUnroll = 8;                   // independent loads in flight per 
 constexpr int kSpec = 32;                    // largest speculative group of stream elements
 constexpr size_t kClusterSmemCap = 200 * 1024;  // bucket bitmap slice per block
 constexpr int kMaskG = 64;                   // largest group of stream slots (mask stage)
+constexpr int kMaskWindow = 512;             // ... slots read ahead (mask stage)
 constexpr int kMaskStrips = 16;              // entries per lane in one warp work item
 constexpr int kMaskItem = 32 * kMaskStrips;  // entries per warp work item
 
@@ -1009,8 +1010,11 @@ __device__ __forceinline__ void mask_item_prefix(int64_t *s_off, int gn, F &&f) 
 }
 
 __global__ void __launch_bounds__(kRGThreads) k_rg_stream_masks(RGArgs a) {
-    __shared__ int32_t s_x[kMaskG];
-    __shared__ int64_t s_beg[kMaskG], s_len[kMaskG];
+    // a window of the stream's slots, read ahead of the groups
+    __shared__ int32_t s_wx[kMaskWindow];
+    __shared__ int64_t s_wbeg[kMaskWindow], s_wlen[kMaskWindow];
+    __shared__ int32_t s_cnt0[kMaskG + 1];           // block 0: elements in the group's first u slots
+    __shared__ int64_t s_len0[kMaskG + 1];           // ... and the entries of their subsets
     __shared__ uint32_t s_g[kMaskG * 64];            // the group's gains, staged once
     __shared__ unsigned long long s_pass[64];        // slots reaching each bucket's threshold
     __shared__ int64_t s_thr[64];
@@ -1047,20 +1051,39 @@ __global__ void __launch_bounds__(kRGThreads) k_rg_stream_masks(RGArgs a) {
         s_scan[threadIdx.x] = 0;
     }
     if (!grid_sync(a.bar, gridDim.x, a.status)) return;
-    int64_t g0 = 0;
+    int64_t g0 = 0, w0 = -1;                         // the window holds slots [w0, w0 + kMaskWindow)
     int G = 8, buf = 0;
     while (g0 < nslots) {
         const int gn = (int)(nslots - g0 < G ? nslots - g0 : G);
-        if (threadIdx.x < gn) {
-            const int64_t t = g0 + threadIdx.x;
-            s_x[threadIdx.x] = __ldcg(a.slot_x + t);
-            s_beg[threadIdx.x] = __ldcg(a.slot_beg + t);
-            s_len[threadIdx.x] = __ldcg(a.slot_len + t);
-            s_acc[threadIdx.x] = 0ull;
+        if (w0 < 0 || g0 + kMaskG > w0 + kMaskWindow) {
+            w0 = g0;
+            for (int i = threadIdx.x; i < kMaskWindow && w0 + i < nslots; i += blockDim.x) {
+                s_wx[i] = __ldcg(a.slot_x + w0 + i);
+                s_wbeg[i] = __ldcg(a.slot_beg + w0 + i);
+                s_wlen[i] = __ldcg(a.slot_len + w0 + i);
+            }
         }
+        const int32_t *s_x = s_wx + (g0 - w0);       // the group's slots
+        const int64_t *s_beg = s_wbeg + (g0 - w0), *s_len = s_wlen + (g0 - w0);
+        if (threadIdx.x < kMaskG) s_acc[threadIdx.x] = 0ull;
         if (threadIdx.x == 0) s_cut = gn;
         __syncthreads();
         mask_item_prefix(s_off, gn, [&](int u) { return (s_len[u] + kMaskItem - 1) / kMaskItem; });
+        if (blockIdx.x == 0 && threadIdx.x >= 32 && threadIdx.x < 64) {
+            const int u0 = 2 * lane, u1 = u0 + 1;
+            const int32_t c0 = u0 < gn && s_x[u0] >= 0, c1 = u1 < gn && s_x[u1] >= 0;
+            const int64_t l0 = c0 ? s_len[u0] : 0, l1 = c1 ? s_len[u1] : 0;
+            const int32_t ci = warp_incl_scan<int32_t>(c0 + c1, lane);
+            const int64_t li = warp_incl_scan<int64_t>(l0 + l1, lane);
+            s_cnt0[u0] = ci - c0 - c1;
+            s_cnt0[u1] = ci - c1;
+            s_len0[u0] = li - l0 - l1;
+            s_len0[u1] = li - l1;
+            if (lane == 31) {
+                s_cnt0[kMaskG] = ci;
+                s_len0[kMaskG] = li;
+            }
+        }
         __syncthreads();
         uint32_t *gb = a.gbuf + (size_t)buf * kMaskG * 64;
         // ---- counts of every slot of the group against the current masks
@@ -1161,12 +1184,11 @@ __global__ void __launch_bounds__(kRGThreads) k_rg_stream_masks(RGArgs a) {
             }
             // diagnostics: slots this bucket considered (up to the cut, or to
             // its accept when that filled it)
-            const int last = (first < cut && s_n[b] == a.k) ? first + 1 : cut;
-            for (int u = 0; u < last; ++u)
-                if (s_x[u] >= 0) {
-                    ++s_eval[b];
-                    s_scan[b] += s_len[u];
-                }
+            if (blockIdx.x == 0) {
+                const int last = (first < cut && s_n[b] == a.k) ? first + 1 : cut;
+                s_eval[b] += s_cnt0[last];
+                s_scan[b] += s_len0[last];
+            }
         }
         __syncthreads();
         // ---- or the accepted subsets into the masks; clear the other buffer
