@@ -9,10 +9,8 @@
 //   3. members are moved into one vertex space (query q's vertex u becomes
 //      vbase[q] + u) so that one radix sort builds the covering subsets of every
 //      query at once;
-//   4. one greedy launch, one block per query, running the lazy greedy of
-//      Alg. 2 with exact tie handling -- the standard greedy's result -- over
-//      a tournament: stale gains of the query's vertices in global memory,
-//      the maximum of every 1024-vertex chunk in shared memory.
+//   4. one launch of the standard greedy for all plain queries, each on a group
+//      of blocks by its share of the members (greedy_many in cover.cu).
 // Each query's result equals what it gets alone (the random stream of a
 // sample depends only on the query's seed and the sample id).
 #include <algorithm>
@@ -45,9 +43,6 @@ struct im_batch {
 namespace im {
 namespace {
 
-constexpr int kBGThreads = 1024;
-constexpr int kChunkV = 1024;      // vertices per tournament chunk
-
 struct BatchQuery {
     int64_t vbase;     // first vertex of the query in the batch vertex space
     int64_t n;
@@ -56,7 +51,6 @@ struct BatchQuery {
     int64_t cbase;     // first word of the query's covered bitmap
     int64_t out;       // row of the query in the seeds output (original index)
     int32_t k;
-    int32_t pad;       // 1: the query runs the grid-wide greedy, not a block
 };
 
 // First member position of every query's sets: out[i] = set_off[qset[i]].
@@ -114,142 +108,6 @@ __global__ void k_shift(const int64_t *in, int64_t count, int64_t by, int64_t *o
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < count;
          i += (int64_t)gridDim.x * blockDim.x)
         out[i] = in[i] + by;
-}
-
-__device__ __forceinline__ unsigned long long bmax(unsigned long long v, unsigned long long *sh) {
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        const unsigned long long t = __shfl_xor_sync(kFull, v, o);
-        v = t > v ? t : v;
-    }
-    if (lane == 0) sh[warp] = v;
-    __syncthreads();
-    if (warp == 0) {
-        unsigned long long x = lane < (int)(blockDim.x >> 5) ? sh[lane] : 0ull;
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) {
-            const unsigned long long t = __shfl_xor_sync(kFull, x, o);
-            x = t > x ? t : x;
-        }
-        if (lane == 0) sh[32] = x;
-    }
-    __syncthreads();
-    const unsigned long long r = sh[32];
-    __syncthreads();
-    return r;
-}
-
-__device__ __forceinline__ long long bsum(long long v, long long *sh) {
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    v = warp_sum<long long>(v);
-    if (lane == 0) sh[warp] = v;
-    __syncthreads();
-    if (warp == 0) {
-        long long x = lane < (int)(blockDim.x >> 5) ? sh[lane] : 0ll;
-        x = warp_sum<long long>(x);
-        if (lane == 0) sh[32] = x;
-    }
-    __syncthreads();
-    const long long r = sh[32];
-    __syncthreads();
-    return r;
-}
-
-__device__ __forceinline__ unsigned long long pack(int32_t gain, int64_t l) {
-    return gain > 0 ? (((unsigned long long)(uint32_t)gain << 32) | (0xffffffffu - (uint32_t)l)) : 0ull;
-}
-
-// Lazy greedy of one query per block.  key[v] is v's marginal gain, exact
-// when stamp[v] equals the current round and an upper bound otherwise; cm[c]
-// is the packed maximum of chunk c.  A fresh winner is the standard greedy's
-// pick (ties to the smallest id); a stale one is re-evaluated.
-__global__ void __launch_bounds__(kBGThreads) k_batch_greedy(
-    const BatchQuery *bq, int32_t nq, const int64_t *vtx_off, const int32_t *set_ids, int32_t *key,
-    int32_t *stamp, uint32_t *covered, int32_t *seeds, int64_t *gains, int32_t kmax,
-    int32_t *nseeds, int64_t *coverage) {
-    extern __shared__ unsigned long long cm[];
-    __shared__ unsigned long long shm[33];
-    __shared__ long long shs[33];
-    for (int qi = blockIdx.x; qi < nq; qi += gridDim.x) {
-        const BatchQuery Q = bq[qi];
-        if (Q.pad) continue;                 // run by the grid-wide greedy instead
-        const int64_t nch = (Q.n + kChunkV - 1) / kChunkV;
-        int32_t *kq = key + Q.vbase;
-        int32_t *sq = stamp + Q.vbase;
-        uint32_t *cov = covered + Q.cbase;
-        const int64_t words = (Q.theta + 31) / 32;
-        for (int64_t x = threadIdx.x; x < words; x += blockDim.x) cov[x] = 0u;
-        for (int64_t v = threadIdx.x; v < Q.n; v += blockDim.x) {
-            const int64_t gv = Q.vbase + v;
-            kq[v] = (int32_t)(vtx_off[gv + 1] - vtx_off[gv]);   // exact: nothing covered yet
-            sq[v] = 0;
-        }
-        __syncthreads();
-        // chunk maxima: one warp per chunk
-        {
-            const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-            for (int64_t c = warp; c < nch; c += blockDim.x >> 5) {
-                unsigned long long m = 0;
-                for (int64_t l = c * kChunkV + lane; l < min(Q.n, (c + 1) * kChunkV); l += 32) {
-                    const unsigned long long p = pack(kq[l], l);
-                    m = p > m ? p : m;
-                }
-                m = warp_max_u64(m);
-                if (lane == 0) cm[c] = m;
-            }
-        }
-        __syncthreads();
-        int32_t j = 0;
-        int64_t total = 0;
-        while (j < Q.k) {
-            unsigned long long best = 0;
-            for (int64_t c = threadIdx.x; c < nch; c += blockDim.x) best = cm[c] > best ? cm[c] : best;
-            best = bmax(best, shm);
-            if (best == 0) break;                                   // every gain is zero
-            const int64_t l = (int64_t)(0xffffffffu - (uint32_t)(best & 0xffffffffu));
-            const int64_t gv = Q.vbase + l;
-            const int64_t sb = vtx_off[gv], se = vtx_off[gv + 1];
-            if (sq[l] != j) {
-                long long miss = 0;
-                for (int64_t t = sb + threadIdx.x; t < se; t += blockDim.x) {
-                    const int64_t i = (int64_t)set_ids[t] - Q.sbase;
-                    miss += !((cov[i >> 5] >> (i & 31)) & 1u);
-                }
-                const long long g = bsum(miss, shs);
-                if (threadIdx.x == 0) {
-                    kq[l] = (int32_t)g;
-                    sq[l] = j;
-                }
-            } else {
-                const int64_t gain = (int64_t)(best >> 32);
-                if (threadIdx.x == 0) {
-                    seeds[Q.out * kmax + j] = (int32_t)l;
-                    gains[Q.out * kmax + j] = gain;
-                    kq[l] = 0;
-                }
-                for (int64_t t = sb + threadIdx.x; t < se; t += blockDim.x) {
-                    const int64_t i = (int64_t)set_ids[t] - Q.sbase;
-                    atomicOr(&cov[i >> 5], 1u << (i & 31));
-                }
-                total += gain;
-                ++j;
-            }
-            __syncthreads();
-            // refresh the maximum of l's chunk
-            const int64_t c = l / kChunkV;
-            const int64_t v = c * kChunkV + threadIdx.x;
-            const unsigned long long p = v < Q.n ? pack(kq[v], v) : 0ull;
-            const unsigned long long m = bmax(p, shm);
-            if (threadIdx.x == 0) cm[c] = m;
-            __syncthreads();
-        }
-        if (threadIdx.x == 0) {
-            nseeds[Q.out] = j;
-            coverage[Q.out] = total;
-        }
-        __syncthreads();
-    }
 }
 
 size_t up256(size_t x) { return (x + 255) & ~(size_t)255; }
@@ -397,7 +255,6 @@ im_status im_solve_batch(im_batch *b, const im_query *qs, int32_t nq, int32_t km
         bq[i].cbase = cb;
         bq[i].out = order[i];
         bq[i].k = Q.k;
-        bq[i].pad = 0;
         vbase[i] = vb;
         qset[i] = sb;
         vb += Q.graph->n;
@@ -426,14 +283,14 @@ im_status im_solve_batch(im_batch *b, const im_query *qs, int32_t nq, int32_t km
                      o_stoff = take((size_t)std::max<int64_t>(sets_total, 1) * 8),
                      o_voff = take((size_t)(n_total + 1) * 8), o_cur = take((size_t)n_total * 4),
                      o_key = take((size_t)n_total * 4), o_stamp = take((size_t)n_total * 4),
-                     o_cov = take((size_t)cov_words * 4), o_bq = take((size_t)nq * sizeof(BatchQuery)),
+                     o_cov = take((size_t)cov_words * 4),
                      o_qset = take((size_t)(nq + 1) * 8), o_vbase = take((size_t)nq * 8),
                      o_tmp = take(std::max(scan_tmp_bytes(std::max(sets_total, n_total)),
                                            (size_t)(2 + 2 * std::max<int64_t>(sets_total, 1)) * 8)),
                      o_out = take(up256((size_t)nq * kmax * 4) + up256((size_t)nq * kmax * 8) +
                                   up256((size_t)nq * 4) + up256((size_t)nq * 8)),
                      o_bounds = take((size_t)(nq + 1) * 8),
-                     o_best = take((size_t)num_sms() * 8 * 8), o_gbar = take(256);
+                     o_many = take(greedy_many_scratch(nq, cap)), o_gbar = take(256);
         im_status s = grow(&b->arena, &b->arena_bytes, off);
         if (s != IM_OK) return s;
         char *A = (char *)b->arena;
@@ -514,8 +371,6 @@ im_status im_solve_batch(im_batch *b, const im_query *qs, int32_t nq, int32_t km
                                 long_sets, st);
         if (s != IM_OK) return s;
         // 3. one vertex space, one index
-        IM_CUDA(cudaMemcpyAsync(A + o_bq, bq.data(), (size_t)nq * sizeof(BatchQuery),
-                                cudaMemcpyHostToDevice, st));
         IM_CUDA(cudaMemcpyAsync(A + o_qset, qset.data(), (size_t)(nq + 1) * 8, cudaMemcpyHostToDevice, st));
         IM_CUDA(cudaMemcpyAsync(A + o_vbase, vbase.data(), (size_t)nq * 8, cudaMemcpyHostToDevice, st));
         int64_t *d_bounds = (int64_t *)(A + o_bounds);
@@ -544,14 +399,7 @@ im_status im_solve_batch(im_batch *b, const im_query *qs, int32_t nq, int32_t km
             s = build_index_raw(set_off, members, sets_total, added, n_total, vtx_off, set_ids,
                                 (int32_t *)(A + o_cur), 1, tmp, st);
         if (s != IM_OK) return s;
-        // 4. seed selection.  A block-per-query lazy greedy suits many small
-        // queries; a query holding a large share of the batch's members would
-        // keep one SM busy long after the rest finish, so those run the
-        // grid-wide greedy, one cooperative launch each.  Cost model (rates
-        // measured on GB300 at the batched mix): a block scans ~0.36 G
-        // entries/s, the grid greedy ~17 G entries/s over a ~0.8 ms floor of
-        // k barrier-bound steps; the largest queries are moved to the grid
-        // while that lowers max(block phase) + sum(grid launches).
+        // 4. seed selection: the plain queries in one launch, on groups of blocks
         int32_t *d_seeds = (int32_t *)(A + o_out);
         int64_t *d_gains = (int64_t *)(A + o_out + up256((size_t)nq * kmax * 4));
         int32_t *d_ns = (int32_t *)((char *)d_gains + up256((size_t)nq * kmax * 8));
@@ -559,72 +407,44 @@ im_status im_solve_batch(im_batch *b, const im_query *qs, int32_t nq, int32_t km
         std::vector<int64_t> hb(nq + 1);
         IM_CUDA(cudaMemcpyAsync(hb.data(), d_bounds, (size_t)(nq + 1) * 8, cudaMemcpyDeviceToHost, st));
         IM_CUDA(cudaStreamSynchronize(st));
-        // RandGreedi queries (pad 2) run after the greedy launches, one by one
-        std::vector<int32_t> by_size;
-        for (int32_t i = 0; i < nq; ++i)
-            if (qs[order[i]].cover.algo != IM_RANDGREEDI) by_size.push_back(i);
-        const int32_t ng = (int32_t)by_size.size();
-        std::sort(by_size.begin(), by_size.end(), [&](int32_t x, int32_t y) {
-            return hb[x + 1] - hb[x] > hb[y + 1] - hb[y];
-        });
-        const double rb = 0.36e9, rg = 17e9, t0 = 0.8e-3;
-        const double slots = 2.0 * num_sms();
-        double rest = 0.0, grid_t = 0.0;
-        for (int32_t x : by_size) rest += (double)(hb[x + 1] - hb[x]);
-        double best_t = std::max((ng ? (double)(hb[by_size[0] + 1] - hb[by_size[0]]) : 0.0) / rb,
-                                 rest / (rb * slots));
-        int32_t n_grid = 0;
-        for (int32_t r = 0; r < ng; ++r) {
-            const double w = (double)(hb[by_size[r] + 1] - hb[by_size[r]]);
-            grid_t += t0 + w / rg;
-            rest -= w;
-            const double next = r + 1 < ng ? (double)(hb[by_size[r + 1] + 1] - hb[by_size[r + 1]]) : 0.0;
-            const double t = grid_t + std::max(next / rb, rest / (rb * slots));
-            if (t < best_t) {
-                best_t = t;
-                n_grid = r + 1;
-            }
-        }
-        for (int32_t i = 0; i < nq; ++i) bq[i].pad = 2;
-        for (int32_t r = 0; r < ng; ++r) bq[by_size[r]].pad = r < n_grid ? 1 : 0;
-        IM_CUDA(cudaMemcpyAsync(A + o_bq, bq.data(), (size_t)nq * sizeof(BatchQuery),
-                                cudaMemcpyHostToDevice, st));
-        int64_t max_nch = 1;
-        for (auto &x : bq) max_nch = std::max<int64_t>(max_nch, (x.n + kChunkV - 1) / kChunkV);
-        const size_t smem = (size_t)max_nch * 8;
-        if (smem > 200 * 1024) {
+        // (a batch takes graphs of at most this many vertices)
+        if ((n_max + 1023) / 1024 * 8 > 200 * 1024) {
             set_error("im_solve_batch: a query graph is too large for the batched greedy");
             return IM_ERR_UNSUPPORTED;
         }
-        IM_TRY(raise_dyn_smem((const void *)k_batch_greedy, smem));
-        if (n_grid < ng) {
-            KernelTimer kt(st, "batch_greedy");
-            k_batch_greedy<<<(unsigned)std::min<int64_t>(nq, (int64_t)num_sms() * 2), kBGThreads, smem,
-                             st>>>((const BatchQuery *)(A + o_bq), nq, vtx_off, set_ids,
-                                   (int32_t *)(A + o_key), (int32_t *)(A + o_stamp),
-                                   (uint32_t *)(A + o_cov), d_seeds, d_gains, kmax, d_ns, d_cov);
-        }
-        IM_CUDA(cudaGetLastError());
-        int *d_gstatus = (int *)(A + o_gbar + sizeof(GridBarrier) + 64);
+        int *d_gstatus = (int *)(A + o_gbar);
         IM_CUDA(cudaMemsetAsync(d_gstatus, 0, sizeof(int), st));
-        for (int32_t r = 0; r < n_grid; ++r) {
-            const BatchQuery &Q = bq[by_size[r]];
-            IM_CUDA(cudaMemsetAsync(A + o_gbar, 0, sizeof(GridBarrier), st));
-            s = greedy_launch_view(Q.n, Q.theta, set_off, members, vtx_off + Q.vbase, set_ids,
-                                   Q.sbase, Q.vbase, Q.k, (int32_t *)(A + o_key) + Q.vbase,
-                                   (uint32_t *)(A + o_cov) + Q.cbase,
-                                   (unsigned long long *)(A + o_best), num_sms() * 8,
-                                   A + o_gbar, d_seeds + Q.out * kmax, d_gains + Q.out * kmax,
-                                   d_ns + Q.out, d_cov + Q.out, d_gstatus, st);
-            if (s != IM_OK) return s;
+        std::vector<GreedyQuery> gq;
+        for (int32_t i = 0; i < nq; ++i) {
+            if (qs[order[i]].cover.algo == IM_RANDGREEDI) continue;
+            const BatchQuery &Q = bq[i];
+            GreedyQuery g;
+            g.n = Q.n;
+            g.theta = Q.theta;
+            g.members = hb[i + 1] - hb[i];
+            g.vtx_off = vtx_off + Q.vbase;
+            g.sshift = Q.sbase;
+            g.vshift = Q.vbase;
+            g.k = Q.k;
+            g.counts = (int32_t *)(A + o_key) + Q.vbase;
+            g.ranks = (int32_t *)(A + o_stamp) + Q.vbase;
+            g.cands = (int32_t *)(A + o_cur) + Q.vbase;
+            g.covered = (uint32_t *)(A + o_cov) + Q.cbase;
+            g.seeds = d_seeds + Q.out * kmax;
+            g.gains = d_gains + Q.out * kmax;
+            g.nseeds = d_ns + Q.out;
+            g.coverage = d_cov + Q.out;
+            gq.push_back(g);
         }
+        s = greedy_many(gq, set_off, members, set_ids, A + o_many, d_gstatus, st);
+        if (s != IM_OK) return s;
         // RandGreedi queries: each on a view of the batch's index, with its own
         // set ids; the partition count picked by timing when the query leaves it open
         std::vector<int32_t> parts_used(nq, 0);
         for (int32_t i = 0; i < nq; ++i) {
             const BatchQuery &Q = bq[i];
-            if (Q.pad != 2) continue;
             const im_query &q = qs[order[i]];
+            if (q.cover.algo != IM_RANDGREEDI) continue;
             {
                 KernelTimer kt(st, "batch_localize");
                 k_localize<<<num_sms() * 4, 256, 0, st>>>(set_ids, vtx_off + Q.vbase, Q.n, Q.sbase);

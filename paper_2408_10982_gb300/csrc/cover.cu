@@ -174,10 +174,10 @@ constexpr int kHubShift = 6;            // hubs: |S(v)| >= max |S(v)| / 64
 // makes the frozen gains exact and every step reads all.
 // Warps take kGreedyChunk-entry chunks of S(v*) from a per-step counter.  Every wait is
 // bounded (grid_sync).
-__global__ void __launch_bounds__(kGreedyThreads, 2) k_greedy(GreedyArgs a) {
-    __shared__ unsigned long long shm[33];
-    const uint32_t nb = gridDim.x;
-    const int64_t tid = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+// Run by block `rank` of `nb`; false: a wait ran out.
+__device__ __forceinline__ bool greedy_steps(const GreedyArgs &a, uint32_t rank, uint32_t nb,
+                                             unsigned long long *shm) {
+    const int64_t tid = (int64_t)rank * blockDim.x + threadIdx.x;
     const int64_t stride = (int64_t)nb * blockDim.x;
     const int lane = threadIdx.x & 31;
     const int64_t gwarp = tid >> 5, nwarps = stride >> 5;
@@ -198,7 +198,7 @@ __global__ void __launch_bounds__(kGreedyThreads, 2) k_greedy(GreedyArgs a) {
         lmax = block_max_u64(lmax, shm);
         if (threadIdx.x == 0 && lmax) atomicMax(a.ctl + 2, (int32_t)lmax);
     }
-    if (!grid_sync(a.bar, nb, a.status)) return;
+    if (!grid_sync(a.bar, nb, a.status)) return false;
     uint32_t tau = 0;                        // > 0: the argmax reads hubs + candidates
     int32_t nhub = 0, ncand = 0;
     if (a.hub_rank) {
@@ -225,7 +225,7 @@ __global__ void __launch_bounds__(kGreedyThreads, 2) k_greedy(GreedyArgs a) {
             a.hub_rank[v] = r;
             if (r == -1 && tau > 0) a.cand[atomicAdd(a.ctl + 1, 1)] = (int32_t)v;
         }
-        if (!grid_sync(a.bar, nb, a.status)) return;
+        if (!grid_sync(a.bar, nb, a.status)) return false;
         nhub = min(__ldcg(a.ctl + 0), a.hub_cap);
         ncand = __ldcg(a.ctl + 1);
     }
@@ -261,8 +261,8 @@ __global__ void __launch_bounds__(kGreedyThreads, 2) k_greedy(GreedyArgs a) {
             consider(c, (uint32_t)__ldcg(a.hub_list + h));
         }
         best = block_max_u64(best, shm);
-        if (threadIdx.x == 0) a.block_best[blockIdx.x] = best;
-        if (!grid_sync(a.bar, nb, a.status)) return;
+        if (threadIdx.x == 0) a.block_best[rank] = best;
+        if (!grid_sync(a.bar, nb, a.status)) return false;
         unsigned long long gbest = 0;
         for (uint32_t b = threadIdx.x; b < nb; b += blockDim.x) {
             const unsigned long long x = __ldcg(a.block_best + b);
@@ -289,13 +289,13 @@ __global__ void __launch_bounds__(kGreedyThreads, 2) k_greedy(GreedyArgs a) {
                 }
             }
             tau = 0;
-            if (!grid_sync(a.bar, nb, a.status)) return;
+            if (!grid_sync(a.bar, nb, a.status)) return false;
             continue;
         }
         if (gbest == 0) break;                       // every remaining gain is zero
         const int32_t vs = (int32_t)(0xffffffffu - (uint32_t)(gbest & 0xffffffffu));
         const int64_t gain = (int64_t)(gbest >> 32);
-        if (blockIdx.x == 0 && threadIdx.x == 0) {
+        if (rank == 0 && threadIdx.x == 0) {
             a.seeds[j] = vs;
             a.gains[j] = gain;
         }
@@ -305,7 +305,7 @@ __global__ void __launch_bounds__(kGreedyThreads, 2) k_greedy(GreedyArgs a) {
         // is cleared meanwhile (its last use ended at the previous step's
         // closing barrier)
         unsigned long long *work = a.work ? a.work + (j & 1) : nullptr;
-        if (work && blockIdx.x == 0 && threadIdx.x == 0) a.work[(j + 1) & 1] = 0ull;
+        if (work && rank == 0 && threadIdx.x == 0) a.work[(j + 1) & 1] = 0ull;
         for (int64_t base = sb + gwarp * kGreedyChunk;;) {
             if (work) {
                 unsigned long long c = 0;
@@ -364,7 +364,7 @@ __global__ void __launch_bounds__(kGreedyThreads, 2) k_greedy(GreedyArgs a) {
             }
             if (!work) base += nwarps * kGreedyChunk;
         }
-        if (!grid_sync(a.bar, nb, a.status)) return;
+        if (!grid_sync(a.bar, nb, a.status)) return false;
         const int64_t np = a.piece ? (int64_t)__ldcg(a.npiece) : 0;
         if (np > 0) {                                // (grid-uniform)
             for (int64_t p = gwarp; p < np; p += nwarps) {
@@ -382,17 +382,49 @@ __global__ void __launch_bounds__(kGreedyThreads, 2) k_greedy(GreedyArgs a) {
                         if (mv[uu] >= 0) decrement(mv[uu], rep);
                 }
             }
-            if (!grid_sync(a.bar, nb, a.status)) return;
+            if (!grid_sync(a.bar, nb, a.status)) return false;
             // (the next pieces are put aside after the next barrier)
-            if (blockIdx.x == 0 && threadIdx.x == 0) *a.npiece = 0ull;
+            if (rank == 0 && threadIdx.x == 0) *a.npiece = 0ull;
         }
         ++j;
     }
-    if (blockIdx.x == 0 && threadIdx.x == 0) {
+    if (rank == 0 && threadIdx.x == 0) {
         *a.nseeds = j;
         *a.coverage = cov;
     }
+    return true;
 }
+
+__global__ void __launch_bounds__(kGreedyThreads, 2) k_greedy(GreedyArgs a) {
+    __shared__ unsigned long long shm[33];
+    greedy_steps(a, blockIdx.x, gridDim.x, shm);
+}
+
+// Many queries at once: group g of the launch, blocks [first[g], first[g + 1]),
+// runs queries g, g + groups, ... of the table, each with its own barrier.  A
+// query of a batch is a chain of short steps that a few SMs feed, and its
+// barriers cost less among a few blocks; one launch after the other over the
+// whole grid took 19 us a step whatever the query's size.
+__global__ void __launch_bounds__(kGreedyThreads, 2) k_greedy_many(const GreedyArgs *tab, int32_t nq,
+                                                                   const int32_t *first,
+                                                                   int32_t groups) {
+    __shared__ unsigned long long shm[33];
+    __shared__ GreedyArgs s_a;
+    __shared__ int32_t s_g;
+    for (int g = threadIdx.x; g < groups; g += blockDim.x)
+        if (first[g] <= (int32_t)blockIdx.x && (int32_t)blockIdx.x < first[g + 1]) s_g = g;
+    __syncthreads();
+    const int32_t g = s_g;
+    const uint32_t rank = blockIdx.x - first[g], nb = first[g + 1] - first[g];
+    for (int32_t q = g; q < nq; q += groups) {
+        __syncthreads();
+        for (int i = threadIdx.x; i < (int)(sizeof(GreedyArgs) / 4); i += blockDim.x)
+            reinterpret_cast<uint32_t *>(&s_a)[i] = reinterpret_cast<const uint32_t *>(tab + q)[i];
+        __syncthreads();
+        if (!greedy_steps(s_a, rank, nb, shm)) return;
+    }
+}
+static_assert(sizeof(GreedyArgs) % 4 == 0, "copied by words");
 
 // ---------------------------------------------------------------------------
 // RandGreedi
@@ -1439,6 +1471,8 @@ __global__ void __launch_bounds__(kFinalThreads) k_rg_final(RGArgs a, int32_t *s
 
 }  // namespace
 
+static size_t align256(size_t x) { return (x + 255) & ~(size_t)255; }
+
 int32_t num_buckets(int32_t k, double delta) {
     double x = 1.0;
     int32_t b = 0;
@@ -1519,26 +1553,12 @@ im_status greedy_plain(im_pool *p, int32_t k, int32_t *d_seeds, int64_t *d_gains
 }
 
 // Launches the standard greedy kernel on caller-provided scratch (used by the
-// allocation-free entry point in noalloc.cu; greedy_plain above is unchanged).
+// allocation-free entry point in noalloc.cu).
 im_status greedy_launch(int64_t n, int64_t theta, const int64_t *set_off, const int32_t *members,
                         const int64_t *vtx_off, const int32_t *set_ids, int32_t k, int32_t *counts,
                         uint32_t *covered, unsigned long long *block_best, int max_grid,
                         void *barrier, int32_t *seeds, int64_t *gains, int32_t *nseeds,
                         int64_t *coverage, int *status, cudaStream_t st) {
-    return greedy_launch_view(n, theta, set_off, members, vtx_off, set_ids, 0, 0, k, counts,
-                              covered, block_best, max_grid, barrier, seeds, gains, nseeds,
-                              coverage, status, st);
-}
-
-// The same over one query of a batch: vtx_off points at the query's first
-// vertex, set_ids / members hold batch-wide set and vertex ids, offset by
-// sshift and vshift from the query's own.
-im_status greedy_launch_view(int64_t n, int64_t theta, const int64_t *set_off,
-                             const int32_t *members, const int64_t *vtx_off,
-                             const int32_t *set_ids, int64_t sshift, int64_t vshift, int32_t k,
-                             int32_t *counts, uint32_t *covered, unsigned long long *block_best,
-                             int max_grid, void *barrier, int32_t *seeds, int64_t *gains,
-                             int32_t *nseeds, int64_t *coverage, int *status, cudaStream_t st) {
     int per_sm = 0;
     IM_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_greedy, kGreedyThreads, 0));
     if (per_sm < 1) return IM_ERR_UNSUPPORTED;
@@ -1561,8 +1581,6 @@ im_status greedy_launch_view(int64_t n, int64_t theta, const int64_t *set_off,
     a.nseeds = nseeds;
     a.coverage = coverage;
     a.status = status;
-    a.sshift = sshift;
-    a.vshift = vshift;
     void *args[] = {&a};
     KernelTimer kt(st, "greedy");
     IM_CUDA(cudaLaunchCooperativeKernel((const void *)k_greedy, dim3(grid), dim3(kGreedyThreads),
@@ -1570,7 +1588,122 @@ im_status greedy_launch_view(int64_t n, int64_t theta, const int64_t *set_off,
     return IM_OK;
 }
 
-static size_t align256(size_t x) { return (x + 255) & ~(size_t)255; }
+// Queries of a batch: scratch of greedy_many for nq queries of `members` members
+// in all (its own arrays; counts, ranks and candidates come with the queries).
+constexpr int32_t kManyHubs = 1024;     // hub rows of a query at most
+
+namespace {
+struct ManyState {                      // zeroed before the launch
+    GridBarrier bar;
+    unsigned long long work[2], npiece;
+    int32_t ctl[4];
+};
+size_t many_pieces(int64_t members) { return (size_t)(2 * members / kGreedyPiece + 1); }
+}  // namespace
+
+size_t greedy_many_scratch(int32_t nq, int64_t members) {
+    return align256((size_t)nq * sizeof(GreedyArgs)) + align256((size_t)(nq + 1) * 4) +
+           align256((size_t)nq * sizeof(ManyState)) + align256((size_t)num_sms() * 2 * 8) +
+           align256((size_t)nq * kManyHubs * kHubRep * 4) + align256((size_t)nq * kManyHubs * 4) +
+           align256((many_pieces(members) + (size_t)nq) * 8);
+}
+
+im_status greedy_many(const std::vector<GreedyQuery> &qs, const int64_t *set_off,
+                      const int32_t *members, const int32_t *set_ids, void *scratch, int *status,
+                      cudaStream_t st) {
+    const int32_t nq = (int32_t)qs.size();
+    if (nq == 0) return IM_OK;
+    int per_sm = 0;
+    IM_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_greedy_many, kGreedyThreads, 0));
+    if (per_sm < 1) return IM_ERR_UNSUPPORTED;
+    const int grid = std::min(per_sm, 2) * num_sms();
+    int64_t total = 0;
+    for (const GreedyQuery &q : qs) total += q.members;
+    char *B = (char *)scratch;
+    auto take = [&](size_t bytes) {
+        char *r = B;
+        B += align256(bytes);
+        return r;
+    };
+    GreedyArgs *tab = (GreedyArgs *)take((size_t)nq * sizeof(GreedyArgs));
+    int32_t *first = (int32_t *)take((size_t)(nq + 1) * 4);
+    ManyState *state = (ManyState *)take((size_t)nq * sizeof(ManyState));
+    unsigned long long *best = (unsigned long long *)take((size_t)num_sms() * 2 * 8);
+    int32_t *hub_cnt = (int32_t *)take((size_t)nq * kManyHubs * kHubRep * 4);
+    int32_t *hub_list = (int32_t *)take((size_t)nq * kManyHubs * 4);
+    unsigned long long *piece = (unsigned long long *)take((many_pieces(total) + (size_t)nq) * 8);
+
+    // largest first; blocks by weight: the members a query may decrement, and a
+    // floor for its steps
+    std::vector<int32_t> order(nq);
+    for (int32_t i = 0; i < nq; ++i) order[i] = i;
+    auto weight = [&](int32_t i) { return (double)qs[i].members + 2e4 * (double)qs[i].k; };
+    std::stable_sort(order.begin(), order.end(),
+                     [&](int32_t x, int32_t y) { return weight(x) > weight(y); });
+    const int32_t groups = std::min<int32_t>(nq, grid);
+    double sum = 0.0;
+    for (int32_t g = 0; g < groups; ++g) sum += weight(order[g]);
+    std::vector<int32_t> hfirst(groups + 1, 0), blocks(groups, 1);
+    int32_t left = grid - groups;
+    for (int32_t g = 0; g < groups; ++g) {
+        const int32_t more = std::min<int32_t>(
+            left, std::max<int32_t>(0, (int32_t)((double)grid * weight(order[g]) / sum) - 1));
+        blocks[g] += more;
+        left -= more;
+    }
+    for (int32_t g = 0; left > 0; g = (g + 1) % groups, --left) ++blocks[g];
+    for (int32_t g = 0; g < groups; ++g) hfirst[g + 1] = hfirst[g] + blocks[g];
+
+    const int32_t cand_shift = (int32_t)tune_value(IM_TUNE_GREEDY_HOT);
+    std::vector<GreedyArgs> h(nq);
+    size_t at = 0;
+    for (int32_t r = 0; r < nq; ++r) {
+        const GreedyQuery &q = qs[order[r]];
+        GreedyArgs &a = h[r];
+        std::memset(&a, 0, sizeof(a));
+        a.n = q.n;
+        a.theta = q.theta;
+        a.set_off = set_off;
+        a.members = members;
+        a.vtx_off = q.vtx_off;
+        a.set_ids = set_ids;
+        a.k = q.k;
+        a.counts = q.counts;
+        a.covered = q.covered;
+        a.block_best = best + hfirst[r % groups];
+        a.bar = &state[r].bar;
+        a.seeds = q.seeds;
+        a.gains = q.gains;
+        a.nseeds = q.nseeds;
+        a.coverage = q.coverage;
+        a.status = status;
+        a.sshift = q.sshift;
+        a.vshift = q.vshift;
+        a.hub_rank = q.ranks;
+        a.hub_cnt = hub_cnt + (size_t)r * kManyHubs * kHubRep;
+        a.hub_list = hub_list + (size_t)r * kManyHubs;
+        a.cand = q.cands;
+        a.ctl = state[r].ctl;
+        a.hub_cap = kManyHubs;
+        a.hub_shift = kHubShift;
+        a.cand_shift = cand_shift;
+        a.work = state[r].work;
+        a.piece = piece + at;
+        a.npiece = &state[r].npiece;
+        at += many_pieces(q.members);
+    }
+    IM_CUDA(cudaMemcpyAsync(tab, h.data(), (size_t)nq * sizeof(GreedyArgs), cudaMemcpyHostToDevice, st));
+    IM_CUDA(cudaMemcpyAsync(first, hfirst.data(), (size_t)(groups + 1) * 4, cudaMemcpyHostToDevice, st));
+    IM_CUDA(cudaMemsetAsync(state, 0, (size_t)nq * sizeof(ManyState), st));
+    const GreedyArgs *ctab = tab;
+    const int32_t *cfirst = first;
+    int32_t cnq = nq, cgroups = groups;
+    void *args[] = {&ctab, &cnq, &cfirst, &cgroups};
+    KernelTimer kt(st, "greedy_many");
+    IM_CUDA(cudaLaunchCooperativeKernel((const void *)k_greedy_many, dim3(grid),
+                                        dim3(kGreedyThreads), args, 0, st));
+    return IM_OK;
+}
 
 im_status randgreedi(im_pool *p, int32_t k, const im_cover_opts *o, int32_t *d_seeds,
                      int64_t *d_gains, int32_t *d_nseeds, int64_t *d_cov, cudaStream_t st,

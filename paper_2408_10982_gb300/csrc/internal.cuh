@@ -442,12 +442,25 @@ im_status greedy_launch(int64_t n, int64_t theta, const int64_t *set_off, const 
                         uint32_t *covered, unsigned long long *block_best, int max_grid,
                         void *barrier, int32_t *seeds, int64_t *gains, int32_t *nseeds,
                         int64_t *coverage, int *status, cudaStream_t st);
-im_status greedy_launch_view(int64_t n, int64_t theta, const int64_t *set_off,
-                             const int32_t *members, const int64_t *vtx_off,
-                             const int32_t *set_ids, int64_t sshift, int64_t vshift, int32_t k,
-                             int32_t *counts, uint32_t *covered, unsigned long long *block_best,
-                             int max_grid, void *barrier, int32_t *seeds, int64_t *gains,
-                             int32_t *nseeds, int64_t *coverage, int *status, cudaStream_t st);
+// The standard greedy of many queries of a batch in one launch (cover.cu).  Set
+// ids in set_ids and vertex ids in members are offset by sshift and vshift (the
+// query's first set and first vertex).
+struct GreedyQuery {
+    int64_t n, theta, members;
+    const int64_t *vtx_off;             // at the query's first vertex
+    int64_t sshift, vshift;
+    int32_t k;
+    int32_t *counts, *ranks, *cands;    // [n] scratch each
+    uint32_t *covered;                  // [ceil(theta / 32)]
+    int32_t *seeds;
+    int64_t *gains;
+    int32_t *nseeds;
+    int64_t *coverage;
+};
+size_t greedy_many_scratch(int32_t nq, int64_t members);
+im_status greedy_many(const std::vector<GreedyQuery> &qs, const int64_t *set_off,
+                      const int32_t *members, const int32_t *set_ids, void *scratch, int *status,
+                      cudaStream_t st);
 // The standard greedy's result on a pool: the lazy kernel (lazy = true, or
 // IM_TUNE_GREEDY_EVALS > 0) or the counts-decrement kernel (cover.cu).
 im_status greedy_select(im_pool *p, int32_t k, bool lazy, int32_t *d_seeds, int64_t *d_gains,
