@@ -138,22 +138,33 @@ constexpr int64_t kICHandCap = 1 << 23;      // members handed over to the secon
 // One sample's draws of one kind (TAG: coins of edge group g, or the LT pick of
 // vertex g): Philox4x32-10 of counter (s, g, 0, TAG), with what does not depend
 // on g computed by begin().  KEYS: the round keys come from rk (kernel
-// parameters, so constant-bank operands); else they are derived from k0, k1 as
-// the rounds go.
-template <uint32_t TAG, bool KEYS>
+// parameters, so constant-bank operands); else they are kept in registers (HELD)
+// or derived from k0, k1 as the rounds go.
+template <uint32_t TAG, bool KEYS, bool HELD = false>
 struct DrawStream {
     uint32_t k0, k1;
     uint32_t gx, c1, ca, cb, cc;
+    uint32_t held[HELD ? 13 : 1];            // K0(3 .. 9), K1(4 .. 9)
     __device__ __forceinline__ uint32_t K0(const uint32_t *rk, int r) const {
-        return KEYS ? rk[2 * r] : k0 + (uint32_t)r * 0x9E3779B9u;
+        return KEYS ? rk[2 * r] : HELD && r >= 3 ? held[r - 3] : k0 + (uint32_t)r * 0x9E3779B9u;
     }
     __device__ __forceinline__ uint32_t K1(const uint32_t *rk, int r) const {
-        return KEYS ? rk[2 * r + 1] : k1 + (uint32_t)r * 0xBB67AE85u;
+        return KEYS ? rk[2 * r + 1] : HELD && r >= 4 ? held[r + 3] : k1 + (uint32_t)r * 0xBB67AE85u;
     }
     __device__ __forceinline__ void begin(const uint32_t *rk, uint32_t s, uint32_t key0,
                                           uint32_t key1) {
         k0 = key0;
         k1 = key1;
+        if (HELD) {
+#pragma unroll
+            for (int r = 3; r < 10; ++r) {
+                held[r - 3] = k0 + (uint32_t)r * 0x9E3779B9u;
+                if (r >= 4) held[r + 3] = k1 + (uint32_t)r * 0xBB67AE85u;
+            }
+            // (kept as values: not to be derived again in the coin loop)
+#pragma unroll
+            for (int i = 0; i < 13; ++i) asm volatile("" : "+r"(held[i]));
+        }
         gx = K0(rk, 0);                                           // round 0: x = g ^ gx
         const uint32_t z1 = __umulhi(0xD2511F53u, s) ^ TAG ^ K1(rk, 0);
         c1 = (0xD2511F53u * s) ^ K1(rk, 1);                       // round 1: z = hi(a) ^ c1
@@ -184,8 +195,8 @@ struct DrawStream {
     }
 };
 
-template <bool KEYS>
-using CoinStream = DrawStream<kStreamCoin, KEYS>;
+template <bool KEYS, bool HELD = false>
+using CoinStream = DrawStream<kStreamCoin, KEYS, HELD>;
 template <bool KEYS>
 using PickStream = DrawStream<kStreamPick, KEYS>;
 
@@ -246,8 +257,8 @@ __device__ __forceinline__ void ic_list(uint32_t m, uint32_t e0, uint32_t *cand,
 // of the warp's 64 groups decides whether any edge is live; the bits, and what
 // lies outside the list in its first and last group, are looked at only then.
 // Unequal weights: the next groups' are loaded while these are tested.
-template <bool KEYS, typename F>
-__device__ __forceinline__ void ic_expand_wide(const CoinStream<KEYS> &cs, const uint32_t *rk,
+template <typename CS, typename F>
+__device__ __forceinline__ void ic_expand_wide(const CS &cs, const uint32_t *rk,
                                                const uint32_t *wgt, const ICItem &o, uint32_t t0,
                                                uint32_t n, int lane, F &&visit) {
     const uint32_t g0 = o.eb >> 2;
@@ -290,8 +301,8 @@ __device__ __forceinline__ void ic_expand_wide(const CoinStream<KEYS> &cs, const
 
 // The same for the lists of a warp's lanes (ng groups in this lane's): those of
 // at least kICWide groups one after another on all lanes, the others packed.
-template <bool KEYS, typename F>
-__device__ __forceinline__ void ic_expand(const CoinStream<KEYS> &cs, const uint32_t *rk,
+template <typename CS, typename F>
+__device__ __forceinline__ void ic_expand(const CS &cs, const uint32_t *rk,
                                           const uint32_t *wgt, const ICItem &it, uint32_t ng,
                                           int lane, F &&visit) {
     unsigned wide = __ballot_sync(kFull, ng >= (uint32_t)kICWide);
@@ -300,7 +311,7 @@ __device__ __forceinline__ void ic_expand(const CoinStream<KEYS> &cs, const uint
         wide &= wide - 1u;
         const ICItem o{__shfl_sync(kFull, it.eb, l), __shfl_sync(kFull, it.ee, l),
                        __shfl_sync(kFull, it.w, l), __shfl_sync(kFull, it.equal, l)};
-        ic_expand_wide<KEYS>(cs, rk, wgt, o, 0u, __shfl_sync(kFull, ng, l), lane, visit);
+        ic_expand_wide(cs, rk, wgt, o, 0u, __shfl_sync(kFull, ng, l), lane, visit);
     }
     const uint32_t ns = ng >= (uint32_t)kICWide ? 0u : ng;
     const uint32_t incl = warp_incl_scan<uint32_t>(ns, lane);
@@ -339,11 +350,12 @@ static_assert(kICHash == 1 << 10, "ic_hash gives a slot of kICHash");
 // -- which moves to the warp's bitmap in global memory (cleared by the warp on
 // its first use, and kept clear) when the set passes kICHashMax members.
 // Shared memory of a warp: visited words, kICQueueSmem queue entries (later
-// entries in global memory), kCandCap listed edges.  Three blocks an SM with
-// the round keys in the arguments (80 registers; four blocks at 64 measured 4 %
-// slower), four without (three: 3 % slower on the batched mix).
+// entries in global memory), kCandCap listed edges.  Three blocks an SM, 80
+// registers: four blocks at 64 measured 4 % slower, and without KEYS the round
+// keys fit as well (held; deriving them in the loop: batched mix 66.9 against
+// 62.5 ms).
 template <bool BITS, bool KEYS>
-__global__ void __launch_bounds__(kSampleThreads, KEYS ? 3 : 4) k_sample_ic(const __grid_constant__ SampleArgs a) {
+__global__ void __launch_bounds__(kSampleThreads, 3) k_sample_ic(const __grid_constant__ SampleArgs a) {
     extern __shared__ uint32_t ic_smem[];
     const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
     const unsigned lt = (1u << lane) - 1u;
@@ -375,7 +387,7 @@ __global__ void __launch_bounds__(kSampleThreads, KEYS ? 3 : 4) k_sample_ic(cons
         const uint64_t seed = V.seed;
         const uint32_t s = V.first + (uint32_t)(j - __ldg(a.qstart + qi));
         const uint32_t root = rrr_root(seed, s, V.n);
-        CoinStream<KEYS> cs;
+        CoinStream<KEYS, !KEYS> cs;
         cs.begin(a.rk, s, seed_lo(seed), seed_hi(seed));
         int32_t head = 0, tail = 1;
         int ncand = 0;
@@ -470,7 +482,7 @@ __global__ void __launch_bounds__(kSampleThreads, KEYS ? 3 : 4) k_sample_ic(cons
                        kICWideEdges);
             sexam += (unsigned long long)deg;
             head += nb;
-            ic_expand<KEYS>(cs, a.rk, wgt, it, ic_groups(it), lane, [&](uint32_t m, uint32_t e0) {
+            ic_expand(cs, a.rk, wgt, it, ic_groups(it), lane, [&](uint32_t m, uint32_t e0) {
                 if (lost) return;
                 ic_list(m, e0, cand, ncand, lane);
                 while (ncand >= 32) flush();
@@ -663,7 +675,7 @@ __global__ void __launch_bounds__(kICBigThreads) k_sample_ic_big(const __grid_co
                     }
                 }
                 __syncwarp();
-                ic_expand<KEYS>(cs, a.rk, wgt, it, ng, lane, visit);
+                ic_expand(cs, a.rk, wgt, it, ng, lane, visit);
             }
             __syncthreads();
             const int nhub = (int)(s_nhub < (unsigned)kICHubCap ? s_nhub : (unsigned)kICHubCap);
@@ -673,7 +685,7 @@ __global__ void __launch_bounds__(kICBigThreads) k_sample_ic_big(const __grid_co
                 const uint32_t per =
                     ((n + kICBigThreads / 32 - 1) / (kICBigThreads / 32) + 31u) & ~31u;
                 const uint32_t t = min(n, warp * per);
-                ic_expand_wide<KEYS>(cs, a.rk, wgt, it, t, min(n, t + per), lane, visit);
+                ic_expand_wide(cs, a.rk, wgt, it, t, min(n, t + per), lane, visit);
             }
             while (ncand > 0) flush();
             __syncthreads();
