@@ -52,6 +52,13 @@ constexpr int kMaskWindow = 512;             // ... slots read ahead (mask stage
 constexpr int kMaskStrips = 16;              // entries per lane in one warp work item
 constexpr int kMaskItem = 32 * kMaskStrips;  // entries per warp work item
 
+// The largest of a warp's values, by 32-bit reductions.
+__device__ __forceinline__ unsigned long long warp_max_key(unsigned long long v) {
+    const uint32_t hi = __reduce_max_sync(kFull, (uint32_t)(v >> 32));
+    const uint32_t lo = __reduce_max_sync(kFull, (uint32_t)(v >> 32) == hi ? (uint32_t)v : 0u);
+    return (unsigned long long)hi << 32 | lo;
+}
+
 __device__ __forceinline__ unsigned long long block_max_u64(unsigned long long v,
                                                             unsigned long long *sh) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -113,7 +120,7 @@ struct GreedyArgs {
     int32_t k;
     int32_t *counts;                    // [n], or [32 ceil(n/32)] with spread
     uint32_t *covered;                  // [ceil(theta/32)]
-    unsigned long long *block_best;     // [grid]
+    unsigned long long *gmax;           // [3] best key of a round
     GridBarrier *bar;
     int32_t *seeds;
     int64_t *gains;
@@ -142,10 +149,15 @@ struct GreedyArgs {
 };
 
 constexpr int kHubRep = 32;             // partial counts of a hub (one per set id mod 32)
-// Entries of S(v*) a warp claims at a time: a chunk's newly covered sets can
-// hold hundreds of members each, so small chunks spread the decrements over
-// more warps (the step waits for the slowest one).
+// Entries of S(v*) a warp takes at a time: its share of the list, at least one
+// (a newly covered set can hold hundreds of members, and the step waits for the
+// slowest warp) and at most kGreedyChunk, beyond which lists are claimed from a
+// counter.  Always claiming 16: 4,096 sets of 200 members (scale 10) .266 against
+// .190 ms, IMM's greedy calls 19.3 against 14.7, 4.2 M LT walks 3.62 against
+// 3.50; claiming half or an eighth of a share at a time: the claims, atomics on
+// one word, cost .7 and 2.7 ms on the LT walks.
 constexpr int kGreedyChunk = 16;
+constexpr int64_t kGreedyTake = 1 << 26;  // members of a set walked at a time
 // A newly covered set longer than this is put aside in pieces of this many
 // members, which the whole grid shares after the claims of the step: the
 // percolating sets of equal-probability IC hold 10^4 to 10^6 members each, and
@@ -172,11 +184,28 @@ constexpr int kHubShift = 6;            // hubs: |S(v)| >= max |S(v)| / 64
 // keeping |S(v)| as a stale bound -- which skips most decrements (low-degree
 // vertices are most members).  Once the best gain falls below tau, one pass
 // makes the frozen gains exact and every step reads all.
-// Warps take kGreedyChunk-entry chunks of S(v*) from a per-step counter.  Every wait is
-// bounded (grid_sync).
+// A warp's first chunk of S(v*) goes by its number, consecutive chunks to
+// different SMs, the others by a per-step counter.  The argmax meets in one word
+// (an atomic per block, no second pass over block results).  Every wait is
+// bounded (grid_sync).  A step is two barriers and the dependent loads between
+// them and the decrements.
+struct GreedyShared {
+    unsigned long long best[2][32];
+};
+
 // Run by block `rank` of `nb`; false: a wait ran out.
 __device__ __forceinline__ bool greedy_steps(const GreedyArgs &a, uint32_t rank, uint32_t nb,
-                                             unsigned long long *shm) {
+                                             GreedyShared &sh) {
+    int par = 0;                             // the buffer of the next block maximum
+    auto block_max = [&](unsigned long long v) {
+        const int l = threadIdx.x & 31;
+        v = warp_max_key(v);
+        if (l == 0) sh.best[par][threadIdx.x >> 5] = v;
+        __syncthreads();
+        const unsigned long long r = warp_max_key(l < (int)(blockDim.x >> 5) ? sh.best[par][l] : 0ull);
+        par ^= 1;                            // (its readers pass a barrier before it is written again)
+        return r;
+    };
     const int64_t tid = (int64_t)rank * blockDim.x + threadIdx.x;
     const int64_t stride = (int64_t)nb * blockDim.x;
     const int lane = threadIdx.x & 31;
@@ -194,8 +223,9 @@ __device__ __forceinline__ bool greedy_steps(const GreedyArgs &a, uint32_t rank,
         lmax = (unsigned long long)d > lmax ? (unsigned long long)d : lmax;
     }
     for (int64_t x = tid; x < words; x += stride) a.covered[x] = 0u;
+    if (tid == 0) a.gmax[0] = a.gmax[1] = a.gmax[2] = 0ull;
     if (a.hub_rank) {
-        lmax = block_max_u64(lmax, shm);
+        lmax = block_max(lmax);
         if (threadIdx.x == 0 && lmax) atomicMax(a.ctl + 2, (int32_t)lmax);
     }
     if (!grid_sync(a.bar, nb, a.status)) return false;
@@ -238,7 +268,8 @@ __device__ __forceinline__ bool greedy_steps(const GreedyArgs &a, uint32_t rank,
     };
     int64_t cov = 0;
     int32_t j = 0;
-    while (j < a.k) {
+    const int64_t claim = (int64_t)(threadIdx.x >> 5) * nb + rank;   // neighbours on different SMs
+    for (int round = 0; j < a.k; ++round) {
         unsigned long long best = 0;
         auto consider = [&](int32_t c, uint32_t v) {
             if (c > 0) {
@@ -260,20 +291,18 @@ __device__ __forceinline__ bool greedy_steps(const GreedyArgs &a, uint32_t rank,
             const int32_t c = warp_sum<int32_t>(__ldcg(a.hub_cnt + h * kHubRep + lane));
             consider(c, (uint32_t)__ldcg(a.hub_list + h));
         }
-        best = block_max_u64(best, shm);
-        if (threadIdx.x == 0) a.block_best[rank] = best;
+        // the grid's maximum by one atomic a block on the round's word; of the
+        // three words, the one of the round before is cleared for the round after
+        // the next (every block has read it: it passed this round's barrier)
+        best = block_max(best);
+        if (threadIdx.x == 0 && best) atomicMax(a.gmax + round % 3, best);
         if (!grid_sync(a.bar, nb, a.status)) return false;
-        unsigned long long gbest = 0;
-        for (uint32_t b = threadIdx.x; b < nb; b += blockDim.x) {
-            const unsigned long long x = __ldcg(a.block_best + b);
-            gbest = x > gbest ? x : gbest;
-        }
-        gbest = block_max_u64(gbest, shm);
+        const unsigned long long gbest = __ldcg(a.gmax + round % 3);
+        if (tid == 0) a.gmax[(round + 2) % 3] = 0ull;
         if (tau > 0 && (uint32_t)(gbest >> 32) < tau) {
             // the best gain fell below tau: the frozen vertices may now win.
             // Make their gains exact against the sets covered so far, thaw
-            // them, and read every gain from here on (block_best is rewritten
-            // only after the barrier below, when every block has read it)
+            // them, and read every gain from here on
             for (int64_t v = gwarp; v < a.n; v += nwarps) {
                 if (__ldcg(a.hub_rank + v) != -2) continue;
                 const int64_t sb = a.vtx_off[v], se = a.vtx_off[v + 1];
@@ -301,21 +330,19 @@ __device__ __forceinline__ bool greedy_steps(const GreedyArgs &a, uint32_t rank,
         }
         cov += gain;
         const int64_t sb = a.vtx_off[vs], se = a.vtx_off[vs + 1];
-        // chunks of S(v*) from this step's counter; the other step's counter
-        // is cleared meanwhile (its last use ended at the previous step's
-        // closing barrier)
-        unsigned long long *work = a.work ? a.work + (j & 1) : nullptr;
-        if (work && rank == 0 && threadIdx.x == 0) a.work[(j + 1) & 1] = 0ull;
-        for (int64_t base = sb + gwarp * kGreedyChunk;;) {
-            if (work) {
-                unsigned long long c = 0;
-                if (lane == 0) c = atomicAdd(work, (unsigned long long)kGreedyChunk);
-                base = sb + (int64_t)__shfl_sync(kFull, c, 0);
-            }
+        // chunks of S(v*): the first by the warp's number, the others from this
+        // step's counter (every warp's first one is taken when it starts); the other
+        // step's counter is cleared meanwhile (its last use ended at the previous
+        // step's closing barrier)
+        const int64_t share = (se - sb + nwarps - 1) / nwarps;
+        const int chunk = (int)(share < 1 ? 1 : share < kGreedyChunk ? share : kGreedyChunk);
+        unsigned long long *work = a.work && se - sb > nwarps * chunk ? a.work + (j & 1) : nullptr;
+        if (a.work && tid == 0) a.work[(j + 1) & 1] = 0ull;
+        for (int64_t base = sb + claim * chunk;;) {
             if (base >= se) break;
             const int64_t t = base + lane;
             int32_t i = -1;
-            if (lane < kGreedyChunk && t < se) i = a.set_ids[t];
+            if (lane < chunk && t < se) i = a.set_ids[t];
             const bool fresh = warp_bitmap_set(a.covered, i >= 0 ? i - a.sshift : -1, lane);
             if (__any_sync(kFull, fresh)) {
                 // decrement the gains of every member of the lane's newly
@@ -337,32 +364,42 @@ __device__ __forceinline__ bool greedy_steps(const GreedyArgs &a, uint32_t rank,
                     }
                     ml = 0;
                 }
-                const int64_t incl = warp_incl_scan<int64_t>(ml, lane);
-                const int64_t tot = __shfl_sync(kFull, incl, 31);
-                constexpr int U = 4;
-                for (int64_t p0 = 0; p0 < tot; p0 += 32 * U) {
-                    int32_t mv[U], ms[U];
+                // (kGreedyTake members of each at a time, so that positions stay
+                // below 2^31 where sets of any length are not cut into pieces)
+                do {
+                    const int32_t mt = (int32_t)(ml < kGreedyTake ? ml : kGreedyTake);
+                    const int32_t incl = warp_incl_scan<int32_t>(mt, lane);
+                    const int32_t tot = __shfl_sync(kFull, incl, 31);
+                    const int64_t from = mo + mt - incl;   // the lane's member for position 0
+                    constexpr int U = 4;
+                    for (int32_t p0 = 0; p0 < tot; p0 += 32 * U) {
+                        int32_t mv[U], ms[U];
 #pragma unroll
-                    for (int uu = 0; uu < U; ++uu) {
-                        const int64_t q = p0 + uu * 32 + lane;
-                        int owner = 0;           // first lane whose inclusive count exceeds q
+                        for (int uu = 0; uu < U; ++uu) {
+                            const int32_t q = p0 + uu * 32 + lane;
+                            int owner = 0;           // first lane whose inclusive count exceeds q
 #pragma unroll
-                        for (int step = 16; step > 0; step >>= 1) {
-                            const int64_t c = __shfl_sync(kFull, incl, owner + step - 1);
-                            if (c <= q) owner += step;
+                            for (int step = 16; step > 0; step >>= 1)
+                                if (__shfl_sync(kFull, incl, owner + step - 1) <= q) owner += step;
+                            const int64_t o_from = __shfl_sync(kFull, from, owner);
+                            ms[uu] = __shfl_sync(kFull, i, owner);
+                            mv[uu] = q < tot ? __ldg(a.members + o_from + q) : -1;
                         }
-                        const int64_t o_incl = __shfl_sync(kFull, incl, owner);
-                        const int64_t o_ml = __shfl_sync(kFull, ml, owner);
-                        const int64_t o_mo = __shfl_sync(kFull, mo, owner);
-                        ms[uu] = __shfl_sync(kFull, i, owner);
-                        mv[uu] = q < tot ? __ldg(a.members + o_mo + (q - (o_incl - o_ml))) : -1;
-                    }
 #pragma unroll
-                    for (int uu = 0; uu < U; ++uu)
-                        if (mv[uu] >= 0) decrement(mv[uu], ms[uu] & (kHubRep - 1));
-                }
+                        for (int uu = 0; uu < U; ++uu)
+                            if (mv[uu] >= 0) decrement(mv[uu], ms[uu] & (kHubRep - 1));
+                    }
+                    mo += mt;
+                    ml -= mt;
+                } while (__any_sync(kFull, ml > 0));
             }
-            if (!work) base += nwarps * kGreedyChunk;
+            if (work) {
+                unsigned long long c = 0;
+                if (lane == 0) c = atomicAdd(work, (unsigned long long)chunk);
+                base = sb + nwarps * chunk + (int64_t)__shfl_sync(kFull, c, 0);
+            } else {
+                base += nwarps * chunk;
+            }
         }
         if (!grid_sync(a.bar, nb, a.status)) return false;
         const int64_t np = a.piece ? (int64_t)__ldcg(a.npiece) : 0;
@@ -396,8 +433,8 @@ __device__ __forceinline__ bool greedy_steps(const GreedyArgs &a, uint32_t rank,
 }
 
 __global__ void __launch_bounds__(kGreedyThreads, 2) k_greedy(GreedyArgs a) {
-    __shared__ unsigned long long shm[33];
-    greedy_steps(a, blockIdx.x, gridDim.x, shm);
+    __shared__ GreedyShared sh;
+    greedy_steps(a, blockIdx.x, gridDim.x, sh);
 }
 
 // Many queries at once: group g of the launch, blocks [first[g], first[g + 1]),
@@ -408,7 +445,7 @@ __global__ void __launch_bounds__(kGreedyThreads, 2) k_greedy(GreedyArgs a) {
 __global__ void __launch_bounds__(kGreedyThreads, 2) k_greedy_many(const GreedyArgs *tab, int32_t nq,
                                                                    const int32_t *first,
                                                                    int32_t groups) {
-    __shared__ unsigned long long shm[33];
+    __shared__ GreedyShared sh;
     __shared__ GreedyArgs s_a;
     __shared__ int32_t s_g;
     for (int g = threadIdx.x; g < groups; g += blockDim.x)
@@ -421,7 +458,7 @@ __global__ void __launch_bounds__(kGreedyThreads, 2) k_greedy_many(const GreedyA
         for (int i = threadIdx.x; i < (int)(sizeof(GreedyArgs) / 4); i += blockDim.x)
             reinterpret_cast<uint32_t *>(&s_a)[i] = reinterpret_cast<const uint32_t *>(tab + q)[i];
         __syncthreads();
-        if (!greedy_steps(s_a, rank, nb, shm)) return;
+        if (!greedy_steps(s_a, rank, nb, sh)) return;
     }
 }
 static_assert(sizeof(GreedyArgs) % 4 == 0, "copied by words");
@@ -494,13 +531,6 @@ constexpr int kProdW = 8;
 
 __device__ __forceinline__ unsigned long long prod_key(int32_t g, int32_t l) {
     return g > 0 ? ((unsigned long long)(uint32_t)g << 32) | (0xffffffffu - (uint32_t)l) : 0ull;
-}
-
-// The largest packed key of a warp's lanes (distinct unless 0).
-__device__ __forceinline__ unsigned long long warp_max_key(unsigned long long v) {
-    const uint32_t hi = __reduce_max_sync(kFull, (uint32_t)(v >> 32));
-    const uint32_t lo = __reduce_max_sync(kFull, (uint32_t)(v >> 32) == hi ? (uint32_t)v : 0u);
-    return (unsigned long long)hi << 32 | lo;
 }
 
 // cmax of chunk c, by one warp
@@ -1501,7 +1531,7 @@ im_status greedy_plain(im_pool *p, int32_t k, int32_t *d_seeds, int64_t *d_gains
     const int64_t vwords = (n + 31) / 32;
     const size_t o_cnt = take((size_t)vwords * 32 * 4),
                  o_cov = take((size_t)std::max<int64_t>(words, 1) * 4),
-                 o_best = take((size_t)grid * 8), o_bar = take(sizeof(GridBarrier)),
+                 o_best = take(3 * 8), o_bar = take(sizeof(GridBarrier)),
                  o_work = take(16), o_hrank = take((size_t)n * 4),
                  o_hcnt = take((size_t)kHubCap * kHubRep * 4), o_hlist = take((size_t)kHubCap * 4),
                  o_cand = take((size_t)n * 4), o_ctl = take(32),
@@ -1526,7 +1556,7 @@ im_status greedy_plain(im_pool *p, int32_t k, int32_t *d_seeds, int64_t *d_gains
     a.k = k;
     a.counts = (int32_t *)(B + o_cnt);
     a.covered = (uint32_t *)(B + o_cov);
-    a.block_best = (unsigned long long *)(B + o_best);
+    a.gmax = (unsigned long long *)(B + o_best);
     a.bar = (GridBarrier *)(B + o_bar);
     a.seeds = d_seeds;
     a.gains = d_gains;
@@ -1574,7 +1604,7 @@ im_status greedy_launch(int64_t n, int64_t theta, const int64_t *set_off, const 
     a.k = k;
     a.counts = counts;
     a.covered = covered;
-    a.block_best = block_best;
+    a.gmax = block_best;
     a.bar = (GridBarrier *)barrier;
     a.seeds = seeds;
     a.gains = gains;
@@ -1595,7 +1625,7 @@ constexpr int32_t kManyHubs = 1024;     // hub rows of a query at most
 namespace {
 struct ManyState {                      // zeroed before the launch
     GridBarrier bar;
-    unsigned long long work[2], npiece;
+    unsigned long long work[2], npiece, gmax[3];
     int32_t ctl[4];
 };
 size_t many_pieces(int64_t members) { return (size_t)(2 * members / kGreedyPiece + 1); }
@@ -1603,7 +1633,7 @@ size_t many_pieces(int64_t members) { return (size_t)(2 * members / kGreedyPiece
 
 size_t greedy_many_scratch(int32_t nq, int64_t members) {
     return align256((size_t)nq * sizeof(GreedyArgs)) + align256((size_t)(nq + 1) * 4) +
-           align256((size_t)nq * sizeof(ManyState)) + align256((size_t)num_sms() * 2 * 8) +
+           align256((size_t)nq * sizeof(ManyState)) +
            align256((size_t)nq * kManyHubs * kHubRep * 4) + align256((size_t)nq * kManyHubs * 4) +
            align256((many_pieces(members) + (size_t)nq) * 8);
 }
@@ -1628,7 +1658,6 @@ im_status greedy_many(const std::vector<GreedyQuery> &qs, const int64_t *set_off
     GreedyArgs *tab = (GreedyArgs *)take((size_t)nq * sizeof(GreedyArgs));
     int32_t *first = (int32_t *)take((size_t)(nq + 1) * 4);
     ManyState *state = (ManyState *)take((size_t)nq * sizeof(ManyState));
-    unsigned long long *best = (unsigned long long *)take((size_t)num_sms() * 2 * 8);
     int32_t *hub_cnt = (int32_t *)take((size_t)nq * kManyHubs * kHubRep * 4);
     int32_t *hub_list = (int32_t *)take((size_t)nq * kManyHubs * 4);
     unsigned long long *piece = (unsigned long long *)take((many_pieces(total) + (size_t)nq) * 8);
@@ -1670,7 +1699,7 @@ im_status greedy_many(const std::vector<GreedyQuery> &qs, const int64_t *set_off
         a.k = q.k;
         a.counts = q.counts;
         a.covered = q.covered;
-        a.block_best = best + hfirst[r % groups];
+        a.gmax = state[r].gmax;
         a.bar = &state[r].bar;
         a.seeds = q.seeds;
         a.gains = q.gains;
