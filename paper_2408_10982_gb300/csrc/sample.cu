@@ -1713,75 +1713,121 @@ template <>
 __device__ __forceinline__ int32_t key_max<int32_t>() { return 0x7fffffff; }
 
 template <typename Key>
-__device__ __forceinline__ Key warp_bitonic32(Key v, int lane) {
-#pragma unroll
-    for (int k = 2; k <= 32; k <<= 1) {
-#pragma unroll
-        for (int j = k >> 1; j > 0; j >>= 1) {
-            const Key o = __shfl_xor_sync(kFull, v, j);
-            const bool keep_min = ((lane & j) == 0) == ((lane & k) == 0);
-            v = keep_min ? (o < v ? o : v) : (o > v ? o : v);
-        }
-    }
-    return v;
+__device__ __forceinline__ void order_pair(Key &x, Key &y) {
+    const Key lo = min(x, y), hi = max(x, y);
+    x = lo;
+    y = hi;
 }
 
-// Bitonic sort of 32 E keys held by a warp in registers, element i = r 32 +
-// lane in v[r] (the layout of a coalesced load).  Partners i ^ j with j < 32
-// sit in other lanes (shuffle), with j >= 32 in the same lane (registers).
-template <typename Key, int E>
-__device__ __forceinline__ void warp_bitonic_regs(Key (&v)[E], int lane) {
+// N keys of one thread ascending (N a power of two, fully unrolled): Batcher's
+// odd-even merge sort, 63 comparators for 16 keys where a bitonic network has 80.
+template <typename Key, int N>
+__device__ __forceinline__ void thread_sort(Key (&v)[N]) {
 #pragma unroll
-    for (int k = 2; k <= 32 * E; k <<= 1) {
+    for (int p = 1; p < N; p <<= 1) {
 #pragma unroll
-        for (int j = k >> 1; j > 0; j >>= 1) {
-            if (j >= 32) {
-                const int jr = j >> 5;
+        for (int d = p; d > 0; d >>= 1) {
 #pragma unroll
-                for (int r = 0; r < E; ++r) {
-                    if (r & jr) continue;
-                    const int r2 = r | jr;
-                    const bool asc = (((r << 5) | lane) & k) == 0;
-                    const Key x = v[r], y = v[r2];
-                    const bool sw = asc ? (y < x) : (x < y);
-                    v[r] = sw ? y : x;
-                    v[r2] = sw ? x : y;
-                }
-            } else {
-                const bool lower = (lane & j) == 0;
-#pragma unroll
-                for (int r = 0; r < E; ++r) {
-                    const bool asc = (((r << 5) | lane) & k) == 0;
-                    const Key x = v[r];
-                    const Key y = __shfl_xor_sync(kFull, x, j);
-                    const Key lo = y < x ? y : x, hi = y < x ? x : y;
-                    v[r] = (lower == asc) ? lo : hi;
-                }
+            for (int i = 0; i < N; ++i) {
+                const int x = i - d % p;             // i heads a pair of this pass?
+                if (x >= 0 && i + d < N && x % (2 * d) < d && i / (2 * p) == (i + d) / (2 * p))
+                    order_pair(v[i], v[i + d]);
             }
         }
     }
 }
 
+// 32 E keys of a warp ascending, the lane's E keys consecutive in that order:
+// bitonic merges whose first pass pairs a block's halves mirrored, so that every
+// pass keeps the smaller key at the lower place.  Whatever E, 15 passes cross
+// lanes (a shuffle and a selected minimum per key); the others are a minimum and
+// a maximum in registers.
 template <typename Key, int E>
-__device__ __forceinline__ void warp_sort_copy(Key *out, const Key *src, int64_t len, int lane) {
+__device__ __forceinline__ void warp_sort_regs(Key (&v)[E], int lane) {
+    thread_sort<Key, E>(v);
+#pragma unroll
+    for (int q = 2; q <= 32; q <<= 1) {              // blocks of q lanes
+        const bool low = (lane & (q >> 1)) == 0;
+#pragma unroll
+        for (int r = 0; r < (E + 1) / 2; ++r) {
+            const Key a = __shfl_xor_sync(kFull, v[r], q - 1);
+            if (r != E - 1 - r) {
+                const Key b = __shfl_xor_sync(kFull, v[E - 1 - r], q - 1);
+                v[r] = low ? min(v[r], b) : max(v[r], b);
+            }
+            v[E - 1 - r] = low ? min(v[E - 1 - r], a) : max(v[E - 1 - r], a);
+        }
+#pragma unroll
+        for (int j = q >> 2; j > 0; j >>= 1) {
+            const bool lo = (lane & j) == 0;
+#pragma unroll
+            for (int r = 0; r < E; ++r) {
+                const Key o = __shfl_xor_sync(kFull, v[r], j);
+                v[r] = lo ? min(v[r], o) : max(v[r], o);
+            }
+        }
+#pragma unroll
+        for (int j = E >> 1; j > 0; j >>= 1) {
+#pragma unroll
+            for (int r = 0; r < E; ++r)
+                if (!(r & j)) order_pair(v[r], v[r | j]);
+        }
+    }
+}
+
+// At most 32 E keys of src, sorted, to buf: key i at word i + i / 32 (the
+// padding keeps either side free of bank conflicts).
+template <typename Key, int E>
+__device__ __forceinline__ void warp_sort_to(Key *buf, const Key *src, int len, int lane) {
     Key v[E];
 #pragma unroll
-    for (int r = 0; r < E; ++r) {
-        const int64_t t = (int64_t)r * 32 + lane;
-        v[r] = t < len ? src[t] : key_max<Key>();
-    }
-    warp_bitonic_regs<Key, E>(v, lane);
+    for (int r = 0; r < E; ++r) v[r] = r * 32 + lane < len ? src[r * 32 + lane] : key_max<Key>();
+    warp_sort_regs<Key, E>(v, lane);
 #pragma unroll
     for (int r = 0; r < E; ++r) {
-        const int64_t t = (int64_t)r * 32 + lane;
-        if (t < len) out[t] = v[r];
+        const int i = lane * E + r;
+        buf[i + (i >> 5)] = v[r];
+    }
+    __syncwarp();
+}
+
+template <typename Key, int E>
+__device__ __forceinline__ void warp_sort_copy(Key *out, const Key *src, int len, Key *buf,
+                                               int lane) {
+    warp_sort_to<Key, E>(buf, src, len, lane);
+#pragma unroll
+    for (int r = 0; r < E; ++r)
+        if (r * 32 + lane < len) out[r * 32 + lane] = buf[r * 33 + lane];
+}
+
+// 513 to 1,024 distinct keys: two sorted runs of 512 at most, then every key to
+// its place in its run plus the number of smaller keys of the other run.
+// (1,024 keys in registers would leave 16 warps an SM.)
+constexpr int kSortRun = 512, kSortRunWords = kSortRun + kSortRun / 32;
+template <typename Key>
+__device__ __forceinline__ void warp_sort_two(Key *out, const Key *src, int len, Key *buf,
+                                              int lane) {
+#pragma unroll 1
+    for (int h = 0; h < 2; ++h)
+        warp_sort_to<Key, kSortRun / 32>(buf + h * kSortRunWords, src + h * kSortRun,
+                                         h ? len - kSortRun : kSortRun, lane);
+    for (int t = lane; t < len; t += 32) {
+        const int h = t >= kSortRun, i = t - h * kSortRun;
+        const Key x = buf[h * kSortRunWords + i + (i >> 5)];
+        const Key *o = buf + (1 - h) * kSortRunWords;
+        int lo = 0, hi = h ? kSortRun : len - kSortRun;
+        while (lo < hi) {
+            const int m = (lo + hi) >> 1;
+            if (o[m + (m >> 5)] < x) lo = m + 1;
+            else hi = m;
+        }
+        out[i + lo] = x;
     }
 }
 
 // bitonic network over buf[0..P) (P a power of two) by `nthreads` threads
 template <typename Key>
-__device__ __forceinline__ void bitonic_smem(Key *buf, int P, int tid, int nthreads,
-                                             bool block_level) {
+__device__ __forceinline__ void bitonic_smem(Key *buf, int P, int tid, int nthreads) {
     for (int k = 2; k <= P; k <<= 1) {
         for (int j = k >> 1; j > 0; j >>= 1) {
             for (int i = tid; i < P; i += nthreads) {
@@ -1795,63 +1841,34 @@ __device__ __forceinline__ void bitonic_smem(Key *buf, int P, int tid, int nthre
                     }
                 }
             }
-            if (block_level) __syncthreads();
-            else __syncwarp();
+            __syncthreads();
         }
     }
 }
 
-// Bitonic sort of N keys held by one thread (N a power of two, fully unrolled).
-template <typename Key, int N>
-__device__ __forceinline__ void thread_bitonic(Key (&v)[N]) {
-#pragma unroll
-    for (int k = 2; k <= N; k <<= 1) {
-#pragma unroll
-        for (int j = k >> 1; j > 0; j >>= 1) {
-#pragma unroll
-            for (int i = 0; i < N; ++i) {
-                const int l = i ^ j;
-                if (l > i) {
-                    const bool asc = (i & k) == 0;
-                    const Key x = v[i], y = v[l];
-                    const bool sw = asc ? (y < x) : (x < y);
-                    v[i] = sw ? y : x;
-                    v[l] = sw ? x : y;
-                }
-            }
-        }
-    }
-}
+constexpr int kSortBuf = 2 * kSortRunWords;  // words of a warp's buffer
+static_assert(kWarpSortKeys == 2 * kSortRun, "two runs");
 
-// One segment sorted by the whole warp (len > kLaneSort): copied from the
-// stage and sorted in registers, or in the warp's shared buffer, or listed in
-// `big` for k_sort_block.
+// One segment sorted by the whole warp in registers (len > kLaneSort), or listed
+// in `big` for k_sort_block.  Instructions bound it.  Against bitonic passes over
+// keys a lane-stride apart (where most passes are shuffles) and, beyond 512 keys,
+// over shared memory: the 5.9 M weighted-cascade sets of an IMM run 3.68 ->
+// 1.02 ms, 4.2 M LT walks of 41 members 1.25 -> .93, 200 k sets at scale 15 .148
+// -> .040.  Five blocks an SM: three cost 5 to 20 % more.
 template <typename Key>
 __device__ __forceinline__ void warp_sort_segment(Key *out, const Key *src, int64_t len, int64_t i,
                                                   Key *buf, int64_t *big, unsigned long long *nbig,
                                                   int lane) {
     if (len <= 32) {
-        Key v = lane < len ? src[lane] : key_max<Key>();
-        v = warp_bitonic32<Key>(v, lane);
-        if (lane < len) out[lane] = v;
-    } else if (len <= 64) {
-        warp_sort_copy<Key, 2>(out, src, len, lane);
-    } else if (len <= 128) {
-        warp_sort_copy<Key, 4>(out, src, len, lane);
-    } else if (len <= 256) {
-        warp_sort_copy<Key, 8>(out, src, len, lane);
-    } else if (len <= 512 && sizeof(Key) == 4) {
-        warp_sort_copy<Key, 16>(out, src, len, lane);
-    } else if (len <= kWarpSortKeys) {
-        int P = 64;
-        while (P < len) P <<= 1;
-        for (int t = lane; t < P; t += 32) buf[t] = t < len ? src[t] : key_max<Key>();
-        __syncwarp();
-        bitonic_smem<Key>(buf, P, lane, 32, false);
-        for (int t = lane; t < len; t += 32) out[t] = buf[t];
-    } else if (lane == 0) {
-        big[atomicAdd(nbig, 1ull)] = i;
-    }
+        Key v[1] = {lane < len ? src[lane] : key_max<Key>()};
+        warp_sort_regs<Key, 1>(v, lane);
+        if (lane < len) out[lane] = v[0];
+    } else if (len <= 64) warp_sort_copy<Key, 2>(out, src, (int)len, buf, lane);
+    else if (len <= 128) warp_sort_copy<Key, 4>(out, src, (int)len, buf, lane);
+    else if (len <= 256) warp_sort_copy<Key, 8>(out, src, (int)len, buf, lane);
+    else if (len <= 512) warp_sort_copy<Key, 16>(out, src, (int)len, buf, lane);
+    else if (len <= kWarpSortKeys) warp_sort_two<Key>(out, src, (int)len, buf, lane);
+    else if (lane == 0) big[atomicAdd(nbig, 1ull)] = i;
     __syncwarp();
 }
 
@@ -1862,12 +1879,12 @@ __device__ __forceinline__ void warp_sort_segment(Key *out, const Key *src, int6
 constexpr int kLaneSort = 16;
 
 template <typename Key>
-__global__ void __launch_bounds__(256) k_sort_small(Key *dst, const int64_t *seg_off, int64_t nseg,
+__global__ void __launch_bounds__(256, 5) k_sort_small(Key *dst, const int64_t *seg_off, int64_t nseg,
                                                     const Key *stage, const int64_t *stage_off,
                                                     int64_t *mid, unsigned long long *nmid,
                                                     bool inline_long, int64_t *big,
                                                     unsigned long long *nbig) {
-    __shared__ Key sbuf[8][kWarpSortKeys];
+    __shared__ Key sbuf[8][kSortBuf];
     const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
     const int64_t nw = (int64_t)gridDim.x * 8;
     for (int64_t i0 = ((int64_t)blockIdx.x * 8 + wib) * 32; i0 < nseg; i0 += nw * 32) {
@@ -1886,7 +1903,7 @@ __global__ void __launch_bounds__(256) k_sort_small(Key *dst, const int64_t *seg
             Key v[kLaneSort];
 #pragma unroll
             for (int r = 0; r < kLaneSort; ++r) v[r] = r < len ? src[r] : key_max<Key>();
-            thread_bitonic<Key, kLaneSort>(v);
+            thread_sort<Key, kLaneSort>(v);
 #pragma unroll
             for (int r = 0; r < kLaneSort; ++r)
                 if (r < len) out[r] = v[r];
@@ -1914,12 +1931,12 @@ __global__ void __launch_bounds__(256) k_sort_small(Key *dst, const int64_t *seg
 // the list): sorted in registers or in the warp's shared buffer; segments
 // longer than that buffer are copied into place and listed in `big`.
 template <typename Key>
-__global__ void __launch_bounds__(256) k_sort_mid(Key *dst, const int64_t *seg_off,
+__global__ void __launch_bounds__(256, 5) k_sort_mid(Key *dst, const int64_t *seg_off,
                                                   const Key *stage, const int64_t *stage_off,
                                                   const int64_t *mid,
                                                   const unsigned long long *nmid, int64_t *big,
                                                   unsigned long long *nbig) {
-    __shared__ Key sbuf[8][kWarpSortKeys];
+    __shared__ Key sbuf[8][kSortBuf];
     const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
     const int64_t nw = (int64_t)gridDim.x * 8;
     const int64_t cnt = (int64_t)*nmid;
@@ -1975,7 +1992,7 @@ __global__ void __launch_bounds__(1024) k_sort_block(Key *dst, const int64_t *se
         while (P < len) P <<= 1;
         for (int t = threadIdx.x; t < P; t += blockDim.x) buf[t] = t < len ? src[t] : key_max<Key>();
         __syncthreads();
-        bitonic_smem<Key>(buf, P, threadIdx.x, blockDim.x, true);
+        bitonic_smem<Key>(buf, P, threadIdx.x, blockDim.x);
         for (int t = threadIdx.x; t < len; t += blockDim.x) dst[o + t] = buf[t];
         __syncthreads();
     }
