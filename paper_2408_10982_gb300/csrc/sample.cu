@@ -1825,27 +1825,6 @@ __device__ __forceinline__ void warp_sort_two(Key *out, const Key *src, int len,
     }
 }
 
-// bitonic network over buf[0..P) (P a power of two) by `nthreads` threads
-template <typename Key>
-__device__ __forceinline__ void bitonic_smem(Key *buf, int P, int tid, int nthreads) {
-    for (int k = 2; k <= P; k <<= 1) {
-        for (int j = k >> 1; j > 0; j >>= 1) {
-            for (int i = tid; i < P; i += nthreads) {
-                const int l = i ^ j;
-                if (l > i) {
-                    const Key x = buf[i], y = buf[l];
-                    const bool asc = (i & k) == 0;
-                    if ((x > y) == asc) {
-                        buf[i] = y;
-                        buf[l] = x;
-                    }
-                }
-            }
-            __syncthreads();
-        }
-    }
-}
-
 constexpr int kSortBuf = 2 * kSortRunWords;  // words of a warp's buffer
 static_assert(kWarpSortKeys == 2 * kSortRun, "two runs");
 
@@ -1949,52 +1928,93 @@ __global__ void __launch_bounds__(256, 5) k_sort_mid(Key *dst, const int64_t *se
     }
 }
 
-// One block per listed segment longer than a warp's buffer: copied from the
-// stage when it is ascending there, else sorted in shared memory, or listed in
-// `giant` for k_sort_giant when it has more than kBlockSortCap keys.
-template <typename Key>
-__global__ void __launch_bounds__(1024) k_sort_block(Key *dst, const int64_t *seg_off,
-                                                     const Key *stage, const int64_t *stage_off,
-                                                     const int64_t *big,
-                                                     const unsigned long long *nbig,
-                                                     int64_t *giant, unsigned long long *ngiant) {
+// A block sorts up to kBlockKeys keys a thread; sets up to kMidSortCap go to
+// blocks of 256, of which an SM holds four, the others to blocks of 1,024.
+constexpr int kBlockKeys = 16;
+constexpr int kMidSortCap = 256 * kBlockKeys;
+static_assert(kBlockSortCap == 1024 * kBlockKeys, "the larger blocks");
+
+// One block of T threads per listed segment of its class: copied from the stage
+// when it is ascending there, or listed in `giant` for k_sort_giant when it has
+// more than kBlockSortCap keys, else sorted: runs of kSortRun keys by the warps,
+// then merged pairwise.  A key's place after a merge is its place in its run plus
+// the number of smaller keys in the other (keys are distinct), found by a binary
+// search; the keys wait in registers while the buffer is rewritten.
+// Against a bitonic network over shared memory (66 to 105 passes of it): the long
+// sets of an IMM run, weighted cascade on the LiveJournal shape, 4.1 -> 1.2 ms.
+template <typename Key, int T>
+__global__ void __launch_bounds__(T, 1024 / T) k_sort_block(Key *dst, const int64_t *seg_off,
+                                                            const Key *stage,
+                                                            const int64_t *stage_off,
+                                                            const int64_t *big,
+                                                            const unsigned long long *nbig,
+                                                            int64_t *giant,
+                                                            unsigned long long *ngiant) {
     extern __shared__ unsigned char sraw[];
     Key *buf = reinterpret_cast<Key *>(sraw);
     const int64_t nb = (int64_t)*nbig;
+    const int tid = threadIdx.x, lane = tid & 31;
     for (int64_t b = blockIdx.x; b < nb; b += gridDim.x) {
         const int64_t i = big[b];
         const int64_t o = seg_off[i];
-        const int64_t len = seg_off[i + 1] - o;
+        const int64_t seg = seg_off[i + 1] - o;
+        if ((T == 256) != (seg <= kMidSortCap)) continue;
         const int64_t so = stage_off[i];
         const Key *src = stage + (so & ~kStageAscending);
         if (so & kStageAscending) {
             constexpr int U = 8;
-            for (int64_t t0 = threadIdx.x; t0 < len; t0 += (int64_t)U * blockDim.x) {
+            for (int64_t t0 = tid; t0 < seg; t0 += (int64_t)U * T) {
                 Key v[U];
 #pragma unroll
                 for (int u = 0; u < U; ++u) {
-                    const int64_t t = t0 + (int64_t)u * blockDim.x;
-                    if (t < len) v[u] = src[t];
+                    const int64_t t = t0 + (int64_t)u * T;
+                    if (t < seg) v[u] = src[t];
                 }
 #pragma unroll
                 for (int u = 0; u < U; ++u) {
-                    const int64_t t = t0 + (int64_t)u * blockDim.x;
-                    if (t < len) dst[o + t] = v[u];
+                    const int64_t t = t0 + (int64_t)u * T;
+                    if (t < seg) dst[o + t] = v[u];
                 }
             }
             continue;
         }
-        if (len > kBlockSortCap) {
-            if (threadIdx.x == 0) giant[atomicAdd(ngiant, 1ull)] = i;
+        if (seg > kBlockSortCap) {
+            if (tid == 0) giant[atomicAdd(ngiant, 1ull)] = i;
             continue;
         }
-        int P = 64;
-        while (P < len) P <<= 1;
-        for (int t = threadIdx.x; t < P; t += blockDim.x) buf[t] = t < len ? src[t] : key_max<Key>();
+        const int len = (int)seg;
+        for (int r = tid >> 5; r * kSortRun < len; r += T / 32)
+            warp_sort_to<Key, kSortRun / 32>(buf + r * kSortRunWords, src + r * kSortRun,
+                                             len - r * kSortRun, lane);
         __syncthreads();
-        bitonic_smem<Key>(buf, P, threadIdx.x, blockDim.x);
-        for (int t = threadIdx.x; t < len; t += blockDim.x) dst[o + t] = buf[t];
-        __syncthreads();
+        for (int w = kSortRun; w < len; w <<= 1) {
+            const bool last = 2 * w >= len;
+            Key x[kBlockKeys];
+            int at[kBlockKeys];
+#pragma unroll
+            for (int u = 0; u < kBlockKeys; ++u) {
+                const int t = tid + u * T;
+                if (t < len) {
+                    x[u] = buf[t + (t >> 5)];
+                    const int first = t & ~(2 * w - 1);          // of the pair of runs
+                    const int from = t & w ? first : min(first + w, len);
+                    int lo = from, hi = t & w ? first + w : min(first + 2 * w, len);
+                    while (lo < hi) {
+                        const int m = (lo + hi) >> 1;
+                        if (buf[m + (m >> 5)] < x[u]) lo = m + 1;
+                        else hi = m;
+                    }
+                    at[u] = first + (t & (w - 1)) + lo - from;
+                    if (last) dst[o + at[u]] = x[u];
+                }
+            }
+            __syncthreads();
+            if (last) break;
+#pragma unroll
+            for (int u = 0; u < kBlockKeys; ++u)
+                if (tid + u * T < len) buf[at[u] + (at[u] >> 5)] = x[u];
+            __syncthreads();
+        }
     }
 }
 
@@ -2434,13 +2454,16 @@ im_status segmented_sort_sets(int32_t *dst, const int64_t *seg_off, int64_t nseg
     }
     IM_CUDA(cudaGetLastError());
     if (long_sets == 0) return IM_OK;
-    const size_t smem = (size_t)kBlockSortCap * 4;
-    IM_TRY(raise_dyn_smem((const void *)k_sort_block<int32_t>, smem));
+    const size_t mid_smem = kMidSortCap / kSortRun * kSortRunWords * sizeof(int32_t);
+    const size_t smem = kBlockSortCap / kSortRun * kSortRunWords * sizeof(int32_t);
+    IM_TRY(raise_dyn_smem((const void *)k_sort_block<int32_t, 1024>, smem));
     IM_CUDA(cudaMemsetAsync(ctr + 1, 0, sizeof(unsigned long long), st));
     {
         KernelTimer kt(st, "sort_sets_block");
-        k_sort_block<int32_t><<<num_sms(), 1024, smem, st>>>(dst, seg_off, stage, stage_off, big,
-                                                             ctr, mid, ctr + 1);
+        k_sort_block<int32_t, 1024><<<num_sms(), 1024, smem, st>>>(dst, seg_off, stage, stage_off,
+                                                                   big, ctr, mid, ctr + 1);
+        k_sort_block<int32_t, 256><<<num_sms() * 4, 256, mid_smem, st>>>(
+            dst, seg_off, stage, stage_off, big, ctr, mid, ctr + 1);
     }
     IM_CUDA(cudaGetLastError());
     const int64_t ngiant = (int64_t)(long_sets >> 32);

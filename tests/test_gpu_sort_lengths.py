@@ -8,8 +8,10 @@ from paper_2408_10982_gb300 import inputs
 pytestmark = pytest.mark.gpu
 
 
-@pytest.mark.parametrize("n,theta", [(20, 40), (70, 1_000_003), (300, 1_500_000), (1100, 9000), (2500, 4000)])
-def test_sorted_at_every_length(n, theta):
+@pytest.mark.parametrize("model,n,theta", [
+    ("IC", 20, 40), ("IC", 70, 1_000_003), ("IC", 300, 1_500_000), ("IC", 1100, 9000), ("IC", 2500, 4000),
+    ("LT", 1030, 9000), ("LT", 2060, 9000), ("LT", 4200, 30_000), ("LT", 17_000, 2500)])
+def test_sorted_at_every_length(model, n, theta):
     from paper_2408_10982_gb300 import im
 
     # a certain chain over shuffled names: the set of place p holds places 0 .. p
@@ -18,7 +20,7 @@ def test_sorted_at_every_length(n, theta):
     in_off, in_src = inputs.in_csr(n, name[:-1], name[1:])
     G = im.Graph(inputs.Graph(n, in_off, in_src, np.full(n - 1, 2**32 - 1, np.uint32)))
     P = im.Pool(G, theta, theta * n)
-    P.sample(im.IM_IC, 17, 0, theta)
+    P.sample(getattr(im, "IM_" + model), 17, 0, theta)
     off, mem = P.export()
     size = np.diff(off)
     assert size.min() >= 1 and size.max() <= n
