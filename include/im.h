@@ -78,8 +78,8 @@ typedef enum { IM_AGG_STREAM = 0, IM_AGG_GREEDY = 1 } im_aggregator;
  *                   as they are produced (streaming overlap, bucket bitmaps in
  *                   global memory); 0 runs them as two launches, the second
  *                   a bucket stage laid out as IM_TUNE_RG_CLUSTER says (by
- *                   default one 64-bit bucket mask per RRR set).  Results
- *                   are identical.
+ *                   default one 64-bit bucket mask per RRR set, or a block
+ *                   per bucket).  Results are identical.
  *   aggregator      RandGreedi only: IM_AGG_STREAM (0) aggregates with the
  *                   streaming buckets of Alg. 5 (Sec. 3.3); IM_AGG_GREEDY (1)
  *                   is Alg. 4's global step as written: the lazy greedy of
@@ -225,11 +225,14 @@ im_status im_pool_sample_bytes(const im_pool *p, int64_t *bytes);
  *                       32 / value walks in lockstep over a fanout-32 search
  *                       tree of the running sums).
  *   IM_TUNE_RG_CLUSTER  RandGreedi two-launch mode, bucket stage: 0 (default)
- *                       keeps one 64-bit bucket mask per RRR set, so one pass
- *                       over a streamed subset counts its gain for every
- *                       bucket, and spreads each group of stream slots over
- *                       the whole GPU (B <= 64; for B > 64 it picks a cluster
- *                       as below); 1..8 keeps each bucket's theta-bit bitmap
+ *                       gives every bucket one block with its theta-bit bitmap
+ *                       in shared memory where the bitmap fits and the pool
+ *                       has at most 2^20 members or B > 64; else keeps one
+ *                       64-bit bucket mask per RRR set, so one pass over a
+ *                       streamed subset counts its gain for every bucket, and
+ *                       spreads each group of stream slots over the whole GPU
+ *                       (B <= 64; for B > 64 it picks a cluster as below);
+ *                       1..8 keeps each bucket's theta-bit bitmap
  *                       in the shared memory of a cluster of at least that
  *                       many blocks (the smallest of 1, 2, 4, 8 that holds
  *                       it); -1 keeps the bitmaps in global memory (one block
@@ -237,9 +240,9 @@ im_status im_pool_sample_bytes(const im_pool *p, int64_t *bytes);
  *   IM_TUNE_INDEX_REPLICAS  covering-subset build: 0 (default) a stable radix
  *                       sort of the (vertex, set id) pairs by vertex, up to 10
  *                       bits a pass, with 0, 8 or 12 bytes of pool scratch per
- *                       member (1, 2 or 3 passes; set ids come out ascending inside every S(v); without the
- *                       memory, the counting build with 4 replicas runs
- *                       instead); 1, 2, 4 or 8: a counting build, histogram
+ *                       member (1, 2 or 3 passes; set ids come out ascending
+ *                       inside every S(v); without the memory, the counting
+ *                       build with 4 replicas runs instead); 1, 2, 4 or 8: a counting build, histogram
  *                       and scatter through per-vertex counters and cursors
  *                       replicated that many times (a member's replica
  *                       follows its position), spreading the atomics on hub
@@ -453,9 +456,9 @@ im_status im_opim(const im_graph *g, im_model model, int32_t k, double eps, doub
  * A query: a resident graph, a model, k, theta (sample ids 0 .. theta-1) and
  * its Philox seed.  im_solve_batch solves nq queries in a fixed number of
  * launches (one sampling launch per model over all their samples, one sort,
- * one covering-subset build over all queries' vertices, one greedy launch
- * with one block per query; RandGreedi queries one after another on the
- * batch's shared index) and gives every query exactly the seeds, gains and
+ * one covering-subset build over all queries' vertices, one greedy launch on
+ * groups of blocks sized by the queries' members; RandGreedi queries one after
+ * another on the batch's shared index) and gives every query exactly the seeds, gains and
  * coverage that im_sample_rrr + im_max_k_cover give it alone.  seeds
  * int32[nq * kmax] and gains int64[nq * kmax] (row q: query q's seeds;
  * entries past num_seeds are unspecified; gains may be NULL), host or
