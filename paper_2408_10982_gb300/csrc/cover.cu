@@ -15,9 +15,10 @@
 // publishes its j-th seed (j < ceil(alpha k)) in slot (j, p) of a device array
 // and raises a release flag; the buckets consume the slots in (j, p) order, so
 // they see the same stream order in every run.  The receiver's B bucketing
-// threads become, by default, k_rg_stream_masks after the producers finish:
-// one 64-bit mask per RRR set holds the buckets covering it, so one pass over
-// a streamed subset counts its gain for every bucket.  Alternatives (tuning
+// threads become, after the producers finish, k_rg_stream_small (a block per
+// bucket: short streams, or more than 64 buckets) or k_rg_stream_masks: one
+// 64-bit mask per RRR set holds the buckets covering it, so one pass over a
+// streamed subset counts its gain for every bucket.  Alternatives (tuning
 // knob values): one "consumer" block or thread-block cluster per bucket, and
 // a fused mode where producers and consumers are one cooperative launch and
 // the consumers read the slots with acquire loads as they are published, the

@@ -216,7 +216,8 @@ struct im_graph {
                          // built on first IC use
     // LT search index, built on first LT use: per-vertex records, per-edge
     // leaves (running weight sum << 31 | source) and upper tree levels
-    uint4 *lt_vrec;                  // [n] {edge offset, in-degree, tree offset | levels << 28, equal in-weight or 0}
+    uint4 *lt_vrec;                  // [n] {edge offset, in-degree, reciprocal of the equal
+                                     // in-weight (else tree offset | levels << 28), that weight or 0}
     unsigned long long *lt_leaf;     // [m]
     unsigned long long *lt_tree;     // [sum over vertices of the upper-level sizes]
     uint4 *lt_guide;                 // [m] inverse-CDF cut points (see k_lt_guide)

@@ -535,7 +535,7 @@ extern "C" im_status im_spread(const im_graph *gc, im_model model, const int32_t
         a.left = (unsigned long long *)(N + o_left);
         IM_CUDA(cudaMemsetAsync(N + o_bars, 0, need - o_bars, st));
         void *args[] = {&a};
-        KernelTimer kt(st, "spread_pull");
+        KernelTimer kt(st, "spread_lt");
         IM_CUDA(cudaLaunchCooperativeKernel((const void *)k_spread_pull, dim3(grid),
                                             dim3(kPullThreads), args, 0, st));
     }
