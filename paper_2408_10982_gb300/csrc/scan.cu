@@ -43,10 +43,19 @@ __global__ void __launch_bounds__(kScanThreads) k_tile_sums(const int32_t *in, i
     __shared__ int64_t sh[33];
     const int64_t base = (int64_t)blockIdx.x * kScanTile;
     int64_t s = 0;
+    if (base + kScanTile <= count && ((uintptr_t)in & 15) == 0) {
+        const int4 *in4 = reinterpret_cast<const int4 *>(in + base);
 #pragma unroll
-    for (int i = 0; i < kScanItems; ++i) {
-        int64_t idx = base + (int64_t)i * kScanThreads + threadIdx.x;
-        if (idx < count) s += in[idx];
+        for (int i = 0; i < kScanItems / 4; ++i) {
+            const int4 x = in4[i * kScanThreads + threadIdx.x];
+            s += (int64_t)x.x + x.y + ((int64_t)x.z + x.w);
+        }
+    } else {
+#pragma unroll
+        for (int i = 0; i < kScanItems; ++i) {
+            int64_t idx = base + (int64_t)i * kScanThreads + threadIdx.x;
+            if (idx < count) s += in[idx];
+        }
     }
     int64_t total;
     block_excl_scan(s, &total, sh);
@@ -91,21 +100,41 @@ __global__ void __launch_bounds__(kScanThreads) k_tile_scan(const int32_t *in, i
         }
         block_excl_scan(s, &prefix, sh);
     }
-    // each thread owns kScanItems consecutive items
+    // each thread owns kScanItems consecutive items, read and written 16 bytes at
+    // a time where the arrays' alignment allows
+    const int64_t at = first + (int64_t)threadIdx.x * kScanItems;
+    const bool whole = at + kScanItems <= count;
     int32_t v[kScanItems];
     int64_t s = 0;
+    if (whole && ((uintptr_t)in & 15) == 0) {
 #pragma unroll
-    for (int i = 0; i < kScanItems; ++i) {
-        int64_t idx = first + (int64_t)threadIdx.x * kScanItems + i;
-        v[i] = idx < count ? in[idx] : 0;
-        s += v[i];
+        for (int i = 0; i < kScanItems; i += 4) {
+            const int4 x = *reinterpret_cast<const int4 *>(in + at + i);
+            v[i] = x.x;
+            v[i + 1] = x.y;
+            v[i + 2] = x.z;
+            v[i + 3] = x.w;
+        }
+    } else {
+#pragma unroll
+        for (int i = 0; i < kScanItems; ++i) v[i] = at + i < count ? in[at + i] : 0;
     }
-    int64_t run = prefix + block_excl_scan(s, &total, sh);
 #pragma unroll
-    for (int i = 0; i < kScanItems; ++i) {
-        int64_t idx = first + (int64_t)threadIdx.x * kScanItems + i;
-        if (idx < count) out[idx] = run;
-        run += v[i];
+    for (int i = 0; i < kScanItems; ++i) s += v[i];
+    int64_t run = prefix + block_excl_scan(s, &total, sh);
+    if (whole && ((uintptr_t)out & 15) == 0) {
+#pragma unroll
+        for (int i = 0; i < kScanItems; i += 2) {
+            const int64_t next = run + v[i];
+            *reinterpret_cast<longlong2 *>(out + at + i) = make_longlong2(run, next);
+            run = next + v[i + 1];
+        }
+    } else {
+#pragma unroll
+        for (int i = 0; i < kScanItems; ++i) {
+            if (at + i < count) out[at + i] = run;
+            run += v[i];
+        }
     }
     // (*base may be out[0]: it is read before, or stays what it is)
     if (blockIdx.x == gridDim.x - 1 && threadIdx.x == 0) out[count] = prefix + total;
