@@ -115,10 +115,10 @@ __device__ __forceinline__ int find_query(const SampleArgs &a, int64_t j) {
 // owner), the short lists packed.
 // Measured against one lane loop that loaded weights and sources with every
 // group and claimed live sources where it found them: weighted cascade on the
-// LiveJournal shape (IMM, 1.6 x 10^11 coins) 597 -> 139 ms, U[0, 0.1] at scale
+// LiveJournal shape (IMM, 1.6 x 10^11 coins) 597 -> 130 ms, U[0, 0.1] at scale
 // 20 (9.8 x 10^9 coins) 55 -> 24.5 ms, trivalency on the LiveJournal shape
-// (6.3 x 10^9) 45 -> 20.7 ms.  ncu, weighted cascade at scale 15: 141
-// instructions per 128 coins, issue 71 % and ALU and FMA-heavy pipes 62 % busy
+// (6.3 x 10^9) 45 -> 20.7 ms.  ncu, weighted cascade at scale 15: 126
+// instructions per 128 coins, issue 64 % and ALU and FMA-heavy pipes 59 % busy
 // while DRAM is idle, so what is left is the instructions of the coins.  Tried
 // and not kept: one call site for all kinds of lists (a state machine; fewer
 // instruction-fetch stalls, more instructions: 31.5 against 23.5 ms at scale
