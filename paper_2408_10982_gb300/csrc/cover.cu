@@ -861,12 +861,12 @@ __device__ void consume(const RGArgs &a, int b, long long *shs) {
 // The producers alone (two-launch mode): one block per part.
 template <bool SB>
 __global__ void __launch_bounds__(kProdThreads) k_rg_local(RGArgs a) {
-    extern __shared__ int32_t key[];
+    extern __shared__ __align__(16) int32_t key[];   // (produce() reads 16 bytes at a time)
     for (int p = blockIdx.x; p < a.P; p += gridDim.x) produce<SB>(a, p, key);
 }
 
 __global__ void __launch_bounds__(kRGThreads) k_randgreedi(RGArgs a) {
-    extern __shared__ int32_t key[];
+    extern __shared__ __align__(16) int32_t key[];
     __shared__ long long shs[33];
     const int r = blockIdx.x;
     if (a.first_role == 0 && r < a.nprod) {

@@ -1950,7 +1950,7 @@ __global__ void __launch_bounds__(T, 1024 / T) k_sort_block(Key *dst, const int6
                                                             const unsigned long long *nbig,
                                                             int64_t *giant,
                                                             unsigned long long *ngiant) {
-    extern __shared__ unsigned char sraw[];
+    extern __shared__ __align__(16) unsigned char sraw[];
     Key *buf = reinterpret_cast<Key *>(sraw);
     const int64_t nb = (int64_t)*nbig;
     const int tid = threadIdx.x, lane = tid & 31;
