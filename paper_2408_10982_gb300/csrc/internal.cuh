@@ -358,10 +358,31 @@ inline im_status dev_alloc(T **p, size_t bytes) {
 }
 
 // A call's temporary memory, from the same cached memory pool but ordered on the
-// call's stream (free it there with cudaFreeAsync): the default memory pool
+// call's stream (held by a CallBuf, which frees it there): the default memory pool
 // unmaps what is freed at the next synchronisation, and mapping it again cost
 // im_spread 2.6 ms a call.
 im_status call_alloc(void **p, size_t bytes, cudaStream_t st);
+
+// The owner of such memory: it is handed back on every way out of the call, failed
+// launches and copies among them, behind the work that the stream then holds.
+class CallBuf {
+  public:
+    explicit CallBuf(cudaStream_t st) : st_(st) {}
+    ~CallBuf() {
+        if (p_) cudaFreeAsync(p_, st_);
+    }
+    CallBuf(const CallBuf &) = delete;
+    CallBuf &operator=(const CallBuf &) = delete;
+    im_status alloc(size_t bytes) { return call_alloc(&p_, bytes, st_); }   // once
+    template <typename T>
+    T *as() const {
+        return static_cast<T *>(p_);
+    }
+
+  private:
+    cudaStream_t st_;
+    void *p_ = nullptr;
+};
 
 // scratch arena of a pool: returns a pointer to at least `bytes` (256-aligned)
 im_status pool_scratch(im_pool *p, size_t bytes, void **out);

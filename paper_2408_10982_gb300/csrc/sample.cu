@@ -2087,18 +2087,7 @@ im_status build_lt_index(im_graph *g, cudaStream_t st) {
     std::lock_guard<std::mutex> lk(g_lt_index_mu);
     if (g->lt_vrec) return IM_OK;   // set only once the whole index is built
     const int64_t n = g->n, m = g->m;
-    // stream-ordered temporaries, freed on every exit
-    struct Temps {
-        cudaStream_t st;
-        int32_t *sizes = nullptr, *big = nullptr;
-        int64_t *toff = nullptr;
-        int *flags = nullptr;   // [0] weights of some vertex sum above 2^32, [1] listed
-                                // vertices, [2] some vertex needs the cut points
-        ~Temps() {
-            for (void *p : {(void *)sizes, (void *)big, (void *)toff, (void *)flags})
-                if (p) cudaFreeAsync(p, st);
-        }
-    } t{st};
+    CallBuf sizes_buf(st), big_buf(st), toff_buf(st), flags_buf(st);
     // the index itself: handed to g once complete, freed on any failure
     struct Index {
         unsigned long long *leaf = nullptr, *tree = nullptr;
@@ -2112,10 +2101,16 @@ im_status build_lt_index(im_graph *g, cudaStream_t st) {
         }
     } x;
     const int64_t big_cap = m / (kLtBlockDeg + 1) + 1;
-    IM_TRY(call_alloc((void **)&t.sizes, (size_t)n * 4, st));
-    IM_TRY(call_alloc((void **)&t.big, (size_t)big_cap * 4, st));
-    IM_TRY(call_alloc((void **)&t.toff, (size_t)(n + 1) * 8 + scan_tmp_bytes(n) + 256, st));
-    IM_TRY(call_alloc((void **)&t.flags, 3 * sizeof(int), st));
+    IM_TRY(sizes_buf.alloc((size_t)n * 4));
+    IM_TRY(big_buf.alloc((size_t)big_cap * 4));
+    IM_TRY(toff_buf.alloc((size_t)(n + 1) * 8 + scan_tmp_bytes(n) + 256));
+    IM_TRY(flags_buf.alloc(3 * sizeof(int)));
+    struct {
+        int32_t *sizes, *big;
+        int64_t *toff;
+        int *flags;             // [0] weights of some vertex sum above 2^32, [1] listed
+                                // vertices, [2] some vertex needs the cut points
+    } t = {sizes_buf.as<int32_t>(), big_buf.as<int32_t>(), toff_buf.as<int64_t>(), flags_buf.as<int>()};
     IM_CUDA(cudaMemsetAsync(t.flags, 0, 3 * sizeof(int), st));
     {
         KernelTimer kt(st, "lt_index");
@@ -2376,10 +2371,10 @@ im_status run_sampling(const SamplingJob &job, const std::function<im_status(siz
         const size_t need2 = (size_t)units * (size_t)per_unit;
         // the first pass's queues and bitmaps are free by now, and mostly enough
         // (mapping fresh memory took 2 to 5 ms a call)
-        int32_t *q2 = nullptr;
         const bool own = need2 > off - o_q;
-        if (own) IM_TRY(call_alloc((void **)&q2, need2, st));
-        else q2 = (int32_t *)(B + o_q);
+        CallBuf q2_buf(st);
+        if (own) IM_TRY(q2_buf.alloc(need2));
+        int32_t *q2 = own ? q2_buf.as<int32_t>() : (int32_t *)(B + o_q);
         uint32_t *vis2 = (uint32_t *)((char *)q2 + (size_t)units * (size_t)n * 4);
         if (ic_big) IM_CUDA(cudaMemsetAsync(vis2, 0, (size_t)units * vis_words * 4, st));
         IM_CUDA(cudaMemsetAsync(ctr, 0, sizeof(unsigned long long), st));
@@ -2400,7 +2395,6 @@ im_status run_sampling(const SamplingJob &job, const std::function<im_status(siz
             launch(nb2, 32);   // one walk per warp: queues of n entries for the longest walks
         }
         IM_CUDA(cudaGetLastError());
-        if (own) IM_CUDA(cudaFreeAsync(q2, st));
         IM_CUDA(cudaMemcpyAsync(hc, ctr, sizeof(hc), cudaMemcpyDeviceToHost, st));
         IM_CUDA(cudaStreamSynchronize(st));
         dev_status = (int)(hc[4] & 0xffffffffu);
@@ -2471,8 +2465,9 @@ im_status segmented_sort_sets(int32_t *dst, const int64_t *seg_off, int64_t nseg
         // an n-bit bitmap per block
         const int64_t gwords = (n_max + 31) / 32;
         const int blocks3 = (int)std::min<int64_t>(ngiant, num_sms());
-        uint32_t *gbm = nullptr;
-        IM_TRY(call_alloc((void **)&gbm, (size_t)blocks3 * gwords * 4, st));
+        CallBuf gbm_buf(st);
+        IM_TRY(gbm_buf.alloc((size_t)blocks3 * gwords * 4));
+        uint32_t *gbm = gbm_buf.as<uint32_t>();
         IM_CUDA(cudaMemsetAsync(gbm, 0, (size_t)blocks3 * gwords * 4, st));
         {
             KernelTimer kt(st, "sort_sets_bitmap");
@@ -2480,7 +2475,6 @@ im_status segmented_sort_sets(int32_t *dst, const int64_t *seg_off, int64_t nseg
                                                    gbm, gwords);
         }
         IM_CUDA(cudaGetLastError());
-        IM_CUDA(cudaFreeAsync(gbm, st));
     }
     return IM_OK;
 }

@@ -369,12 +369,8 @@ im_status build_out_index(im_graph *g, cudaStream_t st) {
     std::lock_guard<std::mutex> lk(g_out_index_mu);
     if (g->out_off) return IM_OK;   // set only once the whole index is built
     const int64_t n = g->n, m = g->m;
-    // stream-ordered temporaries, freed on every exit; the index itself is
-    // handed to g once complete and freed on any failure
+    // the index: handed to g once complete, freed on any failure
     struct Parts {
-        cudaStream_t st;
-        int32_t *cnt = nullptr;
-        void *scan_tmp = nullptr;
         int64_t *off = nullptr;
         uint4 *rec = nullptr;
         ~Parts() {
@@ -383,27 +379,27 @@ im_status build_out_index(im_graph *g, cudaStream_t st) {
                 cudaFree(off);
                 cudaFree(rec);
             }
-            if (cnt) cudaFreeAsync(cnt, st);
-            if (scan_tmp) cudaFreeAsync(scan_tmp, st);
         }
-    } t{st};
-    IM_TRY(call_alloc((void **)&t.cnt, (size_t)n * 4, st));
-    IM_TRY(call_alloc(&t.scan_tmp, scan_tmp_bytes(n), st));
+    } t;
+    CallBuf cnt_buf(st), scan_buf(st);
+    IM_TRY(cnt_buf.alloc((size_t)n * 4));
+    IM_TRY(scan_buf.alloc(scan_tmp_bytes(n)));
+    int32_t *cnt = cnt_buf.as<int32_t>();
     IM_CUDA(cudaMalloc(&t.off, (size_t)(n + 1) * 8));
     IM_CUDA(cudaMalloc(&t.rec, (size_t)std::max<int64_t>(m, 1) * sizeof(uint4)));
-    IM_CUDA(cudaMemsetAsync(t.cnt, 0, (size_t)n * 4, st));
+    IM_CUDA(cudaMemsetAsync(cnt, 0, (size_t)n * 4, st));
     {
         KernelTimer kt(st, "out_index");
-        if (m > 0) k_out_hist<<<num_sms() * 4, 256, 0, st>>>(g->in_src, m, t.cnt);
+        if (m > 0) k_out_hist<<<num_sms() * 4, 256, 0, st>>>(g->in_src, m, cnt);
     }
     IM_CUDA(cudaGetLastError());
-    IM_TRY(exclusive_scan_i32_to_i64(t.cnt, t.off, n, nullptr, t.scan_tmp, scan_tmp_bytes(n), st));
-    IM_CUDA(cudaMemsetAsync(t.cnt, 0, (size_t)n * 4, st));
+    IM_TRY(exclusive_scan_i32_to_i64(cnt, t.off, n, nullptr, scan_buf.as<void>(), scan_tmp_bytes(n), st));
+    IM_CUDA(cudaMemsetAsync(cnt, 0, (size_t)n * 4, st));
     {
         KernelTimer kt(st, "out_index");
         if (m > 0)
             k_out_fill<<<num_sms() * 8, 256, 0, st>>>(g->in_off, g->in_src, g->w, n, t.off,
-                                                      t.cnt, t.rec);
+                                                      cnt, t.rec);
     }
     IM_CUDA(cudaGetLastError());
     IM_CUDA(cudaStreamSynchronize(st));
@@ -470,8 +466,9 @@ extern "C" im_status im_spread(const im_graph *gc, im_model model, const int32_t
                  o_vis = take((size_t)warps * words * 4), o_q = take((size_t)warps * qcap * 4),
                  o_act = take(host_act ? (size_t)runs * 8 : 0),
                  o_hit = take(host_hit ? (size_t)runs : 0);
-    char *B = nullptr;
-    IM_TRY(call_alloc((void **)&B, off, st));
+    CallBuf buf(st), next(st);
+    IM_TRY(buf.alloc(off));
+    char *B = buf.as<char>();
     IM_CUDA(cudaMemsetAsync(B + o_ctr, 0, 4 * 8, st));
     IM_CUDA(cudaMemsetAsync(B + o_vis, 0, (size_t)warps * words * 4, st));
     if (k > 0) IM_CUDA(cudaMemcpyAsync(B + o_seeds, seeds, (size_t)k * 4, cudaMemcpyDefault, st));
@@ -509,7 +506,6 @@ extern "C" im_status im_spread(const im_graph *gc, im_model model, const int32_t
     }
     IM_CUDA(cudaGetLastError());
     unsigned long long hc[4] = {0, 0, 0, 0};
-    int32_t *next = nullptr;
     if (pull) {
         IM_CUDA(cudaMemcpyAsync(hc, ctr, sizeof(hc), cudaMemcpyDeviceToHost, st));
         IM_CUDA(cudaStreamSynchronize(st));
@@ -527,8 +523,8 @@ extern "C" im_status im_spread(const im_graph *gc, im_model model, const int32_t
         const size_t need = o_left + (size_t)a.groups * 4 * 8;
         char *N = B + o_q;
         if (need > (size_t)warps * qcap * 4) {
-            IM_TRY(call_alloc((void **)&next, need, st));
-            N = (char *)next;
+            IM_TRY(next.alloc(need));
+            N = next.as<char>();
         }
         a.next = (int32_t *)N;
         a.bars = (GridBarrier *)(N + o_bars);
@@ -542,8 +538,6 @@ extern "C" im_status im_spread(const im_graph *gc, im_model model, const int32_t
     IM_CUDA(cudaMemcpyAsync(hc, ctr, sizeof(hc), cudaMemcpyDeviceToHost, st));
     if (host_act) IM_CUDA(cudaMemcpyAsync(activated, B + o_act, (size_t)runs * 8, cudaMemcpyDeviceToHost, st));
     if (host_hit) IM_CUDA(cudaMemcpyAsync(root_hit, B + o_hit, (size_t)runs, cudaMemcpyDeviceToHost, st));
-    if (next) IM_CUDA(cudaFreeAsync(next, st));
-    IM_CUDA(cudaFreeAsync(B, st));
     IM_CUDA(cudaStreamSynchronize(st));
     (void)host_seeds;
     const int dev_status = (int)(hc[2] & 0xffffffffu);
