@@ -5,9 +5,10 @@
 // Run r simulates the live-edge world of RRR sample r -- the same IC coins
 // and LT picks the sampler uses -- forward from S by a BFS
 // over out-edges (one block per run, level by level, each warp expanding 32
-// queued vertices at a time).  Under LT a run that activates a large part of the
-// graph is finished by k_spread_pull, which draws every vertex's pick once
-// instead of once per in-edge from an activated vertex.
+// queued vertices at a time).  Under LT a run stops where it would pass n / 8
+// out-edges, and goes on from there or, where that is cheaper (pull_pays), is
+// redone by k_spread_pull, which draws every vertex's pick once instead of once
+// per in-edge from an activated vertex.
 //   IC: in-edge e is live iff lane (e & 3) of Philox(r, e >> 2, e >> 34, coin
 //       tag) is below w[e];
 //   LT: in-edge e into v is live iff v's pick draw x = Philox(r, v, 0, pick
@@ -61,9 +62,15 @@ __global__ void k_out_fill(const int64_t *in_off, const int32_t *in_src, const u
     }
 }
 
+// A run that k_spread stopped before a level: the first `tail` vertices it activated
+// are in its row of the lot, the first `head` of them expanded, at the price of
+// `done` out-edges.
+struct Stopped {
+    unsigned long long run, head, tail, done;
+};
+
 struct SpreadArgs {
     int64_t n;
-    int32_t model;
     uint64_t seed;
     uint64_t first;
     int64_t runs;
@@ -80,10 +87,18 @@ struct SpreadArgs {
     int64_t *activated;               // [runs] or null
     uint8_t *root_hit;                // [runs] or null
     int *status;
-    // LT: runs that examined more than `budget` out-edges, for k_spread_pull
+    int64_t first_new;                // work item w is stopped run again + w, and, past them
+    unsigned long long again, nagain; // all (nagain), run first_new + w - nagain
+    // LT: a run that would pass `budget` out-edges with its next level stops before it
     unsigned long long budget;
-    uint32_t *wide;                   // [runs]
-    unsigned long long *nwide;
+    Stopped *list;                    // [list_cap]
+    unsigned long long list_cap;
+    unsigned long long *nlist;        // how many (or more, where runs found no place)
+    int32_t *lot;                     // [list_cap][lot_row], null: a stopped run is not gone on with
+    int64_t lot_row;
+    unsigned long long *pace;         // [2] out-edges of whole levels, and the blocks' ns for them (with a lot)
+    unsigned long long from, to;      // k_spread_pull: the places it finishes
+    unsigned long long *rest;         // ... and the out-edges they had left, or null
     QueryView view;                   // LT: the graph's pick tables
     int32_t *next;                    // [groups][n] k_spread_pull
     GridBarrier *bars;                // [groups]
@@ -93,27 +108,46 @@ struct SpreadArgs {
 
 // One run per block: a level-synchronous BFS whose warps take 32 vertices
 // of the current level at a time and append the vertices they activate to
-// the block's queue (one atomic per warp and step).
-__global__ void __launch_bounds__(kSpreadThreads) k_spread(SpreadArgs a) {
+// the block's queue (one atomic per warp and step).  LT: a run stops between two
+// levels, when those so far and the next have more than a.budget out-edges.
+template <bool LT>
+__global__ void __launch_bounds__(kSpreadThreads) k_spread(const __grid_constant__ SpreadArgs a) {
     __shared__ unsigned long long s_run;
-    __shared__ unsigned long long s_tail, s_cursor, s_work;
+    __shared__ unsigned long long s_tail, s_cursor, s_edges, s_at;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     uint32_t *vis = a.vis + (int64_t)blockIdx.x * a.words;
     int32_t *q = a.queues + (int64_t)blockIdx.x * a.qcap;
     const uint32_t k0 = seed_lo(a.seed), k1 = seed_hi(a.seed);
-    unsigned long long my_total = 0;
+    unsigned long long my_total = 0, my_edges = 0, my_ns = 0;
     for (;;) {
         if (threadIdx.x == 0) {
             s_run = atomicAdd(a.work, 1ull);
             s_tail = 0;
-            s_work = 0;
+            s_edges = 0;
         }
         __syncthreads();
-        const unsigned long long i = s_run;
-        if (i >= (unsigned long long)a.runs) break;
+        unsigned long long i = s_run;
+        long long head = 0;
+        const bool again = LT && i < a.nagain;   // (block-uniform)
+        if (again) {                         // go on with a stopped run
+            const Stopped r = a.list[a.again + i];
+            const int32_t *row = a.lot + (int64_t)(a.again + i) * a.lot_row;
+            for (int64_t x = threadIdx.x; x < (int64_t)r.tail; x += kSpreadThreads) {
+                const int32_t u = row[x];
+                q[x] = u;
+                atomicOr(&vis[u >> 5], 1u << (u & 31));
+            }
+            i = r.run;
+            head = (long long)r.head;
+            if (threadIdx.x == 0) s_tail = r.tail;
+        } else {
+            i = (unsigned long long)a.first_new + (i - a.nagain);
+            if (i >= (unsigned long long)a.runs) break;
+        }
         const uint32_t s = (uint32_t)(a.first + i);
+        const uint64_t t_begin = LT && a.lot ? global_ns() : 0;
         // the seeds, each once
-        if (warp == 0) {
+        if (warp == 0 && !again) {
             for (int32_t b = 0; b < a.k; b += 32) {
                 bool fresh = false;
                 int32_t u = -1;
@@ -135,22 +169,41 @@ __global__ void __launch_bounds__(kSpreadThreads) k_spread(SpreadArgs a) {
             }
         }
         __syncthreads();
-        long long head = 0;
-        bool wide = false;                   // (block-uniform)
+        unsigned long long done = 0;         // out-edges of the levels before this one
+        unsigned long long budget = LT ? a.budget : ~0ull;
+        bool stop = false;                   // (block-uniform)
         for (;;) {
             const long long lvl_end = (long long)s_tail;
-            if (a.wide && s_work > a.budget) {
-                wide = true;
-                break;
-            }
             if (head >= lvl_end) break;
-            __syncthreads();                 // everyone has read s_tail and s_work
+            __syncthreads();                 // everyone has read s_tail
             if (threadIdx.x == 0) s_cursor = (unsigned long long)head;
+            if (LT && budget != ~0ull) {           // the level's out-edges (the expansion finds what this reads in L1)
+                unsigned long long e = 0;
+                for (long long x = head + threadIdx.x; x < lvl_end; x += kSpreadThreads) {
+                    const int32_t u = q[x];
+                    e += (unsigned long long)(a.out_off[u + 1] - a.out_off[u]);
+                }
+                if (__any_sync(kFull, e != 0ull)) {
+                    e = warp_sum<unsigned long long>(e);
+                    if (lane == 0) atomicAdd(&s_edges, e);
+                }
+            }
             __syncthreads();
+            if (LT && budget != ~0ull) {
+                if (s_edges > budget) {      // (the levels' sum so far)
+                    if (threadIdx.x == 0) {
+                        s_at = atomicAdd(a.nlist, 1ull);
+                    }
+                    __syncthreads();
+                    stop = s_at < a.list_cap;
+                    if (stop) break;
+                    budget = ~0ull;          // no place in the list
+                }
+                done = s_edges;
+            }
             for (;;) {
-                long long base = lvl_end;    // over budget: leave the level
-                if (lane == 0 && !(a.wide && *(volatile unsigned long long *)&s_work > a.budget))
-                    base = (long long)atomicAdd(&s_cursor, 32ull);
+                long long base = 0;
+                if (lane == 0) base = (long long)atomicAdd(&s_cursor, 32ull);
                 base = __shfl_sync(kFull, base, 0);
                 if (base >= lvl_end) break;
                 const int nb = (int)(lvl_end - base < 32 ? lvl_end - base : 32);
@@ -163,11 +216,6 @@ __global__ void __launch_bounds__(kSpreadThreads) k_spread(SpreadArgs a) {
                 const int64_t len = oe - ob;
                 const int64_t incl = warp_incl_scan<int64_t>(len, lane);
                 const int64_t total = __shfl_sync(kFull, incl, 31);
-                if (a.wide) {                // over budget: the run is redone by pulling
-                    unsigned long long w = 0;
-                    if (lane == 0) w = atomicAdd(&s_work, (unsigned long long)total) + (unsigned long long)total;
-                    if (__shfl_sync(kFull, w, 0) > a.budget) break;
-                }
                 for (int64_t eb = 0; eb < total; eb += 32) {
                     const int64_t t = eb + lane;
                     int owner = 0;   // first lane whose inclusive count exceeds t
@@ -186,7 +234,7 @@ __global__ void __launch_bounds__(kSpreadThreads) k_spread(SpreadArgs a) {
                         v = r.x;
                         if (!((__ldcg(vis + (v >> 5)) >> (v & 31)) & 1u)) {
                             bool live;
-                            if (a.model == IM_IC) {
+                            if (!LT) {
                                 const uint32_t e = r.y;   // in-CSR id (< 2^31)
                                 const uint4 c = philox4x32_10(
                                     make_uint4(s, e >> 2, 0u, kStreamCoin), k0, k1);
@@ -218,9 +266,19 @@ __global__ void __launch_bounds__(kSpreadThreads) k_spread(SpreadArgs a) {
             head = lvl_end;
         }
         const long long tail = (long long)s_tail;
-        if (wide) {
-            if (threadIdx.x == 0) a.wide[atomicAdd(a.nwide, 1ull)] = (uint32_t)i;
-        } else if (threadIdx.x == 0) {
+        if (LT && a.lot) {
+            my_edges += stop ? done : s_edges;
+            my_ns += global_ns() - t_begin;
+        }
+        if (LT && stop) {
+            if (threadIdx.x == 0)
+                a.list[s_at] = Stopped{i, (unsigned long long)head, (unsigned long long)tail, done};
+            if (a.lot) {
+                int32_t *row = a.lot + (int64_t)s_at * a.lot_row;
+                for (int64_t x = threadIdx.x; x < tail; x += kSpreadThreads) row[x] = q[x];
+            }
+        }
+        if (!stop && threadIdx.x == 0) {
             const uint32_t root = rrr_root(a.seed, s, (uint32_t)a.n);
             const bool hit = (vis[root >> 5] >> (root & 31)) & 1u;
             if (a.activated) a.activated[i] = tail;
@@ -237,6 +295,10 @@ __global__ void __launch_bounds__(kSpreadThreads) k_spread(SpreadArgs a) {
         __syncthreads();
     }
     if (threadIdx.x == 0 && my_total) atomicAdd(a.total, my_total);
+    if (LT && threadIdx.x == 0 && my_edges) {
+        atomicAdd(a.pace, my_edges);
+        atomicAdd(a.pace + 1, my_ns);
+    }
 }
 
 // The source that vertex v picks in sample s (draw x), or -1: the rules of the LT
@@ -282,8 +344,8 @@ __device__ __forceinline__ int32_t lt_pick_source(const QueryView &V, uint32_t v
 // shorten chains, so rounds work in place.
 // n draws and about ten rounds of n gathers in L2 instead of a draw per out-edge
 // of an activated vertex (1.5 x 10^7 of 1.7 x 10^7 at scale 20 from 100 of the
-// largest vertices): 256 runs 79.9 -> 5.3 ms, 0.7 of them the forward pass.  The groups' pointers together stay
-// below kPullBytes, so that the gathers hit L2.
+// largest vertices): a call of 256 runs 76 -> 4.6 ms.  The groups' pointers together
+// stay below kPullBytes, so that the gathers hit L2.
 constexpr int kPullThreads = 1024;
 constexpr int64_t kPullBytes = 64ll << 20;
 constexpr int kPullU = 4;                    // gathers in flight per thread
@@ -294,11 +356,10 @@ __global__ void __launch_bounds__(kPullThreads) k_spread_pull(const __grid_const
     const uint32_t rank = blockIdx.x / a.groups, nb = (gridDim.x - group + a.groups - 1) / a.groups;
     int32_t *next = a.next + (int64_t)group * a.n;
     GridBarrier *bar = a.bars + group;
-    unsigned long long *left = a.left + 4 * group;       // [0], [1] resolved in a round, [2] activated
+    unsigned long long *left = a.left + 4 * group;       // [0], [1] resolved in a round, [2] activated, [3] their out-edges
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int64_t tid = (int64_t)rank * kPullThreads + threadIdx.x, stride = (int64_t)nb * kPullThreads;
     const uint32_t k0 = seed_lo(a.seed), k1 = seed_hi(a.seed);
-    const int64_t nruns = (int64_t)*a.nwide;
     // adds the block's counts to *to
     auto block_add = [&](unsigned int mine, unsigned long long *to) {
         mine = __reduce_add_sync(kFull, mine);
@@ -310,15 +371,15 @@ __global__ void __launch_bounds__(kPullThreads) k_spread_pull(const __grid_const
         }
         __syncthreads();
     };
-    for (int64_t i = group; i < nruns; i += a.groups) {
-        const uint32_t run = a.wide[i];
+    for (unsigned long long i = a.from + group; i < a.to; i += a.groups) {
+        const unsigned long long run = a.list[i].run;
         const uint32_t s = (uint32_t)(a.first + run);
         for (int64_t v = tid; v < a.n; v += stride) {
             const int32_t u = lt_pick_source(
                 a.view, (uint32_t)v, philox4x32_10(make_uint4(s, (uint32_t)v, 0u, kStreamPick), k0, k1).x);
             next[v] = u >= 0 ? u : -2;
         }
-        if (tid == 0) left[0] = left[1] = left[2] = 0ull;
+        if (tid == 0) left[0] = left[1] = left[2] = left[3] = 0ull;
         if (!grid_sync(bar, nb, a.status)) return;
         for (int64_t b = tid; b < a.k; b += stride) next[a.seeds[b]] = -1;
         if (!grid_sync(bar, nb, a.status)) return;
@@ -349,8 +410,17 @@ __global__ void __launch_bounds__(kPullThreads) k_spread_pull(const __grid_const
             if (!grid_sync(bar, nb, a.status)) return;
         }
         unsigned int act = 0;
-        for (int64_t v = tid; v < a.n; v += stride) act += __ldcg(next + v) == -1;
+        unsigned long long edges = 0;
+        for (int64_t v = tid; v < a.n; v += stride)
+            if (__ldcg(next + v) == -1) {
+                ++act;
+                if (a.rest) edges += (unsigned long long)(a.out_off[v + 1] - a.out_off[v]);
+            }
         block_add(act, left + 2);
+        if (a.rest) {
+            edges = warp_sum<unsigned long long>(edges);
+            if (lane == 0 && edges) atomicAdd(left + 3, edges);
+        }
         if (!grid_sync(bar, nb, a.status)) return;
         if (tid == 0) {
             const unsigned long long t = *(volatile unsigned long long *)(left + 2);
@@ -358,9 +428,43 @@ __global__ void __launch_bounds__(kPullThreads) k_spread_pull(const __grid_const
             if (a.activated) a.activated[run] = (int64_t)t;
             if (a.root_hit) a.root_hit[run] = __ldcg(next + root) == -1 ? 1 : 0;
             atomicAdd(a.total, t);
+            if (a.rest) a.rest[i] = *(volatile unsigned long long *)(left + 3) - a.list[i].done;
         }
         if (!grid_sync(bar, nb, a.status)) return;       // before next and left are rewritten
     }
+}
+
+constexpr int64_t kPullList = 1 << 20;        // runs listed to be pulled at most
+
+// Whether `count` stopped runs cost less to pull than to push to their end, from the
+// out-edges `rest` that the first of them turned out to have left (the runs of a call
+// differ in their random worlds alone) and the pace (out-edges, ns) of the blocks.
+// Neither n, m nor a run's past tells: stopped before 131,072 out-edges at scale 20,
+// runs from 100 of the largest vertices have 1.4 x 10^7 left at 16 out-edges a vertex,
+// and 2.5 x 10^5 at 2 and U[0, 0.1] weights, where pulling all of 3,000 runs took 60
+// ms and pushing them takes 34.
+//   pulling  1 us + 16 ps a vertex of the whole GPU a run (17 us at scale 20; pointers
+//            beyond the L2 cache are gathered from DRAM, at a sixteenth of the rate),
+//            and 100 us for the launch;
+//   pushing  at the blocks' pace, at most 6 x 10^10 out-edges a second together, and
+//            the longest run at a block's.  That lies between a warp's, 2.4 x 10^7 (it
+//            expands a hub, and any 32 vertices, alone), and 3 x 10^8.  Where nothing was
+//            measured, every run having stopped at its first level, it is that of the
+//            warps which that level (run `one`) keeps busy.  The longest run slows
+//            down by half as it comes to the hubs.
+bool pull_pays(const std::vector<unsigned long long> &rest, double count, int64_t n,
+               const unsigned long long *pace, const Stopped &one, int64_t blocks) {
+    double sum = 0.0, most = 0.0;
+    for (const unsigned long long r : rest) {
+        sum += (double)r;
+        most = std::max(most, (double)r);
+    }
+    const double block = pace[1] ? (double)pace[0] * 1e9 / (double)pace[1]         // out-edges a second
+                                 : std::min(3e8, 2.4e7 * (double)((one.tail - one.head + 31) / 32));
+    const double push = std::max(count * sum / (double)rest.size() / std::min(6e10, block * (double)blocks),
+                                 1.5 * most / block);
+    const double pull = 1e-4 + count * (1e-6 + 16e-12 * (double)n * (n * 4 <= kPullBytes ? 1.0 : 16.0));
+    return pull < push;
 }
 
 std::mutex g_out_index_mu;   // graphs are shared between threads
@@ -441,17 +545,33 @@ extern "C" im_status im_spread(const im_graph *gc, im_model model, const int32_t
     // blocks (one run each at a time): occupancy-sized, and the per-block
     // queue (n entries) and bitmap within about 2 GB
     int per_sm = 0;
-    IM_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_spread, kSpreadThreads, 0));
-    const bool pull = model == IM_LT;
-    // LT: out-edges from which drawing all n picks is the cheaper way; a run
-    // examines no more of them here, so its queue holds no more either
+    const void *kern = model == IM_LT ? (const void *)k_spread<true> : (const void *)k_spread<false>;
+    IM_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kSpreadThreads, 0));
+    // LT: runs stop here before they pass this many out-edges (see pull_pays)
     const int64_t budget = std::max<int64_t>(n / 8, 1 << 16);
-    const int64_t qcap = pull ? std::min<int64_t>(n, budget + k) : n;
-    const int64_t per_block = qcap * 4 + words * 4;
+    bool pull = model == IM_LT && g->m > budget;
+    int pull_grid = 0;
+    if (pull) {
+        int per = 0;
+        IM_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_spread_pull, kPullThreads, 0));
+        pull_grid = per * num_sms();
+        pull = per > 0;
+    }
+    const int64_t per_block = n * 4 + words * 4;
     int64_t blocks = std::max(1, per_sm) * (int64_t)num_sms();
     blocks = std::min<int64_t>(blocks, std::max<int64_t>(1, (2ll << 30) / per_block));
     blocks = std::min<int64_t>(blocks, (int64_t)runs);
-    const int64_t warps = blocks;   // one visited bitmap and queue per block
+    const int64_t groups = std::max<int64_t>(
+        1, std::min<int64_t>({blocks, (int64_t)pull_grid / 4, kPullBytes / (n * 4)}));
+    // LT: the runs that find room in a lot of 1 GB if they stop, which tell how to go on
+    // with the others; what a run activates before it stops is bounded by the budget
+    const int64_t lot_row = std::min<int64_t>(n, budget + k);
+    int64_t head_runs = std::min<int64_t>((int64_t)runs, std::max<int64_t>(1, (1ll << 30) / (lot_row * 4)));
+    CallBuf lot(st);
+    if (pull && lot.alloc((size_t)head_runs * lot_row * 4) != IM_OK) pull = false;
+    if (!pull) head_runs = (int64_t)runs;
+    const int64_t list = pull ? std::max(head_runs, std::min<int64_t>((int64_t)runs - head_runs, kPullList)) : 0;
+    const int64_t qcap = pull ? lot_row : n;
     const bool host_act = activated && !is_device_ptr(activated);
     const bool host_hit = root_hit && !is_device_ptr(root_hit);
     const bool host_seeds = k > 0 && !is_device_ptr(seeds);
@@ -461,23 +581,25 @@ extern "C" im_status im_spread(const im_graph *gc, im_model model, const int32_t
         off += (bytes + 255) & ~(size_t)255;
         return at;
     };
-    const size_t o_wide = take(pull ? (size_t)runs * 4 : 0);
-    const size_t o_ctr = take(4 * 8), o_seeds = take((size_t)std::max(k, 1) * 4),
-                 o_vis = take((size_t)warps * words * 4), o_q = take((size_t)warps * qcap * 4),
+    const size_t o_ctr = take(6 * 8), o_seeds = take((size_t)std::max(k, 1) * 4),
+                 o_vis = take((size_t)blocks * words * 4), o_q = take((size_t)blocks * qcap * 4),
                  o_act = take(host_act ? (size_t)runs * 8 : 0),
-                 o_hit = take(host_hit ? (size_t)runs : 0);
-    CallBuf buf(st), next(st);
+                 o_hit = take(host_hit ? (size_t)runs : 0),
+                 o_list = take((size_t)list * sizeof(Stopped)),
+                 o_rest = take(pull ? (size_t)groups * 8 : 0),
+                 o_bars = take(pull ? (size_t)groups * sizeof(GridBarrier) : 0),
+                 o_left = take(pull ? (size_t)groups * 4 * 8 : 0);
+    CallBuf buf(st), next(st), queues(st);
     IM_TRY(buf.alloc(off));
     char *B = buf.as<char>();
-    IM_CUDA(cudaMemsetAsync(B + o_ctr, 0, 4 * 8, st));
-    IM_CUDA(cudaMemsetAsync(B + o_vis, 0, (size_t)warps * words * 4, st));
+    IM_CUDA(cudaMemsetAsync(B + o_ctr, 0, 6 * 8, st));
+    IM_CUDA(cudaMemsetAsync(B + o_vis, 0, (size_t)blocks * words * 4, st));
     if (k > 0) IM_CUDA(cudaMemcpyAsync(B + o_seeds, seeds, (size_t)k * 4, cudaMemcpyDefault, st));
     SpreadArgs a;
     a.n = n;
-    a.model = model;
     a.seed = seed;
     a.first = first_run;
-    a.runs = (int64_t)runs;
+    a.runs = head_runs;
     a.seeds = (const int32_t *)(B + o_seeds);
     a.k = k;
     a.out_off = g->out_off;
@@ -485,55 +607,109 @@ extern "C" im_status im_spread(const im_graph *gc, im_model model, const int32_t
     a.vis = (uint32_t *)(B + o_vis);
     a.words = words;
     a.queues = (int32_t *)(B + o_q);
+    a.qcap = qcap;
     unsigned long long *ctr = (unsigned long long *)(B + o_ctr);
     a.work = ctr;
     a.total = ctr + 1;
     a.status = (int *)(ctr + 2);
-    a.nwide = ctr + 3;
-    a.wide = pull ? (uint32_t *)(B + o_wide) : nullptr;
-    a.budget = (unsigned long long)budget;
-    a.qcap = qcap;
+    a.nlist = ctr + 3;
+    a.pace = ctr + 4;
+    a.first_new = 0;
+    a.again = a.nagain = 0;
+    a.budget = pull ? (unsigned long long)budget : ~0ull;
+    a.list = (Stopped *)(B + o_list);
+    a.list_cap = (unsigned long long)head_runs;
+    a.lot = pull ? lot.as<int32_t>() : nullptr;
+    a.lot_row = lot_row;
+    a.from = a.to = 0;
+    a.rest = nullptr;
     a.view = query_view(g, seed, first_run);
     a.next = nullptr;
-    a.bars = nullptr;
-    a.left = nullptr;
+    a.bars = (GridBarrier *)(B + o_bars);
+    a.left = (unsigned long long *)(B + o_left);
     a.groups = 0;
     a.activated = host_act ? (int64_t *)(B + o_act) : activated;
     a.root_hit = host_hit ? (uint8_t *)(B + o_hit) : root_hit;
-    {
-        KernelTimer kt(st, model == IM_LT ? "spread_lt" : "spread_ic");
-        k_spread<<<(unsigned)blocks, kSpreadThreads, 0, st>>>(a);
-    }
-    IM_CUDA(cudaGetLastError());
-    unsigned long long hc[4] = {0, 0, 0, 0};
-    if (pull) {
-        IM_CUDA(cudaMemcpyAsync(hc, ctr, sizeof(hc), cudaMemcpyDeviceToHost, st));
-        IM_CUDA(cudaStreamSynchronize(st));
-    }
-    if (hc[3] > 0 && (int)(hc[2] & 0xffffffffu) == kDevOk) {
-        int per = 0;
-        IM_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_spread_pull, kPullThreads, 0));
-        if (per < 1) return IM_ERR_UNSUPPORTED;
-        const int grid = per * num_sms();
-        a.groups = (int32_t)std::max<int64_t>(
-            1, std::min<int64_t>({(int64_t)hc[3], (int64_t)grid / 4, kPullBytes / (n * 4)}));
-        // the forward pass's queues are free by now
-        const size_t o_bars = ((size_t)a.groups * n * 4 + 255) & ~(size_t)255;
-        const size_t o_left = o_bars + (((size_t)a.groups * sizeof(GridBarrier) + 255) & ~(size_t)255);
-        const size_t need = o_left + (size_t)a.groups * 4 * 8;
-        char *N = B + o_q;
-        if (need > (size_t)warps * qcap * 4) {
-            IM_TRY(next.alloc(need));
-            N = next.as<char>();
-        }
-        a.next = (int32_t *)N;
-        a.bars = (GridBarrier *)(N + o_bars);
-        a.left = (unsigned long long *)(N + o_left);
-        IM_CUDA(cudaMemsetAsync(N + o_bars, 0, need - o_bars, st));
+    unsigned long long hc[6] = {0, 0, 0, 0, 0, 0};
+    auto pull_runs = [&](unsigned long long from, unsigned long long to, unsigned long long *rest) -> im_status {
+        a.from = from;
+        a.to = to;
+        a.rest = rest;
+        a.groups = (int32_t)std::min<unsigned long long>(groups, to - from);
+        IM_CUDA(cudaMemsetAsync(B + o_bars, 0, (size_t)groups * sizeof(GridBarrier), st));
         void *args[] = {&a};
         KernelTimer kt(st, "spread_lt");
-        IM_CUDA(cudaLaunchCooperativeKernel((const void *)k_spread_pull, dim3(grid),
+        IM_CUDA(cudaLaunchCooperativeKernel((const void *)k_spread_pull, dim3(pull_grid),
                                             dim3(kPullThreads), args, 0, st));
+        return IM_OK;
+    };
+    auto push_runs = [&]() -> im_status {
+        KernelTimer kt(st, model == IM_LT ? "spread_lt" : "spread_ic");
+        if (model == IM_LT) k_spread<true><<<(unsigned)blocks, kSpreadThreads, 0, st>>>(a);
+        else k_spread<false><<<(unsigned)blocks, kSpreadThreads, 0, st>>>(a);
+        IM_CUDA(cudaGetLastError());
+        return IM_OK;
+    };
+    auto read_counters = [&]() -> im_status {
+        IM_CUDA(cudaMemcpyAsync(hc, ctr, sizeof(hc), cudaMemcpyDeviceToHost, st));
+        IM_CUDA(cudaStreamSynchronize(st));
+        return IM_OK;
+    };
+    auto dev_ok = [&] { return (int)(hc[2] & 0xffffffffu) == kDevOk; };
+    IM_TRY(push_runs());
+    if (pull) {
+        IM_TRY(read_counters());
+        const unsigned long long stopped = hc[3];        // (every one has its place in the list)
+        const int64_t later = (int64_t)runs - head_runs;
+        if (dev_ok() && (stopped > 0 || later > 0)) {
+            // the first of them are pulled in any case (no room for their pointers: none is)
+            unsigned long long pulled = 0;
+            bool push = next.alloc((size_t)groups * n * 4) != IM_OK;
+            a.next = next.as<int32_t>();
+            if (stopped > 0 && !push) {
+                pulled = std::min<unsigned long long>(stopped, groups);
+                IM_TRY(pull_runs(0, pulled, (unsigned long long *)(B + o_rest)));
+                if (later > 0 || stopped > 2 * pulled) {
+                    std::vector<unsigned long long> rest(pulled);
+                    IM_CUDA(cudaMemcpyAsync(rest.data(), B + o_rest, pulled * 8, cudaMemcpyDeviceToHost, st));
+                    Stopped one;
+                    IM_CUDA(cudaMemcpyAsync(&one, a.list, sizeof(one), cudaMemcpyDeviceToHost, st));
+                    IM_CUDA(cudaStreamSynchronize(st));
+                    const double count = (double)(stopped - pulled) + (double)stopped * later / head_runs;
+                    push = !pull_pays(rest, count, n, hc + 4, one, blocks);
+                }
+                if (!push && stopped > pulled) {
+                    IM_TRY(pull_runs(pulled, stopped, nullptr));
+                    pulled = stopped;
+                }
+            }
+            if (pulled < stopped || later > 0) {
+                // push on the runs that still wait, then the later ones: to their end,
+                // or until they stop (for good, to be pulled)
+                IM_CUDA(cudaMemsetAsync(a.work, 0, 8, st));
+                IM_CUDA(cudaMemsetAsync(a.nlist, 0, 8, st));
+                a.again = pulled;
+                a.nagain = stopped - pulled;
+                a.first_new = head_runs;
+                a.runs = (int64_t)runs;
+                if (push) a.budget = ~0ull;
+                else a.lot = nullptr;
+                a.list_cap = (unsigned long long)list;
+                if (push || later > list) {              // runs that do not stop
+                    while (queues.alloc((size_t)blocks * n * 4) != IM_OK) {
+                        if (blocks == 1) return IM_ERR_OOM;
+                        blocks /= 2;
+                    }
+                    a.queues = queues.as<int32_t>();
+                    a.qcap = n;
+                }
+                IM_TRY(push_runs());
+                if (!push) {
+                    IM_TRY(read_counters());
+                    if (hc[3] > 0 && dev_ok()) IM_TRY(pull_runs(0, std::min(hc[3], a.list_cap), nullptr));
+                }
+            }
+        }
     }
     IM_CUDA(cudaMemcpyAsync(hc, ctr, sizeof(hc), cudaMemcpyDeviceToHost, st));
     if (host_act) IM_CUDA(cudaMemcpyAsync(activated, B + o_act, (size_t)runs * 8, cudaMemcpyDeviceToHost, st));
