@@ -505,8 +505,9 @@ im_status im_solve_batch(im_batch *b, const im_query *q, int32_t nq, int32_t kma
  * graph and model; a worker with nothing in flight always admits one), run
  * them through im_solve_batch and publish the results.  Requests arriving
  * while batches run join the next batch (one alone in the queue waits up to 3
- * ms for others then); with workers > 1 batches overlap on the device.  Every
- * result equals the query's result alone. */
+ * ms for others while a request of the heavy lane is being sampled); with
+ * workers > 1 batches overlap on the device.  Every result equals the query's
+ * result alone. */
 typedef struct {
     int32_t workers;          /* batches in flight at once, 1..16 */
     int32_t max_batch;        /* requests per batch, >= 1 */

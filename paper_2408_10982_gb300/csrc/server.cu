@@ -32,10 +32,7 @@ namespace {
 
 using Clock = std::chrono::steady_clock;
 
-// How long a request that is alone in the queue waits for company while other
-// batches run (not when the device is idle).  A query of the batched mix takes
-// 1 to 10 ms by itself; at 200 such requests a second, p50 and p99 with and
-// without the wait are equal within their spread (5.2 and 31 ms).
+// How long a request waits at most for company while the heavy lane samples.
 constexpr std::chrono::milliseconds kGather(3);
 
 struct Request {
@@ -66,6 +63,7 @@ struct im_server {
     int32_t in_flight = 0;
     uint64_t next_ticket = 1;
     bool stop = false;
+    bool heavy_sampling = false;   // the heavy lane runs its sampling kernels
     // counters
     int64_t batches = 0, batched_queries = 0;
 };
@@ -95,11 +93,20 @@ double est_members(im_server *s, const im_query &q) {
     return (double)q.theta * per;
 }
 
+// Whether the heavy lane is in its sampling kernels (see worker_main).
+void set_sampling(im_server *s, bool on) {
+    {
+        std::lock_guard<std::mutex> lk(s->mu);
+        s->heavy_sampling = on;
+    }
+    if (!on) s->cv_work.notify_all();
+}
+
 // A heavy request on its own, as im_sample_rrr + im_max_k_cover on a pool of
 // its graph and model that worker 0 keeps between requests (recreated larger
 // when theta or the members outgrow it).  For one large query this is the
 // library's fastest path: the per-query kernels, the whole GPU.
-im_status solve_alone(std::map<std::pair<const im_graph *, int32_t>, im_pool *> &pools,
+im_status solve_alone(im_server *s, std::map<std::pair<const im_graph *, int32_t>, im_pool *> &pools,
                       const im_query &q, int64_t want_entries, int32_t *seeds, im_result *res,
                       cudaStream_t st) {
     im_pool *&p = pools[{q.graph, q.model}];
@@ -116,7 +123,9 @@ im_status solve_alone(std::map<std::pair<const im_graph *, int32_t>, im_pool *> 
         }
         r = im_pool_reset(p);
         if (r != IM_OK) return r;
+        set_sampling(s, true);
         r = im_sample_rrr(q.graph, (im_model)q.model, q.seed, 0, (uint64_t)q.theta, p, st);
+        set_sampling(s, false);
         if (r != IM_ERR_CAPACITY) break;
         want_entries *= 4;                        // the sets were larger than estimated
     }
@@ -157,23 +166,25 @@ void worker_main(im_server *s, int32_t wid) {
         });
         // stop requested and nothing left for this worker (worker 0 drains the heavy lane)
         if (first_mine() == s->queue.end()) break;
-        // a single request while other batches have the device: it shares the GPU
-        // with them either way, so it waits a moment for others to share its
-        // launches (another worker may take it meanwhile)
+        // The heavy lane's sampling kernels are persistent and hold most of every SM,
+        // so a batch that starts meanwhile mostly stands behind them: a single
+        // request waits for others to share its launches instead, until they have
+        // ended or for kGather (another worker may take it).  Nothing else is
+        // waited for, and nothing without a heavy lane.  256 requests at 200/s, three
+        // workers with the lane, the 80 smallest: mean 5.8 ms, median 4.8, 253
+        // batches; with no wait 5.6, 4.0 and 255 or 256; waiting for any batch,
+        // lane or not, 6.1, 5.0 and 252.
         auto waiting = [&]() {
             int32_t c = 0;
-            for (const uint64_t t : s->queue) {
-                const Request &r = s->reqs[t];
-                if (any && r.heavy && s->opts.heavy_members > 0) return 2;   // not batched
-                c += any || !r.heavy;
-                if (c >= 2) break;
-            }
+            for (const uint64_t t : s->queue)
+                if ((c += !s->reqs[t].heavy) > 1) break;
             return c;
         };
-        if (s->opts.max_batch > 1 && s->in_flight > 0 && !s->stop && waiting() == 1) {
-            s->cv_work.wait_for(lk, kGather, [&] {
-                return s->stop || s->in_flight == 0 || waiting() != 1;
-            });
+        auto alone_behind_heavy = [&] {
+            return !any && s->heavy_sampling && !s->stop && waiting() == 1;
+        };
+        if (s->opts.max_batch > 1 && alone_behind_heavy()) {
+            s->cv_work.wait_for(lk, kGather, [&] { return !alone_behind_heavy(); });
             const auto it = first_mine();
             if (it == s->queue.end()) continue;
             if (s->in_flight > 0 && s->mem_in_use + s->reqs[*it].footprint > s->opts.mem_budget)
@@ -219,7 +230,7 @@ void worker_main(im_server *s, int32_t wid) {
         std::vector<int32_t> seeds((size_t)qs.size() * kmax);
         std::vector<im_result> res(qs.size());
         const im_status st_batch =
-            alone ? solve_alone(pools, qs[0], want_entries, seeds.data(), res.data(), st)
+            alone ? solve_alone(s, pools, qs[0], want_entries, seeds.data(), res.data(), st)
                   : im_solve_batch(b, qs.data(), (int32_t)qs.size(), kmax, seeds.data(), nullptr,
                                    res.data(), st);
         const std::string err = st_batch == IM_OK ? std::string() : std::string(im_last_error());
