@@ -40,14 +40,18 @@ constexpr int kWarpSortKeys = 1024;          // sets up to this length are sorte
 constexpr int64_t kStageAscending = (int64_t)1 << 62;
 constexpr int kBlockSortCap = 16384;         // ... by one block in shared memory (int32)
 
-// An IC sample that a warp gave up: its members so far are hand[off .. off +
-// tail), of which the first `head` are expanded (examined in-edges so far);
-// off < 0: start again from the root.
+// An IC sample that a warp handed over: its members so far are hand[off .. off +
+// tail), of which the first `head` are expanded (examined in-edges so far).  tail is
+// at least kICWarpFront, so that off / kICWarpFront is a place of its own in the
+// table, and the table is as long as the buffer of members allows, whatever the
+// number of samples.  The entry in ovf_list is the sample's index, with that
+// place + 1 in the bits from kHandedShift on; 0 there: start again from the root.
 struct Handed {
     int64_t off;
     unsigned long long examined;
     int32_t head, tail;
 };
+constexpr int kHandedShift = 44;
 
 struct SampleArgs {
     const QueryView *qv;      // [nq] graphs and streams of the queries of this launch
@@ -70,7 +74,7 @@ struct SampleArgs {
     int64_t *ovf_list;
     unsigned long long *ovf_count;
     int *status;
-    struct Handed *handed;    // [count] state of the samples in ovf_list (IC)
+    struct Handed *handed;    // [hand_cap / kICWarpFront + 1] state of handed-over samples (IC)
     int32_t *hand;            // their members
     int64_t hand_cap;
     unsigned long long *hand_cursor;
@@ -506,8 +510,13 @@ __global__ void __launch_bounds__(kSampleThreads, 3) k_sample_ic(const __grid_co
                 a.sizes[j] = -1;
                 a.stage_off[j] = 0;
                 const unsigned long long at = atomicAdd(a.ovf_count, 1ull);
-                a.ovf_list[at] = j;
-                a.handed[at] = Handed{(int64_t)off, ex, head, tail};
+                if (off != ~0ull) {
+                    const int64_t place = (int64_t)off / kICWarpFront;
+                    a.handed[place] = Handed{(int64_t)off, ex, head, tail};
+                    a.ovf_list[at] = j | (place + 1) << kHandedShift;
+                } else {
+                    a.ovf_list[at] = j;
+                }
             }
         } else {
             unsigned long long pos = 0;
@@ -590,7 +599,8 @@ __global__ void __launch_bounds__(kICBigThreads) k_sample_ic_big(const __grid_co
         __syncthreads();
         const unsigned long long jw = s_item;
         if (jw >= (unsigned long long)a.count) break;
-        const int64_t j = a.list ? a.list[jw] : (int64_t)jw;
+        const int64_t entry = a.list[jw];
+        const int64_t j = entry & (((int64_t)1 << kHandedShift) - 1), place = (entry >> kHandedShift) - 1;
         const int qi = find_query(a, j);
         const QueryView &V = a.qv[qi];
         const uint4 *rec = V.ic_rec;
@@ -601,8 +611,8 @@ __global__ void __launch_bounds__(kICBigThreads) k_sample_ic_big(const __grid_co
         cs.begin(a.rk, s, seed_lo(V.seed), seed_hi(V.seed));
         unsigned long long sexam = 0;
         unsigned int head = 0;
-        const Handed hd = a.handed[jw];
-        if (hd.off >= 0) {                   // go on where the warp stopped
+        if (place >= 0) {                    // go on where the warp stopped
+            const Handed hd = a.handed[place];
             for (int32_t x = threadIdx.x; x < hd.tail; x += kICBigThreads) {
                 const int32_t u = a.hand[hd.off + x];
                 q[x] = u;
@@ -2282,8 +2292,8 @@ im_status run_sampling(const SamplingJob &job, const std::function<im_status(siz
     const size_t o_ovf = take((size_t)cnt * 8);
     const size_t o_scan = take(scan_tmp_bytes(cnt));
     const size_t o_sort = take((size_t)(2 + 2 * cnt) * 8);
-    const size_t o_handed = take(model == IM_IC ? (size_t)cnt * sizeof(Handed) : 0);
     const int64_t hand_cap = model == IM_IC ? std::min<int64_t>(kICHandCap, cnt * qcap) : 0;
+    const size_t o_handed = take(model == IM_IC ? (size_t)(hand_cap / kICWarpFront + 1) * sizeof(Handed) : 0);
     const size_t o_hand = take((size_t)hand_cap * 4);
     const size_t o_recs = take(lt1 ? (size_t)slots * kLT1Recs * sizeof(uint2) : 0);
     const size_t o_q = take((size_t)slots * qcap * 4);
