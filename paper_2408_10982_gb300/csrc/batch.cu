@@ -263,6 +263,9 @@ im_status im_solve_batch(im_batch *b, const im_query *qs, int32_t nq, int32_t km
     }
     qset[nq] = sb;
     const int64_t cov_words = std::max<int64_t>(cb, 1);
+    std::vector<int64_t> greedy_n;                   // vertices of the queries of greedy_many
+    for (int32_t q = 0; q < nq; ++q)
+        if (qs[q].cover.algo != IM_RANDGREEDI) greedy_n.push_back(qs[q].graph->n);
 
     for (int attempt = 0; attempt < 8; ++attempt) {
         int64_t cap = 1024;
@@ -290,7 +293,7 @@ im_status im_solve_batch(im_batch *b, const im_query *qs, int32_t nq, int32_t km
                      o_out = take(up256((size_t)nq * kmax * 4) + up256((size_t)nq * kmax * 8) +
                                   up256((size_t)nq * 4) + up256((size_t)nq * 8)),
                      o_bounds = take((size_t)(nq + 1) * 8),
-                     o_many = take(greedy_many_scratch(nq, cap)), o_gbar = take(256);
+                     o_many = take(greedy_many_scratch(greedy_n, cap)), o_gbar = take(256);
         im_status s = grow(&b->arena, &b->arena_bytes, off);
         if (s != IM_OK) return s;
         char *A = (char *)b->arena;

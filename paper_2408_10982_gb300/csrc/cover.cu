@@ -1619,8 +1619,9 @@ im_status greedy_launch(int64_t n, int64_t theta, const int64_t *set_off, const 
     return IM_OK;
 }
 
-// Queries of a batch: scratch of greedy_many for nq queries of `members` members
-// in all (its own arrays; counts, ranks and candidates come with the queries).
+// Queries of a batch: scratch of greedy_many for queries of n[] vertices and
+// `members` members in all (its own arrays; counts, ranks and candidates come with
+// the queries).
 constexpr int32_t kManyHubs = 1024;     // hub rows of a query at most
 
 namespace {
@@ -1632,11 +1633,18 @@ struct ManyState {                      // zeroed before the launch
 size_t many_pieces(int64_t members) { return (size_t)(2 * members / kGreedyPiece + 1); }
 }  // namespace
 
-size_t greedy_many_scratch(int32_t nq, int64_t members) {
-    return align256((size_t)nq * sizeof(GreedyArgs)) + align256((size_t)(nq + 1) * 4) +
-           align256((size_t)nq * sizeof(ManyState)) +
-           align256((size_t)nq * kManyHubs * kHubRep * 4) + align256((size_t)nq * kManyHubs * 4) +
-           align256((many_pieces(members) + (size_t)nq) * 8);
+int64_t greedy_hub_rows(int64_t n) { return std::min<int64_t>(n, kManyHubs); }
+
+size_t greedy_query_bytes(int64_t n) {
+    return sizeof(GreedyArgs) + 4 + sizeof(ManyState) + (size_t)greedy_hub_rows(n) * (kHubRep + 1) * 4 + 8;
+}
+
+size_t greedy_many_scratch(const std::vector<int64_t> &n, int64_t members) {
+    size_t rows = 0;
+    for (const int64_t x : n) rows += (size_t)greedy_hub_rows(x);
+    const size_t nq = n.size();
+    return align256(nq * sizeof(GreedyArgs)) + align256((nq + 1) * 4) + align256(nq * sizeof(ManyState)) +
+           align256(rows * kHubRep * 4) + align256(rows * 4) + align256((many_pieces(members) + nq) * 8);
 }
 
 im_status greedy_many(const std::vector<GreedyQuery> &qs, const int64_t *set_off,
@@ -1649,7 +1657,11 @@ im_status greedy_many(const std::vector<GreedyQuery> &qs, const int64_t *set_off
     if (per_sm < 1) return IM_ERR_UNSUPPORTED;
     const int grid = std::min(per_sm, 2) * num_sms();
     int64_t total = 0;
-    for (const GreedyQuery &q : qs) total += q.members;
+    size_t rows = 0;
+    for (const GreedyQuery &q : qs) {
+        total += q.members;
+        rows += (size_t)greedy_hub_rows(q.n);
+    }
     char *B = (char *)scratch;
     auto take = [&](size_t bytes) {
         char *r = B;
@@ -1659,8 +1671,8 @@ im_status greedy_many(const std::vector<GreedyQuery> &qs, const int64_t *set_off
     GreedyArgs *tab = (GreedyArgs *)take((size_t)nq * sizeof(GreedyArgs));
     int32_t *first = (int32_t *)take((size_t)(nq + 1) * 4);
     ManyState *state = (ManyState *)take((size_t)nq * sizeof(ManyState));
-    int32_t *hub_cnt = (int32_t *)take((size_t)nq * kManyHubs * kHubRep * 4);
-    int32_t *hub_list = (int32_t *)take((size_t)nq * kManyHubs * 4);
+    int32_t *hub_cnt = (int32_t *)take(rows * kHubRep * 4);
+    int32_t *hub_list = (int32_t *)take(rows * 4);
     unsigned long long *piece = (unsigned long long *)take((many_pieces(total) + (size_t)nq) * 8);
 
     // largest first; blocks by weight: the members a query may decrement, and a
@@ -1686,7 +1698,7 @@ im_status greedy_many(const std::vector<GreedyQuery> &qs, const int64_t *set_off
 
     const int32_t cand_shift = (int32_t)tune_value(IM_TUNE_GREEDY_HOT);
     std::vector<GreedyArgs> h(nq);
-    size_t at = 0;
+    size_t at = 0, row = 0;
     for (int32_t r = 0; r < nq; ++r) {
         const GreedyQuery &q = qs[order[r]];
         GreedyArgs &a = h[r];
@@ -1710,11 +1722,12 @@ im_status greedy_many(const std::vector<GreedyQuery> &qs, const int64_t *set_off
         a.sshift = q.sshift;
         a.vshift = q.vshift;
         a.hub_rank = q.ranks;
-        a.hub_cnt = hub_cnt + (size_t)r * kManyHubs * kHubRep;
-        a.hub_list = hub_list + (size_t)r * kManyHubs;
+        a.hub_cnt = hub_cnt + row * kHubRep;
+        a.hub_list = hub_list + row;
         a.cand = q.cands;
         a.ctl = state[r].ctl;
-        a.hub_cap = kManyHubs;
+        a.hub_cap = (int32_t)greedy_hub_rows(q.n);
+        row += (size_t)a.hub_cap;
         a.hub_shift = kHubShift;
         a.cand_shift = cand_shift;
         a.work = state[r].work;

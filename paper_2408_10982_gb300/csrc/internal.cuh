@@ -479,7 +479,8 @@ struct GreedyQuery {
     int32_t *nseeds;
     int64_t *coverage;
 };
-size_t greedy_many_scratch(int32_t nq, int64_t members);
+size_t greedy_many_scratch(const std::vector<int64_t> &n, int64_t members);   // n: the queries' vertices
+size_t greedy_query_bytes(int64_t n);                                         // ... a query's own part
 im_status greedy_many(const std::vector<GreedyQuery> &qs, const int64_t *set_off,
                       const int32_t *members, const int32_t *set_ids, void *scratch, int *status,
                       cudaStream_t st);

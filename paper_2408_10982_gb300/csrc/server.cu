@@ -71,9 +71,9 @@ struct im_server {
 namespace {
 
 // device bytes a request needs inside a batch: stage + members + covering
-// subsets (12 B per member) and the buffers of their sort (12 B), set offsets
-// and sizes (20 B per set), the covered bitmap, and per-vertex greedy state
-// (24 B per vertex)
+// subsets (12 B per member) and the buffers and digit tables of their sort (12 and
+// up to 1.5 B), set offsets and sizes (20 B per set), the covered bitmap,
+// per-vertex greedy state (24 B per vertex) and the greedy's rows
 int64_t footprint(im_server *s, const im_query &q) {
     auto it = s->per_set.find({q.graph, q.model});
     const double per = it != s->per_set.end() ? it->second : 64.0;
@@ -82,8 +82,9 @@ int64_t footprint(im_server *s, const im_query &q) {
         const int64_t P = q.cover.partitions > 0 ? q.cover.partitions : 148;
         rg = P * ((q.theta + 31) / 32) * 4 + q.theta * 8 + q.graph->n * 16;
     }
-    return (int64_t)((double)q.theta * per * 1.5 * 24.0) + q.theta * 20 + q.theta / 8 +
-           q.graph->n * 24 + rg + 4096;
+    return (int64_t)((double)q.theta * per * 1.5 * 25.5) + q.theta * 20 + q.theta / 8 +
+           q.graph->n * 24 + rg + 4096 +
+           (q.cover.algo == IM_RANDGREEDI ? 0 : (int64_t)im::greedy_query_bytes(q.graph->n));
 }
 
 // Estimated RRR members of a request (theta x members per set seen so far).
