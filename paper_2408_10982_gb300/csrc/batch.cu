@@ -43,6 +43,11 @@ struct im_batch {
 namespace im {
 namespace {
 
+// Vertices of a query's graph at most.  No kernel of the batch needs the limit (one
+// that kept its bounds in shared memory did); callers that meet it have the
+// one-query path, and it is known before any work is done.
+constexpr int64_t kBatchMaxN = 200 * 1024 / 8 * 1024;
+
 struct BatchQuery {
     int64_t vbase;     // first vertex of the query in the batch vertex space
     int64_t n;
@@ -239,6 +244,10 @@ im_status im_solve_batch(im_batch *b, const im_query *qs, int32_t nq, int32_t km
         set_error("im_solve_batch: the batch's vertices exceed 2^31");
         return IM_ERR_CAPACITY;
     }
+    if (n_max > kBatchMaxN) {
+        set_error("im_solve_batch: a query graph is too large for the batched greedy");
+        return IM_ERR_UNSUPPORTED;
+    }
     // batch order: IC queries, then LT queries (one sampling launch each)
     std::vector<int32_t> order(nq);
     std::iota(order.begin(), order.end(), 0);
@@ -410,11 +419,6 @@ im_status im_solve_batch(im_batch *b, const im_query *qs, int32_t nq, int32_t km
         std::vector<int64_t> hb(nq + 1);
         IM_CUDA(cudaMemcpyAsync(hb.data(), d_bounds, (size_t)(nq + 1) * 8, cudaMemcpyDeviceToHost, st));
         IM_CUDA(cudaStreamSynchronize(st));
-        // (a batch takes graphs of at most this many vertices)
-        if ((n_max + 1023) / 1024 * 8 > 200 * 1024) {
-            set_error("im_solve_batch: a query graph is too large for the batched greedy");
-            return IM_ERR_UNSUPPORTED;
-        }
         int *d_gstatus = (int *)(A + o_gbar);
         IM_CUDA(cudaMemsetAsync(d_gstatus, 0, sizeof(int), st));
         std::vector<GreedyQuery> gq;
