@@ -201,20 +201,25 @@ im_status im_randgreedi_details(const im_pool *p, int32_t *P_out, int32_t *B_out
 /* Algorithmic bytes of all sampling into this pool so far -- the bytes a
  * sampler must move, by this formula (visited-set and queue traffic is
  * on-chip and not counted):
- *   IC: per member 16 (its in-CSR offset pair) + 4 (member write),
- *       per examined edge 8 (source id + weight), per set 8 (offset);
+ *   IC: per member 16 (its vertex record) + 4 (member write), per examined
+ *       edge 8 (source id + weight), per set 8 (offset).  The kernels read
+ *       less: no weights where all in-edges of a vertex weigh the same, and
+ *       the sources of live edges only (a few in a hundred of the edges, or
+ *       in ten thousand under weighted cascade), so that this count is not
+ *       their traffic;
  *   LT, one walk per thread (the default): per set 8 (offset) + 4 (root
- *       write); per step 16 (the vertex record), + 16 (one cut point) when the
- *       in-degree is > 0; when the draw lies past the cut point's edge, 8 per
- *       binary-search probe actually made + 8 (the picked leaf); 4 per member
- *       added.
+ *       write); per step 16 (the vertex record); at a vertex whose in-edges
+ *       weigh the same, 4 (the source) when one is picked; at any other with
+ *       in-edges, 16 (one cut point), and when the draw lies past the cut
+ *       point's edge, 8 per search probe actually made + 8 (the picked leaf);
+ *       4 per member added.
  *   LT, G lanes per walk: per walk step at a vertex of in-degree d: 16
  *       (offset pair) + 8 (floor(log2 d) + 1) when d > 0 (search of the
  *       cumulative weights) + 4 when an edge is picked (its source) + 4
  *       (member write), per set 8 (offset).
- * These are the bytes the kernels' own loads need, not a linear scan of the
- * in-edges the examined-edge count covers (the LT pick reads one cut point,
- * not the e + 1 edges it decides over). */
+ * Under LT these are the bytes the kernels' own loads need, not a linear scan
+ * of the in-edges the examined-edge count covers (the pick reads one source or
+ * cut point, not the e + 1 edges it decides over). */
 im_status im_pool_sample_bytes(const im_pool *p, int64_t *bytes);
 
 /* ---- tuning knobs (process-wide; results never depend on them) ---------------
@@ -240,9 +245,10 @@ im_status im_pool_sample_bytes(const im_pool *p, int64_t *bytes);
  *   IM_TUNE_INDEX_REPLICAS  covering-subset build: 0 (default) a stable radix
  *                       sort of the (vertex, set id) pairs by vertex, up to 10
  *                       bits a pass, with 0, 8 or 12 bytes of pool scratch per
- *                       member (1, 2 or 3 passes; set ids come out ascending
- *                       inside every S(v); without the memory, the counting
- *                       build with 4 replicas runs instead); 1, 2, 4 or 8: a counting build, histogram
+ *                       member (1, 2 or 3 passes) and up to 1.5 for the digit
+ *                       tables (set ids come out ascending inside every S(v);
+ *                       without the memory, the counting build with 4 replicas
+ *                       runs instead); 1, 2, 4 or 8: a counting build, histogram
  *                       and scatter through per-vertex counters and cursors
  *                       replicated that many times (a member's replica
  *                       follows its position), spreading the atomics on hub

@@ -6,7 +6,8 @@
 // is a grid-wide argmax over the marginal gains counts[v] (packed as
 // gain << 32 | ~v so that ties go to the smallest id), a grid barrier, the
 // cover of S(v*) (atomicOr on a theta-bit bitmap; every newly covered set
-// decrements the gains of its members), and a second barrier.  Barriers wait
+// decrements the gains of its members), and a second barrier (a third after
+// sets that were cut into pieces).  Barriers wait
 // at most kWaitLimitNs and then report IM_ERR_TIMEOUT.
 //
 // RandGreedi: the paper's m sender machines are m "producer" blocks, each
@@ -172,7 +173,8 @@ constexpr int kHubShift = 6;            // hubs: |S(v)| >= max |S(v)| / 64
 // Standard greedy (Sec. 3.2), all k steps in one cooperative launch: a step
 // takes the argmax of the gains (packed gain << 32 | ~v: ties to the smallest
 // id), covers S(v*) on the theta-bit bitmap and decrements the gain of every
-// member of every newly covered set; two grid barriers per step.
+// member of every newly covered set; two grid barriers per step, three where it
+// put pieces of long sets aside.
 //
 // On graphs with hubs most decrements land on a few vertices, and atomics on
 // one address serialise in its L2 slice: with hub rows, a hub's gain is the
@@ -188,7 +190,7 @@ constexpr int kHubShift = 6;            // hubs: |S(v)| >= max |S(v)| / 64
 // A warp's first chunk of S(v*) goes by its number, consecutive chunks to
 // different SMs, the others by a per-step counter.  The argmax meets in one word
 // (an atomic per block, no second pass over block results).  Every wait is
-// bounded (grid_sync).  A step is two barriers and the dependent loads between
+// bounded (grid_sync).  A step is its barriers and the dependent loads between
 // them and the decrements.
 struct GreedyShared {
     unsigned long long best[2][32];
@@ -1980,7 +1982,9 @@ im_status randgreedi(im_pool *p, int32_t k, const im_cover_opts *o, int32_t *d_s
             IM_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_rg_stream_masks,
                                                                   kRGThreads, 0));
             if (per < 1) return IM_ERR_UNSUPPORTED;
-            const int grid = std::min(per, 2) * num_sms();
+            // one block an SM: 128 registers a thread fit no second (at 64, two
+            // blocks measured 2.07 ms against 2.03)
+            const int grid = num_sms();
             void *args[] = {&a};
             KernelTimer kt(st, "randgreedi_stream");
             IM_CUDA(cudaLaunchCooperativeKernel((const void *)k_rg_stream_masks, dim3(grid),

@@ -15,7 +15,8 @@ namespace {
 
 // Scratch of every im_max_k_cover_noalloc call on a device, 256-byte aligned:
 //   [0, 256)                 grid barrier and device status word
-//   [256, 256 + 8 * 4096)    per-block maxima (at most 4096 blocks)
+//   [256, 256 + 8 * 4096)    the rounds' best keys, three of these words (the others are
+//                            kept free, as what fits the array is part of the interface)
 //   then counts int32[n], then the covered bitmap uint32[ceil(theta / 32)].
 constexpr size_t kNoAllocScratchBytes = (size_t)64 << 20;   // 64 MiB
 constexpr int kNoAllocMaxGrid = 4096;

@@ -1918,7 +1918,7 @@ __global__ void __launch_bounds__(256, 5) k_sort_small(Key *dst, const int64_t *
 
 // One warp per listed segment longer than kLaneSort keys (grid-stride over
 // the list): sorted in registers or in the warp's shared buffer; segments
-// longer than that buffer are copied into place and listed in `big`.
+// longer than that buffer are listed in `big`.
 template <typename Key>
 __global__ void __launch_bounds__(256, 5) k_sort_mid(Key *dst, const int64_t *seg_off,
                                                   const Key *stage, const int64_t *stage_off,
